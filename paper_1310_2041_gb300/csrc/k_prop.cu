@@ -132,8 +132,9 @@ __device__ __forceinline__ int box_row(int lx, int ly, int lz, int o) {
 // ------------------------------------------------------------------ tcgen05 data gradients
 //
 // The data-gradient convolutions of training (a convolution of the back-
-// propagated gradient with flipped, transposed weights, no bias, FP32 out) on
-// the fifth-generation tensor cores.  A CTA (one warpgroup) works on tiles of
+// propagated gradient with flipped, transposed weights, no bias), multiplied by
+// the SiLU derivative of the layer below in the epilogue, on the
+// fifth-generation tensor cores.  A CTA (one warpgroup) works on tiles of
 // 8 x 16 x 4 voxels of the plain channels-last layout [V][16]; a
 // z-plane of a tile is 128 voxels = the 128 rows of one MMA (eight
 // x-consecutive voxels per 8-row core-matrix group, one group per y row).
@@ -274,13 +275,32 @@ __device__ __forceinline__ void tc_zero_cols16(uint32_t taddr) {
         : "memory");
 }
 
+// g SiLU'(z).
+__device__ __forceinline__ float silu_backward(float g, float z) {
+    const float s = 1.0f / (1.0f + expf(-z));
+    return g * s * (1.0f + z * (1.0f - s));
+}
+
 // Epilogue of one output plane: the warp's 32 accumulator rows (lanes 32w ..)
-// from columns col .. col + 15, voxel (x0 + row % 8, y0 + row / 8, z), FP32.
+// from columns col .. col + 15, voxel (x0 + row % 8, y0 + row / 8, z): the
+// gradient of the layer input through the SiLU of the layer below (its FP32
+// pre-activations z_in [V][16]), in BF16 for the next tensor-core passes.
+// Multiplying here instead of in an elementwise pass keeps the FP32 gradient
+// out of memory (44 MB written and read back per layer at 70^3).
 __device__ __forceinline__ void tc_epilogue(uint32_t tcol, const PropGeom& g, int x0, int y0,
-                                            int z, float* __restrict__ f_out) {
+                                            int z, const float* __restrict__ z_in,
+                                            __nv_bfloat16* __restrict__ gz_out) {
     const int lane = threadIdx.x & 31, w = (threadIdx.x >> 5) & 3;  // lane quarter
     const uint32_t taddr = tcol + ((uint32_t)(32 * w) << 16);
-    float acc[16];
+    const int row = 32 * w + lane;
+    const int X = x0 + (row & 7), Y = y0 + (row >> 3);
+    const bool valid = X < g.mx && Y < g.my && z < g.mz;
+    const size_t gv = ((size_t)z * g.my + Y) * g.mx + X;
+    float4 zz[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        zz[q] = valid ? __ldg(reinterpret_cast<const float4*>(z_in + gv * kPC) + q)
+                      : make_float4(0.f, 0.f, 0.f, 0.f);
     uint32_t r[16];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, "
@@ -290,25 +310,32 @@ __device__ __forceinline__ void tc_epilogue(uint32_t tcol, const PropGeom& g, in
           "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    if (!valid) return;
+    uint4* o = reinterpret_cast<uint4*>(gz_out + gv * kPC);
 #pragma unroll
-    for (int c = 0; c < 16; ++c) acc[c] = __uint_as_float(r[c]);
-    const int row = 32 * w + lane;
-    const int X = x0 + (row & 7), Y = y0 + (row >> 3);
-    if (X >= g.mx || Y >= g.my || z >= g.mz) return;
-    const size_t gv = ((size_t)z * g.my + Y) * g.mx + X;
-    float4* fo = reinterpret_cast<float4*>(f_out + gv * kPC);
+    for (int h = 0; h < 2; ++h) {
+        __nv_bfloat162 v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-        fo[q] = make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+        for (int q = 0; q < 2; ++q) {
+            const float4 zq = zz[2 * h + q];
+            const uint32_t* a = r + 8 * h + 4 * q;
+            v[2 * q] = __floats2bfloat162_rn(silu_backward(__uint_as_float(a[0]), zq.x),
+                                             silu_backward(__uint_as_float(a[1]), zq.y));
+            v[2 * q + 1] = __floats2bfloat162_rn(silu_backward(__uint_as_float(a[2]), zq.z),
+                                                 silu_backward(__uint_as_float(a[3]), zq.w));
+        }
+        o[h] = *reinterpret_cast<uint4*>(v);
+    }
 }
 
-// Wp: a packed weight image (k_pack_tc_image) of the data-gradient weights
+// Wp: a packed weight image (k_pack_images) of the data-gradient weights
 // [27][16 out][16 in], offset index 9 dz_index + in-plane offset (dy, dx);
 // K = 16 input channels of the plain layout [V][16].
 template <int kBuf>
 __global__ void __launch_bounds__(kTcThreads, kBuf == 1 ? 4 : 1)
     k_conv_tc(const __nv_bfloat16* __restrict__ in, const uint4* __restrict__ Wp,
-              float* __restrict__ f_out, PropGeom g, int n_tiles, int* __restrict__ flag) {
+              const float* __restrict__ z_in, __nv_bfloat16* __restrict__ gz_out, PropGeom g,
+              int n_tiles, int* __restrict__ flag) {
     constexpr int kRows = kTcRows16, kIP = kTcInPlane;
     extern __shared__ __align__(128) uint4 tc_smem[];
     uint4* boxp = tc_smem;                    // [buffer][channel half][kTcBox]
@@ -330,7 +357,9 @@ __global__ void __launch_bounds__(kTcThreads, kBuf == 1 ? 4 : 1)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&bar[2])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // B, pre-packed in its shared-memory layout (tc_pack_weights): one bulk
+    griddep_wait();
+    griddep_launch_dependents();
+    // B, pre-packed in its shared-memory layout (k_pack_images): one bulk
     // copy from one of kTcWCopies replicas of the image in global memory
     constexpr uint32_t kWBytes = (uint32_t)sizeof(uint4) * 2 * kIP * kRows;
     if (tid == 0) {
@@ -449,7 +478,8 @@ __global__ void __launch_bounds__(kTcThreads, kBuf == 1 ? 4 : 1)
             const uint32_t accp = tmem + (uint32_t)(kTcCols * (b ^ 1));
 #pragma unroll 1
             for (int p = 2 * (w >> 2); p < 2 * (w >> 2) + 2; ++p)
-                tc_epilogue(accp + (uint32_t)(16 * (kTcZ - 1 - p)), g, px0, py0, pz0 + p, f_out);
+                tc_epilogue(accp + (uint32_t)(16 * (kTcZ - 1 - p)), g, px0, py0, pz0 + p, z_in,
+                            gz_out);
         }
         px0 = x0;
         py0 = y0;
@@ -466,7 +496,8 @@ __global__ void __launch_bounds__(kTcThreads, kBuf == 1 ? 4 : 1)
             const uint32_t accp = tmem + (uint32_t)(kTcCols * pb);
 #pragma unroll 1
             for (int p = 2 * (w >> 2); p < 2 * (w >> 2) + 2; ++p)
-                tc_epilogue(accp + (uint32_t)(16 * (kTcZ - 1 - p)), g, px0, py0, pz0 + p, f_out);
+                tc_epilogue(accp + (uint32_t)(16 * (kTcZ - 1 - p)), g, px0, py0, pz0 + p, z_in,
+                            gz_out);
         }
     }
     if (failed) {
@@ -501,30 +532,14 @@ void conv_tc_setup() {
     });
 }
 
-// Data-gradient convolution of in [V][16] with weight image k of tcw into
-// f_out [V][16] FP32.
-void launch_conv_tc(const __nv_bfloat16* in, const uint4* tcw, int k, float* f_out,
-                    const PropGeom& g, int* flag, cudaStream_t s) {
+// Data-gradient convolution of in [V][16] with weight image k of tcw, through
+// the SiLU at pre-activations z_in [V][16], into gz_out [V][16] (not in).
+void launch_conv_tc(const __nv_bfloat16* in, const uint4* tcw, int k, const float* z_in,
+                    __nv_bfloat16* gz_out, const PropGeom& g, int* flag, cudaStream_t s) {
     conv_tc_setup();
     const int n = conv_tc_tiles(g);
-    k_conv_tc<1><<<n, kTcThreads, tc_smem_bytes(1), s>>>(in, tcw + tc_image_offset(k), f_out, g,
-                                                         n, flag);
-}
-
-// Weight image k in the B layout of k_conv_tc, kTcWCopies times: from the
-// padded BF16 weights W [27][16 out][16 in] (offset 9 dz_index + in-plane
-// offset), row n = dz_index 16 + out channel.
-__global__ void k_pack_tc_image(const __nv_bfloat16* __restrict__ W, int k,
-                                uint4* __restrict__ tcw) {
-    const int per = kTcImageWords, rows = kTcRows16, ip = kTcInPlane;
-    const uint4* W4 = reinterpret_cast<const uint4*>(W);
-    uint4* out = tcw + tc_image_offset(k);
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-        const int half = e / (ip * rows), rest = e % (ip * rows);
-        const int o9 = rest / rows, n = rest % rows;
-        const uint4 v = W4[(((n / 16) * ip + o9) * kPC + n % 16) * 2 + half];
-        for (int c = 0; c < kTcWCopies; ++c) out[c * per + e] = v;
-    }
+    launch_pdl(k_conv_tc<1>, dim3(n), dim3(kTcThreads), tc_smem_bytes(1), s, in,
+               tcw + tc_image_offset(k), z_in, gz_out, g, n, flag);
 }
 
 // ------------------------------------------------------------------ z-sweep convolution
@@ -609,7 +624,7 @@ struct SweepArgs {
     const float* bias;         // [16]
     float* z_out;              // hidden: pre-activations [V][16] FP32 (optional)
     __nv_bfloat16* act_out;    // hidden: SiLU output, padded layout [2][Mz + 2][PY][PX][8]
-    float* f_out;              // last: [V][16] FP32, channels 0 and 1 (optional)
+    float* f_out;              // last: [V][2] FP32 (optional)
     float* y_out;              // last: planar [2][V], times inv_scale (optional)
     float inv_scale;
     int* flag;
@@ -1148,7 +1163,7 @@ __global__ void __launch_bounds__(kSwThreads, kSwPerSM)
                                __shfl_down_sync(0xffffffffu, v[4 + c], 1);
                     if (valid) {
                         if (a.f_out)
-                            *reinterpret_cast<float2*>(a.f_out + gv * kPC) = make_float2(o[0], o[1]);
+                            *reinterpret_cast<float2*>(a.f_out + 2 * gv) = make_float2(o[0], o[1]);
                         if (a.y_out) {
                             const size_t V = (size_t)a.mx * a.my * a.mz;
                             a.y_out[gv] = o[0] * a.inv_scale;
@@ -1241,44 +1256,26 @@ void launch_conv_sweep(const CUtensorMap& tmap, const SweepArgs& a, int ctas, cu
     if (grid > 0) launch_pdl(k_conv_sweep<kL>, grid, kSwThreads, sw_smem_bytes(kL), s, tmap, a);
 }
 
-// Weight image of layer kL in the B layout of k_conv_sweep, kTcWCopies times:
-// [half][dy index][row][8 channels], row = dz index C + column, column = co
-// (first layer), dx index 16 + co (second), dx index 2 + co < 6 (last); from
-// the forward weights wf [o][co][ci] (o = 9 dz index + 3 dy index + dx index)
-// or, for the first layer, wx [3 dz index + dy index][co][K].
-__global__ void k_pack_sweep_images(const __nv_bfloat16* __restrict__ wf,
-                                    const __nv_bfloat16* __restrict__ wx, uint4* __restrict__ out) {
-    const int L = blockIdx.x;
-    const int C = sw_cols(L), RW = sw_rows(L), per = sw_image_words(L);
-    const uint4* wf4 = reinterpret_cast<const uint4*>(wf + (size_t)L * kOffsets * kPC * kPC);
-    const uint4* wx4 = reinterpret_cast<const uint4*>(wx);
-    uint4* o = out + sw_image_offset(L);
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-        const int half = e / (3 * RW), dyi = (e / RW) % 3, row = e % RW;
-        const int dzi = row / C, c = row % C;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (L == 0) {
-            v = wx4[((dzi * 3 + dyi) * kPC + c) * 2 + half];
-        } else if (L == 1) {
-            const int dxi = c / 16, co = c % 16;
-            v = wf4[((dzi * 9 + dyi * 3 + dxi) * kPC + co) * 2 + half];
-        } else if (c < 6) {
-            const int dxi = c / 2, co = c % 2;
-            v = wf4[((dzi * 9 + dyi * 3 + dxi) * kPC + co) * 2 + half];
-        }
-        for (int k = 0; k < kTcWCopies; ++k) o[k * per + e] = v;
-    }
-}
-
 // dW[o][ci][co] = sum_n in(n + d_o)[ci] gz(n)[co]: a voxel reduction on the
 // tensor cores.  Warp w owns offsets w, w + 8, w + 16 (and 24 for w < 3); a
 // CTA walks tiles grid-stride and writes its register sums to its own slice
-// part[blockIdx.x] (every entry, once); k_sum_partials adds the slices in a
-// fixed order, so the gradient is deterministic.
-__global__ void __launch_bounds__(256) k_conv_wgrad(const __nv_bfloat16* __restrict__ in,
-                                                    const __nv_bfloat16* __restrict__ gz,
-                                                    float* __restrict__ part, PropGeom g,
-                                                    ActLayout L) {
+// part[blockIdx.x] (every entry, once); k_sum_grads adds the slices in a
+// fixed order, so the gradient is deterministic.  The shared-memory matrix
+// loads bound it, so a k-step's gradient fragment is loaded once for all of
+// the warp's offsets (five loads for four offsets instead of eight), and with
+// kHalf (the two-channel last layer) only the first eight channels are
+// multiplied.  The bias gradient, the sum of gz itself, comes from the same
+// tiles in FP32: thread t sums channel half t & 1 of voxels t / 2 + 128 j,
+// into the slice's last 16 entries.
+constexpr int kGradEntries = kOffsets * kPC * kPC + kPC;  // a slice: weights, then biases
+
+template <bool kHalf>
+__global__ void __launch_bounds__(256, 2) k_conv_wgrad(const __nv_bfloat16* __restrict__ in,
+                                                       const __nv_bfloat16* __restrict__ gz,
+                                                       float* __restrict__ part, PropGeom g,
+                                                       ActLayout L) {
+    griddep_wait();
+    griddep_launch_dependents();
     __shared__ uint4 box[kBoxVox * 2];
     __shared__ uint4 gt[kTileVox * 2];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -1289,6 +1286,9 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(const __nv_bfloat16* __restr
         for (int j = 0; j < 2; ++j)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[s][j][c] = 0.f;
+    float bsum[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) bsum[c] = 0.f;
     // A = in^T (ci x voxels) by ldmatrix.trans of voxel rows: lane -> voxel
     // (lane & 7) + 8 (lane >= 16), channel half ((lane >> 3) & 1), so that
     // a0 = ci 0-7 / vox 0-7, a1 = ci 8-15 / vox 0-7, a2 = ci 0-7 / vox 8-15,
@@ -1299,6 +1299,14 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(const __nv_bfloat16* __restr
     // co 8-15, b3 = vox 8-15 / co 8-15
     const int g_vox = (lane & 7) + (((lane >> 3) & 1) << 3), g_half = lane >> 4;
     const uint32_t box_s = saddr(box), gt_s = saddr(gt);
+    int row0[4];  // box row of the lane's first voxel shifted by the warp's offset s
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        int lx, ly, lz;
+        warp_voxel(0, r_vox, lx, ly, lz);
+        row0[s] = box_row(lx, ly, lz, w + 8 * s < kOffsets ? w + 8 * s : w);
+    }
+    const bool four = w + 24 < kOffsets;
     for (int t = blockIdx.x; t < g.tiles; t += gridDim.x) {
         int x0, y0, z0;
         tile_origin(g, t, x0, y0, z0);
@@ -1315,22 +1323,33 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(const __nv_bfloat16* __restr
         }
         cp_async_wait_all();
         __syncthreads();
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const int o = w + 8 * s;
-            if (o >= kOffsets) break;
 #pragma unroll 4
-            for (int ks = 0; ks < kTileVox / 16; ++ks) {  // 16 voxels per k-step
-                int lx, ly, lz;
-                warp_voxel(ks, r_vox, lx, ly, lz);
-                uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
-                ldsm_x4_t(box_s + 16 * swz(box_row(lx, ly, lz, o), r_half), a0, a1, a2, a3);
-                ldsm_x4_t(gt_s + 16 * swz(16 * ks + g_vox, g_half), b0, b1, b2, b3);
+        for (int ks = 0; ks < kTileVox / 16; ++ks) {  // 16 voxels per k-step: two y rows
+            // k-step ks starts 2 y rows (20 box rows) further, a z-plane every fourth
+            const int step = (ks >> 2) * kBY * kBX + (ks & 3) * 2 * kBX;
+            uint32_t b0, b1, b2, b3;
+            ldsm_x4_t(gt_s + 16 * swz(16 * ks + g_vox, g_half), b0, b1, b2, b3);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                if (s == 3 && !four) break;
+                uint32_t a0, a1, a2, a3;
+                ldsm_x4_t(box_s + 16 * swz(row0[s] + step, r_half), a0, a1, a2, a3);
                 mma_bf16(acc[s][0], a0, a1, a2, a3, b0, b1);
-                mma_bf16(acc[s][1], a0, a1, a2, a3, b2, b3);
+                if (!kHalf) mma_bf16(acc[s][1], a0, a1, a2, a3, b2, b3);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kTileVox / 128; ++j) {
+            const uint4 v = gt[swz((tid >> 1) + 128 * j, tid & 1)];
+            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                bsum[2 * c] += __uint_as_float(u[c] << 16);
+                bsum[2 * c + 1] += __uint_as_float(u[c] & 0xffff0000u);
             }
         }
     }
+    float* out = part + (size_t)blockIdx.x * kGradEntries;
     const int gq = lane >> 2, q = lane & 3;
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -1341,9 +1360,22 @@ __global__ void __launch_bounds__(256) k_conv_wgrad(const __nv_bfloat16* __restr
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int ci = gq + 8 * (c >> 1), co = 8 * j + 2 * q + (c & 1);
-                part[(size_t)blockIdx.x * kOffsets * kPC * kPC + (o * kPC + ci) * kPC + co] =
-                    acc[s][j][c];
+                out[(o * kPC + ci) * kPC + co] = acc[s][j][c];
             }
+    }
+    __shared__ float rows[8][kPC];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+#pragma unroll
+        for (int m = 2; m < 32; m <<= 1) bsum[c] += __shfl_xor_sync(0xffffffffu, bsum[c], m);
+        if (lane < 2) rows[w][8 * lane + c] = bsum[c];
+    }
+    __syncthreads();
+    if (tid < kPC) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t += rows[k][tid];
+        out[kOffsets * kPC * kPC + tid] = t;
     }
 }
 
@@ -1372,9 +1404,11 @@ __device__ __forceinline__ void input_features(const float* __restrict__ x, int 
 // the padded plane; halo
 // included, each halo voxel a copy of the opposite face): out_x in the padded
 // layout of the forward convolutions [2][Mz + 2][py][px][8]; out (optional, for the
-// weight gradient): the plain four channels [V][16] at the interior voxels.
+// weight gradient): the plain four channels [V][16] at the interior voxels;
+// diff (with phi_next, for the loss): the change phi_next - phi(t) [V][2].
 __global__ void k_pack_input(const float* __restrict__ x, PropGeom g, int px, int py, float scale,
-                             __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ out_x) {
+                             __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ out_x,
+                             const float* __restrict__ phi_next, float2* __restrict__ diff) {
     // the first convolution (a programmatic launch) may start its prologue now;
     // it waits for this grid before reading what it writes
     griddep_launch_dependents();
@@ -1404,6 +1438,9 @@ __global__ void k_pack_input(const float* __restrict__ x, PropGeom g, int px, in
         uint4* o = reinterpret_cast<uint4*>(out + (size_t)(row + xi) * kPC);
         o[0] = reinterpret_cast<uint4*>(vals)[0];
         o[1] = reinterpret_cast<uint4*>(vals)[1];
+        const int v = row + xi;
+        diff[v] = make_float2(__fsub_rn(phi_next[v], f[1][2]),
+                              __fsub_rn(phi_next[(size_t)g.V + v], f[1][3]));
     }
 }
 
@@ -1420,30 +1457,28 @@ __global__ void k_rollout_shift(float* __restrict__ x, const float* __restrict__
     }
 }
 
-// Mean squared error of the network output y against scale * (phi_next -
-// phi_cur) (planar [2][V] each) and its gradient 2 (y - target) / (2V) in BF16.
-__global__ void __launch_bounds__(256) k_loss(const float* __restrict__ y,
-                                              const float* __restrict__ phi_cur,
-                                              const float* __restrict__ phi_next, int V,
-                                              float scale,
+// Mean squared error of the network output y against scale * diff, diff =
+// phi_next - phi_cur ([V][2] each), and its gradient 2 (y - target) / (2V) in
+// BF16; the loss in FP64 per thread, one partial per block.
+constexpr int kLossBlocks = 608;
+
+__global__ void __launch_bounds__(256) k_loss(const float2* __restrict__ y,
+                                              const float2* __restrict__ diff, int V, float scale,
                                               __nv_bfloat16* __restrict__ gy,
                                               double* __restrict__ loss_part) {
+    griddep_wait();
+    griddep_launch_dependents();
     __shared__ double sh[8];
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
     double l = 0.0;
-    if (v < V) {
-        __nv_bfloat16 vals[kPC];
-#pragma unroll
-        for (int c = 0; c < kPC; ++c) vals[c] = __float2bfloat16_rn(0.f);
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const size_t k = (size_t)c * V + v;
-            const float d = y[(size_t)v * kPC + c] - scale * (phi_next[k] - phi_cur[k]);
-            l += (double)d * d;
-            vals[c] = __float2bfloat16_rn(d / (float)V);
-        }
-        reinterpret_cast<uint4*>(gy + (size_t)v * kPC)[0] = reinterpret_cast<uint4*>(vals)[0];
-        reinterpret_cast<uint4*>(gy + (size_t)v * kPC)[1] = reinterpret_cast<uint4*>(vals)[1];
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
+        const float2 yv = y[v], dv = diff[v];
+        const float a = fmaf(-scale, dv.x, yv.x), b = fmaf(-scale, dv.y, yv.y);
+        l += (double)a * a;
+        l += (double)b * b;
+        const __nv_bfloat162 g2 = __floats2bfloat162_rn(a / (float)V, b / (float)V);
+        uint4* o = reinterpret_cast<uint4*>(gy + (size_t)v * kPC);
+        o[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&g2), 0u, 0u, 0u);
+        o[1] = make_uint4(0u, 0u, 0u, 0u);
     }
     for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = l;
@@ -1465,104 +1500,164 @@ __global__ void k_sum_partials(const T* __restrict__ part, int nb, int m, T* __r
     out[j] = s;
 }
 
-// gz = gh * SiLU'(z), in BF16 for the next tensor-core pass.
-__global__ void k_silu_backward(const float* __restrict__ gh, const float* __restrict__ z,
-                                long long n, __nv_bfloat16* __restrict__ gz) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float zz = z[i];
-    const float s = 1.0f / (1.0f + expf(-zz));
-    gz[i] = __float2bfloat16_rn(gh[i] * s * (1.0f + zz * (1.0f - s)));
-}
-
-// Bias gradient partials: part[block][co] = sum over the block's voxels of
-// gz(n)[co] (16 voxel rows x 16 channels per pass).
-__global__ void __launch_bounds__(256) k_bias_grad(const __nv_bfloat16* __restrict__ gz, int V,
-                                                   float* __restrict__ part) {
-    __shared__ float rows[16][kPC];
-    const int c = threadIdx.x & (kPC - 1), r = threadIdx.x >> 4;
-    float s = 0.f;
-    for (long long v = (long long)blockIdx.x * 16 + r; v < V; v += (long long)gridDim.x * 16)
-        s += __bfloat162float(gz[v * kPC + c]);
-    rows[r][c] = s;
-    __syncthreads();
-    if (threadIdx.x < kPC) {
-        float t = 0.f;
-        for (int k = 0; k < 16; ++k) t += rows[k][threadIdx.x];
-        part[blockIdx.x * kPC + threadIdx.x] = t;
-    }
-}
-
-// Packed FP32 parameters -> padded BF16 forward weights [o][co][ci], data-
-// gradient weights [o'][ci][co] (o' = the opposite offset) and FP32 biases.
-// wx: the first layer's weights for its x-im2col input, [dz_index * 3 + dy_index]
-// [co][K = (dx + 1) * 4 + ci], zeros from K = 12 on.
-__global__ void k_pack_weights(const float* __restrict__ params, __nv_bfloat16* __restrict__ wf,
-                               __nv_bfloat16* __restrict__ wb, float* __restrict__ bias,
-                               __nv_bfloat16* __restrict__ wx) {
-    const int layer = blockIdx.x;
-    const int ci_n = layer_in(layer), co_n = layer_out(layer);
-    int off = 0;
-    for (int l = 0; l < layer; ++l) off += kOffsets * layer_in(l) * layer_out(l) + layer_out(l);
-    const float* Wl = params + off;
-    const float* bl = Wl + kOffsets * ci_n * co_n;
-    __nv_bfloat16* f = wf + (size_t)layer * kOffsets * kPC * kPC;
-    __nv_bfloat16* b = wb + (size_t)layer * kOffsets * kPC * kPC;
-    for (int e = threadIdx.x; e < kOffsets * kPC * kPC; e += blockDim.x) {
-        const int o = e / (kPC * kPC), r = (e / kPC) % kPC, c = e % kPC;
-        // forward: [o][co = r][ci = c]
-        const float vf = (r < co_n && c < ci_n) ? Wl[(o * ci_n + c) * co_n + r] : 0.f;
-        f[e] = __float2bfloat16_rn(vf);
-        // data gradient: output channel = ci (r), input channel = co (c), offset flipped
-        const int of = kOffsets - 1 - o;
-        const float vb = (r < ci_n && c < co_n) ? Wl[(of * ci_n + r) * co_n + c] : 0.f;
-        b[e] = __float2bfloat16_rn(vb);
-    }
-    if (threadIdx.x < kPC) bias[layer * kPC + threadIdx.x] = threadIdx.x < co_n ? bl[threadIdx.x] : 0.f;
-    if (layer == 0) {
-        for (int e = threadIdx.x; e < 9 * kPC * kPC; e += blockDim.x) {
-            const int o = e / (kPC * kPC), co = (e / kPC) % kPC, k = e % kPC;
-            const int dzi = o / 3, dyi = o % 3, dxi = k >> 2, ci = k & 3;
-            const float v = k < 12 ? Wl[((dzi * 9 + dyi * 3 + dxi) * ci_n + ci) * co_n + co] : 0.f;
-            wx[e] = __float2bfloat16_rn(v);
-        }
-    }
-}
-
-// Padded weight / bias gradients -> packed gradient vector.
-__global__ void k_pack_grads(const float* __restrict__ dW, const float* __restrict__ db,
-                             float* __restrict__ grads) {
-    const int layer = blockIdx.x;
-    const int ci_n = layer_in(layer), co_n = layer_out(layer);
-    int off = 0;
-    for (int l = 0; l < layer; ++l) off += kOffsets * layer_in(l) * layer_out(l) + layer_out(l);
-    const float* d = dW + (size_t)layer * kOffsets * kPC * kPC;
-    for (int e = threadIdx.x; e < kOffsets * ci_n * co_n; e += blockDim.x) {
-        const int o = e / (ci_n * co_n), ci = (e / co_n) % ci_n, co = e % co_n;
-        grads[off + e] = d[(o * kPC + ci) * kPC + co];
-    }
-    if (threadIdx.x < co_n)
-        grads[off + kOffsets * ci_n * co_n + threadIdx.x] = db[layer * kPC + threadIdx.x];
+// First packed parameter of layer l.
+__host__ __device__ constexpr int param_offset(int l) {
+    return l == 0 ? 0 : param_offset(l - 1) + kOffsets * layer_in(l - 1) * layer_out(l - 1) +
+                            layer_out(l - 1);
 }
 
 // Adam (Kingma & Ba, 2015) on the FP32 master parameters.
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, int n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
+struct AdamArgs {
+    float *p, *m, *v;  // p null: no update
+    float lr, c1, c2;  // c1, c2: the bias corrections 1 - b^t
+};
+
+__device__ __forceinline__ void adam_update(const AdamArgs& a, int i, float g) {
+    constexpr float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    const float mi = b1 * a.m[i] + (1.f - b1) * g;
+    const float vi = b2 * a.v[i] + (1.f - b2) * g * g;
+    a.m[i] = mi;
+    a.v[i] = vi;
+    a.p[i] -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + eps);
+}
+
+__global__ void k_adam(const AdamArgs a, const float* __restrict__ g, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    if (i < n) adam_update(a, i, g[i]);
+}
+
+// The weight gradients' slices added up: block (x, layer) takes 32 consecutive
+// entries of that layer, eight threads per entry each adding every eighth
+// slice (nb of them), then the eight sums in order -- a fixed order, with every load
+// of a thread in flight together instead of one thread walking all slices.
+// The packed gradient goes to grads and, with adam.p, straight into the Adam
+// update.  One more block adds the loss partials.
+constexpr int kSumEntries = 32;
+constexpr int kSumBlocks = (kGradEntries + kSumEntries - 1) / kSumEntries;
+
+__global__ void __launch_bounds__(256) k_sum_grads(const float* __restrict__ part, int nb,
+                                                   float* __restrict__ grads, const AdamArgs adam,
+                                                   const double* __restrict__ loss_part, int nl,
+                                                   double* __restrict__ loss) {
+    griddep_wait();
+    griddep_launch_dependents();
+    const int tid = threadIdx.x, layer = blockIdx.y;
+    if (blockIdx.x == kSumBlocks) {
+        if (layer != 0) return;
+        __shared__ double shd[8];
+        double l = 0.0;
+        for (int k = tid; k < nl; k += 256) l += loss_part[k];
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
+        if ((tid & 31) == 0) shd[tid >> 5] = l;
+        __syncthreads();
+        if (tid == 0) {
+            double t = 0.0;
+            for (int k = 0; k < 8; ++k) t += shd[k];
+            *loss = t;
+        }
+        return;
+    }
+    __shared__ float sh[8][kSumEntries];
+    const int e = blockIdx.x * kSumEntries + (tid & 31), slice = tid >> 5;
+    // entry e: offset o, input channel ci, output channel co; the biases follow the weights
+    const int ci_n = layer_in(layer), co_n = layer_out(layer);
+    const bool bias = e >= kOffsets * kPC * kPC;
+    const int o = e / (kPC * kPC), ci = (e / kPC) % kPC, co = e % kPC;
+    const bool valid = e < kGradEntries && co < co_n && (bias || ci < ci_n);
+    float s = 0.f;
+    if (valid) {
+        const float* p = part + (size_t)layer * nb * kGradEntries + e;
+#pragma unroll 8
+        for (int b = slice; b < nb; b += 8) s += p[(size_t)b * kGradEntries];
+    }
+    sh[slice][tid & 31] = s;
+    __syncthreads();
+    if (slice != 0 || !valid) return;
+    s = sh[0][tid];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) s += sh[k][tid];
+    const int j = (layer == 0 ? param_offset(0) : (layer == 1 ? param_offset(1) : param_offset(2))) +
+                  (bias ? kOffsets * ci_n * co_n + co : (o * ci_n + ci) * co_n + co);
+    grads[j] = s;
+    if (adam.p) adam_update(adam, j, s);
+}
+
+// The tensor-core weight images and the padded biases from the FP32
+// parameters, kTcWCopies replicas each, one thread per 16-byte word (eight
+// channels of one row).  Forward images (k_conv_sweep), layer L:
+// [half][dy index][row], row = dz index C + column, column = co (first layer,
+// K index (dx + 1) 4 + ci of its x-im2col input, zeros from 12 on), dx index 16 + co
+// (second), dx index 2 + co < 6 (last).  Data-gradient images (k_conv_tc),
+// layer L = 1, 2: [half][in-plane offset][dz index 16 + input channel], the
+// kernel offset flipped and the channels transposed.
+constexpr int kSweepWords = sw_image_words(0) + sw_image_words(1) + sw_image_words(2);
+constexpr int kPackWords = kSweepWords + kTcImages * kTcImageWords;
+
+__global__ void k_pack_images(const float* __restrict__ params, uint4* __restrict__ sww,
+                              uint4* __restrict__ tcw, float* __restrict__ bias) {
+    griddep_wait();
+    griddep_launch_dependents();
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 3 * kPC) {
+        const int L = t / kPC, c = t % kPC, co_n = layer_out(L);
+        const float* Wl = params + (L == 0 ? param_offset(0) : (L == 1 ? param_offset(1) : param_offset(2)));
+        bias[t] = c < co_n ? Wl[kOffsets * layer_in(L) * co_n + c] : 0.f;
+    }
+    if (t >= kPackWords) return;
+    // which image, which word of it
+    const bool fwd = t < kSweepWords;
+    int L = 0, e = t;
+    if (fwd) {
+        while (e >= sw_image_words(L)) e -= sw_image_words(L++);
+    } else {
+        e -= kSweepWords;
+        L = 1 + e / kTcImageWords;
+        e %= kTcImageWords;
+    }
+    const int ci_n = layer_in(L), co_n = layer_out(L);
+    const float* Wl = params + (L == 0 ? param_offset(0) : (L == 1 ? param_offset(1) : param_offset(2)));
+    float v[8];
+    uint4* out;
+    int per;
+    if (fwd) {
+        const int C = sw_cols(L), RW = sw_rows(L);
+        const int half = e / (3 * RW), dyi = (e / RW) % 3, row = e % RW;
+        const int dzi = row / C, c = row % C;
+        const int cols = L == 1 ? 16 : 2;  // columns per dx block
+        const int co = L == 0 ? c : c % cols;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int k = 8 * half + j;
+            const int dxi = L == 0 ? k >> 2 : c / cols, ci = L == 0 ? k & 3 : k;
+            const bool on = dxi < 3 && ci < ci_n && co < co_n;
+            v[j] = on ? Wl[((dzi * 9 + dyi * 3 + dxi) * ci_n + ci) * co_n + co] : 0.f;
+        }
+        out = sww + (L == 0 ? sw_image_offset(0) : (L == 1 ? sw_image_offset(1) : sw_image_offset(2))) + e;
+        per = sw_image_words(L);
+    } else {
+        const int half = e / (kTcInPlane * kTcRows16), rest = e % (kTcInPlane * kTcRows16);
+        const int o9 = rest / kTcRows16, n = rest % kTcRows16;
+        const int o = (n / 16) * kTcInPlane + o9, ci = n % 16;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int co = 8 * half + j;
+            const bool on = ci < ci_n && co < co_n;
+            v[j] = on ? Wl[((kOffsets - 1 - o) * ci_n + ci) * co_n + co] : 0.f;
+        }
+        out = tcw + tc_image_offset(L - 1) + e;
+        per = kTcImageWords;
+    }
+    __nv_bfloat162 h[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+    const uint4 w = *reinterpret_cast<uint4*>(h);
+#pragma unroll
+    for (int k = 0; k < kTcWCopies; ++k) out[k * per] = w;
 }
 
 // ------------------------------------------------------------------ learned-step mesh kernels
 
 constexpr int kErrBlocks = 1216;  // blocks of the force-error reduction (8 per SM)
-constexpr int kBiasBlocks = 152;
 
 // phi_K(n) = D_K(n) phi_c: the volume fractions of an int64 fixed-point mesh.
 __global__ void k_mesh_to_phi(const unsigned long long* __restrict__ D, long long n, double phi_c,
@@ -1710,27 +1805,22 @@ struct hpf_prop {
     float* adam_m = nullptr;
     float* adam_v = nullptr;
     int adam_t = 0;
-    __nv_bfloat16* wf = nullptr;  // [3][27][16][16]
-    __nv_bfloat16* wb = nullptr;
     float* bias = nullptr;        // [3][16]
-    float* dW = nullptr;          // [3][27][16][16]
-    float* db = nullptr;          // [3][16]
-    float* wpart = nullptr;       // weight-gradient partials [grid_wgrad][27][16][16]
-    float* bpart = nullptr;       // bias-gradient partials [152][16]
-    double* lpart = nullptr;      // loss partials [ceil(V / 256)]
+    float* wpart = nullptr;       // gradient slices [3][grid_wgrad][kGradEntries]
+    double* lpart = nullptr;      // loss partials [kLossBlocks]
     // act[0]: the plain input [V][16] (training only); act[1], act[2]: the
-    // hidden activations in the padded layout [2][Mz + 2][py][px][8]; act[3]:
-    // a gradient buffer [V][16]
-    __nv_bfloat16* act[4] = {};
+    // hidden activations in the padded layout [2][Mz + 2][py][px][8]; act[3],
+    // act[4]: gradient buffers [V][16]
+    __nv_bfloat16* act[5] = {};
     __nv_bfloat16* act_x = nullptr;  // the input as x-im2col, padded layout
-    __nv_bfloat16* wx = nullptr;     // first-layer weights for it [9][16][16]
     uint4* tcw = nullptr;            // packed weight images of the data-gradient convolutions
     uint4* sww = nullptr;            // packed weight images of the forward convolutions
     CUtensorMap tmap[3];             // act_x, act[1], act[2]
     int px = 0, py = 0;              // padded pitches
     int ctas = 1;                    // CTAs of the persistent convolutions (kSwPerSM per SM)
     float* z[2] = {};             // pre-activations of layers 1, 2 [V][16]
-    float* fbuf = nullptr;        // FP32 [V][16]: output / data gradient
+    float* fbuf = nullptr;        // FP32 output [V][2]
+    float2* diff = nullptr;       // the change to learn [V][2]
     float* xin = nullptr;         // staging of the planar input [4][V]
     float* tin = nullptr;         // staging of the planar next densities [2][V]
     float* yout = nullptr;        // planar output [2][V]
@@ -1757,14 +1847,10 @@ hpf_status prop_copy_out(hpf_prop* p, void* dst, const void* src, size_t bytes) 
     return HPF_OK;
 }
 
-// The padded BF16 weights, biases and the tensor-core weight images from the
-// FP32 parameters.
+// The biases and the tensor-core weight images from the FP32 parameters.
 void pack_all_weights(hpf_prop* p, cudaStream_t s) {
-    const size_t wl = (size_t)kOffsets * kPC * kPC;
-    k_pack_weights<<<3, 256, 0, s>>>(p->params, p->wf, p->wb, p->bias, p->wx);
-    k_pack_sweep_images<<<3, 256, 0, s>>>(p->wf, p->wx, p->sww);
-    k_pack_tc_image<<<1, 256, 0, s>>>(p->wb + wl, 0, p->tcw);
-    k_pack_tc_image<<<1, 256, 0, s>>>(p->wb + 2 * wl, 1, p->tcw);
+    launch_pdl(k_pack_images, dim3((kPackWords + 127) / 128), dim3(128), 0, s,
+               (const float*)p->params, p->sww, p->tcw, p->bias);
 }
 
 SweepArgs sweep_args(const hpf_prop* p, int layer, int* flag) {
@@ -1783,66 +1869,61 @@ SweepArgs sweep_args(const hpf_prop* p, int layer, int* flag) {
     return a;
 }
 
-// Forward pass of planar input x [4][V] (device).  keep_z: the pre-activations
-// and the plain input are stored and the FP32 output goes to fbuf [V][16] for
-// a backward pass; y_planar (optional): the predicted change [2][V] (the
-// output divided by scale).
-void prop_forward(hpf_prop* p, const float* x, bool keep_z, cudaStream_t s, int* flag,
+// Forward pass of planar input x [4][V] (device).  With phi_next (training):
+// the pre-activations, the plain input and the change phi_next - x[2:4] are
+// stored and the FP32 output goes to fbuf [V][2] for a backward pass (the
+// first kernel alone reads x and phi_next); y_planar (optional): the
+// predicted change [2][V] (the output divided by scale).
+void prop_forward(hpf_prop* p, const float* x, const float* phi_next, cudaStream_t s, int* flag,
                   float* y_planar = nullptr) {
+    const bool train = phi_next != nullptr;
     const int hp = (p->g.mx + 2) * (p->g.my + 2);  // padded voxels per plane
     k_pack_input<<<dim3((unsigned)((hp + 255) / 256), (unsigned)(p->g.mz + 2)), 256, 0, s>>>(
-        x, p->g, p->px, p->py, p->scale, keep_z ? p->act[0] : nullptr, p->act_x);
+        x, p->g, p->px, p->py, p->scale, train ? p->act[0] : nullptr, p->act_x, phi_next, p->diff);
     SweepArgs a = sweep_args(p, 0, flag);
-    a.z_out = keep_z ? p->z[0] : nullptr;
+    a.z_out = train ? p->z[0] : nullptr;
     a.act_out = p->act[1];
     launch_conv_sweep<0>(p->tmap[0], a, p->ctas, s);
     a = sweep_args(p, 1, flag);
-    a.z_out = keep_z ? p->z[1] : nullptr;
+    a.z_out = train ? p->z[1] : nullptr;
     a.act_out = p->act[2];
     launch_conv_sweep<1>(p->tmap[1], a, p->ctas, s);
     a = sweep_args(p, 2, flag);
-    a.f_out = keep_z ? p->fbuf : nullptr;
+    a.f_out = train ? p->fbuf : nullptr;
     a.y_out = y_planar;
     launch_conv_sweep<2>(p->tmap[2], a, p->ctas, s);
 }
 
-// Loss and packed gradients (p->grads, p->loss) after prop_forward(keep_z) of
-// x; the target is phi_next - x[2:4].
-void prop_backward(hpf_prop* p, const float* x, const float* phi_next) {
-    const int V = p->g.V, tb = (V + 255) / 256;
-    const long long nv = (long long)V * kPC;
-    const size_t wl = (size_t)kOffsets * kPC * kPC;
+// Loss and packed gradients (p->grads, p->loss) after a training forward
+// pass, and with adam.p the parameter update.
+void prop_backward(hpf_prop* p, const AdamArgs& adam) {
+    const int V = p->g.V, nb = p->grid_wgrad;
+    const int lb = (V + 255) / 256 < kLossBlocks ? (V + 255) / 256 : kLossBlocks;
     cudaStream_t s = p->stream;
-    __nv_bfloat16* gbuf = p->act[3];
+    const ActLayout plain{p->g.mx, p->g.my, 0, kPC, 8};
+    const ActLayout padded{p->px, p->py, 1, 8, 8ll * (p->g.mz + 2) * p->py * p->px};
+    const size_t slices = (size_t)nb * kGradEntries;
     // the last layer has no activation: its gz is dL/dy
-    k_loss<<<tb, 256, 0, s>>>(p->fbuf, x + 2 * (size_t)V, phi_next, V, p->scale, gbuf, p->lpart);
-    k_sum_partials<double><<<1, 32, 0, s>>>(p->lpart, tb, 1, p->loss);
-    for (int layer = 2; layer >= 0; --layer) {
-        const ActLayout lay =
-            layer == 0 ? ActLayout{p->g.mx, p->g.my, 0, kPC, 8}
-                       : ActLayout{p->px, p->py, 1, 8, 8ll * (p->g.mz + 2) * p->py * p->px};
-        k_conv_wgrad<<<p->grid_wgrad, 256, 0, s>>>(p->act[layer], gbuf, p->wpart, p->g, lay);
-        k_sum_partials<float><<<(unsigned)((wl + 255) / 256), 256, 0, s>>>(
-            p->wpart, p->grid_wgrad, (int)wl, p->dW + layer * wl);
-        k_bias_grad<<<kBiasBlocks, 256, 0, s>>>(gbuf, V, p->bpart);
-        k_sum_partials<float><<<1, 32, 0, s>>>(p->bpart, kBiasBlocks, kPC, p->db + layer * kPC);
-        if (layer == 0) break;
-        // the data gradient of the layer input, then through the SiLU below it
-        launch_conv_tc(gbuf, p->tcw, layer - 1, p->fbuf, p->g, p->flag, s);
-        k_silu_backward<<<(unsigned)((nv + 255) / 256), 256, 0, s>>>(p->fbuf, p->z[layer - 1], nv,
-                                                                      gbuf);
-    }
-    k_pack_grads<<<3, 256, 0, s>>>(p->dW, p->db, p->grads);
+    launch_pdl(k_loss, dim3(lb), dim3(256), 0, s, (const float2*)p->fbuf, (const float2*)p->diff, V,
+               p->scale, p->act[3], p->lpart);
+    launch_pdl(k_conv_wgrad<true>, dim3(nb), dim3(256), 0, s, (const __nv_bfloat16*)p->act[2],
+               (const __nv_bfloat16*)p->act[3], p->wpart + 2 * slices, p->g, padded);
+    launch_conv_tc(p->act[3], p->tcw, 1, p->z[1], p->act[4], p->g, p->flag, s);
+    launch_pdl(k_conv_wgrad<false>, dim3(nb), dim3(256), 0, s, (const __nv_bfloat16*)p->act[1],
+               (const __nv_bfloat16*)p->act[4], p->wpart + slices, p->g, padded);
+    launch_conv_tc(p->act[4], p->tcw, 0, p->z[0], p->act[3], p->g, p->flag, s);
+    launch_pdl(k_conv_wgrad<false>, dim3(nb), dim3(256), 0, s, (const __nv_bfloat16*)p->act[0],
+               (const __nv_bfloat16*)p->act[3], p->wpart, p->g, plain);
+    launch_pdl(k_sum_grads, dim3(kSumBlocks + 1, 3), dim3(256), 0, s, (const float*)p->wpart, nb,
+               p->grads, adam, (const double*)p->lpart, lb, p->loss);
 }
 
-void prop_adam(hpf_prop* p, const float* grads, float lr) {
+// The next Adam step's arguments.
+AdamArgs adam_args(hpf_prop* p, float lr) {
     p->adam_t += 1;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = (float)(1.0 - pow(0.9, (double)p->adam_t));
-    const float c2 = (float)(1.0 - pow(0.999, (double)p->adam_t));
-    k_adam<<<(p->np + 255) / 256, 256, 0, p->stream>>>(p->params, grads, p->adam_m, p->adam_v,
-                                                      p->np, lr, b1, b2, 1e-8f, c1, c2);
-    pack_all_weights(p, p->stream);
+    return AdamArgs{p->params, p->adam_m, p->adam_v, lr,
+                    (float)(1.0 - pow(0.9, (double)p->adam_t)),
+                    (float)(1.0 - pow(0.999, (double)p->adam_t))};
 }
 
 // Planar inputs are staged into library buffers (host or device sources).
@@ -1915,7 +1996,7 @@ bool prop_mesh_is(const hpf_prop* p, const MeshGeom& g) {
 }
 
 void prop_predict(hpf_prop* p, const float* x, float* dphi, cudaStream_t s, int* flag) {
-    prop_forward(p, x, false, s, flag ? flag : p->flag, dphi);
+    prop_forward(p, x, nullptr, s, flag ? flag : p->flag, dphi);
 }
 
 }  // namespace hpf
@@ -1952,24 +2033,20 @@ hpf_status hpf_prop_init(const int32_t mesh[3], void* stream, hpf_prop** out) {
     p->ctas = kSwPerSM * sms;
     sweep_pitches(g, p->px, p->py);
     const size_t Vp = (size_t)(g.mz + 2) * p->py * p->px;  // padded voxels
-    const size_t wl = (size_t)kOffsets * kPC * kPC, Vs = (size_t)g.V;
+    const size_t Vs = (size_t)g.V;
     cudaError_t e = cudaSuccess;
     e = e ? e : cudaMalloc(&p->params, sizeof(float) * p->np);
     e = e ? e : cudaMalloc(&p->grads, sizeof(float) * p->np);
     e = e ? e : cudaMalloc(&p->adam_m, sizeof(float) * p->np);
     e = e ? e : cudaMalloc(&p->adam_v, sizeof(float) * p->np);
-    e = e ? e : cudaMalloc(&p->wf, sizeof(__nv_bfloat16) * 3 * wl);
-    e = e ? e : cudaMalloc(&p->wb, sizeof(__nv_bfloat16) * 3 * wl);
     e = e ? e : cudaMalloc(&p->bias, sizeof(float) * 3 * kPC);
-    e = e ? e : cudaMalloc(&p->dW, sizeof(float) * 3 * wl);
-    e = e ? e : cudaMalloc(&p->db, sizeof(float) * 3 * kPC);
-    e = e ? e : cudaMalloc(&p->wpart, sizeof(float) * (size_t)p->grid_wgrad * wl);
-    e = e ? e : cudaMalloc(&p->bpart, sizeof(float) * kBiasBlocks * kPC);
-    e = e ? e : cudaMalloc(&p->lpart, sizeof(double) * ((Vs + 255) / 256));
-    for (int k = 0; k < 4; ++k)
+    e = e ? e : cudaMalloc(&p->wpart, sizeof(float) * 3 * (size_t)p->grid_wgrad * kGradEntries);
+    e = e ? e : cudaMalloc(&p->lpart, sizeof(double) * kLossBlocks);
+    for (int k = 0; k < 5; ++k)
         e = e ? e : cudaMalloc(&p->act[k], sizeof(__nv_bfloat16) * (k == 1 || k == 2 ? Vp : Vs) * kPC);
     for (int k = 0; k < 2; ++k) e = e ? e : cudaMalloc(&p->z[k], sizeof(float) * Vs * kPC);
-    e = e ? e : cudaMalloc(&p->fbuf, sizeof(float) * Vs * kPC);
+    e = e ? e : cudaMalloc(&p->fbuf, sizeof(float) * Vs * 2);
+    e = e ? e : cudaMalloc(&p->diff, sizeof(float2) * Vs);
     e = e ? e : cudaMalloc(&p->xin, sizeof(float) * Vs * 4);
     e = e ? e : cudaMalloc(&p->tin, sizeof(float) * Vs * 2);
     e = e ? e : cudaMalloc(&p->yout, sizeof(float) * Vs * 2);
@@ -1978,7 +2055,6 @@ hpf_status hpf_prop_init(const int32_t mesh[3], void* stream, hpf_prop** out) {
     e = e ? e : cudaMalloc(&p->flag, sizeof(int));
     e = e ? e : cudaMalloc(&p->act_x, sizeof(__nv_bfloat16) * Vp * kPC);
     e = e ? e : cudaMalloc(&p->sww, sizeof(uint4) * sw_image_offset(3));
-    e = e ? e : cudaMalloc(&p->wx, sizeof(__nv_bfloat16) * 9 * kPC * kPC);
     e = e ? e : cudaMalloc(&p->tcw, sizeof(uint4) * tc_image_offset(kTcImages));
     e = e ? e : cudaMallocHost(&p->h_flag, sizeof(int));
     if (e == cudaSuccess) {
@@ -2018,17 +2094,13 @@ hpf_status hpf_prop_destroy(hpf_prop* p) {
     cudaFree(p->grads);
     cudaFree(p->adam_m);
     cudaFree(p->adam_v);
-    cudaFree(p->wf);
-    cudaFree(p->wb);
     cudaFree(p->bias);
-    cudaFree(p->dW);
-    cudaFree(p->db);
     cudaFree(p->wpart);
-    cudaFree(p->bpart);
     cudaFree(p->lpart);
-    for (int k = 0; k < 4; ++k) cudaFree(p->act[k]);
+    for (int k = 0; k < 5; ++k) cudaFree(p->act[k]);
     for (int k = 0; k < 2; ++k) cudaFree(p->z[k]);
     cudaFree(p->fbuf);
+    cudaFree(p->diff);
     cudaFree(p->xin);
     cudaFree(p->tin);
     cudaFree(p->yout);
@@ -2037,7 +2109,6 @@ hpf_status hpf_prop_destroy(hpf_prop* p) {
     cudaFree(p->flag);
     cudaFreeHost(p->h_flag);
     cudaFree(p->act_x);
-    cudaFree(p->wx);
     cudaFree(p->tcw);
     cudaFree(p->sww);
     cudaGetLastError();
@@ -2146,14 +2217,31 @@ hpf_status hpf_prop_rollout(hpf_prop* p, const float* x, int32_t steps, float* p
     return dev ? HPF_OK : prop_flag_status(p);
 }
 
+// Forward and backward of x against phi_next: device arrays of the current
+// device are read in place (by the first kernel alone), host arrays go through
+// the handle's staging buffers.
+static hpf_status prop_gradients(hpf_prop* p, const float* x, const float* phi_next,
+                                 const AdamArgs& adam) {
+    hpf_status s = HPF_OK;
+    if (!prop_on_device(x)) {
+        s = prop_stage(p, p->xin, x, (size_t)p->g.V * 4);
+        x = p->xin;
+    }
+    if (s == HPF_OK && !prop_on_device(phi_next)) {
+        s = prop_stage(p, p->tin, phi_next, (size_t)p->g.V * 2);
+        phi_next = p->tin;
+    }
+    if (s != HPF_OK) return s;
+    prop_forward(p, x, phi_next, p->stream, p->flag);
+    prop_backward(p, adam);
+    return HPF_OK;
+}
+
 hpf_status hpf_prop_backward(hpf_prop* p, const float* x, const float* phi_next, float* grads,
                              double* loss) {
-    if (!p) return HPF_ERR_INVALID;
-    hpf_status s = prop_stage(p, p->xin, x, (size_t)p->g.V * 4);
-    if (s == HPF_OK) s = prop_stage(p, p->tin, phi_next, (size_t)p->g.V * 2);
+    if (!p || !x || !phi_next) return HPF_ERR_INVALID;
+    hpf_status s = prop_gradients(p, x, phi_next, AdamArgs{});
     if (s != HPF_OK) return s;
-    prop_forward(p, p->xin, true, p->stream, p->flag);
-    prop_backward(p, p->xin, p->tin);
     if ((s = prop_launched(p)) != HPF_OK) return s;
     if ((s = prop_copy_out(p, grads, p->grads, sizeof(float) * p->np)) != HPF_OK) return s;
     return prop_read_loss(p, loss);
@@ -2163,19 +2251,21 @@ hpf_status hpf_prop_adam_step(hpf_prop* p, const float* grads, float lr) {
     if (!p || !grads || !(lr > 0.f)) return HPF_ERR_INVALID;
     hpf_status s = prop_stage(p, p->grads, grads, (size_t)p->np);
     if (s != HPF_OK) return s;
-    prop_adam(p, p->grads, lr);
+    k_adam<<<(p->np + 255) / 256, 256, 0, p->stream>>>(adam_args(p, lr), p->grads, p->np);
+    pack_all_weights(p, p->stream);
     return prop_launched(p);
 }
 
 hpf_status hpf_prop_train_step(hpf_prop* p, const float* x, const float* phi_next, float lr,
                                double* loss) {
-    if (!p || !(lr > 0.f)) return HPF_ERR_INVALID;
-    hpf_status s = prop_stage(p, p->xin, x, (size_t)p->g.V * 4);
-    if (s == HPF_OK) s = prop_stage(p, p->tin, phi_next, (size_t)p->g.V * 2);
-    if (s != HPF_OK) return s;
-    prop_forward(p, p->xin, true, p->stream, p->flag);
-    prop_backward(p, p->xin, p->tin);
-    prop_adam(p, p->grads, lr);
+    if (!p || !x || !phi_next || !(lr > 0.f)) return HPF_ERR_INVALID;
+    const int t = p->adam_t;
+    hpf_status s = prop_gradients(p, x, phi_next, adam_args(p, lr));
+    if (s != HPF_OK) {
+        p->adam_t = t;  // nothing was launched
+        return s;
+    }
+    pack_all_weights(p, p->stream);
     if ((s = prop_launched(p)) != HPF_OK) return s;
     return prop_read_loss(p, loss);
 }
