@@ -58,11 +58,10 @@ struct hpf_ctx {
     CUtensorMap tmap[2];              // over mesh buffers 0 and 1
     float* out_f = nullptr;           // 2 x 3n floats of tag-order output staging
     void* stage = nullptr;            // set_state input staging
-    int* dflag = nullptr;             // [0] kernel flags, [1..4] validation counters
+    int* dflag = nullptr;             // [0] kernel flags, [1..4] validation counters, [5] ticket
     int* hflag = nullptr;             // pinned mirror
     double* partials = nullptr;
-    double* d_out6 = nullptr;
-    double* h_out6 = nullptr;         // pinned
+    double* h_out6 = nullptr;         // pinned, written by the observables' last kernel
     bool has_state = false;
     bool field_valid = false;
     long long step = 0;
@@ -97,7 +96,7 @@ struct hpf_ctx {
     bool up_ready = false;    // stream, events and both slots exist
     bool up_pending = false;
     bool energy_pending = false;  // hpf_energy_start issued, hpf_energy_finish not yet
-    cudaEvent_t energy_ev = nullptr;  // after hpf_energy_start's copies to the host
+    cudaEvent_t energy_ev = nullptr;  // after hpf_energy_start's kernels
 };
 
 // Buffers of the learned-propagator driver and the density judge.
@@ -711,9 +710,9 @@ hpf_status check_flags(hpf_ctx* c) {
     return flag_status(c, c->hflag[0]);
 }
 
-// The observables of the current step: kernels and the copies of the six
-// sums (and the Nose-Hoover state) to the context's pinned mirrors, all
-// asynchronous on the context's stream.
+// The observables of the current step: kernels, the last of which writes the
+// six sums, the error word (hflag[7]) and the Nose-Hoover state to the
+// context's pinned mirrors, all asynchronous on the context's stream.
 hpf_status energy_launch(hpf_ctx* c) {
     if (!c->has_state) return fail(c, HPF_ERR_STATE, "no state loaded");
     hpf_status s = ensure_field(c);
@@ -725,31 +724,24 @@ hpf_status energy_launch(hpf_ctx* c) {
     if ((s = scatter_current(c)) != HPF_OK) return s;
     {
         const long long* Dm = reinterpret_cast<const long long*>(mesh_buf(c, c->dmesh));
+        const EnergyOut eo{c->h_out6, c->dflag, c->hflag + 7,
+                           c->nh ? reinterpret_cast<const double*>(c->nh) : nullptr, c->h_nh};
         if (c->obs_step == c->step) {
             // the bead terms came with the step launch: node sums and combination
             StageScope sc(c, HPF_STAGE_ENERGY, 2);
             launch_energy_nodes_only(c->n, c->geom, Dm, c->ec, c->obs_part, c->obs_nb,
-                                     c->partials, c->d_out6, c->stream);
+                                     c->partials, eo, c->stream);
         } else {
             StageScope sc(c, HPF_STAGE_ENERGY, energy_launches(c->n, c->S));
             launch_energy(cur_state(c), c->meta, c->n, c->geom, c->G, c->sc, c->step, Dm, c->ec,
-                          c->partials, c->d_out6, c->stream);
+                          c->partials, eo, c->stream);
         }
     }
     LAUNCH_CHECK(c);
-    CUDA_TRY(c, cudaMemcpyAsync(c->h_out6, c->d_out6, sizeof(double) * 6, cudaMemcpyDeviceToHost,
-                                c->stream));
-    if (c->nh)
-        CUDA_TRY(c, cudaMemcpyAsync(c->h_nh, c->nh, sizeof(double) * 2, cudaMemcpyDeviceToHost,
-                                    c->stream));
-    // the error word as it stands after these kernels, for hpf_energy_finish
-    CUDA_TRY(c, cudaMemcpyAsync(c->hflag + 7, c->dflag, sizeof(int), cudaMemcpyDeviceToHost,
-                                c->stream));
-    CUDA_TRY(c, cudaEventRecord(c->energy_ev, c->stream));
     return HPF_OK;
 }
 
-// After the stream has reached energy_launch's copies: the six values.
+// After the stream has reached energy_launch's last kernel: the six values.
 void energy_finish(const hpf_ctx* c, double out[6]) {
     memcpy(out, c->h_out6, sizeof(double) * 6);
     if (c->nh) {
@@ -820,7 +812,6 @@ hpf_status hpf_init(const hpf_params* params, void* stream, hpf_ctx** out) {
     e = e ? e : cudaMalloc(&c->partials,
                            sizeof(double) * energy_partials_needed(c->n, c->geom.nodes,
                                                                    c->p.n_species));
-    e = e ? e : cudaMalloc(&c->d_out6, sizeof(double) * 8);
     e = e ? e : cudaMallocHost(&c->h_out6, sizeof(double) * 8);
     e = e ? e : cudaEventCreateWithFlags(&c->energy_ev, cudaEventDisableTiming);
     e = e ? e : cudaMalloc(&c->obs_part, sizeof(float2) * kBeadVals * step_warp_grid_cap());
@@ -895,7 +886,6 @@ hpf_status hpf_destroy(hpf_ctx* c) {
     cudaFree(c->dflag);
     cudaFreeHost(c->hflag);
     cudaFree(c->partials);
-    cudaFree(c->d_out6);
     cudaFreeHost(c->h_out6);
     if (c->energy_ev) cudaEventDestroy(c->energy_ev);
     cudaFree(c->obs_part);
@@ -1137,21 +1127,43 @@ hpf_status hpf_apply_state(hpf_ctx* c, int64_t step) {
     return HPF_OK;
 }
 
+// Whether kernels may write n floats at p in place of a copy: memory of the
+// current device, aligned.
+static bool device_floats(const void* p) {
+    cudaPointerAttributes a;
+    int dev = -1;
+    const bool ok = cudaPointerGetAttributes(&a, p) == cudaSuccess &&
+                    cudaGetDevice(&dev) == cudaSuccess && a.type == cudaMemoryTypeDevice &&
+                    a.device == dev && (reinterpret_cast<uintptr_t>(p) & 3u) == 0;
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
 hpf_status hpf_get_state(hpf_ctx* c, float* pos, float* vel, int64_t* step) {
     if (!c) return HPF_ERR_INVALID;
     if (!c->has_state) return fail(c, HPF_ERR_STATE, "no state loaded");
-    float* pt = c->out_f;
-    float* vt = c->out_f + 3 * (size_t)c->n;
+    // device outputs that do not overlap are written in place; others (host
+    // memory above all) take the staged arrays and a copy
+    const size_t bytes = sizeof(float) * 3 * (size_t)c->n;
+    const uintptr_t pa = reinterpret_cast<uintptr_t>(pos), va = reinterpret_cast<uintptr_t>(vel);
+    const bool direct = (!pos || device_floats(pos)) && (!vel || device_floats(vel)) &&
+                        (!pos || !vel || pa + bytes <= va || va + bytes <= pa);
+    float* pt = direct ? pos : (pos ? c->out_f : nullptr);
+    float* vt = direct ? vel : (vel ? c->out_f + 3 * (size_t)c->n : nullptr);
     {
         StageScope sc(c, HPF_STAGE_OTHER, c->n > 0 ? 1 : 0);
-        launch_unpermute(cur_state(c), c->meta, c->n, pt, vt, c->dflag, c->stream);
+        launch_unpermute(cur_state(c), c->meta, c->n, pt, vt, c->dflag,
+                         reinterpret_cast<unsigned*>(c->dflag + 5), c->hflag, c->stream);
     }
     LAUNCH_CHECK(c);
-    hpf_status s;
-    if ((s = copy_out(c, pos, pt, sizeof(float) * 3 * c->n)) != HPF_OK) return s;
-    if ((s = copy_out(c, vel, vt, sizeof(float) * 3 * c->n)) != HPF_OK) return s;
+    if (!direct && bytes > 0) {
+        if (pos) CUDA_TRY(c, cudaMemcpyAsync(pos, pt, bytes, cudaMemcpyDefault, c->stream));
+        if (vel) CUDA_TRY(c, cudaMemcpyAsync(vel, vt, bytes, cudaMemcpyDefault, c->stream));
+    }
     if (step) *step = c->step;
-    return check_flags(c);
+    if (c->n == 0) return check_flags(c);
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    return flag_status(c, c->hflag[0]);
 }
 
 hpf_status hpf_get_order(hpf_ctx* c, int32_t* order) {
@@ -1349,7 +1361,8 @@ hpf_status hpf_energy(hpf_ctx* c, double out[6]) {
     if (c->energy_pending) return fail(c, HPF_ERR_STATE, "hpf_energy_start is pending");
     hpf_status s = energy_launch(c);
     if (s != HPF_OK) return s;
-    if ((s = check_flags(c)) != HPF_OK) return s;
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    if ((s = flag_status(c, c->hflag[7])) != HPF_OK) return s;
     energy_finish(c, out);
     return HPF_OK;
 }
@@ -1359,6 +1372,7 @@ hpf_status hpf_energy_start(hpf_ctx* c) {
     if (c->energy_pending) return fail(c, HPF_ERR_STATE, "hpf_energy_start is pending");
     const hpf_status s = energy_launch(c);
     if (s != HPF_OK) return s;
+    CUDA_TRY(c, cudaEventRecord(c->energy_ev, c->stream));
     c->energy_pending = true;
     return HPF_OK;
 }
@@ -1367,7 +1381,7 @@ hpf_status hpf_energy_finish(hpf_ctx* c, double out[6]) {
     if (!c || !out) return fail(c, HPF_ERR_INVALID, "out is required");
     if (!c->energy_pending) return fail(c, HPF_ERR_STATE, "no hpf_energy_start pending");
     c->energy_pending = false;
-    // waits for the observables' own copies only: work enqueued after
+    // waits for the observables' own kernels only: work enqueued after
     // hpf_energy_start (the next step's upload, permutation, step) keeps running
     CUDA_TRY(c, cudaEventSynchronize(c->energy_ev));
     const hpf_status s = flag_status(c, c->hflag[7]);
@@ -1779,8 +1793,9 @@ hpf_status hpf_batch_energy(hpf_batch* b, double* out) {
         hpf_status s = energy_launch(c);
         if (s != HPF_OK) return s;
     }
+    CUDA_TRY(b->rep[0], cudaStreamSynchronize(b->stream));
     for (hpf_ctx* c : b->rep) {
-        hpf_status s = check_flags(c);
+        hpf_status s = flag_status(c, c->hflag[7]);
         if (s != HPF_OK) return s;
     }
     for (size_t r = 0; r < b->rep.size(); ++r) energy_finish(b->rep[r], out + 6 * r);

@@ -924,6 +924,15 @@ __device__ __forceinline__ void warp_bonded_forces(float x0, float y0, float z0,
 
 // ------------------------------------------------------------------ launchers
 
+// Where the observables go: mapped host memory, written by the last kernel.
+struct EnergyOut {
+    double* out6;     // the six sums
+    const int* flag;  // the error word as it stands after the kernels, to h_flag
+    int* h_flag;
+    const double* nh;  // xi, eta of a Nose-Hoover context (NULL: none), to h_nh
+    double* h_nh;
+};
+
 // Mesh, box, species, rho0, kT, 1/kappa and chi of a parameter block:
 // HPF_OK or HPF_ERR_INVALID.
 hpf_status validate_field_params(const hpf_params* p);
@@ -944,12 +953,12 @@ void launch_step(StateBuf in, StateBuf out, const uint32_t* meta, int n, int n_s
                  unsigned long long* D_next, int* flag, cudaStream_t s);
 void launch_energy(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const float4* G,
                    StepConsts c, long long step, const long long* D, const EnergyConsts& e,
-                   double* partials, double* out6, cudaStream_t s);
+                   double* partials, const EnergyOut& out, cudaStream_t s);
 void launch_order(const uint32_t* meta, int n, int32_t* order, cudaStream_t s);
 void launch_advance_counter(long long* step, long long by, cudaStream_t s);
 void launch_set_counter(long long* step, long long v, cudaStream_t s);
 void launch_unpermute(StateBuf st, const uint32_t* meta, int n, float* pos_tag, float* vel_tag,
-                      int* flag, cudaStream_t s);
+                      int* flag, unsigned* ticket, int* h_flag, cudaStream_t s);
 void launch_repermute(const float* pos_tag, const float* vel_tag, const uint32_t* meta, int n,
                       StateBuf st, const MeshGeom& g, unsigned long long* D, int* flag,
                       cudaStream_t s);
@@ -998,7 +1007,7 @@ int energy_partials_needed(int n, int nodes, int S);
 int energy_launches(int n, int S);  // kernels launch_energy issues
 void launch_energy_nodes_only(int n, MeshGeom g, const long long* D, const EnergyConsts& e,
                               const float2* bead_part, int nb_bead, double* partials,
-                              double* out6, cudaStream_t s);
+                              const EnergyOut& out, cudaStream_t s);
 
 // learned density propagator (the network lives in k_prop.cu)
 bool prop_mesh_is(const hpf_prop* p, const MeshGeom& g);

@@ -291,13 +291,13 @@ __global__ void __launch_bounds__(kRedBlock, 4) k_energy_main(StateBuf st,
 // One block: the bead partials (float-float) and the node partials (exact
 // 128-bit) summed over the blocks in a fixed order -- each thread a strided
 // share of the blocks, its loads all in flight together, then its warp, then
-// one lane per value over the warps -- and combined in FP64.
+// one lane per value over the warps -- and combined in FP64, then written to the host.
 template <int kS>
 __global__ void __launch_bounds__(kFinalBlock) k_energy_final(const float2* __restrict__ bead_part,
                                                               int nb,
                                                               const unsigned long long* __restrict__ node_part,
                                                               int nn, int nodes, EnergyConsts e,
-                                                              double* __restrict__ out6) {
+                                                              EnergyOut out) {
     constexpr int kP = kS * (kS + 1) / 2;
     constexpr int kQ = kP + 2;
     constexpr int kW = kFinalBlock / 32;
@@ -362,12 +362,17 @@ __global__ void __launch_bounds__(kFinalBlock) k_energy_final(const float2* __re
                                                              (double)nodes));
         const double ke = 0.5 * e.mass * res[0], ub = res[1];
         const double px = e.mass * res[2], py = e.mass * res[3], pz = e.mass * res[4];
-        out6[0] = ke;
-        out6[1] = ub;
-        out6[2] = w_f;
-        out6[3] = ke + ub + w_f;
-        out6[4] = sqrt(px * px + py * py + pz * pz);
-        out6[5] = e.n > 0 ? 2.0 * ke / (3.0 * (double)e.n) : 0.0;
+        out.out6[0] = ke;
+        out.out6[1] = ub;
+        out.out6[2] = w_f;
+        out.out6[3] = ke + ub + w_f;
+        out.out6[4] = sqrt(px * px + py * py + pz * pz);
+        out.out6[5] = e.n > 0 ? 2.0 * ke / (3.0 * (double)e.n) : 0.0;
+        *out.h_flag = *out.flag;
+        if (out.nh) {
+            out.h_nh[0] = out.nh[0];
+            out.h_nh[1] = out.nh[1];
+        }
     }
 }
 
@@ -391,7 +396,7 @@ static int energy_blocks(int count, int per_thread) {
 
 void launch_energy(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const float4* G,
                    StepConsts c, long long step, const long long* D, const EnergyConsts& e,
-                   double* partials, double* out6, cudaStream_t s) {
+                   double* partials, const EnergyOut& out, cudaStream_t s) {
     const int nb = energy_blocks(n, kBeadsPerThread);
     const int nn = energy_blocks(g.nodes, kNodesPerThread);
     // bead partials: kBeadVals float-float pairs (one double's room each) per block
@@ -425,7 +430,7 @@ void launch_energy(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const f
 #define HPF_FINAL(k)                                                                        \
     case k:                                                                                 \
         launch_pdl(k_energy_final<k>, dim3(1), dim3(kFinalBlock), 0, s, (const float2*)bead_part, \
-                   nb, (const unsigned long long*)node_part, nn, g.nodes, e, out6);         \
+                   nb, (const unsigned long long*)node_part, nn, g.nodes, e, out);         \
         break;
         HPF_FINAL(1) HPF_FINAL(2) HPF_FINAL(3) HPF_FINAL(4)
         HPF_FINAL(5) HPF_FINAL(6) HPF_FINAL(7) HPF_FINAL(8)
@@ -437,7 +442,7 @@ void launch_energy(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const f
 // (nb_bead CTAs' worth, by the step launch that ended at this state).
 void launch_energy_nodes_only(int n, MeshGeom g, const long long* D, const EnergyConsts& e,
                               const float2* bead_part, int nb_bead, double* partials,
-                              double* out6, cudaStream_t s) {
+                              const EnergyOut& out, cudaStream_t s) {
     const int nb = energy_blocks(n, kBeadsPerThread);
     const int nn = energy_blocks(g.nodes, kNodesPerThread);
     unsigned long long* node_part =
@@ -452,7 +457,7 @@ void launch_energy_nodes_only(int n, MeshGeom g, const long long* D, const Energ
         else                                                                                \
             k_energy_nodes<k><<<nn, kRedBlock, 0, s>>>(D, g.nodes, node_part);              \
         launch_pdl(k_energy_final<k>, dim3(1), dim3(kFinalBlock), 0, s, bead_part, nb_bead, \
-                   (const unsigned long long*)node_part, nn, g.nodes, e, out6);             \
+                   (const unsigned long long*)node_part, nn, g.nodes, e, out);             \
         break;
         HPF_ONLY(1) HPF_ONLY(2) HPF_ONLY(3) HPF_ONLY(4)
         HPF_ONLY(5) HPF_ONLY(6) HPF_ONLY(7) HPF_ONLY(8)

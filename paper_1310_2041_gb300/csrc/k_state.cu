@@ -44,28 +44,41 @@ __global__ void k_mark_bonds(const int32_t* __restrict__ bonds, long long nb, in
     atomicOr(meta + hi, kBondPrev);
 }
 
-// Storage order -> tag order, with a finiteness check of the state.
+// Storage order -> tag order, with a finiteness check of the state.  The last
+// block to finish (ticket, left at zero) writes the error word to the mapped
+// host word h_flag, which saves the read-back its copy: a frame of a small
+// system is a few microseconds of work, and every copy on the stream costs
+// about as much again.
 __global__ void k_unpermute(StateBuf st, const uint32_t* __restrict__ meta, int n,
-                            float* __restrict__ pos_tag, float* __restrict__ vel_tag,
-                            int* __restrict__ flag) {
+                            float* __restrict__ pos_tag, float* __restrict__ vel_tag, int* flag,
+                            unsigned* ticket, volatile int* h_flag) {
+    griddep_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t tag = meta[i] & kTagMask;
-    const float x = st.x[i], y = st.y[i], z = st.z[i];
-    const float vx = st.vx[i], vy = st.vy[i], vz = st.vz[i];
-    if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(vx) && isfinite(vy) &&
-          isfinite(vz)))
-        atomicOr(flag, kFlagNonFinite);
-    if (pos_tag) {
-        pos_tag[3 * tag] = x;
-        pos_tag[3 * tag + 1] = y;
-        pos_tag[3 * tag + 2] = z;
+    if (i < n) {
+        const uint32_t tag = meta[i] & kTagMask;
+        const float x = st.x[i], y = st.y[i], z = st.z[i];
+        const float vx = st.vx[i], vy = st.vy[i], vz = st.vz[i];
+        if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(vx) && isfinite(vy) &&
+              isfinite(vz)))
+            atomicOr(flag, kFlagNonFinite);
+        if (pos_tag) {
+            pos_tag[3 * tag] = x;
+            pos_tag[3 * tag + 1] = y;
+            pos_tag[3 * tag + 2] = z;
+        }
+        if (vel_tag) {
+            vel_tag[3 * tag] = vx;
+            vel_tag[3 * tag + 1] = vy;
+            vel_tag[3 * tag + 2] = vz;
+        }
     }
-    if (vel_tag) {
-        vel_tag[3 * tag] = vx;
-        vel_tag[3 * tag + 1] = vy;
-        vel_tag[3 * tag + 2] = vz;
-    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(ticket, 1u) != gridDim.x - 1) return;
+    *ticket = 0u;
+    __threadfence();
+    *h_flag = atomicOr(flag, 0);
 }
 
 // New positions and velocities given in tag order, written in storage order
@@ -141,9 +154,10 @@ void launch_repermute(const float* pos_tag, const float* vel_tag, const uint32_t
 }
 
 void launch_unpermute(StateBuf st, const uint32_t* meta, int n, float* pos_tag, float* vel_tag,
-                      int* flag, cudaStream_t s) {
+                      int* flag, unsigned* ticket, int* h_flag, cudaStream_t s) {
     if (n <= 0) return;
-    k_unpermute<<<(n + 255) / 256, 256, 0, s>>>(st, meta, n, pos_tag, vel_tag, flag);
+    launch_pdl(k_unpermute, dim3((n + 255) / 256), dim3(256), 0, s, st, meta, n, pos_tag, vel_tag,
+               flag, ticket, (volatile int*)h_flag);
 }
 
 }  // namespace hpf

@@ -9,6 +9,7 @@ there is no fallback of any kind when it is missing.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 import threading
 
@@ -214,6 +215,10 @@ def make_params(n_beads, n_species, mesh, box, kT=1.0, rho0=3.0, inv_kappa=0.1, 
     return p
 
 
+_TORCH_NAMES = {np.float32: "float32", np.int32: "int32", np.int64: "int64",
+                np.float64: "float64"}
+
+
 def _ptr(a, dtype, shape=None, name="array"):
     """Raw pointer of a numpy array or torch tensor after dtype / layout checks."""
     if a is None:
@@ -221,15 +226,14 @@ def _ptr(a, dtype, shape=None, name="array"):
     if isinstance(a, np.ndarray):
         if a.dtype != dtype or not a.flags.c_contiguous:
             a = np.ascontiguousarray(a, dtype=dtype)
-        if shape is not None and a.size != int(np.prod(shape)):
+        if shape is not None and a.size != math.prod(shape):
             raise ValueError(f"{name}: expected {shape}, got {a.shape}")
         return a.ctypes.data, a
     import torch  # tensors only
-    tdt = {np.float32: torch.float32, np.int32: torch.int32, np.int64: torch.int64,
-           np.float64: torch.float64}[np.dtype(dtype).type]
+    tdt = getattr(torch, _TORCH_NAMES[dtype])
     if a.dtype != tdt or not a.is_contiguous():
         raise ValueError(f"{name}: needs a contiguous {tdt} tensor")
-    if shape is not None and a.numel() != int(np.prod(shape)):
+    if shape is not None and a.numel() != math.prod(shape):
         raise ValueError(f"{name}: expected {shape}, got {tuple(a.shape)}")
     return a.data_ptr(), a
 
