@@ -25,7 +25,7 @@
 namespace hpf {
 
 constexpr int kPC = 16;                      // padded channels
-constexpr int kTX = 8, kTY = 8, kTZ = 8;     // output tile: one z-plane of 64 voxels per warp
+constexpr int kTX = 8, kTY = 8, kTZ = 8;     // tile of the weight gradients
 constexpr int kBX = kTX + 2, kBY = kTY + 2, kBZ = kTZ + 2;
 constexpr int kBoxVox = kBX * kBY * kBZ;     // 1000 (32 000 bytes)
 constexpr int kTileVox = kTX * kTY * kTZ;    // 512
@@ -48,26 +48,8 @@ __device__ __forceinline__ uint32_t saddr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2,
-                                        uint32_t& r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(addr));
-}
-
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2,
-                                          uint32_t& r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(addr));
-}
-
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
@@ -83,50 +65,6 @@ __device__ __forceinline__ void tile_origin(const PropGeom& g, int t, int& x0, i
     x0 = (t % g.tiles_x) * kTX;
     y0 = ((t / g.tiles_x) % g.tiles_y) * kTY;
     z0 = (t / (g.tiles_x * g.tiles_y)) * kTZ;
-}
-
-// Shared-memory rows are 16 channels = two 16-byte halves.  The halves of
-// every other group of four rows are swapped so that the eight rows an
-// ldmatrix phase reads (always eight consecutive rows here) hit distinct banks.
-__device__ __forceinline__ int swz(int row, int half) { return 2 * row + (half ^ ((row >> 2) & 1)); }
-
-// Where the voxels of an activation buffer live: channel half h (8 channels)
-// of voxel (x, y, z) at element (((z + off) ly + y + off) lx + x + off) vs +
-// h hs -- the plain layout [V][16] (lx = Mx, ly = My, off = 0, vs = 16, hs =
-// 8) or the padded one of the forward convolutions [2][Mz + 2][PY][PX][8]
-// (off = 1, vs = 8, hs = (Mz + 2) PY PX 8).
-struct ActLayout {
-    int lx, ly, off;
-    long long vs, hs;
-};
-
-// Periodic input box of a tile (all 16 channels), 16-byte asynchronous copies.
-__device__ __forceinline__ void load_box(const __nv_bfloat16* __restrict__ in, const PropGeom& g,
-                                         const ActLayout& L, int x0, int y0, int z0, uint4* box) {
-    const uint32_t box_s = saddr(box);
-    for (int e = threadIdx.x; e < kBoxVox * 2; e += blockDim.x) {
-        const int v = e >> 1, half = e & 1;
-        const int bx = v % kBX, by = (v / kBX) % kBY, bz = v / (kBX * kBY);
-        const int gx = pwrap(x0 - 1 + bx, g.mx), gy = pwrap(y0 - 1 + by, g.my),
-                  gz = pwrap(z0 - 1 + bz, g.mz);
-        const size_t gv = ((size_t)(gz + L.off) * L.ly + gy + L.off) * L.lx + gx + L.off;
-        cp_async16(box_s + 16 * swz(v, half), in + gv * L.vs + half * L.hs);
-    }
-}
-
-// Voxel r (0..15) of 16-voxel row tile mt (0..31) of the tile: (lx, ly, lz);
-// row tiles 4w .. 4w + 3 are the z-plane lz = w.
-__device__ __forceinline__ void warp_voxel(int mt, int r, int& lx, int& ly, int& lz) {
-    const int m = 16 * mt + r;
-    lx = m % kTX;
-    ly = (m / kTX) % kTY;
-    lz = m / (kTX * kTY);
-}
-
-// Box row of tile voxel (lx, ly, lz) shifted by kernel offset o.
-__device__ __forceinline__ int box_row(int lx, int ly, int lz, int o) {
-    const int dz = o / 9 - 1, dy = (o / 3) % 3 - 1, dx = o % 3 - 1;
-    return ((lz + 1 + dz) * kBY + (ly + 1 + dy)) * kBX + (lx + 1 + dx);
 }
 
 // ------------------------------------------------------------------ tcgen05 data gradients
@@ -231,7 +169,7 @@ __device__ __forceinline__ int tc_wrap(int i, int m, bool near) {
 }
 
 // A thread's share of the box copies: elements e = tid + kTcThreads k of the
-// [voxel][half] order, their box coordinates and shared-memory offsets, the
+// [half][voxel] order, their box coordinates and shared-memory offsets, the
 // same for every tile.
 constexpr int kTcSlots = (kTcBox * 2 + kTcThreads - 1) / kTcThreads;
 
@@ -244,7 +182,7 @@ __device__ __forceinline__ void tc_slots(TcSlots& sl) {
 #pragma unroll
     for (int k = 0; k < kTcSlots; ++k) {
         const int e = threadIdx.x + kTcThreads * k;
-        const int v = e >> 1, half = e & 1;
+        const int half = e / kTcBox, v = e % kTcBox;
         const int bx = v % kTcBX, by = (v / kTcBX) % kTcBY, bz = v / kTcPlane;
         sl.c[k] = e < kTcBox * 2 ? (bx | (by << 8) | (bz << 16) | (half << 24)) : -1;
         sl.s[k] = (uint32_t)sizeof(uint4) * (uint32_t)(half * kTcBox + v);
@@ -262,7 +200,7 @@ __device__ __forceinline__ void tc_load_box(const __nv_bfloat16* __restrict__ in
         const int gy = tc_wrap(y0 - 1 + ((c >> 8) & 0xff), g.my, near);
         const int gz = tc_wrap(z0 - 1 + ((c >> 16) & 0xff), g.mz, near);
         const int gv = (gz * g.my + gy) * g.mx + gx;
-        cp_async16(box_s + sl.s[k], in + (size_t)gv * kPC + 8 * (c >> 24));
+        cp_async16(box_s + sl.s[k], in + ((size_t)(c >> 24) * g.V + gv) * 8);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -284,7 +222,8 @@ __device__ __forceinline__ float silu_backward(float g, float z) {
 // Epilogue of one output plane: the warp's 32 accumulator rows (lanes 32w ..)
 // from columns col .. col + 15, voxel (x0 + row % 8, y0 + row / 8, z): the
 // gradient of the layer input through the SiLU of the layer below (its FP32
-// pre-activations z_in [V][16]), in BF16 for the next tensor-core passes.
+// pre-activations z_in [V][16]), in BF16 for the next tensor-core passes
+// (planar channel halves [2][V][8]).
 // Multiplying here instead of in an elementwise pass keeps the FP32 gradient
 // out of memory (44 MB written and read back per layer at 70^3).
 __device__ __forceinline__ void tc_epilogue(uint32_t tcol, const PropGeom& g, int x0, int y0,
@@ -311,7 +250,7 @@ __device__ __forceinline__ void tc_epilogue(uint32_t tcol, const PropGeom& g, in
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
     if (!valid) return;
-    uint4* o = reinterpret_cast<uint4*>(gz_out + gv * kPC);
+    uint4* o = reinterpret_cast<uint4*>(gz_out) + gv;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         __nv_bfloat162 v[4];
@@ -324,13 +263,13 @@ __device__ __forceinline__ void tc_epilogue(uint32_t tcol, const PropGeom& g, in
             v[2 * q + 1] = __floats2bfloat162_rn(silu_backward(__uint_as_float(a[2]), zq.z),
                                                  silu_backward(__uint_as_float(a[3]), zq.w));
         }
-        o[h] = *reinterpret_cast<uint4*>(v);
+        o[(size_t)h * g.V] = *reinterpret_cast<uint4*>(v);
     }
 }
 
 // Wp: a packed weight image (k_pack_images) of the data-gradient weights
 // [27][16 out][16 in], offset index 9 dz_index + in-plane offset (dy, dx);
-// K = 16 input channels of the plain layout [V][16].
+// K = 16 input channels of the planar layout [2][V][8].
 template <int kBuf>
 __global__ void __launch_bounds__(kTcThreads, kBuf == 1 ? 4 : 1)
     k_conv_tc(const __nv_bfloat16* __restrict__ in, const uint4* __restrict__ Wp,
@@ -532,8 +471,8 @@ void conv_tc_setup() {
     });
 }
 
-// Data-gradient convolution of in [V][16] with weight image k of tcw, through
-// the SiLU at pre-activations z_in [V][16], into gz_out [V][16] (not in).
+// Data-gradient convolution of in [2][V][8] with weight image k of tcw, through
+// the SiLU at pre-activations z_in [V][16], into gz_out [2][V][8] (not in).
 void launch_conv_tc(const __nv_bfloat16* in, const uint4* tcw, int k, const float* z_in,
                     __nv_bfloat16* gz_out, const PropGeom& g, int* flag, cudaStream_t s) {
     conv_tc_setup();
@@ -1247,6 +1186,24 @@ bool make_act_tensor_map(CUtensorMap* map, __nv_bfloat16* act, const PropGeom& g
     return encode_tiled_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, act, dims, strides, box);
 }
 
+// The weight gradients' boxes: a tile with one neighbour on every side of the
+// padded activations (both channel halves), and a tile of the gradients.
+bool make_wgrad_tensor_maps(CUtensorMap* in, CUtensorMap* gzm, __nv_bfloat16* act,
+                            __nv_bfloat16* gz, const PropGeom& g) {
+    int px, py;
+    sweep_pitches(g, px, py);
+    const cuuint64_t pz = (cuuint64_t)g.mz + 2;
+    const cuuint64_t dims[4] = {8ull * px, (cuuint64_t)py, pz, 2};
+    const cuuint64_t strides[3] = {16ull * px, 16ull * px * py, 16ull * px * py * pz};
+    const cuuint32_t box[4] = {8 * kBX, kBY, kBZ, 2};
+    const cuuint64_t mx = g.mx, my = g.my, mz = g.mz;
+    const cuuint64_t gdims[4] = {8 * mx, my, mz, 2};
+    const cuuint64_t gstrides[3] = {16 * mx, 16 * mx * my, 16 * mx * my * mz};
+    const cuuint32_t gbox[4] = {8 * kTX, kTY, kTZ, 2};
+    return encode_tiled_map(in, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, act, dims, strides, box) &&
+           encode_tiled_map(gzm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, gz, gdims, gstrides, gbox);
+}
+
 template <int kL>
 void launch_conv_sweep(const CUtensorMap& tmap, const SweepArgs& a, int ctas, cudaStream_t s) {
     conv_sweep_setup();
@@ -1257,28 +1214,109 @@ void launch_conv_sweep(const CUtensorMap& tmap, const SweepArgs& a, int ctas, cu
 }
 
 // dW[o][ci][co] = sum_n in(n + d_o)[ci] gz(n)[co]: a voxel reduction on the
-// tensor cores.  Warp w owns offsets w, w + 8, w + 16 (and 24 for w < 3); a
-// CTA walks tiles grid-stride and writes its register sums to its own slice
-// part[blockIdx.x] (every entry, once); k_sum_grads adds the slices in a
-// fixed order, so the gradient is deterministic.  The shared-memory matrix
-// loads bound it, so a k-step's gradient fragment is loaded once for all of
-// the warp's offsets (five loads for four offsets instead of eight), and with
-// kHalf (the two-channel last layer) only the first eight channels are
-// multiplied.  The bias gradient, the sum of gz itself, comes from the same
-// tiles in FP32: thread t sums channel half t & 1 of voxels t / 2 + 128 j,
-// into the slice's last 16 entries.
+// tensor cores (warp-level MMAs, A = in^T and B = gz by ldmatrix.trans).  A
+// persistent CTA walks tiles of 8^3 voxels grid-stride and writes its register
+// sums to its own slice part[blockIdx.x] (every entry that is read, once);
+// k_sum_grads adds the slices in a fixed order, so the gradient is
+// deterministic.  Index arithmetic bound the form with cp.async copies of a
+// periodic box and swizzled rows (ALU pipe 46 % busy, tensor pipe 18 %, 33 us
+// a layer at 70^3): here one thread issues two TMA boxes per tile -- the
+// padded activations hold their periodic halo, and boxes past the mesh arrive
+// as zeros -- into one of two stages, the other being multiplied.  Both
+// operands sit in shared memory as planar channel halves, 16 bytes per voxel,
+// so the eight x-consecutive voxels of an ldmatrix phase are 128 contiguous
+// bytes (no bank conflict, no swizzle) and every address is a per-lane base
+// plus a constant.  A k-step's gradient fragment is loaded once for all of a
+// warp's offsets.  Layer kL: 1, 2 (27 offsets): warp w owns offsets w, w + 8,
+// w + 16 and, w < 3, w + 24; the two-channel last layer (2) multiplies only
+// the first eight output channels.  0: the x-im2col input carries the three dx
+// as channels (dx + 1) 4 + ci, so nine offsets (dz, dy) do: warp w owns offset
+// w, and all warps share the ninth, each over its z-plane.  The bias gradient,
+// the sum of gz itself, comes from the same stages in FP32, into the slice's
+// last 16 entries.
 constexpr int kGradEntries = kOffsets * kPC * kPC + kPC;  // a slice: weights, then biases
+constexpr uint32_t kWgBoxHalf = 16u * kBoxVox, kWgBoxBytes = 2u * kWgBoxHalf;
+constexpr uint32_t kWgTileHalf = 16u * kTileVox, kWgTileBytes = 2u * kWgTileHalf;
+constexpr uint32_t kWgBoxPitch = (kWgBoxBytes + 127u) & ~127u;  // TMA targets: 128-byte aligned
+constexpr uint32_t kWgStage = kWgBoxPitch + kWgTileBytes;
+constexpr size_t kWgSmem = 2 * (size_t)kWgStage + 128 + 64;
 
-template <bool kHalf>
-__global__ void __launch_bounds__(256, 2) k_conv_wgrad(const __nv_bfloat16* __restrict__ in,
-                                                       const __nv_bfloat16* __restrict__ gz,
-                                                       float* __restrict__ part, PropGeom g,
-                                                       ActLayout L) {
+template <int kOff>
+__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4 + %5];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr), "n"(kOff));
+}
+
+// k-step kKs (16 voxels: two y rows) of the offsets at lane bases a[0 .. n).
+template <int kKs, int kN, bool kHalf>
+__device__ __forceinline__ void wgrad_step(const uint32_t (&a)[4], uint32_t b, bool last,
+                                           float (&acc)[4][2][4]) {
+    // two y rows further in the box per k-step, a z-plane every fourth
+    constexpr int kStep = 16 * ((kKs >> 2) * kBY * kBX + (kKs & 3) * 2 * kBX);
+    uint32_t gb[4];
+    ldsm_x4_t<256 * kKs>(b, gb);
+#pragma unroll
+    for (int s = 0; s < kN; ++s) {
+        if (s == 3 && !last) break;
+        uint32_t ga[4];
+        ldsm_x4_t<kStep>(a[s], ga);
+        mma_bf16(acc[s][0], ga[0], ga[1], ga[2], ga[3], gb[0], gb[1]);
+        if (!kHalf) mma_bf16(acc[s][1], ga[0], ga[1], ga[2], ga[3], gb[2], gb[3]);
+    }
+}
+
+template <int kL, int kKs = 0>
+__device__ __forceinline__ void wgrad_tile(const uint32_t (&a)[4], uint32_t b, bool last,
+                                           float (&acc)[4][2][4]) {
+    if constexpr (kKs < kTileVox / 16) {
+        wgrad_step<kKs, kL == 0 ? 1 : 4, kL == 2>(a, b, last, acc);
+        wgrad_tile<kL, kKs + 1>(a, b, last, acc);
+    }
+}
+
+template <int kL>
+__global__ void __launch_bounds__(256, 2)
+    k_conv_wgrad(const __grid_constant__ CUtensorMap in, const __grid_constant__ CUtensorMap gz,
+                 float* __restrict__ part, const PropGeom g, int* __restrict__ flag) {
+    extern __shared__ uint8_t wg_raw[];
+    __shared__ __align__(8) unsigned long long bars[2];
+    const uint32_t stage_s = (saddr(wg_raw) + 127u) & ~127u;
+    const uint8_t* base = wg_raw + (stage_s - saddr(wg_raw));
+    const uint32_t bar = saddr(bars);
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     griddep_wait();
     griddep_launch_dependents();
-    __shared__ uint4 box[kBoxVox * 2];
-    __shared__ uint4 gt[kTileVox * 2];
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int mine = (g.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    // tile i of this CTA into stage i & 1: the voxels with one neighbour on every
+    // side (padded coordinates start at 0) and their gradients
+    auto issue = [&](int i) {
+        int x0, y0, z0;
+        tile_origin(g, (int)blockIdx.x + i * (int)gridDim.x, x0, y0, z0);
+        const uint32_t st = stage_s + (i & 1) * kWgStage, fb = bar + 8 * (i & 1);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
+                     "r"(kWgBoxBytes + kWgTileBytes)
+                     : "memory");
+        asm volatile(
+            "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(st),
+            "l"(reinterpret_cast<uint64_t>(&in)), "r"(8 * x0), "r"(y0), "r"(z0), "r"(0), "r"(fb)
+            : "memory");
+        asm volatile(
+            "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(st + kWgBoxPitch),
+            "l"(reinterpret_cast<uint64_t>(&gz)), "r"(8 * x0), "r"(y0), "r"(z0), "r"(0), "r"(fb)
+            : "memory");
+    };
+    if (tid == 0) {
+        for (int i = 0; i < 2 && i < mine; ++i) issue(i);
+    }
+    __syncthreads();  // the barriers are initialised
     float acc[4][2][4];
 #pragma unroll
     for (int s = 0; s < 4; ++s)
@@ -1289,94 +1327,119 @@ __global__ void __launch_bounds__(256, 2) k_conv_wgrad(const __nv_bfloat16* __re
     float bsum[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) bsum[c] = 0.f;
-    // A = in^T (ci x voxels) by ldmatrix.trans of voxel rows: lane -> voxel
-    // (lane & 7) + 8 (lane >= 16), channel half ((lane >> 3) & 1), so that
+    // A: lane -> voxel (lane & 7) + 8 (lane >= 16), channel half ((lane >> 3) & 1), so that
     // a0 = ci 0-7 / vox 0-7, a1 = ci 8-15 / vox 0-7, a2 = ci 0-7 / vox 8-15,
-    // a3 = ci 8-15 / vox 8-15
-    const int r_vox = (lane & 7) + ((lane >> 4) << 3), r_half = (lane >> 3) & 1;
-    // B = gz (voxels x co): lane -> voxel (lane & 7) + 8 ((lane >> 3) & 1), co half
-    // (lane >> 4): b0 = vox 0-7 / co 0-7, b1 = vox 8-15 / co 0-7, b2 = vox 0-7 /
-    // co 8-15, b3 = vox 8-15 / co 8-15
-    const int g_vox = (lane & 7) + (((lane >> 3) & 1) << 3), g_half = lane >> 4;
-    const uint32_t box_s = saddr(box), gt_s = saddr(gt);
-    int row0[4];  // box row of the lane's first voxel shifted by the warp's offset s
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        int lx, ly, lz;
-        warp_voxel(0, r_vox, lx, ly, lz);
-        row0[s] = box_row(lx, ly, lz, w + 8 * s < kOffsets ? w + 8 * s : w);
-    }
-    const bool four = w + 24 < kOffsets;
-    for (int t = blockIdx.x; t < g.tiles; t += gridDim.x) {
-        int x0, y0, z0;
-        tile_origin(g, t, x0, y0, z0);
-        __syncthreads();
-        load_box(in, g, L, x0, y0, z0, box);
-        for (int e = tid; e < kTileVox * 2; e += blockDim.x) {
-            const int m = e >> 1, half = e & 1;
-            const int X = x0 + m % kTX, Y = y0 + (m / kTX) % kTY, Z = z0 + m / (kTX * kTY);
-            if (X < g.mx && Y < g.my && Z < g.mz)
-                cp_async16(gt_s + 16 * swz(m, half),
-                           gz + (((size_t)Z * g.my + Y) * g.mx + X) * kPC + 8 * half);
-            else
-                gt[swz(m, half)] = make_uint4(0u, 0u, 0u, 0u);  // outside the mesh: adds nothing
-        }
-        cp_async_wait_all();
-        __syncthreads();
-#pragma unroll 4
-        for (int ks = 0; ks < kTileVox / 16; ++ks) {  // 16 voxels per k-step: two y rows
-            // k-step ks starts 2 y rows (20 box rows) further, a z-plane every fourth
-            const int step = (ks >> 2) * kBY * kBX + (ks & 3) * 2 * kBX;
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4_t(gt_s + 16 * swz(16 * ks + g_vox, g_half), b0, b1, b2, b3);
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                if (s == 3 && !four) break;
-                uint32_t a0, a1, a2, a3;
-                ldsm_x4_t(box_s + 16 * swz(row0[s] + step, r_half), a0, a1, a2, a3);
-                mma_bf16(acc[s][0], a0, a1, a2, a3, b0, b1);
-                if (!kHalf) mma_bf16(acc[s][1], a0, a1, a2, a3, b2, b3);
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < kTileVox / 128; ++j) {
-            const uint4 v = gt[swz((tid >> 1) + 128 * j, tid & 1)];
-            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                bsum[2 * c] += __uint_as_float(u[c] << 16);
-                bsum[2 * c + 1] += __uint_as_float(u[c] & 0xffff0000u);
-            }
-        }
-    }
-    float* out = part + (size_t)blockIdx.x * kGradEntries;
-    const int gq = lane >> 2, q = lane & 3;
+    // a3 = ci 8-15 / vox 8-15.  B: lane -> voxel (lane & 7) + 8 ((lane >> 3) & 1), co half
+    // (lane >> 4): b0 = vox 0-7 / co 0-7, b1 = vox 8-15 / co 0-7, b2, b3 the same of co 8-15
+    auto box_at = [&](int o) {  // the lane's A row at kernel offset o of the first k-step
+        const int dz = o / 9, dy = (o / 3) % 3, dx = o % 3;
+        return ((lane >> 3) & 1) * kWgBoxHalf +
+               16u * (uint32_t)((dz * kBY + dy + (lane >> 4)) * kBX + dx + (lane & 7));
+    };
+    const bool last = w + 24 < kOffsets;
+    uint32_t off[4];
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
         const int o = w + 8 * s;
+        off[s] = kL == 0 ? box_at(3 * (s == 0 ? w : 8) + 1) : box_at(o < kOffsets ? o : w);
+    }
+    const uint32_t b_off = (lane >> 4) * kWgTileHalf +
+                           16u * (uint32_t)((lane & 7) + (((lane >> 3) & 1) << 3));
+    bool failed = false;
+    int i = 0;
+    for (; i < mine; ++i) {
+        const bool ok = tc_wait(bar + 8 * (i & 1), (i >> 1) & 1);
+        if (ok) {
+            const uint32_t st = stage_s + (i & 1) * kWgStage;
+            const uint32_t a[4] = {st + off[0], st + off[1], st + off[2], st + off[3]};
+            const uint32_t b = st + kWgBoxPitch + b_off;
+            wgrad_tile<kL>(a, b, last, acc);
+            if (kL == 0) {  // the ninth offset over z-plane w: k-steps 4 w .. 4 w + 3
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t ga[4], gb[4];
+                    ldsm_x4_t<0>(b + 256u * (4 * w + q), gb);
+                    ldsm_x4_t<0>(a[1] + 16u * (w * kBY * kBX + 2 * q * kBX), ga);
+                    mma_bf16(acc[1][0], ga[0], ga[1], ga[2], ga[3], gb[0], gb[1]);
+                    mma_bf16(acc[1][1], ga[0], ga[1], ga[2], ga[3], gb[2], gb[3]);
+                }
+            }
+            const uint4* gt = reinterpret_cast<const uint4*>(base + (i & 1) * kWgStage + kWgBoxPitch) +
+                              (tid >> 7) * kTileVox + (tid & 127);
+#pragma unroll
+            for (int j = 0; j < kTileVox / 128; ++j) {
+                const uint4 v = gt[128 * j];
+                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    bsum[2 * c] += __uint_as_float(u[c] << 16);
+                    bsum[2 * c + 1] += __uint_as_float(u[c] & 0xffff0000u);
+                }
+            }
+        }
+        if (__syncthreads_or(!ok)) {  // every thread is done with the stage
+            failed = true;
+            break;
+        }
+        if (tid == 0 && i + 2 < mine) issue(i + 2);
+    }
+    if (failed) {
+        // report; the copies issued for this and the next tile land (bounded) before the CTA ends
+        if (tid == 0) {
+            atomicOr(flag, kFlagTimeout);
+            for (int k = i; k < i + 2 && k < mine; ++k) tc_wait(bar + 8 * (k & 1), (k >> 1) & 1);
+        }
+        return;
+    }
+    float* out = part + (size_t)blockIdx.x * kGradEntries;
+    const int gq = lane >> 2, q = lane & 3;
+    auto entry = [&](int c, int j) { return (gq + 8 * (c >> 1)) * kPC + 8 * j + 2 * q + (c & 1); };
+#pragma unroll
+    for (int s = 0; s < (kL == 0 ? 1 : 4); ++s) {
+        const int o = w + 8 * s;
         if (o >= kOffsets) break;
+#pragma unroll
+        for (int j = 0; j < (kL == 2 ? 1 : 2); ++j)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) out[o * kPC * kPC + entry(c, j)] = acc[s][j][c];
+    }
+    // across the warps, through the stages: the first layer's ninth offset, the biases
+    float* sums = reinterpret_cast<float*>(const_cast<uint8_t*>(base));
+    float* rows = sums + 8 * kPC * kPC;
+    if (kL == 0) {
 #pragma unroll
         for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int ci = gq + 8 * (c >> 1), co = 8 * j + 2 * q + (c & 1);
-                out[(o * kPC + ci) * kPC + co] = acc[s][j][c];
-            }
+            for (int c = 0; c < 4; ++c) sums[w * kPC * kPC + entry(c, j)] = acc[1][j][c];
     }
-    __shared__ float rows[8][kPC];
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
 #pragma unroll
-        for (int m = 2; m < 32; m <<= 1) bsum[c] += __shfl_xor_sync(0xffffffffu, bsum[c], m);
-        if (lane < 2) rows[w][8 * lane + c] = bsum[c];
+        for (int m = 1; m < 32; m <<= 1) bsum[c] += __shfl_xor_sync(0xffffffffu, bsum[c], m);
+        if (lane == 0) rows[w * 8 + c] = bsum[c];
     }
     __syncthreads();
-    if (tid < kPC) {
-        float t = 0.f;
+    if (kL == 0) {
+        float t = sums[tid];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) t += rows[k][tid];
-        out[kOffsets * kPC * kPC + tid] = t;
+        for (int k = 1; k < 8; ++k) t += sums[k * kPC * kPC + tid];
+        out[8 * kPC * kPC + tid] = t;
     }
+    if (tid < kPC) {  // warps 0-3 hold the first channel half, 4-7 the second
+        const float* r = rows + (tid >> 3) * 32 + (tid & 7);
+        out[kOffsets * kPC * kPC + tid] = (r[0] + r[8]) + (r[16] + r[24]);
+    }
+}
+
+template <int kL>
+void launch_conv_wgrad(const CUtensorMap& in, const CUtensorMap& gz, float* part,
+                       const PropGeom& g, int blocks, int* flag, cudaStream_t s) {
+    static std::once_flag once[64];
+    once_per_device(once, [] {
+        cudaFuncSetAttribute(k_conv_wgrad<kL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kWgSmem);
+    });
+    launch_pdl(k_conv_wgrad<kL>, dim3(blocks), dim3(256), kWgSmem, s, in, gz, part, g, flag);
 }
 
 // ------------------------------------------------------------------ elementwise
@@ -1403,12 +1466,11 @@ __device__ __forceinline__ void input_features(const float* __restrict__ x, int 
 // One thread per voxel of the padded array [Mz + 2][My + 2][Mx + 2] (grid y:
 // the padded plane; halo
 // included, each halo voxel a copy of the opposite face): out_x in the padded
-// layout of the forward convolutions [2][Mz + 2][py][px][8]; out (optional, for the
-// weight gradient): the plain four channels [V][16] at the interior voxels;
-// diff (with phi_next, for the loss): the change phi_next - phi(t) [V][2].
+// layout of the forward convolutions [2][Mz + 2][py][px][8]; with phi_next
+// (training, for the loss) diff: the change phi_next - phi(t) [V][2].
 __global__ void k_pack_input(const float* __restrict__ x, PropGeom g, int px, int py, float scale,
-                             __nv_bfloat16* __restrict__ out, __nv_bfloat16* __restrict__ out_x,
-                             const float* __restrict__ phi_next, float2* __restrict__ diff) {
+                             __nv_bfloat16* __restrict__ out_x, const float* __restrict__ phi_next,
+                             float2* __restrict__ diff) {
     // the first convolution (a programmatic launch) may start its prologue now;
     // it waits for this grid before reading what it writes
     griddep_launch_dependents();
@@ -1425,19 +1487,13 @@ __global__ void k_pack_input(const float* __restrict__ x, PropGeom g, int px, in
     input_features(x, g.V, row + xm, scale, f[0]);
     input_features(x, g.V, row + xi, scale, f[1]);
     input_features(x, g.V, row + xp, scale, f[2]);
-    __nv_bfloat16 vals[kPC], cols[kPC];
+    __nv_bfloat16 cols[kPC];
 #pragma unroll
-    for (int c = 0; c < kPC; ++c) {
-        vals[c] = __float2bfloat16_rn(c < 4 ? f[1][c] : 0.f);
-        cols[c] = __float2bfloat16_rn(c < 12 ? f[c >> 2][c & 3] : 0.f);
-    }
+    for (int c = 0; c < kPC; ++c) cols[c] = __float2bfloat16_rn(c < 12 ? f[c >> 2][c & 3] : 0.f);
     uint4* ox = reinterpret_cast<uint4*>(out_x) + ((size_t)hz * py + hy) * px + hx;
     ox[0] = reinterpret_cast<uint4*>(cols)[0];
     ox[(size_t)wz * py * px] = reinterpret_cast<uint4*>(cols)[1];
-    if (out && hx >= 1 && hx <= g.mx && hy >= 1 && hy <= g.my && hz >= 1 && hz <= g.mz) {
-        uint4* o = reinterpret_cast<uint4*>(out + (size_t)(row + xi) * kPC);
-        o[0] = reinterpret_cast<uint4*>(vals)[0];
-        o[1] = reinterpret_cast<uint4*>(vals)[1];
+    if (phi_next && hx >= 1 && hx <= g.mx && hy >= 1 && hy <= g.my && hz >= 1 && hz <= g.mz) {
         const int v = row + xi;
         diff[v] = make_float2(__fsub_rn(phi_next[v], f[1][2]),
                               __fsub_rn(phi_next[(size_t)g.V + v], f[1][3]));
@@ -1459,7 +1515,8 @@ __global__ void k_rollout_shift(float* __restrict__ x, const float* __restrict__
 
 // Mean squared error of the network output y against scale * diff, diff =
 // phi_next - phi_cur ([V][2] each), and its gradient 2 (y - target) / (2V) in
-// BF16; the loss in FP64 per thread, one partial per block.
+// BF16 (the first channel half of a planar buffer, whose second half stays
+// zero); the loss in FP64 per thread, one partial per block.
 constexpr int kLossBlocks = 608;
 
 __global__ void __launch_bounds__(256) k_loss(const float2* __restrict__ y,
@@ -1476,9 +1533,8 @@ __global__ void __launch_bounds__(256) k_loss(const float2* __restrict__ y,
         l += (double)a * a;
         l += (double)b * b;
         const __nv_bfloat162 g2 = __floats2bfloat162_rn(a / (float)V, b / (float)V);
-        uint4* o = reinterpret_cast<uint4*>(gy + (size_t)v * kPC);
-        o[0] = make_uint4(*reinterpret_cast<const uint32_t*>(&g2), 0u, 0u, 0u);
-        o[1] = make_uint4(0u, 0u, 0u, 0u);
+        reinterpret_cast<uint4*>(gy)[v] =
+            make_uint4(*reinterpret_cast<const uint32_t*>(&g2), 0u, 0u, 0u);
     }
     for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = l;
@@ -1527,15 +1583,15 @@ __global__ void k_adam(const AdamArgs a, const float* __restrict__ g, int n) {
 }
 
 // The weight gradients' slices added up: block (x, layer) takes 32 consecutive
-// entries of that layer, eight threads per entry each adding every eighth
-// slice (nb of them), then the eight sums in order -- a fixed order, with every load
-// of a thread in flight together instead of one thread walking all slices.
+// entries of that layer, sixteen threads per entry each adding every sixteenth
+// slice (nb of them), then the sixteen sums in order -- a fixed order, with the
+// loads of a thread in flight together instead of one thread walking all slices.
 // The packed gradient goes to grads and, with adam.p, straight into the Adam
 // update.  One more block adds the loss partials.
-constexpr int kSumEntries = 32;
+constexpr int kSumEntries = 32, kSumShare = 16;
 constexpr int kSumBlocks = (kGradEntries + kSumEntries - 1) / kSumEntries;
 
-__global__ void __launch_bounds__(256) k_sum_grads(const float* __restrict__ part, int nb,
+__global__ void __launch_bounds__(kSumEntries * kSumShare) k_sum_grads(const float* __restrict__ part, int nb,
                                                    float* __restrict__ grads, const AdamArgs adam,
                                                    const double* __restrict__ loss_part, int nl,
                                                    double* __restrict__ loss) {
@@ -1544,38 +1600,45 @@ __global__ void __launch_bounds__(256) k_sum_grads(const float* __restrict__ par
     const int tid = threadIdx.x, layer = blockIdx.y;
     if (blockIdx.x == kSumBlocks) {
         if (layer != 0) return;
-        __shared__ double shd[8];
+        __shared__ double shd[kSumShare];
         double l = 0.0;
-        for (int k = tid; k < nl; k += 256) l += loss_part[k];
+        for (int k = tid; k < nl; k += kSumEntries * kSumShare) l += loss_part[k];
         for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
         if ((tid & 31) == 0) shd[tid >> 5] = l;
         __syncthreads();
         if (tid == 0) {
             double t = 0.0;
-            for (int k = 0; k < 8; ++k) t += shd[k];
+            for (int k = 0; k < kSumShare; ++k) t += shd[k];
             *loss = t;
         }
         return;
     }
-    __shared__ float sh[8][kSumEntries];
+    __shared__ float sh[kSumShare][kSumEntries];
     const int e = blockIdx.x * kSumEntries + (tid & 31), slice = tid >> 5;
-    // entry e: offset o, input channel ci, output channel co; the biases follow the weights
+    // entry e: offset o, input channel ci, output channel co; the biases follow the
+    // weights.  First layer: offset 3 dz index + dy index, channel (dx index) 4 + ci.
     const int ci_n = layer_in(layer), co_n = layer_out(layer);
     const bool bias = e >= kOffsets * kPC * kPC;
-    const int o = e / (kPC * kPC), ci = (e / kPC) % kPC, co = e % kPC;
-    const bool valid = e < kGradEntries && co < co_n && (bias || ci < ci_n);
+    int o = e / (kPC * kPC), ci = (e / kPC) % kPC;
+    const int co = e % kPC;
+    bool valid = e < kGradEntries && co < co_n && (bias || ci < ci_n);
+    if (layer == 0 && !bias) {
+        valid = o < 9 && ci < 12;
+        o = 3 * o + (ci >> 2);
+        ci &= 3;
+    }
     float s = 0.f;
     if (valid) {
         const float* p = part + (size_t)layer * nb * kGradEntries + e;
-#pragma unroll 8
-        for (int b = slice; b < nb; b += 8) s += p[(size_t)b * kGradEntries];
+#pragma unroll 10
+        for (int b = slice; b < nb; b += kSumShare) s += p[(size_t)b * kGradEntries];
     }
     sh[slice][tid & 31] = s;
     __syncthreads();
     if (slice != 0 || !valid) return;
     s = sh[0][tid];
 #pragma unroll
-    for (int k = 1; k < 8; ++k) s += sh[k][tid];
+    for (int k = 1; k < kSumShare; ++k) s += sh[k][tid];
     const int j = (layer == 0 ? param_offset(0) : (layer == 1 ? param_offset(1) : param_offset(2))) +
                   (bias ? kOffsets * ci_n * co_n + co : (o * ci_n + ci) * co_n + co);
     grads[j] = s;
@@ -1808,14 +1871,18 @@ struct hpf_prop {
     float* bias = nullptr;        // [3][16]
     float* wpart = nullptr;       // gradient slices [3][grid_wgrad][kGradEntries]
     double* lpart = nullptr;      // loss partials [kLossBlocks]
-    // act[0]: the plain input [V][16] (training only); act[1], act[2]: the
-    // hidden activations in the padded layout [2][Mz + 2][py][px][8]; act[3],
-    // act[4]: gradient buffers [V][16]
-    __nv_bfloat16* act[5] = {};
+    // act[1], act[2]: the hidden activations in the padded layout
+    // [2][Mz + 2][py][px][8]
+    __nv_bfloat16* act[3] = {};
+    // back-propagated gradients of the three layers' outputs, [2][V][8] (the
+    // last layer's second half is zero)
+    __nv_bfloat16* gz[3] = {};
     __nv_bfloat16* act_x = nullptr;  // the input as x-im2col, padded layout
     uint4* tcw = nullptr;            // packed weight images of the data-gradient convolutions
     uint4* sww = nullptr;            // packed weight images of the forward convolutions
     CUtensorMap tmap[3];             // act_x, act[1], act[2]
+    CUtensorMap wmap[3];             // the same, for the weight gradients' boxes
+    CUtensorMap gmap[3];             // gz
     int px = 0, py = 0;              // padded pitches
     int ctas = 1;                    // CTAs of the persistent convolutions (kSwPerSM per SM)
     float* z[2] = {};             // pre-activations of layers 1, 2 [V][16]
@@ -1879,7 +1946,7 @@ void prop_forward(hpf_prop* p, const float* x, const float* phi_next, cudaStream
     const bool train = phi_next != nullptr;
     const int hp = (p->g.mx + 2) * (p->g.my + 2);  // padded voxels per plane
     k_pack_input<<<dim3((unsigned)((hp + 255) / 256), (unsigned)(p->g.mz + 2)), 256, 0, s>>>(
-        x, p->g, p->px, p->py, p->scale, train ? p->act[0] : nullptr, p->act_x, phi_next, p->diff);
+        x, p->g, p->px, p->py, p->scale, p->act_x, phi_next, p->diff);
     SweepArgs a = sweep_args(p, 0, flag);
     a.z_out = train ? p->z[0] : nullptr;
     a.act_out = p->act[1];
@@ -1900,21 +1967,16 @@ void prop_backward(hpf_prop* p, const AdamArgs& adam) {
     const int V = p->g.V, nb = p->grid_wgrad;
     const int lb = (V + 255) / 256 < kLossBlocks ? (V + 255) / 256 : kLossBlocks;
     cudaStream_t s = p->stream;
-    const ActLayout plain{p->g.mx, p->g.my, 0, kPC, 8};
-    const ActLayout padded{p->px, p->py, 1, 8, 8ll * (p->g.mz + 2) * p->py * p->px};
     const size_t slices = (size_t)nb * kGradEntries;
     // the last layer has no activation: its gz is dL/dy
     launch_pdl(k_loss, dim3(lb), dim3(256), 0, s, (const float2*)p->fbuf, (const float2*)p->diff, V,
-               p->scale, p->act[3], p->lpart);
-    launch_pdl(k_conv_wgrad<true>, dim3(nb), dim3(256), 0, s, (const __nv_bfloat16*)p->act[2],
-               (const __nv_bfloat16*)p->act[3], p->wpart + 2 * slices, p->g, padded);
-    launch_conv_tc(p->act[3], p->tcw, 1, p->z[1], p->act[4], p->g, p->flag, s);
-    launch_pdl(k_conv_wgrad<false>, dim3(nb), dim3(256), 0, s, (const __nv_bfloat16*)p->act[1],
-               (const __nv_bfloat16*)p->act[4], p->wpart + slices, p->g, padded);
-    launch_conv_tc(p->act[4], p->tcw, 0, p->z[0], p->act[3], p->g, p->flag, s);
-    launch_pdl(k_conv_wgrad<false>, dim3(nb), dim3(256), 0, s, (const __nv_bfloat16*)p->act[0],
-               (const __nv_bfloat16*)p->act[3], p->wpart, p->g, plain);
-    launch_pdl(k_sum_grads, dim3(kSumBlocks + 1, 3), dim3(256), 0, s, (const float*)p->wpart, nb,
+               p->scale, p->gz[2], p->lpart);
+    launch_conv_wgrad<2>(p->wmap[2], p->gmap[2], p->wpart + 2 * slices, p->g, nb, p->flag, s);
+    launch_conv_tc(p->gz[2], p->tcw, 1, p->z[1], p->gz[1], p->g, p->flag, s);
+    launch_conv_wgrad<1>(p->wmap[1], p->gmap[1], p->wpart + slices, p->g, nb, p->flag, s);
+    launch_conv_tc(p->gz[1], p->tcw, 0, p->z[0], p->gz[0], p->g, p->flag, s);
+    launch_conv_wgrad<0>(p->wmap[0], p->gmap[0], p->wpart, p->g, nb, p->flag, s);
+    launch_pdl(k_sum_grads, dim3(kSumBlocks + 1, 3), dim3(kSumEntries * kSumShare), 0, s, (const float*)p->wpart, nb,
                p->grads, adam, (const double*)p->lpart, lb, p->loss);
 }
 
@@ -2042,8 +2104,8 @@ hpf_status hpf_prop_init(const int32_t mesh[3], void* stream, hpf_prop** out) {
     e = e ? e : cudaMalloc(&p->bias, sizeof(float) * 3 * kPC);
     e = e ? e : cudaMalloc(&p->wpart, sizeof(float) * 3 * (size_t)p->grid_wgrad * kGradEntries);
     e = e ? e : cudaMalloc(&p->lpart, sizeof(double) * kLossBlocks);
-    for (int k = 0; k < 5; ++k)
-        e = e ? e : cudaMalloc(&p->act[k], sizeof(__nv_bfloat16) * (k == 1 || k == 2 ? Vp : Vs) * kPC);
+    for (int k = 1; k < 3; ++k) e = e ? e : cudaMalloc(&p->act[k], sizeof(__nv_bfloat16) * Vp * kPC);
+    for (int k = 0; k < 3; ++k) e = e ? e : cudaMalloc(&p->gz[k], sizeof(__nv_bfloat16) * Vs * kPC);
     for (int k = 0; k < 2; ++k) e = e ? e : cudaMalloc(&p->z[k], sizeof(float) * Vs * kPC);
     e = e ? e : cudaMalloc(&p->fbuf, sizeof(float) * Vs * 2);
     e = e ? e : cudaMalloc(&p->diff, sizeof(float2) * Vs);
@@ -2063,7 +2125,11 @@ hpf_status hpf_prop_init(const int32_t mesh[3], void* stream, hpf_prop** out) {
         cudaMemsetAsync(p->act_x, 0, sizeof(__nv_bfloat16) * Vp * kPC, p->stream);
         cudaMemsetAsync(p->act[1], 0, sizeof(__nv_bfloat16) * Vp * kPC, p->stream);
         cudaMemsetAsync(p->act[2], 0, sizeof(__nv_bfloat16) * Vp * kPC, p->stream);
-        if (!make_act_tensor_map(&p->tmap[0], p->act_x, g) ||
+        cudaMemsetAsync(p->gz[2], 0, sizeof(__nv_bfloat16) * Vs * kPC, p->stream);
+        if (!make_wgrad_tensor_maps(&p->wmap[0], &p->gmap[0], p->act_x, p->gz[0], g) ||
+            !make_wgrad_tensor_maps(&p->wmap[1], &p->gmap[1], p->act[1], p->gz[1], g) ||
+            !make_wgrad_tensor_maps(&p->wmap[2], &p->gmap[2], p->act[2], p->gz[2], g) ||
+            !make_act_tensor_map(&p->tmap[0], p->act_x, g) ||
             !make_act_tensor_map(&p->tmap[1], p->act[1], g) ||
             !make_act_tensor_map(&p->tmap[2], p->act[2], g))
             e = cudaErrorNotSupported;
@@ -2097,7 +2163,10 @@ hpf_status hpf_prop_destroy(hpf_prop* p) {
     cudaFree(p->bias);
     cudaFree(p->wpart);
     cudaFree(p->lpart);
-    for (int k = 0; k < 5; ++k) cudaFree(p->act[k]);
+    for (int k = 0; k < 3; ++k) {
+        cudaFree(p->act[k]);
+        cudaFree(p->gz[k]);
+    }
     for (int k = 0; k < 2; ++k) cudaFree(p->z[k]);
     cudaFree(p->fbuf);
     cudaFree(p->diff);

@@ -99,6 +99,28 @@ def test_forward_matches_oracle(hpf_gpu, mesh):
     assert np.max(np.abs(y - yo)) < 0.1 * np.max(np.abs(yo))
 
 
+@pytest.mark.parametrize("mesh,rep", [((33, 35, 31), 2), ((9, 18, 7), 4)],
+                         ids=["66x70x62", "36x72x28"])
+def test_gradients_of_a_repeated_input(hpf_gpu, mesh, rep):
+    # a periodic input repeated along every axis has the gradients of one copy; on
+    # the larger mesh a weight-gradient CTA takes up to three tiles, ragged ones
+    # among them.  rep^3 is a power of two, so the loss gradient d / V rounds alike
+    # and only the FP32 accumulation order differs: the same bars
+    params = rand_params(3)
+    x = rand_phi(grid(mesh), 4).astype(np.float32)
+    nxt = (x[2:] + 0.1 * rand_phi(grid(mesh), 5, 2)).astype(np.float32)
+    big = tuple(rep * m for m in mesh)
+    with hpf_gpu.Propagator(big) as net:
+        net.set_weights(hpf_gpu.pack_params(params))
+        tile = (1, rep, rep, rep)
+        loss, g = net.backward(np.tile(x, tile), np.tile(nxt, tile))
+    lo, go = E.backward(params, x, nxt)
+    assert abs(loss - lo) < EMU_LOSS * lo
+    for (W, b), (Wo, bo) in zip(hpf_gpu.unpack_params(g), go):
+        within_emulated(W, Wo, "weights")
+        within_emulated(b, bo, "biases")
+
+
 @pytest.mark.parametrize("ctas", [1, 3, 7])
 def test_forward_does_not_depend_on_the_cta_split(hpf_gpu, ctas):
     # few CTAs: long sweeps through many columns, the accumulator ring wrapping
