@@ -22,9 +22,10 @@ struct hpf_ctx {
     StepConsts sc{};
     FieldCoef coef{};
     EnergyConsts ec{};
-    float* state_mem = nullptr;     // 2 x 6 x n floats
+    float* state_mem = nullptr;     // 2 x 6 arrays of bead_stride(n) floats
     StateBuf st[2]{};
     int cur = 0;
+    uint32_t* meta_mem = nullptr;     // 2 arrays of bead_stride(n) words
     uint32_t* meta = nullptr;
     uint32_t* meta2 = nullptr;        // sort target
     SortBufs sb{};
@@ -343,6 +344,11 @@ size_t stage_bytes(int n) {
     return (size_t)n * (3 + 3 + 1 + 2) * 4 + 256;
 }
 
+// The six arrays of one state buffer, from its x to the end of its vz.
+size_t state_bytes(const hpf_ctx* c) {
+    return sizeof(float) * (5 * bead_stride(c->n) + (size_t)c->n);
+}
+
 StateBuf& cur_state(hpf_ctx* c) { return c->st[c->cur]; }
 
 size_t mesh_words(const hpf_ctx* c) { return (size_t)c->geom.nodes * c->S; }
@@ -576,7 +582,11 @@ hpf_status advance(hpf_ctx* c, int chunk, bool fuse, const float4* lerp_G2 = nul
     c->obs_step = -1;
     {
         StageScope sc(c, HPF_STAGE_STEP, c->n > 0 ? 1 : 0);
-        if (c->warp_mode) {
+        if (chunk == 1 && !lerp_G2 && !obs && step_one_supports(c->sc)) {
+            launch_step_one(c->st[c->cur], c->st[c->cur ^ 1], c->meta, c->n, c->step, c->geom, c->G,
+                            c->sc, c->warp_mode, fuse ? mesh_buf(c, c->dmesh ^ 1) : nullptr,
+                            c->dflag, c->stream);
+        } else if (c->warp_mode) {
             // the batch step kernel instantiated for one replica
             SingleStepParams p;
             memset(&p, 0, sizeof p);
@@ -634,7 +644,7 @@ hpf_status advance_nh(hpf_ctx* c, int chunk, bool fuse) {
     {
         StageScope sc(c, HPF_STAGE_STEP, c->n > 0 ? chunk + 1 : 0);
         if (c->n > 0) {
-            const size_t n = (size_t)c->n;
+            const size_t m = bead_stride(c->n);
             NhParams p;
             memset(&p, 0, sizeof p);
             p.meta = c->meta;
@@ -651,8 +661,8 @@ hpf_status advance_nh(hpf_ctx* c, int chunk, bool fuse) {
                 p.in = c->st[c->cur];
                 p.out = c->st[c->cur ^ 1];
                 for (int a = 0; a < 3; ++a) {
-                    p.Fin[a] = c->nh_F + ((size_t)c->nh_f * 3 + a) * n;
-                    p.Fout[a] = c->nh_F + ((size_t)(c->nh_f ^ 1) * 3 + a) * n;
+                    p.Fin[a] = c->nh_F + kBeadPad + ((size_t)c->nh_f * 3 + a) * m;
+                    p.Fout[a] = c->nh_F + kBeadPad + ((size_t)(c->nh_f ^ 1) * 3 + a) * m;
                 }
                 p.kick_drift = kick_drift ? 1 : 0;
                 p.force_kick = force_kick ? 1 : 0;
@@ -794,9 +804,8 @@ hpf_status hpf_init(const hpf_params* params, void* stream, hpf_ctx** out) {
         return s;
     };
     cudaError_t e = cudaSuccess;
-    e = e ? e : cudaMalloc(&c->state_mem, sizeof(float) * 12 * n);
-    e = e ? e : cudaMalloc(&c->meta, sizeof(uint32_t) * n);
-    e = e ? e : cudaMalloc(&c->meta2, sizeof(uint32_t) * n);
+    e = e ? e : cudaMalloc(&c->state_mem, sizeof(float) * 12 * bead_stride(c->n));
+    e = e ? e : cudaMalloc(&c->meta_mem, sizeof(uint32_t) * 2 * bead_stride(c->n));
     const long long K = sort_key_space(c->geom);
     const long long scan_words = scan_scratch_words(K > (long long)n ? K : (long long)n);
     const size_t sort_words = 13 * n + 2 * (n / 256 + 2) + 3 * (size_t)K + (size_t)scan_words + 64;
@@ -818,7 +827,7 @@ hpf_status hpf_init(const hpf_params* params, void* stream, hpf_ctx** out) {
     if (params->thermostat == 1) {
         e = e ? e : cudaMalloc(&c->nh, sizeof(NhDev));
         e = e ? e : cudaMalloc(&c->nh_part, sizeof(double) * (nh_blocks((int)n) + 1));
-        e = e ? e : cudaMalloc(&c->nh_F, sizeof(float) * 6 * n);
+        e = e ? e : cudaMalloc(&c->nh_F, sizeof(float) * 6 * bead_stride(c->n));
         e = e ? e : cudaMallocHost(&c->h_nh, sizeof(double) * 2);
         e = e ? e : cudaMemsetAsync(c->nh, 0, sizeof(NhDev), c->stream);
     }
@@ -850,9 +859,12 @@ hpf_status hpf_init(const hpf_params* params, void* stream, hpf_ctx** out) {
         b.scratch = w;
     }
     for (int b = 0; b < 2; ++b) {
-        float* base = c->state_mem + (size_t)b * 6 * n;
-        c->st[b] = StateBuf{base, base + n, base + 2 * n, base + 3 * n, base + 4 * n, base + 5 * n};
+        const size_t m = bead_stride(c->n);
+        float* base = c->state_mem + (size_t)b * 6 * m + kBeadPad;
+        c->st[b] = StateBuf{base, base + m, base + 2 * m, base + 3 * m, base + 4 * m, base + 5 * m};
     }
+    c->meta = c->meta_mem + kBeadPad;
+    c->meta2 = c->meta + bead_stride(c->n);
     if (cudaMemcpyAsync(c->d_coef, &c->coef, sizeof(FieldCoef), cudaMemcpyHostToDevice,
                         c->stream) != cudaSuccess ||
         cudaStreamSynchronize(c->stream) != cudaSuccess ||
@@ -874,8 +886,7 @@ hpf_status hpf_destroy(hpf_ctx* c) {
     }
     for (auto e : c->ev_free) cudaEventDestroy(e);
     cudaFree(c->state_mem);
-    cudaFree(c->meta);
-    cudaFree(c->meta2);
+    cudaFree(c->meta_mem);
     cudaFree(c->sort_mem);
     cudaFree(c->D);
     cudaFree(c->G);
@@ -1916,7 +1927,7 @@ hpf_status ensure_learned(hpf_ctx* c) {
     e = e ? e : cudaMalloc(&L->Dp, sizeof(unsigned long long) * S * M);
     e = e ? e : cudaMalloc(&L->x, sizeof(float) * xs * M);
     e = e ? e : cudaMalloc(&L->dphi, sizeof(float) * S * M);
-    e = e ? e : cudaMalloc(&L->snap, sizeof(float) * 6 * (size_t)(c->n > 0 ? c->n : 1));
+    e = e ? e : cudaMalloc(&L->snap, sizeof(float) * 6 * bead_stride(c->n));
     e = e ? e : cudaMalloc(&L->acc, sizeof(double) * (2 + 2 * (size_t)force_error_partials()));
     e = e ? e : cudaMallocHost(&L->h_acc, sizeof(double) * 2);
     e = e ? e : cudaMalloc(&L->G2, sizeof(float4) * S * (size_t)c->geom.gnodes);
@@ -2145,7 +2156,7 @@ hpf_status hpf_step_learned(hpf_ctx* c, hpf_prop* prop, int32_t n_windows, int32
         double eps = 0.0;
         if (have_hist && !skip && !L->plain_mode) {
             // learned window: steps t .. t+K-1 on predicted densities
-            CUDA_TRY(c, cudaMemcpyAsync(L->snap, cur_state(c).x, sizeof(float) * 6 * c->n,
+            CUDA_TRY(c, cudaMemcpyAsync(L->snap, cur_state(c).x, state_bytes(c),
                                         cudaMemcpyDeviceToDevice, c->stream));
             if (L->tmap_tile != c->field_tile) {
                 L->tmap_ok = make_mesh_tensor_map(&L->tmap,
@@ -2196,7 +2207,7 @@ hpf_status hpf_step_learned(hpf_ctx* c, hpf_prop* prop, int32_t n_windows, int32
             } else {
                 // roll back to t and take the plain update instead
                 st.rejected += 1;
-                CUDA_TRY(c, cudaMemcpyAsync(cur_state(c).x, L->snap, sizeof(float) * 6 * c->n,
+                CUDA_TRY(c, cudaMemcpyAsync(cur_state(c).x, L->snap, state_bytes(c),
                                             cudaMemcpyDeviceToDevice, c->stream));
                 c->step = t;
                 c->field_valid = false;

@@ -5,6 +5,7 @@
 //             (ping-pong) because the step kernel reads neighbours' old positions
 //   meta    : uint32 per bead = tag (24 bits) | species (3 bits) << 24
 //             | bonded-to-previous << 27 | bonded-to-next << 28
+//             | second bead of its lane in a warp segment << 29
 //   D       : int64 density [S][Mz][My][Mx], fixed point with 2^39 per bead
 //   G       : float4 field  [S][Mz+1][My+1][Mx+1] = (dV/dx, dV/dy, dV/dz, V), with one
 //             periodic ghost layer per axis so a cell's upper corner is always lo + 1
@@ -29,6 +30,7 @@ constexpr int kTypeShift = 24;
 constexpr uint32_t kTypeMask = 0x7u;
 constexpr uint32_t kBondPrev = 1u << 27;
 constexpr uint32_t kBondNext = 1u << 28;
+constexpr uint32_t kSlotOdd = 1u << 29;
 constexpr int kFrac = HPF_FRAC_BITS;
 constexpr int kOne = 1 << kFrac;
 constexpr float kCoordLimit = 262144.0f;  // |mesh coordinate| < 2^18 keeps 2^13 s in int32
@@ -37,6 +39,12 @@ constexpr float kCoordLimit = 262144.0f;  // |mesh coordinate| < 2^18 keeps 2^13
 constexpr int kFlagNonFinite = 1;
 constexpr int kFlagRange = 2;
 constexpr int kFlagTimeout = 4;
+
+// Per-bead arrays start kBeadPad elements into their allocation and are
+// bead_stride(n) elements apart: whole chunks of beads with their halo can be
+// copied without bounds checks (chunk_pipe.cuh), and every array is 64-byte aligned.
+constexpr int kBeadPad = 16;
+inline size_t bead_stride(int n) { return (size_t)((n + 255) / 256) * 256 + 2 * kBeadPad; }
 
 struct MeshGeom {
     int mx, my, mz;
@@ -398,30 +406,49 @@ __device__ __forceinline__ void scatter_bead(unsigned long long* __restrict__ Dt
 }
 
 // -trilinear interpolation of the nodal gradient of one species (ghosted
-// field array: the eight corners are base + {0, 1} + {0, gx} + {0, gxy}).
+// field array: the eight corners are base + {0, 1} + {0, gx} + {0, gxy}), in
+// two parts so that a kernel can have the loads in flight during other work.
+struct FieldCorners {
+    float4 c000, c001, c010, c011, c100, c101, c110, c111;  // z, y, x
+};
+
+__device__ __forceinline__ FieldCorners load_field(const float4* __restrict__ Gt, const MeshGeom& g,
+                                                   const AxisCoord& ax, const AxisCoord& ay,
+                                                   const AxisCoord& az) {
+    const int o00 = az.lo * g.gxy + ay.lo * g.gx + ax.lo;
+    const int o01 = o00 + g.gx, o10 = o00 + g.gxy, o11 = o10 + g.gx;
+    FieldCorners k;
+    k.c000 = __ldg(Gt + o00);
+    k.c001 = __ldg(Gt + o00 + 1);
+    k.c010 = __ldg(Gt + o01);
+    k.c011 = __ldg(Gt + o01 + 1);
+    k.c100 = __ldg(Gt + o10);
+    k.c101 = __ldg(Gt + o10 + 1);
+    k.c110 = __ldg(Gt + o11);
+    k.c111 = __ldg(Gt + o11 + 1);
+    return k;
+}
+
+__device__ __forceinline__ void apply_field(const FieldCorners& k, float wx1, float wy1, float wz1,
+                                            float& fx, float& fy, float& fz) {
+    const float wx0 = 1.0f - wx1, wy0 = 1.0f - wy1, wz0 = 1.0f - wz1;
+    const float w00 = wz0 * wy0, w01 = wz0 * wy1, w10 = wz1 * wy0, w11 = wz1 * wy1;
+    float gx = w00 * (wx0 * k.c000.x + wx1 * k.c001.x) + w01 * (wx0 * k.c010.x + wx1 * k.c011.x) +
+               w10 * (wx0 * k.c100.x + wx1 * k.c101.x) + w11 * (wx0 * k.c110.x + wx1 * k.c111.x);
+    float gy = w00 * (wx0 * k.c000.y + wx1 * k.c001.y) + w01 * (wx0 * k.c010.y + wx1 * k.c011.y) +
+               w10 * (wx0 * k.c100.y + wx1 * k.c101.y) + w11 * (wx0 * k.c110.y + wx1 * k.c111.y);
+    float gz = w00 * (wx0 * k.c000.z + wx1 * k.c001.z) + w01 * (wx0 * k.c010.z + wx1 * k.c011.z) +
+               w10 * (wx0 * k.c100.z + wx1 * k.c101.z) + w11 * (wx0 * k.c110.z + wx1 * k.c111.z);
+    fx -= gx;
+    fy -= gy;
+    fz -= gz;
+}
+
 __device__ __forceinline__ void gather_field(const float4* __restrict__ Gt, const MeshGeom& g,
                                              const AxisCoord& ax, const AxisCoord& ay,
                                              const AxisCoord& az, float& fx, float& fy,
                                              float& fz) {
-    const float wx1 = ax.f, wx0 = 1.0f - ax.f;
-    const float wy1 = ay.f, wy0 = 1.0f - ay.f;
-    const float wz1 = az.f, wz0 = 1.0f - az.f;
-    const int o00 = az.lo * g.gxy + ay.lo * g.gx + ax.lo;
-    const int o01 = o00 + g.gx, o10 = o00 + g.gxy, o11 = o10 + g.gx;
-    const float4 c000 = __ldg(Gt + o00), c001 = __ldg(Gt + o00 + 1);
-    const float4 c010 = __ldg(Gt + o01), c011 = __ldg(Gt + o01 + 1);
-    const float4 c100 = __ldg(Gt + o10), c101 = __ldg(Gt + o10 + 1);
-    const float4 c110 = __ldg(Gt + o11), c111 = __ldg(Gt + o11 + 1);
-    const float w00 = wz0 * wy0, w01 = wz0 * wy1, w10 = wz1 * wy0, w11 = wz1 * wy1;
-    float gx = w00 * (wx0 * c000.x + wx1 * c001.x) + w01 * (wx0 * c010.x + wx1 * c011.x) +
-               w10 * (wx0 * c100.x + wx1 * c101.x) + w11 * (wx0 * c110.x + wx1 * c111.x);
-    float gy = w00 * (wx0 * c000.y + wx1 * c001.y) + w01 * (wx0 * c010.y + wx1 * c011.y) +
-               w10 * (wx0 * c100.y + wx1 * c101.y) + w11 * (wx0 * c110.y + wx1 * c111.y);
-    float gz = w00 * (wx0 * c000.z + wx1 * c001.z) + w01 * (wx0 * c010.z + wx1 * c011.z) +
-               w10 * (wx0 * c100.z + wx1 * c101.z) + w11 * (wx0 * c110.z + wx1 * c111.z);
-    fx -= gx;
-    fy -= gy;
-    fz -= gz;
+    apply_field(load_field(Gt, g, ax, ay, az), ax.f, ay.f, az.f, fx, fy, fz);
 }
 
 // The exact derivative of the CIC field energy at a bead: minus the gradient
@@ -644,16 +671,31 @@ __host__ __device__ __forceinline__ BondFF bond_ff(const EnergyConsts& e) {
 
 // Harmonic bond U = k (r - r0)^2 seen from bead i: F_i += -2k (1 - r0 / r) d, d = x_i - x_j,
 // with 1 / r from the hardware reciprocal square root (2 ulp: about 1e-6 of a
-// typical bond force).
+// typical bond force).  kOrder fixes the rounding of |d|^2 where two kernels
+// have to form the same bits: kLaneBond the bond between the two beads of a
+// lane of the warp form, kCrossBond the one to the next lane's first bead (the
+// two orders are the ones every release of the warp kernel has had); 0 leaves
+// it to the compiler.
+constexpr int kLaneBond = 1, kCrossBond = 2;
+template <int kOrder = 0>
 __device__ __forceinline__ void bond_force(float dx, float dy, float dz, float two_k, float r0,
                                            float& fx, float& fy, float& fz) {
+    float rr = dx * dx + dy * dy + dz * dz;
+    if (kOrder == kLaneBond) rr = fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
+    if (kOrder == kCrossBond) rr = fmaf(dz, dz, fmaf(dx, dx, __fmul_rn(dy, dy)));
     // r^2 is clamped so that a masked bond (two_k = 0, zero vector) adds exactly zero
-    const float r2 = fmaxf(dx * dx + dy * dy + dz * dz, 1e-30f);
+    const float r2 = fmaxf(rr, 1e-30f);
     const float ir = rsqrtf(r2);
     const float s = -two_k * fmaf(-r0, ir, 1.0f);
-    fx += s * dx;
-    fy += s * dy;
-    fz += s * dz;
+    if (kOrder != 0) {  // a share on its own: rounded before it is summed
+        fx = __fmul_rn(s, dx);
+        fy = __fmul_rn(s, dy);
+        fz = __fmul_rn(s, dz);
+    } else {
+        fx += s * dx;
+        fy += s * dy;
+        fz += s * dz;
+    }
 }
 
 // Angle at a middle bead j with u = x_a - x_j, w = x_b - x_j: forces on the
@@ -840,12 +882,22 @@ __device__ __forceinline__ void warp_bonded_forces(float x0, float y0, float z0,
     const float dy = __shfl_down_sync(0xffffffffu, y0, 1);
     const float dz = __shfl_down_sync(0xffffffffu, z0, 1);
     float ax = 0.f, ay = 0.f, az = 0.f;  // on bead 2l from bead 2l + 1
-    bond_force(x0 - x1, y0 - y1, z0 - z1, n0 ? c.two_k : 0.0f, c.r0, ax, ay, az);
+    constexpr int kIn = kBonded == 0 ? kLaneBond : 0, kOut = kBonded == 0 ? kCrossBond : 0;
+    bond_force<kIn>(x0 - x1, y0 - y1, z0 - z1, n0 ? c.two_k : 0.0f, c.r0, ax, ay, az);
     float nx = 0.f, ny = 0.f, nz = 0.f;  // on bead 2l + 1 from bead 2l + 2
-    bond_force(x1 - dx, y1 - dy, z1 - dz, n1 ? c.two_k : 0.0f, c.r0, nx, ny, nz);
+    bond_force<kOut>(x1 - dx, y1 - dy, z1 - dz, n1 ? c.two_k : 0.0f, c.r0, nx, ny, nz);
     const float ux = __shfl_up_sync(0xffffffffu, nx, 1);  // previous lane's share
     const float uy = __shfl_up_sync(0xffffffffu, ny, 1);
     const float uz = __shfl_up_sync(0xffffffffu, nz, 1);
+    if (kBonded == 0) {
+        w0x = p0 ? __fsub_rn(ax, ux) : ax;
+        w0y = p0 ? __fsub_rn(ay, uy) : ay;
+        w0z = p0 ? __fsub_rn(az, uz) : az;
+        w1x = __fsub_rn(nx, ax);
+        w1y = __fsub_rn(ny, ay);
+        w1z = __fsub_rn(nz, az);
+        return;
+    }
     // angles, each evaluated once by the lane of its middle bead: at bead 2l
     // (ends 2l - 1, 2l + 1) and at bead 2l + 1 (ends 2l, 2l + 2); the shares
     // of the end beads held by the neighbouring lanes go there by one shuffle
@@ -975,6 +1027,12 @@ int launch_sort(const SortBufs& b, StateBuf in, StateBuf out, const uint32_t* me
                 uint32_t* meta_out, int n, int C, MeshGeom g, cudaStream_t s);
 
 int step_halo_max();
+// One step of a single context, one bead per thread (k_one.cu): the bits of
+// the warp form, or of the halo form.  Bonds only, force_mode 0.
+bool step_one_supports(const StepConsts& c);
+void launch_step_one(StateBuf in, StateBuf out, const uint32_t* meta, int n, long long step,
+                     const MeshGeom& g, const float4* G, const StepConsts& c, bool warp_order,
+                     unsigned long long* D_next, int* flag, cudaStream_t s);
 void launch_step_warp_batch(const BatchStepParams& p, int max_seg_total, int therm,
                             cudaStream_t s);
 // A single context's launch that also writes the observables' bead partials

@@ -12,7 +12,7 @@
 // tile shape is chosen per mesh by timing the candidates (hpf_api.cu).
 #include <cuda.h>
 
-#include "hpf_internal.cuh"
+#include "chunk_pipe.cuh"
 
 namespace hpf {
 
@@ -26,8 +26,6 @@ constexpr int kTileShapes[kTileCandidates][3] = {
     {32, 8, 4}, {32, 8, 8}, {16, 16, 4}, {64, 4, 4}, {16, 16, 8}, {32, 4, 8}, {0, 0, 0},
     {2, 1, 1}};
 constexpr int kPairTile = 7;
-constexpr unsigned kWaitLimit = 1u << 22;          // polls of an mbarrier before giving up
-constexpr unsigned long long kWaitNs = 200000000ull;  // or 0.2 s, whichever comes first
 
 int field_tile_candidates() { return kTileCandidates; }
 
@@ -42,35 +40,6 @@ size_t field_tile_smem(int id, int S) {
 }
 
 bool field_tile_is_plain(int id) { return kTileShapes[id][0] == 0 || id == kPairTile; }
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Returns false if the barrier did not complete within kWaitLimit polls or
-// kWaitNs nanoseconds (a tensor copy completes within microseconds).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    const unsigned long long t0 = global_ns();
-    for (unsigned it = 0; it < kWaitLimit; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if ((it & 63) == 63 && global_ns() - t0 > kWaitNs) return false;
-    }
-    return false;
-}
 
 // Self-test of the bounded wait: an mbarrier nothing ever arrives on (no
 // copy is issued), so the wait must give up, raise the timeout flag and

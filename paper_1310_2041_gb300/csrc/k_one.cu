@@ -1,0 +1,189 @@
+// k_one.cu -- one step per launch: the step kernel of schedules that refresh
+// the field every step, one bead per thread.
+//
+// The field-period kernels (k_step.cu) keep beads on chip over many steps and
+// pay for it once per launch: a segment's beads, their cell polynomials in
+// shared memory, two CTAs of 256 threads per SM.  A single step amortises none
+// of that, and the chain segment -> state -> corners of dependent loads at 16
+// warps per SM was what such a launch took its time for.  Here the beads
+// stream through shared memory ahead of their use (chunk_pipe.cuh), the eight
+// corner loads of a bead are in flight while its noise and bonds are formed,
+// and the polynomial stays in registers.  The arithmetic, operation by
+// operation, is that of the field-period kernels: kWarp takes the order of
+// the warp form's bond sums, else that of the halo form, so that a run gives
+// the same bits whichever kernel its steps go through.
+#include "cell_poly.cuh"
+#include "chunk_pipe.cuh"
+
+namespace hpf {
+
+namespace {
+
+constexpr int kOneArrays = 7;  // x y z vx vy vz meta
+constexpr int kOnePerSM = 3;    // resident CTAs (80 registers; four, at 64, spill)
+
+struct OneParams {
+    const void* src[kOneArrays];
+    StateBuf out;
+    int n;
+    long long step;
+    MeshGeom g;
+    const float4* G;
+    StepConsts c;
+    unsigned long long* D_next;
+    int* flag;
+};
+
+template <int kTherm, bool kWarp>
+__global__ void __launch_bounds__(kChunk, kOnePerSM) k_step_one(const __grid_constant__ OneParams p) {
+    __shared__ __align__(128) float smem[kChunkStages * kOneArrays * kSpan];
+    __shared__ __align__(8) unsigned long long bars[kChunkStages];
+    const int tid = threadIdx.x;
+    ChunkPipe<kOneArrays> pipe;
+    pipe.begin(smem, bars, p.n);
+    griddep_wait();
+    griddep_launch_dependents();
+    const void* src = nullptr;
+    if (tid < kOneArrays) src = p.src[tid];
+    if (tid < 32) {
+        __syncwarp();
+        for (int i = 0; i < kChunkStages && i < pipe.count; ++i) pipe.issue(i, src);
+    }
+    __syncthreads();  // the barriers are initialised
+    const MeshGeom& g = p.g;
+    const StepConsts& c = p.c;
+    for (int i = 0; i < pipe.count; ++i) {
+        const bool ok = pipe.wait(i);
+        const float(*s)[kSpan] = pipe.stage[i % kChunkStages];
+        const int bead = pipe.bead0(i) + tid, e = tid + kChunkHalo;
+        if (ok && bead < p.n) {
+            float x = s[0][e], y = s[1][e], z = s[2][e];
+            float vx = s[3][e], vy = s[4][e], vz = s[5][e];
+            const uint32_t m = __float_as_uint(s[6][e]);
+            const float s0 = __fmul_rn(x, g.inv_h[0]), s1 = __fmul_rn(y, g.inv_h[1]),
+                        s2 = __fmul_rn(z, g.inv_h[2]);
+            const float flx = floorf(s0), fly = floorf(s1), flz = floorf(s2);
+            const Corners k = load_corners(p.G + (size_t)((m >> kTypeShift) & kTypeMask) * g.gnodes,
+                                           g, flx, fly, flz);
+            // while they arrive: the chain neighbours' bonds and the noise
+            float nx = 0.f, ny = 0.f, nz = 0.f, qx = 0.f, qy = 0.f, qz = 0.f;
+            if (kWarp) {
+                // one bond of a bead lies inside its lane, the other crosses lanes
+                const bool odd = (m & kSlotOdd) != 0;
+                const float ax = x - s[0][e + 1], ay = y - s[1][e + 1], az = z - s[2][e + 1];
+                const float bx = s[0][e - 1] - x, by = s[1][e - 1] - y, bz = s[2][e - 1] - z;
+                if (odd) {
+                    if (m & kBondNext) bond_force<kCrossBond>(ax, ay, az, c.two_k, c.r0, nx, ny, nz);
+                    if (m & kBondPrev) bond_force<kLaneBond>(bx, by, bz, c.two_k, c.r0, qx, qy, qz);
+                } else {
+                    if (m & kBondNext) bond_force<kLaneBond>(ax, ay, az, c.two_k, c.r0, nx, ny, nz);
+                    if (m & kBondPrev) bond_force<kCrossBond>(bx, by, bz, c.two_k, c.r0, qx, qy, qz);
+                }
+                nx = __fsub_rn(nx, qx);
+                ny = __fsub_rn(ny, qy);
+                nz = __fsub_rn(nz, qz);
+            }
+            const uint32_t tag = m & kTagMask;
+            float gx = 0.f, gy = 0.f, gz = 0.f;
+            bool coll = false;
+            if (kTherm == 1) gauss3(c, tag, p.step, gx, gy, gz);
+            if (kTherm == 2) {
+                coll = andersen_collides(c, tag, p.step);
+                if (coll) gauss3(c, tag, p.step, gx, gy, gz);
+            }
+            const float f0 = __fsub_rn(s0, flx), f1 = __fsub_rn(s1, fly), f2 = __fsub_rn(s2, flz);
+            float fx = -c.fric * vx, fy = -c.fric * vy, fz = -c.fric * vz;
+            float4 lo, hi;
+            cell_coefs(HPF_CORNERS(k, x), lo, hi);
+            fx -= cell_poly(lo, hi, f0, f1, f2);
+            cell_coefs(HPF_CORNERS(k, y), lo, hi);
+            fy -= cell_poly(lo, hi, f0, f1, f2);
+            cell_coefs(HPF_CORNERS(k, z), lo, hi);
+            fz -= cell_poly(lo, hi, f0, f1, f2);
+            if (kTherm == 1) {
+                fx = fmaf(c.sigma, gx, fx);
+                fy = fmaf(c.sigma, gy, fy);
+                fz = fmaf(c.sigma, gz, fz);
+            }
+            if (kWarp) {
+                fx += nx;
+                fy += ny;
+                fz += nz;
+            } else {
+                if (m & kBondPrev)
+                    bond_force(x - s[0][e - 1], y - s[1][e - 1], z - s[2][e - 1], c.two_k, c.r0, fx,
+                               fy, fz);
+                if (m & kBondNext)
+                    bond_force(x - s[0][e + 1], y - s[1][e + 1], z - s[2][e + 1], c.two_k, c.r0, fx,
+                               fy, fz);
+            }
+            if (kTherm == 2 && coll) {
+                const float h = 0.5f * c.dt_m;
+                vx = fmaf(h, fx, c.sig_v * gx);
+                vy = fmaf(h, fy, c.sig_v * gy);
+                vz = fmaf(h, fz, c.sig_v * gz);
+            } else {
+                vx = fmaf(c.dt_m, fx, vx);
+                vy = fmaf(c.dt_m, fy, vy);
+                vz = fmaf(c.dt_m, fz, vz);
+            }
+            x = fmaf(c.dt, vx, x);
+            y = fmaf(c.dt, vy, y);
+            z = fmaf(c.dt, vz, z);
+            p.out.x[bead] = x;
+            p.out.y[bead] = y;
+            p.out.z[bead] = z;
+            p.out.vx[bead] = vx;
+            p.out.vy[bead] = vy;
+            p.out.vz[bead] = vz;
+            const bool finite = isfinite(x) && isfinite(y) && isfinite(z) && isfinite(vx) &&
+                                isfinite(vy) && isfinite(vz);
+            if (!finite) atomicOr(p.flag, kFlagNonFinite);
+            else if (!(coord_in_range(x, g.inv_h[0]) && coord_in_range(y, g.inv_h[1]) &&
+                       coord_in_range(z, g.inv_h[2])))
+                atomicOr(p.flag, kFlagRange);
+            if (p.D_next) {
+                const AxisCoord ax = axis_coord(x, g.inv_h[0], g.mx, g.inv_m[0]);
+                const AxisCoord ay = axis_coord(y, g.inv_h[1], g.my, g.inv_m[1]);
+                const AxisCoord az = axis_coord(z, g.inv_h[2], g.mz, g.inv_m[2]);
+                scatter_bead(p.D_next + (size_t)((m >> kTypeShift) & kTypeMask) * g.nodes, g, ax, ay,
+                             az);
+            }
+        }
+        if (__syncthreads_or(!ok)) {  // every thread is done with the stage
+            if (tid == 0) atomicOr(p.flag, kFlagTimeout);
+            pipe.drain(i);
+            return;
+        }
+        if (tid < 32 && i + kChunkStages < pipe.count) pipe.issue(i + kChunkStages, src);
+    }
+}
+
+}  // namespace
+
+bool step_one_supports(const StepConsts& c) { return c.force_mode == 0 && bonded_level(c) == 0; }
+
+void launch_step_one(StateBuf in, StateBuf out, const uint32_t* meta, int n, long long step,
+                     const MeshGeom& g, const float4* G, const StepConsts& c, bool warp_order,
+                     unsigned long long* D_next, int* flag, cudaStream_t s) {
+    if (n <= 0) return;
+    static std::once_flag once[64];
+    static int sms[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    once_per_device(once, [dev] {
+        cudaDeviceGetAttribute(&sms[dev & 63], cudaDevAttrMultiProcessorCount, dev);
+    });
+    const int chunks = (n + kChunk - 1) / kChunk, cap = kOnePerSM * (sms[dev & 63] > 0 ? sms[dev & 63] : 1);
+    const int blocks = chunks < cap ? chunks : cap;
+    const OneParams p{{in.x, in.y, in.z, in.vx, in.vy, in.vz, meta}, out, n, step, g, G, c, D_next,
+                      flag};
+    const int th = step_thermostat(c);
+#define HPF_ONE(T, W) launch_pdl(k_step_one<T, W>, dim3(blocks), dim3(kChunk), 0, s, p)
+    if (th == 1) warp_order ? HPF_ONE(1, true) : HPF_ONE(1, false);
+    else if (th == 2) warp_order ? HPF_ONE(2, true) : HPF_ONE(2, false);
+    else warp_order ? HPF_ONE(0, true) : HPF_ONE(0, false);
+#undef HPF_ONE
+}
+
+}  // namespace hpf

@@ -258,6 +258,20 @@ __global__ void k_gather_segments(const int* __restrict__ tmp_start,
     if (slot == 0) *n_seg = (int)(chunk_off[n_chunks - 1] + chunk_nseg[n_chunks - 1]);
 }
 
+// Marks the second bead of every lane of the warp form (a lane of a segment
+// holds beads 2l and 2l + 1), one warp per segment: the one-step kernel
+// (k_one.cu) rounds a bond as the warp form does by it.
+__global__ void k_mark_slots(const int* __restrict__ seg_start, const int* __restrict__ seg_count,
+                             const int* __restrict__ n_seg, uint32_t* __restrict__ meta) {
+    const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (w >= *n_seg) return;
+    const int start = seg_start[w], count = seg_count[w];
+    for (int j = lane; j < count; j += 32) {
+        const uint32_t m = meta[start + j];
+        meta[start + j] = (j & 1) ? m | kSlotOdd : m & ~kSlotOdd;
+    }
+}
+
 // ------------------------------------------------------------------ host side
 
 long long sort_key_space(const MeshGeom& g) {
@@ -309,7 +323,8 @@ int launch_sort(const SortBufs& b, StateBuf in, StateBuf out, const uint32_t* me
         launched += 1 + scan_exclusive(b.chunk_nseg, b.chunk_off, n_chunks, b.scratch, s);
         k_gather_segments<<<cb, 256, 0, s>>>(b.seg_tmp, b.seg_tmp + C, b.chunk_nseg, b.chunk_off,
                                              C, n_chunks, b.seg_start, b.seg_count, b.n_seg);
-        ++launched;
+        k_mark_slots<<<(C + 7) / 8, 256, 0, s>>>(b.seg_start, b.seg_count, b.n_seg, meta_out);
+        launched += 2;
     }
     return launched;
 }

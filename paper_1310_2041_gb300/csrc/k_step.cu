@@ -1,5 +1,5 @@
 // k_step.cu -- field gather, bonds, Langevin velocity-Verlet (the fused field-period kernels).
-#include "hpf_internal.cuh"
+#include "cell_poly.cuh"
 
 namespace hpf {
 
@@ -71,65 +71,19 @@ constexpr int kCachePlanes = 6;
 constexpr size_t kStepSmem = sizeof(float4) * kCachePlanes * kStepBlock +
                              sizeof(float) * 3 * 2 * kStepBlock;
 
-// Ghosted-array index of the lower corner of cell (flx, fly, flz) (periodic
-// image; see axis_gather for why no fix-up is needed).
-__device__ __forceinline__ int cell_base(const MeshGeom& g, float flx, float fly, float flz) {
-    const float fmx = (float)g.mx, fmy = (float)g.my, fmz = (float)g.mz;
-    float wx = __fmaf_rn(-fmx, floorf((flx + 0.5f) * g.inv_m[0]), flx);
-    float wy = __fmaf_rn(-fmy, floorf((fly + 0.5f) * g.inv_m[1]), fly);
-    float wz = __fmaf_rn(-fmz, floorf((flz + 0.5f) * g.inv_m[2]), flz);
-    wx = fminf(fmaxf(wx, 0.0f), fmx - 1.0f);
-    wy = fminf(fmaxf(wy, 0.0f), fmy - 1.0f);
-    wz = fminf(fmaxf(wz, 0.0f), fmz - 1.0f);
-    return (int)wz * g.gxy + (int)wy * g.gx + (int)wx;
-}
-
-// The eight corners (x, y, z offsets in {0, 1}) of cell (flx, fly, flz).
-struct Corners {
-    float4 g000, g100, g010, g110, g001, g101, g011, g111;
-};
-
-__device__ __forceinline__ Corners load_corners(const float4* __restrict__ Gt, const MeshGeom& g,
-                                                float flx, float fly, float flz) {
-    const int o00 = cell_base(g, flx, fly, flz);
-    const int o01 = o00 + g.gx, o10 = o00 + g.gxy, o11 = o10 + g.gx;
-    Corners k;
-    k.g000 = __ldg(Gt + o00);
-    k.g100 = __ldg(Gt + o00 + 1);
-    k.g010 = __ldg(Gt + o01);
-    k.g110 = __ldg(Gt + o01 + 1);
-    k.g001 = __ldg(Gt + o10);
-    k.g101 = __ldg(Gt + o10 + 1);
-    k.g011 = __ldg(Gt + o11);
-    k.g111 = __ldg(Gt + o11 + 1);
-    return k;
-}
-
 // The cell polynomial's coefficients from its corners into cache slot t
 // (component-major: planes 2j, 2j + 1 hold c0..c7 of component j; kForce 1:
 // planes 0 and 1 hold the polynomial of V).
 template <int kForce>
 __device__ __forceinline__ void store_cell_coefs(const Corners& k, float4* __restrict__ cache, int t,
                                                  int stride) {
-#define HPF_COEF(comp, j)                                                                        \
-    {                                                                                            \
-        const float a0 = k.g000.comp, a1 = k.g100.comp - k.g000.comp;                            \
-        const float a2 = k.g010.comp - k.g000.comp, a3 = k.g001.comp - k.g000.comp;              \
-        const float a4 = (k.g110.comp - k.g100.comp) - a2;                                       \
-        const float a5 = (k.g101.comp - k.g100.comp) - a3;                                       \
-        const float a6 = (k.g011.comp - k.g010.comp) - a3;                                       \
-        const float a7 = ((k.g111.comp - k.g110.comp) - (k.g101.comp - k.g100.comp)) - a6;       \
-        cache[(2 * j) * stride + t] = make_float4(a0, a1, a2, a3);                               \
-        cache[(2 * j + 1) * stride + t] = make_float4(a4, a5, a6, a7);                           \
-    }
     if (kForce == 1) {
-        HPF_COEF(w, 0)
+        cell_coefs(HPF_CORNERS(k, w), cache[t], cache[stride + t]);
     } else {
-        HPF_COEF(x, 0)
-        HPF_COEF(y, 1)
-        HPF_COEF(z, 2)
+        cell_coefs(HPF_CORNERS(k, x), cache[t], cache[stride + t]);
+        cell_coefs(HPF_CORNERS(k, y), cache[2 * stride + t], cache[3 * stride + t]);
+        cell_coefs(HPF_CORNERS(k, z), cache[4 * stride + t], cache[5 * stride + t]);
     }
-#undef HPF_COEF
 }
 
 // kForce 1: planes 0 and 1 hold the trilinear polynomial of V instead (the
@@ -155,19 +109,6 @@ __device__ __forceinline__ void fill_cell_cache(const float4* __restrict__ Gt, c
 template <int kForce>
 __device__ __forceinline__ float cache_key(float s) {
     return kForce == 2 ? stag_vertex(s) : floorf(s);
-}
-
-// -(trilinear polynomial) of the cached cell at offset (fx, fy, fz).
-__device__ __forceinline__ float cell_poly(const float4 lo, const float4 hi, float fx, float fy,
-                                           float fz) {
-    // lo = (c0, c1, c2, c3), hi = (c4, c5, c6, c7)
-    float a = fmaf(fz, hi.w, hi.x);
-    a = fmaf(fy, a, lo.y);
-    a = fmaf(fz, hi.y, a);
-    const float b = fmaf(fz, hi.z, lo.z);
-    float v = fmaf(fx, a, lo.x);
-    v = fmaf(fy, b, v);
-    return fmaf(fz, lo.w, v);
 }
 
 template <int kForce>
