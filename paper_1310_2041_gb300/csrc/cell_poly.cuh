@@ -24,20 +24,23 @@ struct Corners {
     float4 g000, g100, g010, g110, g001, g101, g011, g111;
 };
 
+// q: the cell's lower corner in the ghosted field array of one species.
+__device__ __forceinline__ Corners load_corners_at(const float4* __restrict__ q, const MeshGeom& g) {
+    Corners k;
+    k.g000 = __ldg(q);
+    k.g100 = __ldg(q + 1);
+    k.g010 = __ldg(q + g.gx);
+    k.g110 = __ldg(q + g.gx + 1);
+    k.g001 = __ldg(q + g.gxy);
+    k.g101 = __ldg(q + g.gxy + 1);
+    k.g011 = __ldg(q + g.gxy + g.gx);
+    k.g111 = __ldg(q + g.gxy + g.gx + 1);
+    return k;
+}
+
 __device__ __forceinline__ Corners load_corners(const float4* __restrict__ Gt, const MeshGeom& g,
                                                 float flx, float fly, float flz) {
-    const int o00 = cell_base(g, flx, fly, flz);
-    const int o01 = o00 + g.gx, o10 = o00 + g.gxy, o11 = o10 + g.gx;
-    Corners k;
-    k.g000 = __ldg(Gt + o00);
-    k.g100 = __ldg(Gt + o00 + 1);
-    k.g010 = __ldg(Gt + o01);
-    k.g110 = __ldg(Gt + o01 + 1);
-    k.g001 = __ldg(Gt + o10);
-    k.g101 = __ldg(Gt + o10 + 1);
-    k.g011 = __ldg(Gt + o11);
-    k.g111 = __ldg(Gt + o11 + 1);
-    return k;
+    return load_corners_at(Gt + cell_base(g, flx, fly, flz), g);
 }
 
 // One component's polynomial c0 + c1 fx + c2 fy + c3 fz + c4 fx fy + c5 fx fz

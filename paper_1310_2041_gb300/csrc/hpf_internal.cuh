@@ -385,23 +385,25 @@ __device__ __forceinline__ bool coord_in_range(float x, float inv_h) {
     return fabsf(s) < kCoordLimit;
 }
 
-// Add one bead's eight fixed-point CIC weights to its species' mesh.
+// Add one bead's eight fixed-point CIC weights to its species' mesh.  A weight
+// is a product of three 13-bit numbers: the first two fit 32 bits, the third
+// factor one widening multiply.
 __device__ __forceinline__ void scatter_bead(unsigned long long* __restrict__ Dt, const MeshGeom& g,
                                              const AxisCoord& ax, const AxisCoord& ay,
                                              const AxisCoord& az) {
-    const unsigned long long wx0 = (unsigned long long)(kOne - ax.q), wx1 = (unsigned long long)ax.q;
-    const unsigned long long wy[2] = {(unsigned long long)(kOne - ay.q), (unsigned long long)ay.q};
-    const unsigned long long wz[2] = {(unsigned long long)(kOne - az.q), (unsigned long long)az.q};
+    const uint32_t wx0 = (uint32_t)(kOne - ax.q), wx1 = (uint32_t)ax.q;
+    const uint32_t wy[2] = {(uint32_t)(kOne - ay.q), (uint32_t)ay.q};
+    const uint32_t wz[2] = {(uint32_t)(kOne - az.q), (uint32_t)az.q};
     const int ny[2] = {ay.lo, ay.hi}, nz[2] = {az.lo, az.hi};
 #pragma unroll
     for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
         for (int dy = 0; dy < 2; ++dy) {
-            const unsigned long long wzy = wz[dz] * wy[dy];
+            const uint32_t wzy = wz[dz] * wy[dy];
+            if (wzy == 0) continue;
             unsigned long long* row = Dt + (nz[dz] * g.my + ny[dy]) * g.mx;
-            const unsigned long long a = wzy * wx0, b = wzy * wx1;
-            if (a) atomicAdd(row + ax.lo, a);
-            if (b) atomicAdd(row + ax.hi, b);
+            atomicAdd(row + ax.lo, (unsigned long long)wzy * wx0);  // wx0 >= 1
+            if (wx1) atomicAdd(row + ax.hi, (unsigned long long)wzy * wx1);
         }
 }
 

@@ -386,6 +386,14 @@ void launch_step(StateBuf in, StateBuf out, const uint32_t* meta, int n, int n_s
 // read on the device so a re-sort needs no host synchronisation.
 constexpr int kWarpBlock = 256;
 constexpr size_t kWarpSmem = sizeof(float4) * kCachePlanes * 2 * kWarpBlock;
+// The packed form (advance_pairs below) covers bonds with the interpolated-
+// gradient force; it needs no shared cache.
+__host__ __device__ constexpr bool pair_form(int force, int bonded) {
+    return force == 0 && bonded == 0;
+}
+__host__ __device__ constexpr size_t warp_smem(int force, int bonded) {
+    return pair_form(force, bonded) ? 0 : kWarpSmem;
+}
 
 struct Bead {
     float x, y, z, vx, vy, vz;
@@ -483,6 +491,216 @@ __device__ __forceinline__ void kick_bead(Bead& b, float f0, float f1, float f2,
     }
 }
 
+// ---- two beads a lane in packed FP32 (the interpolated-gradient force)
+//
+// A launch of the warp form is bound by instruction issue (63 % of the issue
+// slots used at 16 warps per SM, about 550 instructions per warp and
+// sub-step) and by the L1 data pipe (56 %, a third of it the reads of the
+// shared polynomial cache).  Here every FP32 operation that a lane does for
+// both of its beads is one packed instruction (add, multiply and
+// multiply-add on float pairs), and the two cell polynomials live in 48
+// registers, paired coefficient by coefficient, instead of shared memory: no
+// loads per evaluation, and the L1 keeps the space.  91.4M -> 75.0M
+// instructions and 124 -> 118 us per 10-step launch of 1M beads (L1 data pipe
+// 56 -> 34 %).  What bounds it now is latency at 16 warps per SM: the refills
+// (a warp meets about one per sub-step; 1.7 of 6.8 stall cycles per
+// instruction) and dependent arithmetic.  Starting a refill's loads a
+// sub-step's noise earlier was slower, whether as L1 prefetches (137 us: they
+// do not fill the L1) or as asynchronous copies into shared memory (126 us).
+// The rounding of every operation is the scalar form's, so the bits are too.
+struct Pair {
+    float2 x, y, z, vx, vy, vz;  // .x: bead 2 lane, .y: bead 2 lane + 1
+    float2 cx, cy, cz;           // cached cells, NaN: none
+    float2 kx[8], ky[8], kz[8];  // their polynomials, c0 .. c7 per component
+    uint32_t m0, m1;
+};
+
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 pair_sub(float2 a, float2 b) {  // a - b
+    return __ffma2_rn(b, both(-1.0f), a);
+}
+
+// -(cell polynomials) added to f: cell_poly of both beads.
+__device__ __forceinline__ float2 pair_poly(float2 f, const float2 (&c)[8], float2 fx, float2 fy,
+                                            float2 fz) {
+    float2 a = __ffma2_rn(fz, c[7], c[4]);
+    a = __ffma2_rn(fy, a, c[1]);
+    a = __ffma2_rn(fz, c[5], a);
+    const float2 b = __ffma2_rn(fz, c[6], c[2]);
+    float2 v = __ffma2_rn(fx, a, c[0]);
+    v = __ffma2_rn(fy, b, v);
+    v = __ffma2_rn(fz, c[3], v);
+    return pair_sub(f, v);
+}
+
+template <int kBead>
+__device__ __forceinline__ void pair_coefs(Pair& b, const Corners& k) {
+    auto put = [](float2 (&c)[8], float4 lo, float4 hi) {
+        const float v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) (kBead == 0 ? c[j].x : c[j].y) = v[j];
+    };
+    float4 lo, hi;
+    cell_coefs(HPF_CORNERS(k, x), lo, hi);
+    put(b.kx, lo, hi);
+    cell_coefs(HPF_CORNERS(k, y), lo, hi);
+    put(b.ky, lo, hi);
+    cell_coefs(HPF_CORNERS(k, z), lo, hi);
+    put(b.kz, lo, hi);
+}
+
+__device__ __forceinline__ const float4* species_field(const float4* __restrict__ G,
+                                                       const MeshGeom& g, uint32_t m) {
+    return G + (size_t)((m >> kTypeShift) & kTypeMask) * g.gnodes;
+}
+
+// floor(s) of both for |s| < 2^22 (the coordinate range ends at 2^18): adding
+// 1.5 2^23 rounded down leaves an integer ulp.
+__device__ __forceinline__ float2 pair_floor(float2 s) {
+    return __fadd2_rn(__fadd2_rd(s, both(12582912.0f)), both(-12582912.0f));
+}
+
+// Uniforms of two Philox words, as open_uniform: the float 1 + (r >> 9) 2^-23
+// (its bits) minus 1 - 2^-24, exact.
+__device__ __forceinline__ float2 pair_uniform(uint32_t r0, uint32_t r1) {
+    return __fadd2_rn(make_float2(__uint_as_float(0x3f800000u | (r0 >> 9)),
+                                  __uint_as_float(0x3f800000u | (r1 >> 9))),
+                      both(-0.999999940395355224609375f));
+}
+
+// The Box-Muller radius sqrt(-2 ln u) of both, negated (log_unit's two forms).
+__device__ __forceinline__ float2 pair_radius_neg(float2 u) {
+    const float2 d = __ffma2_rn(u, both(-1.0f), both(1.0f));
+    const float2 t = __ffma2_rn(__ffma2_rn(d, both(1.0f / 3.0f), both(0.5f)), d, both(1.0f));
+    const float2 series = __fmul2_rn(d, t);
+    const float2 l = __fmul2_rn(make_float2(d.x <= 0.015625f ? series.x : -__logf(u.x),
+                                            d.y <= 0.015625f ? series.y : -__logf(u.y)),
+                                both(2.0f));
+    return __fmul2_rn(l, make_float2(-rsqrtf(l.x), -rsqrtf(l.y)));
+}
+
+// gauss3 of both beads.
+__device__ __forceinline__ void pair_gauss3(const StepConsts& c, uint32_t tag0, uint32_t tag1,
+                                            long long step, float2& gx, float2& gy, float2& gz) {
+    uint32_t a0 = tag0 + c.tag_base, a1 = (uint32_t)step,
+             a2 = (uint32_t)((unsigned long long)step >> 32), a3 = 0u;
+    uint32_t b0 = tag1 + c.tag_base, b1 = a1, b2 = a2, b3 = 0u;
+    philox4x32_10(a0, a1, a2, a3, c.rk0, c.rk1);
+    philox4x32_10(b0, b1, b2, b3, c.rk0, c.rk1);
+    const float2 a = pair_radius_neg(pair_uniform(a0, b0));
+    const float2 b = pair_radius_neg(pair_uniform(a2, b2));
+    const float2 t1 = __fmul2_rn(__fadd2_rn(pair_uniform(a1, b1), both(-0.5f)),
+                                 both(6.28318530717958648f));
+    const float2 t3 = __fmul2_rn(__fadd2_rn(pair_uniform(a3, b3), both(-0.5f)),
+                                 both(6.28318530717958648f));
+    float2 s1, k1;
+    __sincosf(t1.x, &s1.x, &k1.x);
+    __sincosf(t1.y, &s1.y, &k1.y);
+    gx = __fmul2_rn(a, k1);
+    gy = __fmul2_rn(a, s1);
+    gz = __fmul2_rn(b, make_float2(__cosf(t3.x), __cosf(t3.y)));
+}
+
+// The bond forces of a segment (warp_bonded_forces<0>), the lane's two bonds as
+// a pair: the in-lane one (2l, 2l + 1) and the one to the next lane.  The pairs
+// (dx, dy'), (dy, dx'), (dz, dz') give each its own order of |d|^2 (kLaneBond,
+// kCrossBond).
+__device__ __forceinline__ void pair_bonds(const Pair& b, bool p0, float2 minus_k,
+                                           const StepConsts& c, float2& wx, float2& wy,
+                                           float2& wz) {
+    const float dx = __shfl_down_sync(0xffffffffu, b.x.x, 1);
+    const float dy = __shfl_down_sync(0xffffffffu, b.y.x, 1);
+    const float dz = __shfl_down_sync(0xffffffffu, b.z.x, 1);
+    const float2 A = make_float2(__fsub_rn(b.x.x, b.x.y), __fsub_rn(b.y.y, dy));
+    const float2 B = make_float2(__fsub_rn(b.y.x, b.y.y), __fsub_rn(b.x.y, dx));
+    const float2 C = make_float2(__fsub_rn(b.z.x, b.z.y), __fsub_rn(b.z.y, dz));
+    const float2 rr = __ffma2_rn(C, C, __ffma2_rn(B, B, __fmul2_rn(A, A)));
+    const float2 ir = make_float2(rsqrtf(fmaxf(rr.x, 1e-30f)), rsqrtf(fmaxf(rr.y, 1e-30f)));
+    const float2 s = __fmul2_rn(minus_k, __ffma2_rn(both(-c.r0), ir, both(1.0f)));
+    const float2 fa = __fmul2_rn(s, A), fb = __fmul2_rn(s, B), fc = __fmul2_rn(s, C);
+    const float ux = __shfl_up_sync(0xffffffffu, fb.y, 1);  // the previous lane's share
+    const float uy = __shfl_up_sync(0xffffffffu, fa.y, 1);
+    const float uz = __shfl_up_sync(0xffffffffu, fc.y, 1);
+    wx = make_float2(p0 ? __fsub_rn(fa.x, ux) : fa.x, __fsub_rn(fb.y, fa.x));
+    wy = make_float2(p0 ? __fsub_rn(fb.x, uy) : fb.x, __fsub_rn(fa.y, fb.x));
+    wz = make_float2(p0 ? __fsub_rn(fc.x, uz) : fc.x, __fsub_rn(fc.y, fc.x));
+}
+
+// The forces on a lane's two beads at their positions: field, friction, bonds
+// and step `step`'s noise.  coll0, coll1 (Andersen): the bead collides
+// and (gx, gy, gz) holds its normals.
+struct PairForce {
+    float2 fx, fy, fz, gx, gy, gz;
+    bool coll0, coll1;
+};
+
+template <int kTherm>
+__device__ __forceinline__ PairForce pair_force(Pair& b, bool p0, float2 minus_k, long long step,
+                                                const MeshGeom& g, const float4* __restrict__ G,
+                                                const StepConsts& c) {
+    PairForce r;
+    float2 wx, wy, wz;
+    pair_bonds(b, p0, minus_k, c, wx, wy, wz);
+    const float2 s0 = __fmul2_rn(b.x, both(g.inv_h[0])), s1 = __fmul2_rn(b.y, both(g.inv_h[1])),
+                 s2 = __fmul2_rn(b.z, both(g.inv_h[2]));
+    const float2 l0 = pair_floor(s0), l1 = pair_floor(s1), l2 = pair_floor(s2);
+    if (l0.x != b.cx.x || l1.x != b.cy.x || l2.x != b.cz.x)
+        pair_coefs<0>(b, load_corners(species_field(G, g, b.m0), g, l0.x, l1.x, l2.x));
+    if (l0.y != b.cx.y || l1.y != b.cy.y || l2.y != b.cz.y)
+        pair_coefs<1>(b, load_corners(species_field(G, g, b.m1), g, l0.y, l1.y, l2.y));
+    b.cx = l0;
+    b.cy = l1;
+    b.cz = l2;
+    const float2 f0 = pair_sub(s0, l0), f1 = pair_sub(s1, l1), f2 = pair_sub(s2, l2);
+    r.gx = r.gy = r.gz = both(0.f);
+    r.coll0 = r.coll1 = false;
+    const uint32_t t0 = b.m0 & kTagMask, t1 = b.m1 & kTagMask;
+    if (kTherm == 1) pair_gauss3(c, t0, t1, step, r.gx, r.gy, r.gz);
+    if (kTherm == 2) {
+        r.coll0 = andersen_collides(c, t0, step);
+        r.coll1 = andersen_collides(c, t1, step);
+        if (r.coll0) gauss3(c, t0, step, r.gx.x, r.gy.x, r.gz.x);
+        if (r.coll1) gauss3(c, t1, step, r.gx.y, r.gy.y, r.gz.y);
+    }
+    const float2 fric = both(-c.fric);
+    r.fx = pair_poly(__fmul2_rn(fric, b.vx), b.kx, f0, f1, f2);
+    r.fy = pair_poly(__fmul2_rn(fric, b.vy), b.ky, f0, f1, f2);
+    r.fz = pair_poly(__fmul2_rn(fric, b.vz), b.kz, f0, f1, f2);
+    if (kTherm == 1) {
+        r.fx = __ffma2_rn(both(c.sigma), r.gx, r.fx);
+        r.fy = __ffma2_rn(both(c.sigma), r.gy, r.fy);
+        r.fz = __ffma2_rn(both(c.sigma), r.gz, r.fz);
+    }
+    r.fx = __fadd2_rn(r.fx, wx);
+    r.fy = __fadd2_rn(r.fy, wy);
+    r.fz = __fadd2_rn(r.fz, wz);
+    return r;
+}
+
+// Kick by those forces (a colliding bead: redrawn velocity, second half kick) and drift.
+template <int kTherm>
+__device__ __forceinline__ void pair_move(Pair& b, const PairForce& r, const StepConsts& c) {
+    b.vx = __ffma2_rn(both(c.dt_m), r.fx, b.vx);
+    b.vy = __ffma2_rn(both(c.dt_m), r.fy, b.vy);
+    b.vz = __ffma2_rn(both(c.dt_m), r.fz, b.vz);
+    if (kTherm == 2) {
+        const float h = 0.5f * c.dt_m;
+        if (r.coll0) {
+            b.vx.x = fmaf(h, r.fx.x, __fmul_rn(c.sig_v, r.gx.x));
+            b.vy.x = fmaf(h, r.fy.x, __fmul_rn(c.sig_v, r.gy.x));
+            b.vz.x = fmaf(h, r.fz.x, __fmul_rn(c.sig_v, r.gz.x));
+        }
+        if (r.coll1) {
+            b.vx.y = fmaf(h, r.fx.y, __fmul_rn(c.sig_v, r.gx.y));
+            b.vy.y = fmaf(h, r.fy.y, __fmul_rn(c.sig_v, r.gy.y));
+            b.vz.y = fmaf(h, r.fz.y, __fmul_rn(c.sig_v, r.gz.y));
+        }
+    }
+    b.x = __ffma2_rn(both(c.dt), b.vx, b.x);
+    b.y = __ffma2_rn(both(c.dt), b.vy, b.y);
+    b.z = __ffma2_rn(both(c.dt), b.vz, b.z);
+}
+
 __device__ __forceinline__ void finish_bead(const Bead& b, long long i, StateBuf out,
                                             const MeshGeom& g, unsigned long long* D_next,
                                             int* flag) {
@@ -520,56 +738,84 @@ struct ObsArgs {
 };
 
 template <int kTherm>
-__device__ __forceinline__ void observe_segment(Bead& b0, Bead& b1, bool a0, bool a1, bool p0,
-                                                bool n0, bool n1, long long step,
-                                                const MeshGeom& g, const float4* __restrict__ G,
-                                                const StepConsts& c, float4* wcache, int tid,
+__device__ __forceinline__ void observe_segment(Pair& b, bool a0, bool a1, bool p0, bool n0, bool n1,
+                                                float2 minus_k, long long step, const MeshGeom& g,
+                                                const float4* __restrict__ G, const StepConsts& c,
                                                 const ObsArgs& o, FF* acc) {
-    const int lane = tid & 31;
-    float w0x, w0y, w0z, w1x, w1y, w1z;
-    warp_bonded_forces<0>(b0.x, b0.y, b0.z, b1.x, b1.y, b1.z, p0, n0, n1, c, lane, w0x, w0y, w0z,
-                          w1x, w1y, w1z);
-    float f00, f01, f02, f10, f11, f12;
-    cell_check<0>(b0, G, g, wcache, tid, f00, f01, f02);
-    cell_check<0>(b1, G, g, wcache, kWarpBlock + tid, f10, f11, f12);
-    float g0x = 0.f, g0y = 0.f, g0z = 0.f, g1x = 0.f, g1y = 0.f, g1z = 0.f;
-    if (kTherm == 1) {
-        gauss3(c, b0.m & kTagMask, step, g0x, g0y, g0z);
-        gauss3(c, b1.m & kTagMask, step, g1x, g1y, g1z);
-    }
-    float F0x, F0y, F0z, F1x, F1y, F1z;
-    bead_force<kTherm, 0>(b0, f00, f01, f02, g0x, g0y, g0z, w0x, w0y, w0z, c, g, wcache, tid, 0.f,
-                          F0x, F0y, F0z);
-    bead_force<kTherm, 0>(b1, f10, f11, f12, g1x, g1y, g1z, w1x, w1y, w1z, c, g, wcache,
-                          kWarpBlock + tid, 0.f, F1x, F1y, F1z);
+    const PairForce r = pair_force<kTherm>(b, p0, minus_k, step, g, G, c);
     // the next lane's first bead (every lane takes part in the shuffles)
-    const float qx = __shfl_down_sync(0xffffffffu, b0.x, 1);
-    const float qy = __shfl_down_sync(0xffffffffu, b0.y, 1);
-    const float qz = __shfl_down_sync(0xffffffffu, b0.z, 1);
+    const float qx = __shfl_down_sync(0xffffffffu, b.x.x, 1);
+    const float qy = __shfl_down_sync(0xffffffffu, b.y.x, 1);
+    const float qz = __shfl_down_sync(0xffffffffu, b.z.x, 1);
     float uh = acc[1].h, ul = acc[1].l;
-    if (n0) bond_energy_ff(b0.x, b0.y, b0.z, b1.x, b1.y, b1.z, o.bond, uh, ul);
-    if (n1) bond_energy_ff(b1.x, b1.y, b1.z, qx, qy, qz, o.bond, uh, ul);
+    if (n0) bond_energy_ff(b.x.x, b.y.x, b.z.x, b.x.y, b.y.y, b.z.y, o.bond, uh, ul);
+    if (n1) bond_energy_ff(b.x.y, b.y.y, b.z.y, qx, qy, qz, o.bond, uh, ul);
     acc[1] = FF{uh, ul};
-    const float hf = o.half_dt_m;
+    const float2 hf = both(o.half_dt_m);
+    const float2 ux = __ffma2_rn(hf, r.fx, b.vx), uy = __ffma2_rn(hf, r.fy, b.vy),
+                 uz = __ffma2_rn(hf, r.fz, b.vz);
     if (a0) {
-        const float ux = fmaf(hf, F0x, b0.vx), uy = fmaf(hf, F0y, b0.vy), uz = fmaf(hf, F0z, b0.vz);
-        acc[0] = ff_plus(acc[0], fmaf(ux, ux, fmaf(uy, uy, __fmul_rn(uz, uz))));
-        acc[2] = ff_plus(acc[2], ux);
-        acc[3] = ff_plus(acc[3], uy);
-        acc[4] = ff_plus(acc[4], uz);
+        acc[0] = ff_plus(acc[0], fmaf(ux.x, ux.x, fmaf(uy.x, uy.x, __fmul_rn(uz.x, uz.x))));
+        acc[2] = ff_plus(acc[2], ux.x);
+        acc[3] = ff_plus(acc[3], uy.x);
+        acc[4] = ff_plus(acc[4], uz.x);
     }
     if (a1) {
-        const float ux = fmaf(hf, F1x, b1.vx), uy = fmaf(hf, F1y, b1.vy), uz = fmaf(hf, F1z, b1.vz);
-        acc[0] = ff_plus(acc[0], fmaf(ux, ux, fmaf(uy, uy, __fmul_rn(uz, uz))));
-        acc[2] = ff_plus(acc[2], ux);
-        acc[3] = ff_plus(acc[3], uy);
-        acc[4] = ff_plus(acc[4], uz);
+        acc[0] = ff_plus(acc[0], fmaf(ux.y, ux.y, fmaf(uy.y, uy.y, __fmul_rn(uz.y, uz.y))));
+        acc[2] = ff_plus(acc[2], ux.y);
+        acc[3] = ff_plus(acc[3], uy.y);
+        acc[4] = ff_plus(acc[4], uz.y);
     }
 }
 
-// One warp advances one segment (whole chains, base .. base + cnt) by n_sub steps.
-// kObs: also the observables' terms of the final state (observe_segment).
-template <int kTherm, int kForce, int kBonded, int kLerp = 0, int kObs = 0>
+// One warp advances one segment by n_sub steps in packed form (the
+// interpolated-gradient force).  kObs: also the observables' terms of the
+// final state.
+template <int kTherm, int kObs = 0>
+__device__ __forceinline__ void advance_pairs(const StateBuf& in, const StateBuf& out,
+                                              const uint32_t* __restrict__ meta, int base, int cnt,
+                                              int n_sub, long long step0, const MeshGeom& g,
+                                              const float4* __restrict__ G, const StepConsts& c,
+                                              unsigned long long* __restrict__ D_next,
+                                              int* __restrict__ flag, const ObsArgs* obs = nullptr,
+                                              FF* obs_acc = nullptr) {
+    const int lane = threadIdx.x & 31, j0 = 2 * lane;
+    const bool a0 = j0 < cnt, a1 = j0 + 1 < cnt;
+    const long long i = (long long)base + j0;
+    Pair b;
+    auto load = [&](const float* p) { return make_float2(a0 ? p[i] : 0.f, a1 ? p[i + 1] : 0.f); };
+    b.x = load(in.x);
+    b.y = load(in.y);
+    b.z = load(in.z);
+    b.vx = load(in.vx);
+    b.vy = load(in.vy);
+    b.vz = load(in.vz);
+    b.m0 = a0 ? meta[i] : 0u;
+    b.m1 = a1 ? meta[i + 1] : 0u;
+    b.cx = b.cy = b.cz = both(__int_as_float(0x7fc00000));
+#pragma unroll
+    for (int j = 0; j < 8; ++j) b.kx[j] = b.ky[j] = b.kz[j] = both(0.f);
+    // whole chains: every flagged neighbour is inside the segment
+    const bool p0 = (b.m0 & kBondPrev) != 0, n0 = (b.m0 & kBondNext) != 0;
+    const bool n1 = (b.m1 & kBondNext) != 0;  // b1's previous bond is b0's next
+    const float2 minus_k = make_float2(n0 ? -c.two_k : 0.f, n1 ? -c.two_k : 0.f);
+    for (int k = 0; k < n_sub; ++k)
+        pair_move<kTherm>(b, pair_force<kTherm>(b, p0, minus_k, step0 + k, g, G, c), c);
+    if constexpr (kObs != 0)
+        observe_segment<kTherm>(b, a0, a1, p0, n0, n1, minus_k, step0 + n_sub, g, G, c, *obs,
+                                obs_acc);
+    if (a0)
+        finish_bead(Bead{b.x.x, b.y.x, b.z.x, b.vx.x, b.vy.x, b.vz.x, b.m0, 0.f, 0.f, 0.f}, i, out, g,
+                    D_next, flag);
+    if (a1)
+        finish_bead(Bead{b.x.y, b.y.y, b.z.y, b.vx.y, b.vy.y, b.vz.y, b.m1, 0.f, 0.f, 0.f}, i + 1, out,
+                    g, D_next, flag);
+}
+
+// One warp advances one segment (whole chains, base .. base + cnt) by n_sub
+// steps with the polynomials in shared memory: the other force modes, and the
+// interpolated fields of a learned window (two polynomials per bead).
+template <int kTherm, int kForce, int kBonded, int kLerp = 0>
 __device__ __forceinline__ void advance_segment(const StateBuf& in, const StateBuf& out,
                                                 const uint32_t* __restrict__ meta, int base,
                                                 int cnt, int n_sub, long long step0,
@@ -578,9 +824,7 @@ __device__ __forceinline__ void advance_segment(const StateBuf& in, const StateB
                                                 unsigned long long* __restrict__ D_next,
                                                 int* __restrict__ flag, float4* wcache, int tid,
                                                 const float4* __restrict__ G2 = nullptr,
-                                                int lerp_j0 = 0, float lerp_inv_k = 0.f,
-                                                const ObsArgs* obs = nullptr,
-                                                FF* obs_acc = nullptr) {
+                                                int lerp_j0 = 0, float lerp_inv_k = 0.f) {
     const int lane = tid & 31;
     const float nan = __int_as_float(0x7fc00000);
     const int j0 = 2 * lane, j1 = j0 + 1;
@@ -635,9 +879,6 @@ __device__ __forceinline__ void advance_segment(const StateBuf& in, const StateB
         b1.y = fmaf(c.dt, b1.vy, b1.y);
         b1.z = fmaf(c.dt, b1.vz, b1.z);
     }
-    if constexpr (kObs != 0)
-        observe_segment<kTherm>(b0, b1, a0, a1, p0, n0, n1, step0 + n_sub, g, G, c, wcache, tid,
-                                *obs, obs_acc);
     if (a0) finish_bead(b0, (long long)base + j0, out, g, D_next, flag);
     if (a1) finish_bead(b1, (long long)base + j1, out, g, D_next, flag);
 }
@@ -678,10 +919,16 @@ __global__ void __launch_bounds__(kWarpBlock, 2) k_step_warp_batch(
         }
         const BatchStepRep& rp = p.rep[kCap > 1 ? lo : 0];
         const int s = w - s_off[lo];
-        advance_segment<kTherm, kForce, kBonded>(rp.st[p.cur], rp.st[p.cur ^ 1], rp.meta,
-                                                 rp.seg_start[s],
-                                rp.seg_count[s], p.n_sub, step0, rp.g, rp.G, rp.c,
-                                p.fuse ? rp.D[p.dnext] : nullptr, p.flag, wcache, tid);
+        unsigned long long* D = p.fuse ? rp.D[p.dnext] : nullptr;
+        if constexpr (pair_form(kForce, kBonded))
+            advance_pairs<kTherm>(rp.st[p.cur], rp.st[p.cur ^ 1], rp.meta, rp.seg_start[s],
+                                           rp.seg_count[s], p.n_sub, step0, rp.g, rp.G, rp.c, D,
+                                           p.flag);
+        else
+            advance_segment<kTherm, kForce, kBonded>(rp.st[p.cur], rp.st[p.cur ^ 1], rp.meta,
+                                                     rp.seg_start[s], rp.seg_count[s], p.n_sub,
+                                                     step0, rp.g, rp.G, rp.c, D, p.flag, wcache,
+                                                     tid);
     }
 }
 
@@ -694,7 +941,6 @@ __global__ void __launch_bounds__(kWarpBlock, 2) k_step_warp_obs(
     const __grid_constant__ SingleStepParams p, const ObsArgs o) {
     griddep_wait();
     griddep_launch_dependents();
-    extern __shared__ float4 wcache[];
     __shared__ FF sh[kBeadVals][kWarpBlock / 32];
     const int tid = threadIdx.x;
     const BatchStepRep& rp = p.rep[0];
@@ -705,10 +951,9 @@ __global__ void __launch_bounds__(kWarpBlock, 2) k_step_warp_obs(
 #pragma unroll
     for (int k = 0; k < kBeadVals; ++k) acc[k] = FF{0.f, 0.f};
     for (int w = blockIdx.x * (kWarpBlock / 32) + (tid >> 5); w < total; w += warps_total)
-        advance_segment<kTherm, 0, 0, 0, 1>(rp.st[p.cur], rp.st[p.cur ^ 1], rp.meta,
-                                            rp.seg_start[w], rp.seg_count[w], p.n_sub, step0,
-                                            rp.g, rp.G, rp.c, p.fuse ? rp.D[p.dnext] : nullptr,
-                                            p.flag, wcache, tid, nullptr, 0, 0.f, &o, acc);
+        advance_pairs<kTherm, 1>(rp.st[p.cur], rp.st[p.cur ^ 1], rp.meta, rp.seg_start[w],
+                                    rp.seg_count[w], p.n_sub, step0, rp.g, rp.G, rp.c,
+                                    p.fuse ? rp.D[p.dnext] : nullptr, p.flag, &o, acc);
     const int wi = tid >> 5;
 #pragma unroll
     for (int k = 0; k < kBeadVals; ++k) {
@@ -797,15 +1042,10 @@ static int warp_grid_cap() {
     once_per_device(once, [dev] {
         warp_attrs<HPF_MAX_REPLICAS>();
         warp_attrs<1>();
-        cudaFuncSetAttribute(k_step_warp_obs<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kWarpSmem);
-        cudaFuncSetAttribute(k_step_warp_obs<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kWarpSmem);
         int sms = 0, per_sm = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, k_step_warp_batch<1, HPF_MAX_REPLICAS, 0, 0>, kWarpBlock,
-            kWarpSmem);
+            &per_sm, k_step_warp_batch<1, HPF_MAX_REPLICAS, 1, 0>, kWarpBlock, kWarpSmem);
         cudaGetLastError();
         cap[dev & 63] = (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
     });
@@ -816,17 +1056,20 @@ static int warp_grid_cap() {
 // graphs and launched plainly.
 template <int kCap>
 static void launch_warp_k(void (*k)(const BatchStepParamsT<kCap>), const BatchStepParamsT<kCap>& p,
-                          int blocks, cudaStream_t s) {
-    if (kCap == 1) launch_pdl(k, blocks, kWarpBlock, kWarpSmem, s, p);
-    else k<<<blocks, kWarpBlock, kWarpSmem, s>>>(p);
+                          int blocks, size_t smem, cudaStream_t s) {
+    if (kCap == 1) launch_pdl(k, blocks, kWarpBlock, smem, s, p);
+    else k<<<blocks, kWarpBlock, smem, s>>>(p);
 }
 
 template <int kCap, int kTherm, int kForce>
 static void launch_warp_f(const BatchStepParamsT<kCap>& p, int blocks, int bonded,
                           cudaStream_t s) {
-    if (bonded == 2) launch_warp_k(k_step_warp_batch<kTherm, kCap, kForce, 2>, p, blocks, s);
-    else if (bonded == 1) launch_warp_k(k_step_warp_batch<kTherm, kCap, kForce, 1>, p, blocks, s);
-    else launch_warp_k(k_step_warp_batch<kTherm, kCap, kForce, 0>, p, blocks, s);
+#define HPF_WARP(B) \
+    launch_warp_k(k_step_warp_batch<kTherm, kCap, kForce, B>, p, blocks, warp_smem(kForce, B), s)
+    if (bonded == 2) HPF_WARP(2);
+    else if (bonded == 1) HPF_WARP(1);
+    else HPF_WARP(0);
+#undef HPF_WARP
 }
 
 template <int kCap, int kTherm>
@@ -886,8 +1129,8 @@ int launch_step_warp_obs(const SingleStepParams& p, int max_seg, int therm, floa
     const int need = (max_seg + kWarpBlock / 32 - 1) / (kWarpBlock / 32);
     const int blocks = need < cap ? need : cap;
     const ObsArgs o{part, half_dt_m, bond};
-    if (therm == 1) launch_pdl(k_step_warp_obs<1>, blocks, kWarpBlock, kWarpSmem, s, p, o);
-    else launch_pdl(k_step_warp_obs<0>, blocks, kWarpBlock, kWarpSmem, s, p, o);
+    if (therm == 1) launch_pdl(k_step_warp_obs<1>, blocks, kWarpBlock, 0, s, p, o);
+    else launch_pdl(k_step_warp_obs<0>, blocks, kWarpBlock, 0, s, p, o);
     return blocks;
 }
 
