@@ -110,8 +110,8 @@ struct LearnedBufs {
     float* x = nullptr;     // network input [max(4, S)][M]: phi(t - K), phi(t)
     float* dphi = nullptr;  // predicted change [S][M]
     float* snap = nullptr;  // state at the window start [6][n]
-    double* acc = nullptr;  // judge sums [2] and their partials
-    double* h_acc = nullptr;
+    void* judge = nullptr;  // the judge's partial sums
+    double* h_acc = nullptr;  // pinned, written by the judge's kernel
     long long hist_step = -1;  // step whose phi is in x[0:2] (-1: none)
     bool plain_mode = false;   // run plain windows (shadow-judged) until a prediction meets tol
     int backoff = 0;           // plain windows to skip between shadow judgements (doubles per failure)
@@ -919,7 +919,7 @@ hpf_status hpf_destroy(hpf_ctx* c) {
         cudaFree(L->x);
         cudaFree(L->dphi);
         cudaFree(L->snap);
-        cudaFree(L->acc);
+        cudaFree(L->judge);
         cudaFreeHost(L->h_acc);
         cudaFree(L->G2);
         delete L;
@@ -1928,7 +1928,8 @@ hpf_status ensure_learned(hpf_ctx* c) {
     e = e ? e : cudaMalloc(&L->x, sizeof(float) * xs * M);
     e = e ? e : cudaMalloc(&L->dphi, sizeof(float) * S * M);
     e = e ? e : cudaMalloc(&L->snap, sizeof(float) * 6 * bead_stride(c->n));
-    e = e ? e : cudaMalloc(&L->acc, sizeof(double) * (2 + 2 * (size_t)force_error_partials()));
+    e = e ? e : cudaMalloc(&L->judge, judge_scratch_bytes());
+    e = e ? e : cudaMemsetAsync(L->judge, 0, judge_scratch_bytes(), c->stream);
     e = e ? e : cudaMallocHost(&L->h_acc, sizeof(double) * 2);
     e = e ? e : cudaMalloc(&L->G2, sizeof(float4) * S * (size_t)c->geom.gnodes);
     c->learned = L;  // freed by hpf_destroy, also after a failed allocation
@@ -1939,7 +1940,7 @@ hpf_status ensure_learned(hpf_ctx* c) {
         cudaFree(L->x);
         cudaFree(L->dphi);
         cudaFree(L->snap);
-        cudaFree(L->acc);
+        cudaFree(L->judge);
         cudaFreeHost(L->h_acc);
         cudaFree(L->G2);
         delete L;
@@ -1950,39 +1951,42 @@ hpf_status ensure_learned(hpf_ctx* c) {
     return HPF_OK;
 }
 
-// eps of the candidate mesh in Dp against the true density of the current
-// positions, which must be the context's mesh.  Leaves the true field in force.
-hpf_status judge_mesh(hpf_ctx* c, double* eps) {
+// The judge's eps of the fields Ga (candidate) and Gb at the current
+// positions; waits for the stream.
+hpf_status judge_fields(hpf_ctx* c, const float4* Ga, const float4* Gb, double* eps) {
     LearnedBufs* L = c->learned;
-    hpf_status s;
-    if (c->field_tile < 0 && (s = run_field(c)) != HPF_OK) return s;  // picks the tile
-    if (L->tmap_tile != c->field_tile) {
-        L->tmap_ok = c->S <= 4 && make_mesh_tensor_map(&L->tmap,
-                                                       reinterpret_cast<const long long*>(L->Dp),
-                                                       c->geom, c->S, c->field_tile);
-        L->tmap_tile = c->field_tile;
-    }
-    if ((s = field_from(c, L->Dp, L->tmap, L->tmap_ok, nullptr)) != HPF_OK) return s;
-    const long long n3 = 3ll * c->n;
     {
-        StageScope sc(c, HPF_STAGE_OTHER, c->n > 0 ? 1 : 0);
-        launch_forces(cur_state(c), c->meta, c->n, c->geom, c->G, c->sc, HPF_FORCE_FIELD,
-                      c->out_f, c->stream);
-    }
-    if ((s = run_field(c)) != HPF_OK) return s;
-    {
-        StageScope sc(c, HPF_STAGE_OTHER, c->n > 0 ? 2 : 1);
-        launch_forces(cur_state(c), c->meta, c->n, c->geom, c->G, c->sc, HPF_FORCE_FIELD,
-                      c->out_f + n3, c->stream);
-        launch_force_error(c->out_f, c->out_f + n3, n3, L->acc, c->stream);
+        StageScope sc(c, HPF_STAGE_OTHER, 1);
+        launch_judge(cur_state(c), c->meta, c->n, c->geom, Ga, Gb, c->sc.force_mode, L->judge,
+                     L->h_acc, c->dflag, c->hflag, c->stream);
     }
     LAUNCH_CHECK(c);
-    CUDA_TRY(c, cudaMemcpyAsync(L->h_acc, L->acc, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                                c->stream));
-    if ((s = check_flags(c)) != HPF_OK) return s;
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    const hpf_status s = flag_status(c, c->hflag[0]);
+    if (s != HPF_OK) return s;
     const double e2 = L->h_acc[0], r2 = L->h_acc[1];
     *eps = r2 > 0.0 ? sqrt(e2 / r2) : (e2 > 0.0 ? INFINITY : 0.0);
     return HPF_OK;
+}
+
+// eps of a candidate density against the true density of the current
+// positions, which must be the context's mesh.  The candidate is the mesh in
+// Dp, or with have_G2 its field, already in G2.  Leaves the true field in
+// force.
+hpf_status judge_mesh(hpf_ctx* c, bool have_G2, double* eps) {
+    LearnedBufs* L = c->learned;
+    hpf_status s;
+    if ((s = run_field(c)) != HPF_OK) return s;  // also picks the tile
+    if (!have_G2) {
+        if (L->tmap_tile != c->field_tile) {
+            L->tmap_ok = c->S <= 4 &&
+                         make_mesh_tensor_map(&L->tmap, reinterpret_cast<const long long*>(L->Dp),
+                                              c->geom, c->S, c->field_tile);
+            L->tmap_tile = c->field_tile;
+        }
+        if ((s = field_from(c, L->Dp, L->tmap, L->tmap_ok, nullptr, L->G2)) != HPF_OK) return s;
+    }
+    return judge_fields(c, L->G2, c->G, eps);
 }
 
 // K steps with a true scatter and field refresh at every step (the plain
@@ -2032,7 +2036,7 @@ hpf_status hpf_judge_density(hpf_ctx* c, const float* phi, double* eps) {
         launch_mesh_predict(nullptr, L->dphi, n, 1.0 / c->ec.phi_c, L->Dp, c->stream);
     }
     LAUNCH_CHECK(c);
-    return judge_mesh(c, eps);
+    return judge_mesh(c, false, eps);
 }
 
 hpf_status hpf_learned_mode(hpf_ctx* c, int32_t in_launch) {
@@ -2070,7 +2074,7 @@ hpf_status hpf_judge_density_pair(hpf_ctx* c, const float* phi_cand, const float
     hpf_status s = ensure_learned(c);
     if (s != HPF_OK) return s;
     LearnedBufs* L = c->learned;
-    const long long n = (long long)mesh_words(c), n3 = 3ll * c->n;
+    const long long n = (long long)mesh_words(c);
     if ((s = scatter_current(c)) != HPF_OK) return s;
     if (c->field_tile < 0 && (s = run_field(c)) != HPF_OK) return s;  // picks the tile
     CUDA_TRY(c, cudaMemcpyAsync(L->dphi, phi_cand, sizeof(float) * n, cudaMemcpyDefault,
@@ -2088,28 +2092,11 @@ hpf_status hpf_judge_density_pair(hpf_ctx* c, const float* phi_cand, const float
     LAUNCH_CHECK(c);
     CUtensorMap none;
     memset(&none, 0, sizeof none);
-    if ((s = field_from(c, L->Dp, none, false, nullptr)) != HPF_OK) return s;
-    {
-        StageScope sc(c, HPF_STAGE_OTHER, c->n > 0 ? 1 : 0);
-        launch_forces(cur_state(c), c->meta, c->n, c->geom, c->G, c->sc, HPF_FORCE_FIELD,
-                      c->out_f, c->stream);
-    }
+    if ((s = field_from(c, L->Dp, none, false, nullptr, L->G2)) != HPF_OK) return s;
     if ((s = field_from(c, L->Dbase, none, false, nullptr)) != HPF_OK) return s;
-    {
-        StageScope sc(c, HPF_STAGE_OTHER, c->n > 0 ? 2 : 1);
-        launch_forces(cur_state(c), c->meta, c->n, c->geom, c->G, c->sc, HPF_FORCE_FIELD,
-                      c->out_f + n3, c->stream);
-        launch_force_error(c->out_f, c->out_f + n3, n3, L->acc, c->stream);
-    }
-    LAUNCH_CHECK(c);
+    if ((s = judge_fields(c, L->G2, c->G, eps)) != HPF_OK) return s;
     // the field of the true density back in force
-    if ((s = run_field(c)) != HPF_OK) return s;
-    CUDA_TRY(c, cudaMemcpyAsync(L->h_acc, L->acc, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                                c->stream));
-    if ((s = check_flags(c)) != HPF_OK) return s;
-    const double e2 = L->h_acc[0], r2 = L->h_acc[1];
-    *eps = r2 > 0.0 ? sqrt(e2 / r2) : (e2 > 0.0 ? INFINITY : 0.0);
-    return HPF_OK;
+    return run_field(c);
 }
 
 hpf_status hpf_step_learned(hpf_ctx* c, hpf_prop* prop, int32_t n_windows, int32_t K, double tol,
@@ -2169,7 +2156,8 @@ hpf_status hpf_step_learned(hpf_ctx* c, hpf_prop* prop, int32_t n_windows, int32
                                             sizeof(unsigned long long) * SM, c->stream));
                 c->next_zero = true;
             }
-            if (L->in_launch && c->warp_mode && c->sc.force_mode == 0) {
+            const bool in_launch = L->in_launch && c->warp_mode && c->sc.force_mode == 0;
+            if (in_launch) {
                 // one launch: the field of the predicted end density D(t) + dphi in
                 // G2, interpolated with the field of D(t) in the step kernel
                 {
@@ -2194,13 +2182,14 @@ hpf_status hpf_step_learned(hpf_ctx* c, hpf_prop* prop, int32_t n_windows, int32
                 }
             }
             c->field_valid = false;  // the field in force was a predicted one
-            // judge the prediction for t + K against the true scatter there
-            {
+            // judge the prediction for t + K against the true scatter there (its
+            // field is G2's when the window ran in one launch)
+            if (!in_launch) {
                 StageScope sc(c, HPF_STAGE_OTHER, 1);
                 launch_mesh_predict(L->Dbase, L->dphi, SM, inv_phi_c, L->Dp, c->stream);
             }
             LAUNCH_CHECK(c);
-            if ((s = judge_mesh(c, &eps)) != HPF_OK) return s;
+            if ((s = judge_mesh(c, in_launch, &eps)) != HPF_OK) return s;
             judged = true;
             if (eps <= tol) {
                 st.learned += 1;
@@ -2230,7 +2219,7 @@ hpf_status hpf_step_learned(hpf_ctx* c, hpf_prop* prop, int32_t n_windows, int32
                     launch_mesh_predict(L->Dbase, L->dphi, SM, inv_phi_c, L->Dp, c->stream);
                 }
                 LAUNCH_CHECK(c);
-                if ((s = judge_mesh(c, &eps)) != HPF_OK) return s;
+                if ((s = judge_mesh(c, false, &eps)) != HPF_OK) return s;
                 judged = true;
                 if (eps <= tol) {
                     L->plain_mode = false;

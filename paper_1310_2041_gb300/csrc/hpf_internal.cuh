@@ -1079,10 +1079,13 @@ void launch_smooth_phi(const float* in, float* out, float* tmp, int mx, int my, 
                        int passes, cudaStream_t s);
 void launch_mesh_predict(const unsigned long long* D_base, const float* dphi, long long n,
                          double frac_over_phi_c, unsigned long long* D_out, cudaStream_t s);
-// acc[0] = sum (Fa - Fb)^2, acc[1] = sum Fb^2 over n floats, deterministic;
-// acc holds 2 + 2 force_error_partials() doubles (the tail is scratch)
-void launch_force_error(const float* Fa, const float* Fb, long long n, double* acc,
-                        cudaStream_t s);
-int force_error_partials();
+// The judge: h_acc[0] = sum |Fa - Fb|^2, h_acc[1] = sum |Fb|^2 over the beads, Fa
+// and Fb the field forces of fields Ga and Gb at the current positions, and
+// the error word to h_flag, both in mapped host memory; deterministic.
+// scratch: judge_scratch_bytes(), its first word (the ticket) zero.
+size_t judge_scratch_bytes();
+void launch_judge(StateBuf st, const uint32_t* meta, int n, const MeshGeom& g, const float4* Ga,
+                  const float4* Gb, int force_mode, void* scratch, double* h_acc, const int* flag,
+                  int* h_flag, cudaStream_t s);
 
 }  // namespace hpf

@@ -1546,16 +1546,6 @@ __global__ void __launch_bounds__(256) k_loss(const float2* __restrict__ y,
     }
 }
 
-// out[j] = sum_b part[b][j], b in order (deterministic reductions).
-template <class T>
-__global__ void k_sum_partials(const T* __restrict__ part, int nb, int m, T* __restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m) return;
-    T s = 0;
-    for (int b = 0; b < nb; ++b) s += part[(size_t)b * m + j];
-    out[j] = s;
-}
-
 // First packed parameter of layer l.
 __host__ __device__ constexpr int param_offset(int l) {
     return l == 0 ? 0 : param_offset(l - 1) + kOffsets * layer_in(l - 1) * layer_out(l - 1) +
@@ -1720,7 +1710,6 @@ __global__ void k_pack_images(const float* __restrict__ params, uint4* __restric
 
 // ------------------------------------------------------------------ learned-step mesh kernels
 
-constexpr int kErrBlocks = 1216;  // blocks of the force-error reduction (8 per SM)
 
 // phi_K(n) = D_K(n) phi_c: the volume fractions of an int64 fixed-point mesh.
 __global__ void k_mesh_to_phi(const unsigned long long* __restrict__ D, long long n, double phi_c,
@@ -1738,38 +1727,6 @@ __global__ void k_mesh_predict(const unsigned long long* D_base, const float* __
     const long long base = D_base ? (long long)D_base[i] : 0ll;
     long long d = base + __double2ll_rn((double)dphi[i] * frac_over_phi_c);
     D_out[i] = (unsigned long long)(d > 0 ? d : 0ll);
-}
-
-// Partials part[block] = (sum (Fa - Fb)^2, sum Fb^2) in FP64.
-__global__ void __launch_bounds__(256) k_force_error(const float* __restrict__ Fa,
-                                                     const float* __restrict__ Fb, long long n,
-                                                     double* __restrict__ part) {
-    __shared__ double sh[2][8];
-    double e = 0.0, r = 0.0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const double b = Fb[i], d = (double)Fa[i] - b;
-        e += d * d;
-        r += b * b;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        e += __shfl_down_sync(0xffffffffu, e, o);
-        r += __shfl_down_sync(0xffffffffu, r, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        sh[0][threadIdx.x >> 5] = e;
-        sh[1][threadIdx.x >> 5] = r;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double se = 0.0, sr = 0.0;
-        for (int k = 0; k < 8; ++k) {
-            se += sh[0][k];
-            sr += sh[1][k];
-        }
-        part[2 * blockIdx.x] = se;
-        part[2 * blockIdx.x + 1] = sr;
-    }
 }
 
 // One pass of the periodic binomial filter (1/4, 1/2, 1/4) along one axis of
@@ -1833,17 +1790,6 @@ void launch_mesh_predict(const unsigned long long* D_base, const float* dphi, lo
     if (n > 0)
         k_mesh_predict<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(D_base, dphi, n,
                                                                    frac_over_phi_c, D_out);
-}
-
-int force_error_partials() { return kErrBlocks; }
-
-void launch_force_error(const float* Fa, const float* Fb, long long n, double* acc,
-                        cudaStream_t s) {
-    long long blocks = (n + 255) / 256;
-    if (blocks > kErrBlocks) blocks = kErrBlocks;
-    if (blocks < 1) blocks = 1;
-    k_force_error<<<(unsigned)blocks, 256, 0, s>>>(Fa, Fb, n, acc + 2);
-    k_sum_partials<double><<<1, 32, 0, s>>>(acc + 2, (int)blocks, 2, acc);
 }
 
 // ------------------------------------------------------------------ host side
