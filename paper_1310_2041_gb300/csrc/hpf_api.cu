@@ -320,10 +320,16 @@ void derive_constants(hpf_ctx* c) {
     e.cos0 = p.angle_cos0;
     e.angle_form = p.angle_form;
     e.theta0 = p.angle_theta0;
-    e.dih_k = p.dihedral_k;
     e.dih_n = p.dihedral_k != 0.0 ? p.dihedral_n : 1;
-    e.dih_cd = cos(p.dihedral_delta);
-    e.dih_sd = sin(p.dihedral_delta);
+    auto split = [](float (&f)[2], double v) {
+        f[0] = (float)v;
+        f[1] = (float)(v - (double)f[0]);
+    };
+    split(e.ff_angle_k, p.angle_k);
+    split(e.ff_cos0, p.angle_cos0);
+    split(e.ff_dih_k, p.dihedral_k);
+    split(e.ff_dih_cd, cos(p.dihedral_delta));
+    split(e.ff_dih_sd, sin(p.dihedral_delta));
     e.inv_kappa = p.inv_kappa;
     e.phi_c = phi_c;
     e.w_scale = p.rho0 * vol;

@@ -118,9 +118,9 @@ struct EnergyConsts {
     double angle_k, cos0;  // angle potential
     int angle_form;        // 0 cosine, 1 harmonic (theta0)
     double theta0;
-    double dih_k;          // dihedral potential k [1 + cos(n phi - delta)]
-    int dih_n;
-    double dih_cd, dih_sd; // cos delta, sin delta
+    int dih_n;             // dihedral potential k [1 + cos(n phi - delta)]
+    // float-float pairs (high, low) of angle_k, cos0, the dihedral's k, cos delta, sin delta
+    float ff_angle_k[2], ff_cos0[2], ff_dih_k[2], ff_dih_cd[2], ff_dih_sd[2];
 };
 
 struct StateBuf {
@@ -591,6 +591,37 @@ __device__ __forceinline__ FF ff_plus(FF a, FF b) {
     float s, t;
     two_sum(a.h, b.h, s, t);
     return ff_norm(s, __fadd_rn(t, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ FF ff_mul(FF a, FF b) {  // about 2^-46 relative
+    const float p = __fmul_rn(a.h, b.h);
+    return ff_norm(p, fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p))));
+}
+__device__ __forceinline__ FF ff_neg(FF a) { return FF{-a.h, -a.l}; }
+__device__ __forceinline__ FF ff_diff(float a, float b) {  // exact
+    FF r;
+    two_sum(a, -b, r.h, r.l);
+    return r;
+}
+// 1 / sqrt(d): the hardware's y with 1 - d y^2 = r (about 2^-22) evaluated in
+// float-float, y (1 + r/2 + 3 r^2 / 8), about 2^-46 relative; NaN for d = 0
+// (an undefined angle).
+__device__ __forceinline__ FF ff_rsqrt(FF d) {
+    const float y = rsqrtf(d.h);
+    const float p = __fmul_rn(y, y);
+    const FF t = ff_mul(d, FF{p, fmaf(y, y, -p)});
+    const float r = __fsub_rn(__fsub_rn(1.0f, t.h), t.l);
+    return ff_norm(y, __fmul_rn(y, fmaf(__fmul_rn(0.375f, r), r, __fmul_rn(0.5f, r))));
+}
+struct FF3 {
+    FF x, y, z;
+};
+__device__ __forceinline__ FF ff_dot(const FF3& a, const FF3& b) {
+    return ff_plus(ff_plus(ff_mul(a.x, b.x), ff_mul(a.y, b.y)), ff_mul(a.z, b.z));
+}
+__device__ __forceinline__ FF3 ff_cross(const FF3& a, const FF3& b) {
+    return FF3{ff_plus(ff_mul(a.y, b.z), ff_neg(ff_mul(a.z, b.y))),
+               ff_plus(ff_mul(a.z, b.x), ff_neg(ff_mul(a.x, b.z))),
+               ff_plus(ff_mul(a.x, b.y), ff_neg(ff_mul(a.y, b.x)))};
 }
 __device__ __forceinline__ FF ff_from_double(double v) {
     const float h = (float)v;

@@ -48,52 +48,58 @@ __device__ __forceinline__ double norm_fp64(double r2) {
     return r2 * y;
 }
 
-// Dihedral energy k [1 + cos(n phi - delta)] of the quadruplet i .. i + 3 in
-// FP64 from the FP32 positions: cos phi = A.B / (|A||B|), sin phi =
-// |b2| b1.B / (|A||B|) with A = b1 x b2, B = b2 x b3, and cos(n phi),
-// sin(n phi) by the n-th power of cos phi + i sin phi.
-__device__ __forceinline__ double dihedral_energy_fp64(const StateBuf& st, int i,
-                                                       const EnergyConsts& e) {
-    double b[3][3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        b[k][0] = (double)st.x[i + k + 1] - st.x[i + k];
-        b[k][1] = (double)st.y[i + k + 1] - st.y[i + k];
-        b[k][2] = (double)st.z[i + k + 1] - st.z[i + k];
-    }
-    double A[3], B[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int u = (a + 1) % 3, v = (a + 2) % 3;
-        A[a] = b[0][u] * b[1][v] - b[0][v] * b[1][u];
-        B[a] = b[1][u] * b[2][v] - b[1][v] * b[2][u];
-    }
-    const double AA = A[0] * A[0] + A[1] * A[1] + A[2] * A[2];
-    const double BB = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
-    const double L = norm_fp64(b[1][0] * b[1][0] + b[1][1] * b[1][1] + b[1][2] * b[1][2]);
-    const double den = norm_fp64(AA) * norm_fp64(BB);
-    const double cp = (A[0] * B[0] + A[1] * B[1] + A[2] * B[2]) / den;
-    const double sp = L * (b[0][0] * B[0] + b[0][1] * B[1] + b[0][2] * B[2]) / den;
-    double cn = cp, sn = sp;
+// Bond vector x[j] - x[i], exactly.
+__device__ __forceinline__ FF3 bond_ff3(const StateBuf& st, int i, int j) {
+    return FF3{ff_diff(st.x[j], st.x[i]), ff_diff(st.y[j], st.y[i]), ff_diff(st.z[j], st.z[i])};
+}
+__device__ __forceinline__ FF ff_of(const float (&v)[2]) { return FF{v[0], v[1]}; }
+
+// Angle energy k (cos theta - cos0)^2 at the middle bead i of i - 1, i, i + 1.
+__device__ __forceinline__ FF angle_energy_ff(const StateBuf& st, int i, const EnergyConsts& e) {
+    const FF3 u = bond_ff3(st, i, i - 1), w = bond_ff3(st, i, i + 1);
+    const FF c = ff_mul(ff_dot(u, w), ff_mul(ff_rsqrt(ff_dot(u, u)), ff_rsqrt(ff_dot(w, w))));
+    const FF d = ff_plus(c, ff_neg(ff_of(e.ff_cos0)));
+    return ff_mul(ff_of(e.ff_angle_k), ff_mul(d, d));
+}
+
+// Dihedral energy k [1 + cos(n phi - delta)] of the quadruplet i .. i + 3: cos
+// phi = A.B / (|A||B|), sin phi = |b2| b1.B / (|A||B|) with A = b1 x b2, B =
+// b2 x b3, and cos(n phi), sin(n phi) by the n-th power of cos phi + i sin phi.
+__device__ __forceinline__ FF dihedral_energy_ff(const StateBuf& st, int i, const EnergyConsts& e) {
+    const FF3 b1 = bond_ff3(st, i, i + 1), b2 = bond_ff3(st, i + 1, i + 2),
+              b3 = bond_ff3(st, i + 2, i + 3);
+    const FF3 A = ff_cross(b1, b2), B = ff_cross(b2, b3);
+    const FF b22 = ff_dot(b2, b2);
+    const FF inv = ff_mul(ff_rsqrt(ff_dot(A, A)), ff_rsqrt(ff_dot(B, B)));
+    const FF cp = ff_mul(ff_dot(A, B), inv);
+    const FF sp = ff_mul(ff_mul(ff_mul(b22, ff_rsqrt(b22)), ff_dot(b1, B)), inv);
+    FF cn = cp, sn = sp;
     for (int k = 1; k < e.dih_n; ++k) {
-        const double t = cn * cp - sn * sp;
-        sn = sn * cp + cn * sp;
+        const FF t = ff_plus(ff_mul(cn, cp), ff_neg(ff_mul(sn, sp)));
+        sn = ff_plus(ff_mul(sn, cp), ff_mul(cn, sp));
         cn = t;
     }
-    return e.dih_k * (1.0 + cn * e.dih_cd + sn * e.dih_sd);
+    const FF v = ff_plus(ff_plus(FF{1.0f, 0.f}, ff_mul(cn, ff_of(e.ff_dih_cd))),
+                         ff_mul(sn, ff_of(e.ff_dih_sd)));
+    return ff_mul(ff_of(e.ff_dih_k), v);
 }
 
 // Per bead: F_n with the terms the step kernel's kick uses (bonds, the field
 // by a direct trilinear gather, friction, step n's noise), the on-step velocity
 // v_n = v + dt/(2m) F_n, then kinetic energy, momentum and the bond energy of
-// the bond to the next bead (each bond once).  The bond energy is formed in
-// float-float (bond_energy_ff), the angle and dihedral energies in FP64, all
-// from the FP32 positions with exact differences; v_n and |v_n|^2 are FP32
+// the bond to the next bead (each bond once).  The bond, cosine-angle and
+// dihedral energies are formed in float-float (about 2^-46 per operation, like
+// the FP64 forms they replace, whose lengths carried one Newton step from an
+// FP32 seed: 3e-14), the harmonic angle's in FP64 for its arc tangent, all
+// from the FP32 positions with exact differences (the FP64 pipe bound the
+// angle and dihedral terms: 98 us for 200k beads with both); v_n and |v_n|^2 are FP32
 // (the FP32 force already limits them to ~1e-7) and are summed in float-float
 // over the thread's beads, its warp and its block, into one float-float
 // partial per observable and block (kinetic energy without the factor m/2 and
 // momentum without m, both applied in FP64 in k_energy_final).
 // Block blk of nb bead blocks (grid-stride over the beads within them).
+// kBonded: bonded_level(c).
+template <int kBonded>
 __device__ __forceinline__ void energy_beads_block(const StateBuf& st,
                                                    const uint32_t* __restrict__ meta, int n,
                                                    const MeshGeom& g,
@@ -102,8 +108,8 @@ __device__ __forceinline__ void energy_beads_block(const StateBuf& st,
                                                    const EnergyConsts& e,
                                                    float2* __restrict__ partials, int blk, int nb,
                                                    FF (*sh)[kRedBlock / 32]) {
-    double ub = 0.0;           // angle and dihedral energies (FP64)
-    float uh = 0.f, ul = 0.f;  // bond energy, float-float
+    double ub = 0.0;           // harmonic angle energies (FP64)
+    float uh = 0.f, ul = 0.f;  // the other bonded energies, float-float
     FF kf{0.f, 0.f}, pfx{0.f, 0.f}, pfy{0.f, 0.f}, pfz{0.f, 0.f};
     for (int i = blk * kRedBlock + threadIdx.x; i < n; i += nb * kRedBlock) {
         const float x = st.x[i], y = st.y[i], z = st.z[i];
@@ -117,35 +123,39 @@ __device__ __forceinline__ void energy_beads_block(const StateBuf& st,
             bond_force(x - xj, y - yj, z - zj, c.two_k, c.r0, fx, fy, fz);
             bond_energy_ff(x, y, z, xj, yj, zj, bond_ff(e), uh, ul);
         }
-        if (c.two_ka != 0.f) {
+        if (kBonded >= 1 && c.two_ka != 0.f) {
             angle_forces_of(st, meta, i, m, c, fx, fy, fz);
-            if ((m & kBondPrev) && (m & kBondNext)) {
-                // the angle centred here, once, in FP64 from the FP32 positions
-                const double ux = (double)st.x[i - 1] - x, uy = (double)st.y[i - 1] - y,
-                             uz = (double)st.z[i - 1] - z;
-                const double wx = (double)st.x[i + 1] - x, wy = (double)st.y[i + 1] - y,
-                             wz = (double)st.z[i + 1] - z;
-                const double uu = ux * ux + uy * uy + uz * uz, ww = wx * wx + wy * wy + wz * wz;
-                const double uw = ux * wx + uy * wy + uz * wz;
+            if ((m & kBondPrev) && (m & kBondNext)) {  // the angle centred here, once
                 if (e.angle_form == 1) {
                     // harmonic: theta = atan2(|u x w|, u.w)
+                    const double ux = (double)st.x[i - 1] - x, uy = (double)st.y[i - 1] - y,
+                                 uz = (double)st.z[i - 1] - z;
+                    const double wx = (double)st.x[i + 1] - x, wy = (double)st.y[i + 1] - y,
+                                 wz = (double)st.z[i + 1] - z;
                     const double qx = uy * wz - uz * wy, qy = uz * wx - ux * wz,
                                  qz = ux * wy - uy * wx;
-                    const double d = atan2(norm_fp64(qx * qx + qy * qy + qz * qz), uw) - e.theta0;
+                    const double d = atan2(norm_fp64(qx * qx + qy * qy + qz * qz),
+                                           ux * wx + uy * wy + uz * wz) -
+                                     e.theta0;
                     ub += e.angle_k * d * d;
                 } else {
-                    const double cth = uw / norm_fp64(uu * ww);
-                    ub += e.angle_k * (cth - e.cos0) * (cth - e.cos0);
+                    const FF u = ff_plus(FF{uh, ul}, angle_energy_ff(st, i, e));
+                    uh = u.h;
+                    ul = u.l;
                 }
             }
         }
-        if (c.kd != 0.f) {
+        if (kBonded == 2) {
             int back, fwd;
             chain_reach(meta, i, m, back, fwd);
             dihedral_forces_of(
                 [&](int d) { return make_float3(st.x[i + d], st.y[i + d], st.z[i + d]); }, back,
                 fwd, c, fx, fy, fz);
-            if (fwd == 3) ub += dihedral_energy_fp64(st, i, e);  // the one starting here, once
+            if (fwd == 3) {  // the one starting here, once
+                const FF u = ff_plus(FF{uh, ul}, dihedral_energy_ff(st, i, e));
+                uh = u.h;
+                ul = u.l;
+            }
         }
         const float4* Gt = G + (size_t)((m >> kTypeShift) & kTypeMask) * g.gnodes;
         gather_field_mode(Gt, g, c.force_mode, x, y, z, fx, fy, fz);
@@ -175,7 +185,7 @@ __device__ __forceinline__ void energy_beads_block(const StateBuf& st,
         pfz = ff_plus(pfz, uz);
     }
     FF v[kBeadVals] = {kf, ff_norm(uh, ul), pfx, pfy, pfz};
-    if (c.two_ka != 0.f || c.kd != 0.f) v[1] = ff_plus(v[1], ff_from_double(ub));
+    if (kBonded >= 1) v[1] = ff_plus(v[1], ff_from_double(ub));
     const int w = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < kBeadVals; ++k) {
@@ -256,8 +266,8 @@ __global__ void __launch_bounds__(kRedBlock) k_energy_nodes(const long long* __r
 
 // One launch for the bead and node sums: blocks 0 .. nn - 1 take the nodes
 // (kN species; 0: none), the rest the beads, so the two run side by side.
-template <int kN>
-__global__ void __launch_bounds__(kRedBlock, 4) k_energy_main(StateBuf st,
+template <int kN, int kBonded>
+__global__ void __launch_bounds__(kRedBlock, kBonded == 0 ? 4 : 3) k_energy_main(StateBuf st,
                                                               const uint32_t* __restrict__ meta,
                                                               int n, MeshGeom g,
                                                               const float4* __restrict__ G,
@@ -282,7 +292,7 @@ __global__ void __launch_bounds__(kRedBlock, 4) k_energy_main(StateBuf st,
         }
         blk -= nn;
     }
-    energy_beads_block(st, meta, n, g, G, c, step, e, bead_part, blk, nb,
+    energy_beads_block<kBonded>(st, meta, n, g, G, c, step, e, bead_part, blk, nb,
                        reinterpret_cast<FF(*)[kRedBlock / 32]>(sm));
     // the combining kernel may be scheduled once every block is here
     griddep_launch_dependents();
@@ -405,20 +415,24 @@ void launch_energy(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const f
         reinterpret_cast<unsigned long long*>(partials + (size_t)nb * kBeadVals);
     // up to three species: node and bead sums in one launch; more species:
     // the node sums in a launch of their own, after the beads
-    if (e.S <= 3) {
-        switch (e.S) {
-#define HPF_MAIN(k)                                                                              \
-    case k:                                                                                      \
-        k_energy_main<k><<<nn + nb, kRedBlock, 0, s>>>(st, meta, n, g, G, c, step, e, bead_part, \
-                                                       nb, D, node_part, nn);                    \
-        break;
-            HPF_MAIN(1) HPF_MAIN(2) HPF_MAIN(3)
-#undef HPF_MAIN
-        }
+    const int bonded = bonded_level(c);
+#define HPF_MAIN_B(k, B, blocks, nn_)                                                             \
+    k_energy_main<k, B><<<blocks, kRedBlock, 0, s>>>(st, meta, n, g, G, c, step, e, bead_part, nb, \
+                                                     D, node_part, nn_)
+#define HPF_MAIN(k, blocks, nn_)                           \
+    if (bonded == 2) HPF_MAIN_B(k, 2, blocks, nn_);        \
+    else if (bonded == 1) HPF_MAIN_B(k, 1, blocks, nn_);   \
+    else HPF_MAIN_B(k, 0, blocks, nn_);
+    if (e.S == 1) {
+        HPF_MAIN(1, nn + nb, nn)
+    } else if (e.S == 2) {
+        HPF_MAIN(2, nn + nb, nn)
+    } else if (e.S == 3) {
+        HPF_MAIN(3, nn + nb, nn)
     } else {
-        if (nb > 0)
-            k_energy_main<0><<<nb, kRedBlock, 0, s>>>(st, meta, n, g, G, c, step, e, bead_part, nb,
-                                                      D, node_part, 0);
+        if (nb > 0) {
+            HPF_MAIN(0, nb, 0)
+        }
         switch (e.S) {
 #define HPF_NODES(k)                                                                     \
     case k: k_energy_nodes<k><<<nn, kRedBlock, 0, s>>>(D, g.nodes, node_part); break;
@@ -426,6 +440,8 @@ void launch_energy(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const f
 #undef HPF_NODES
         }
     }
+#undef HPF_MAIN
+#undef HPF_MAIN_B
     switch (e.S) {
 #define HPF_FINAL(k)                                                                        \
     case k:                                                                                 \
@@ -451,7 +467,7 @@ void launch_energy_nodes_only(int n, MeshGeom g, const long long* D, const Energ
 #define HPF_ONLY(k)                                                                         \
     case k:                                                                                 \
         if (k <= 3)                                                                         \
-            k_energy_main<(k <= 3 ? k : 0)><<<nn, kRedBlock, 0, s>>>(                       \
+            k_energy_main<(k <= 3 ? k : 0), 0><<<nn, kRedBlock, 0, s>>>(                       \
                 StateBuf{}, nullptr, 0, g, nullptr, StepConsts{}, 0, e, nullptr, 0, D,      \
                 node_part, nn);                                                             \
         else                                                                                \
