@@ -603,6 +603,7 @@ __device__ __forceinline__ bool sw_late(unsigned it, unsigned long long t0) {
 // Bounded wait that also gives up when another role has aborted.
 __device__ __forceinline__ bool sw_wait(uint32_t bar, uint32_t parity, volatile int* abort_w,
                                         int* flag) {
+    if (mbar_test(bar, parity)) return true;  // without a look at the clock
     const unsigned long long t0 = sw_now();
     for (unsigned it = 0; it < kTcWaitLimit && !sw_late(it, t0); ++it) {
         if (mbar_test(bar, parity)) return true;
@@ -763,29 +764,48 @@ __device__ __forceinline__ void sw_reset_slot(uint32_t taddr, int g, const float
     }
 }
 
-// One channel half (8 BF16 channels) of a voxel to the padded layout, with
-// its periodic copies in the halo when it lies on a face (up to eight at a
-// corner).
-__device__ __forceinline__ void sw_store_half(__nv_bfloat16* __restrict__ act, const SweepArgs& a,
-                                              int X, int Y, int Z, int h, uint4 v) {
-    const int xs[2] = {X + 1, X == 0 ? a.mx + 1 : (X == a.mx - 1 ? 0 : -1)};
-    const int ys[2] = {Y + 1, Y == 0 ? a.my + 1 : (Y == a.my - 1 ? 0 : -1)};
-    const int zs[2] = {Z + 1, Z == 0 ? a.mz + 1 : (Z == a.mz - 1 ? 0 : -1)};
-    uint4* base = reinterpret_cast<uint4*>(act) + (size_t)h * (a.mz + 2) * a.py * a.px;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        if (zs[k] < 0) continue;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            if (ys[j] < 0) continue;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                if (xs[i] < 0) continue;
-                base[((size_t)zs[k] * a.py + ys[j]) * a.px + xs[i]] = v;
-            }
+// u / (1 + e^-u) from the hardware's 2^x and reciprocal (flushing subnormals,
+// which keeps their range handling out of the epilogue's inner loop).
+__device__ __forceinline__ float silu(float u) {
+    float e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(u * -1.44269504088896341f));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
+    return u * r;
+}
+
+// Where an epilogue lane stores its channel half (8 BF16 channels, 16 bytes)
+// of a voxel in the padded layout: the voxel itself and, when it lies on a
+// face, its periodic copies in the halo (up to eight places at a corner).  All
+// but the plane is the same for a whole run of planes, so it is worked out
+// once per run: the words from a plane's start, and the steps to the copies
+// beyond the x and y faces (0: none).
+struct HalfStore {
+    uint4* base;       // channel half, voxel (X, Y) of padded plane 0
+    int plane;         // words per padded plane
+    int dx, dy;
+    bool faces;        // some lane of the warp stores copies in x or y
+    __device__ __forceinline__ void begin(const SweepArgs& a, int X, int Y, int h, bool valid) {
+        plane = a.py * a.px;
+        base = reinterpret_cast<uint4*>(a.act_out) + (size_t)h * (a.mz + 2) * plane +
+               (Y + 1) * a.px + X + 1;
+        dx = !valid ? 0 : (X == 0 ? a.mx : (X == a.mx - 1 ? -a.mx : 0));
+        dy = !valid ? 0 : (Y == 0 ? a.my * a.px : (Y == a.my - 1 ? -a.my * a.px : 0));
+        faces = __any_sync(0xffffffffu, (dx | dy) != 0);
+    }
+    __device__ __forceinline__ void put(uint4* p, uint4 v) const {
+        *p = v;
+        if (faces) {
+            if (dx) p[dx] = v;
+            if (dy) p[dy] = v;
+            if (dx && dy) p[dx + dy] = v;
         }
     }
-}
+    __device__ __forceinline__ void operator()(const SweepArgs& a, int Z, uint4 v) const {
+        put(base + (size_t)(Z + 1) * plane, v);
+        if (Z == 0) put(base + (size_t)(a.mz + 1) * plane, v);
+        if (Z == a.mz - 1) put(base, v);
+    }
+};
 
 // The output planes [q0, q1) of this CTA in the order q = column Mz + z.
 __device__ __forceinline__ void sw_share(const SweepArgs& a, long long& q0, long long& q1) {
@@ -1067,6 +1087,8 @@ __global__ void __launch_bounds__(kSwThreads, kSwPerSM)
             sw_chunk(a, q, q1, x0, y0, zs, ze);
             const int X = x0 - 1 + bx, Y = y0 + by;
             const bool valid = bx >= 1 && bx <= kSwOX && X < a.mx && Y < a.my;
+            HalfStore store;
+            if (kL != 2) store.begin(a, X, Y, eg, valid);
             for (int zo = zs; zo < ze; ++zo, ++k) {
                 const int slot = k % kSwRing;
                 int got = 1;
@@ -1129,11 +1151,9 @@ __global__ void __launch_bounds__(kSwThreads, kSwPerSM)
                         __nv_bfloat162 h[4];
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
-                            const float u = o[2 * c], w = o[2 * c + 1];
-                            h[c] = __floats2bfloat162_rn(__fdividef(u, 1.0f + __expf(-u)),
-                                                         __fdividef(w, 1.0f + __expf(-w)));
+                            h[c] = __floats2bfloat162_rn(silu(o[2 * c]), silu(o[2 * c + 1]));
                         }
-                        sw_store_half(a.act_out, a, X, Y, zo, eg, *reinterpret_cast<uint4*>(h));
+                        store(a, zo, *reinterpret_cast<uint4*>(h));
                     }
                 }
             }
