@@ -11,14 +11,9 @@ __global__ void __launch_bounds__(256) k_scatter(StateBuf st, const uint32_t* __
                                                  int n, MeshGeom g,
                                                  unsigned long long* __restrict__ D) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float x = st.x[i], y = st.y[i], z = st.z[i];
-    const uint32_t m = meta[i];
-    const int T = (m >> kTypeShift) & kTypeMask;
-    const AxisCoord ax = axis_coord(x, g.inv_h[0], g.mx, g.inv_m[0]);
-    const AxisCoord ay = axis_coord(y, g.inv_h[1], g.my, g.inv_m[1]);
-    const AxisCoord az = axis_coord(z, g.inv_h[2], g.mz, g.inv_m[2]);
-    scatter_bead(D + (size_t)T * g.nodes, g, ax, ay, az);
+    const bool on = i < n;
+    scatter_paired(D, g, on ? st.x[i] : 0.f, on ? st.y[i] : 0.f, on ? st.z[i] : 0.f,
+                   on ? meta[i] : 0u, on);
 }
 
 void launch_scatter(StateBuf st, const uint32_t* meta, int n, MeshGeom g, unsigned long long* D,

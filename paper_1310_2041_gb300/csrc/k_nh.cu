@@ -124,6 +124,37 @@ __device__ __forceinline__ void bonded_of(const NhParams& p, const Drift& d, int
     }
 }
 
+// Stores a bead's state and checks it: whether it is finite and in range.
+__device__ __forceinline__ bool store_state(const NhParams& p, int i, float x, float y, float z,
+                                            float vx, float vy, float vz) {
+    p.out.x[i] = x;
+    p.out.y[i] = y;
+    p.out.z[i] = z;
+    p.out.vx[i] = vx;
+    p.out.vy[i] = vy;
+    p.out.vz[i] = vz;
+    const bool finite = isfinite(x) && isfinite(y) && isfinite(z) && isfinite(vx) &&
+                        isfinite(vy) && isfinite(vz);
+    const bool range = coord_in_range(x, p.g.inv_h[0]) && coord_in_range(y, p.g.inv_h[1]) &&
+                       coord_in_range(z, p.g.inv_h[2]);
+    if (!finite) atomicOr(p.flag, kFlagNonFinite);
+    else if (!range) atomicOr(p.flag, kFlagRange);
+    return finite && range;
+}
+
+// Kick, drift and deposit of bead i (a launch that ends on a refresh step).
+__device__ __forceinline__ void deposit_drift(const NhParams& p, const Drift& d, int i) {
+    float x = 0.f, y = 0.f, z = 0.f, vx, vy, vz;
+    uint32_t m = 0;
+    bool on = i < p.n;
+    if (on) {
+        m = p.meta[i];
+        moved(p, d, i, x, y, z, vx, vy, vz);
+        on = store_state(p, i, x, y, z, vx, vy, vz);
+    }
+    scatter_paired(p.D_next, p.g, x, y, z, m, on);
+}
+
 __device__ __forceinline__ double nh_rate(const NhConsts& t, double K) {
     return t.dof_kT > 0.0 ? fma(K, t.two_over_dof_kT, -1.0) * t.inv_tau2 : 0.0;
 }
@@ -157,6 +188,11 @@ __global__ void __launch_bounds__(kNhBlock) k_nh_step(const __grid_constant__ Nh
     d.hdt_m = 0.5f * p.c.dt_m;
     d.dt = p.c.dt;
     FF ke{0.f, 0.f};  // this thread's beads, float-float (FP32 pipe) up to the last block
+    if (p.D_next) {  // no force: the next field comes first; the warps' lanes stay together
+        for (int i0 = blockIdx.x * kNhBlock; i0 < p.n; i0 += gridDim.x * kNhBlock)
+            deposit_drift(p, d, i0 + tid);
+        return;
+    }
 #pragma unroll 2
     for (int i = blockIdx.x * kNhBlock + tid; i < p.n; i += gridDim.x * kNhBlock) {
         const uint32_t m = p.meta[i];
@@ -175,25 +211,7 @@ __global__ void __launch_bounds__(kNhBlock) k_nh_step(const __grid_constant__ Nh
             vz = fmaf(d.hdt_m, fz, vz);
             ke = ff_plus(ke, fmaf(vx, vx, fmaf(vy, vy, vz * vz)));
         }
-        p.out.x[i] = x;
-        p.out.y[i] = y;
-        p.out.z[i] = z;
-        p.out.vx[i] = vx;
-        p.out.vy[i] = vy;
-        p.out.vz[i] = vz;
-        const bool finite = isfinite(x) && isfinite(y) && isfinite(z) && isfinite(vx) &&
-                            isfinite(vy) && isfinite(vz);
-        if (!finite) atomicOr(p.flag, kFlagNonFinite);
-        else if (!(coord_in_range(x, p.g.inv_h[0]) && coord_in_range(y, p.g.inv_h[1]) &&
-                   coord_in_range(z, p.g.inv_h[2])))
-            atomicOr(p.flag, kFlagRange);
-        else if (p.D_next) {
-            const AxisCoord ax = axis_coord(x, p.g.inv_h[0], p.g.mx, p.g.inv_m[0]);
-            const AxisCoord ay = axis_coord(y, p.g.inv_h[1], p.g.my, p.g.inv_m[1]);
-            const AxisCoord az = axis_coord(z, p.g.inv_h[2], p.g.mz, p.g.inv_m[2]);
-            scatter_bead(p.D_next + (size_t)((m >> kTypeShift) & kTypeMask) * p.g.nodes, p.g,
-                         ax, ay, az);
-        }
+        store_state(p, i, x, y, z, vx, vy, vz);
     }
     if (!p.force_kick) return;
     // the kinetic-energy sum in float-float on the FP32 pipe (this GPU's FP64

@@ -56,10 +56,15 @@ __global__ void __launch_bounds__(kChunk, kOnePerSM) k_step_one(const __grid_con
         const bool ok = pipe.wait(i);
         const float(*s)[kSpan] = pipe.stage[i % kChunkStages];
         const int bead = pipe.bead0(i) + tid, e = tid + kChunkHalo;
-        if (ok && bead < p.n) {
-            float x = s[0][e], y = s[1][e], z = s[2][e];
+        const bool live = ok && bead < p.n;
+        float x = 0.f, y = 0.f, z = 0.f;
+        uint32_t m = 0;
+        if (live) {
+            x = s[0][e];
+            y = s[1][e];
+            z = s[2][e];
+            m = __float_as_uint(s[6][e]);
             float vx = s[3][e], vy = s[4][e], vz = s[5][e];
-            const uint32_t m = __float_as_uint(s[6][e]);
             const float s0 = __fmul_rn(x, g.inv_h[0]), s1 = __fmul_rn(y, g.inv_h[1]),
                         s2 = __fmul_rn(z, g.inv_h[2]);
             const float flx = floorf(s0), fly = floorf(s1), flz = floorf(s2);
@@ -142,14 +147,8 @@ __global__ void __launch_bounds__(kChunk, kOnePerSM) k_step_one(const __grid_con
             else if (!(coord_in_range(x, g.inv_h[0]) && coord_in_range(y, g.inv_h[1]) &&
                        coord_in_range(z, g.inv_h[2])))
                 atomicOr(p.flag, kFlagRange);
-            if (p.D_next) {
-                const AxisCoord ax = axis_coord(x, g.inv_h[0], g.mx, g.inv_m[0]);
-                const AxisCoord ay = axis_coord(y, g.inv_h[1], g.my, g.inv_m[1]);
-                const AxisCoord az = axis_coord(z, g.inv_h[2], g.mz, g.inv_m[2]);
-                scatter_bead(p.D_next + (size_t)((m >> kTypeShift) & kTypeMask) * g.nodes, g, ax, ay,
-                             az);
-            }
         }
+        if (p.D_next) scatter_paired(p.D_next, g, x, y, z, m, live);
         if (__syncthreads_or(!ok)) {  // every thread is done with the stage
             if (tid == 0) atomicOr(p.flag, kFlagTimeout);
             pipe.drain(i);

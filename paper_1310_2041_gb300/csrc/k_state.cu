@@ -90,26 +90,27 @@ __global__ void k_repermute(const float* __restrict__ pos_tag, const float* __re
                             const uint32_t* __restrict__ meta, int n, StateBuf st, MeshGeom g,
                             unsigned long long* __restrict__ D, int* __restrict__ flag) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t m = meta[i];
-    const uint32_t tag = m & kTagMask;
-    const float x = pos_tag[3 * tag], y = pos_tag[3 * tag + 1], z = pos_tag[3 * tag + 2];
-    const float vx = vel_tag[3 * tag], vy = vel_tag[3 * tag + 1], vz = vel_tag[3 * tag + 2];
-    if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(vx) && isfinite(vy) &&
-          isfinite(vz)))
-        atomicOr(flag, kFlagNonFinite);
-    st.x[i] = x;
-    st.y[i] = y;
-    st.z[i] = z;
-    st.vx[i] = vx;
-    st.vy[i] = vy;
-    st.vz[i] = vz;
-    if (D) {
-        const AxisCoord ax = axis_coord(x, g.inv_h[0], g.mx, g.inv_m[0]);
-        const AxisCoord ay = axis_coord(y, g.inv_h[1], g.my, g.inv_m[1]);
-        const AxisCoord az = axis_coord(z, g.inv_h[2], g.mz, g.inv_m[2]);
-        scatter_bead(D + (size_t)((m >> kTypeShift) & kTypeMask) * g.nodes, g, ax, ay, az);
+    const bool on = i < n;
+    uint32_t m = 0;
+    float x = 0.f, y = 0.f, z = 0.f;
+    if (on) {
+        m = meta[i];
+        const uint32_t tag = m & kTagMask;
+        x = pos_tag[3 * tag];
+        y = pos_tag[3 * tag + 1];
+        z = pos_tag[3 * tag + 2];
+        const float vx = vel_tag[3 * tag], vy = vel_tag[3 * tag + 1], vz = vel_tag[3 * tag + 2];
+        if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(vx) && isfinite(vy) &&
+              isfinite(vz)))
+            atomicOr(flag, kFlagNonFinite);
+        st.x[i] = x;
+        st.y[i] = y;
+        st.z[i] = z;
+        st.vx[i] = vx;
+        st.vy[i] = vy;
+        st.vz[i] = vz;
     }
+    if (D) scatter_paired(D, g, x, y, z, m, on);
 }
 
 __global__ void k_order(const uint32_t* __restrict__ meta, int n, int32_t* __restrict__ order) {

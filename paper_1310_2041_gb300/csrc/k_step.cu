@@ -296,7 +296,8 @@ __global__ void __launch_bounds__(kStepBlock, 2) k_step(StateBuf in, StateBuf ou
         y = fmaf(c.dt, vy, y);
         z = fmaf(c.dt, vz, z);
     }
-    if (live && t >= halo && t < kStepBlock - halo) {
+    const bool mine = live && t >= halo && t < kStepBlock - halo;
+    if (mine) {
         out.x[i] = x;
         out.y[i] = y;
         out.z[i] = z;
@@ -309,15 +310,9 @@ __global__ void __launch_bounds__(kStepBlock, 2) k_step(StateBuf in, StateBuf ou
         else if (!(coord_in_range(x, g.inv_h[0]) && coord_in_range(y, g.inv_h[1]) &&
                    coord_in_range(z, g.inv_h[2])))
             atomicOr(flag, kFlagRange);
-        if (D_next) {
-            // this launch ends on a refresh step: deposit the final positions
-            const AxisCoord ax = axis_coord(x, g.inv_h[0], g.mx, g.inv_m[0]);
-            const AxisCoord ay = axis_coord(y, g.inv_h[1], g.my, g.inv_m[1]);
-            const AxisCoord az = axis_coord(z, g.inv_h[2], g.mz, g.inv_m[2]);
-            scatter_bead(D_next + (size_t)((m >> kTypeShift) & kTypeMask) * g.nodes, g, ax, ay,
-                         az);
-        }
     }
+    // a launch that ends on a refresh step deposits the final positions
+    if (D_next) scatter_paired(D_next, g, x, y, z, m, mine);
 }
 
 template <int kTherm, int kForce, int kBonded>
@@ -702,8 +697,7 @@ __device__ __forceinline__ void pair_move(Pair& b, const PairForce& r, const Ste
 }
 
 __device__ __forceinline__ void finish_bead(const Bead& b, long long i, StateBuf out,
-                                            const MeshGeom& g, unsigned long long* D_next,
-                                            int* flag) {
+                                            const MeshGeom& g, int* flag) {
     out.x[i] = b.x;
     out.y[i] = b.y;
     out.z[i] = b.z;
@@ -716,12 +710,6 @@ __device__ __forceinline__ void finish_bead(const Bead& b, long long i, StateBuf
     else if (!(coord_in_range(b.x, g.inv_h[0]) && coord_in_range(b.y, g.inv_h[1]) &&
                coord_in_range(b.z, g.inv_h[2])))
         atomicOr(flag, kFlagRange);
-    if (D_next) {
-        const AxisCoord ax = axis_coord(b.x, g.inv_h[0], g.mx, g.inv_m[0]);
-        const AxisCoord ay = axis_coord(b.y, g.inv_h[1], g.my, g.inv_m[1]);
-        const AxisCoord az = axis_coord(b.z, g.inv_h[2], g.mz, g.inv_m[2]);
-        scatter_bead(D_next + (size_t)((b.m >> kTypeShift) & kTypeMask) * g.nodes, g, ax, ay, az);
-    }
 }
 
 // The observables' bead terms of a segment's final state (what the next
@@ -806,10 +794,14 @@ __device__ __forceinline__ void advance_pairs(const StateBuf& in, const StateBuf
                                 obs_acc);
     if (a0)
         finish_bead(Bead{b.x.x, b.y.x, b.z.x, b.vx.x, b.vy.x, b.vz.x, b.m0, 0.f, 0.f, 0.f}, i, out, g,
-                    D_next, flag);
+                    flag);
     if (a1)
         finish_bead(Bead{b.x.y, b.y.y, b.z.y, b.vx.y, b.vy.y, b.vz.y, b.m1, 0.f, 0.f, 0.f}, i + 1, out,
-                    g, D_next, flag);
+                    g, flag);
+    if (D_next) {
+        scatter_paired(D_next, g, b.x.x, b.y.x, b.z.x, b.m0, a0);
+        scatter_paired(D_next, g, b.x.y, b.y.y, b.z.y, b.m1, a1);
+    }
 }
 
 // One warp advances one segment (whole chains, base .. base + cnt) by n_sub
@@ -879,8 +871,12 @@ __device__ __forceinline__ void advance_segment(const StateBuf& in, const StateB
         b1.y = fmaf(c.dt, b1.vy, b1.y);
         b1.z = fmaf(c.dt, b1.vz, b1.z);
     }
-    if (a0) finish_bead(b0, (long long)base + j0, out, g, D_next, flag);
-    if (a1) finish_bead(b1, (long long)base + j1, out, g, D_next, flag);
+    if (a0) finish_bead(b0, (long long)base + j0, out, g, flag);
+    if (a1) finish_bead(b1, (long long)base + j1, out, g, flag);
+    if (D_next) {
+        scatter_paired(D_next, g, b0.x, b0.y, b0.z, b0.m, a0);
+        scatter_paired(D_next, g, b1.x, b1.y, b1.z, b1.m, a1);
+    }
 }
 
 // All replicas of a batch in one persistent launch (a single context is a
