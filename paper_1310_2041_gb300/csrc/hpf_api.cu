@@ -832,7 +832,7 @@ hpf_status hpf_init(const hpf_params* params, void* stream, hpf_ctx** out) {
     e = e ? e : cudaMalloc(&c->obs_part, sizeof(float2) * kBeadVals * step_warp_grid_cap());
     if (params->thermostat == 1) {
         e = e ? e : cudaMalloc(&c->nh, sizeof(NhDev));
-        e = e ? e : cudaMalloc(&c->nh_part, sizeof(double) * (nh_blocks((int)n) + 1));
+        e = e ? e : cudaMalloc(&c->nh_part, sizeof(double) * (nh_max_blocks((int)n) + 1));
         e = e ? e : cudaMalloc(&c->nh_F, sizeof(float) * 6 * bead_stride(c->n));
         e = e ? e : cudaMallocHost(&c->h_nh, sizeof(double) * 2);
         e = e ? e : cudaMemsetAsync(c->nh, 0, sizeof(NhDev), c->stream);

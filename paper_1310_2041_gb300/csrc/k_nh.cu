@@ -18,8 +18,8 @@
 // also deposits the positions into the next density mesh, then the refresh,
 // then force_kick).
 //
-// A fixed grid (at most kNhGrid blocks, set by n alone, so the summation
-// order is the same on every GPU) whose threads loop over the beads; the
+// A fixed grid (at most kNhGrid blocks, set by n and the bonded terms, so
+// the summation order is the same on every GPU) whose threads loop over the beads; the
 // state and the stored force are read from one buffer and written to the
 // other.  A bead's bonded force after the drift
 // needs its chain neighbours' new positions (two beads each way with angles,
@@ -29,12 +29,22 @@
 // is needed and every bit agrees.  Any chain length works.
 #include "nh_internal.cuh"
 
+#include <algorithm>
+
 namespace hpf {
 
 namespace {
 
 constexpr int kNhBlock = 256;
-constexpr int kNhGrid = 1024;  // at most this many blocks, each thread loops over beads
+// At most this many blocks, each thread looping over its beads: one wave of 5
+// CTAs on each of 152 SMs (48 registers), with dihedrals three waves of 2 (96).
+// 1M beads, a step's launch: 1024 blocks at 4 per SM (64 registers) took 32.6
+// us, two waves of which the second was two thirds full; 608 at 4 per SM 29.6,
+// 760 at 5 28.2, 912 at 6 31, 1216 at 8 40 (spills).  With angles 760 blocks
+// took 858 us for 20 steps against 1021 at 1024 blocks, with dihedrals 912
+// blocks 1342 against 1391.
+constexpr int kNhGrid[3] = {760, 760, 912};
+constexpr int kNhPerSM = 5;
 
 struct Drift {
     float s1, s2, hdt_m, dt;
@@ -172,15 +182,32 @@ __device__ __forceinline__ double nh_half(const NhConsts& t, double& xi, double&
     return s;
 }
 
+// Sum over the block in a fixed order (a tree over the lanes, then over the
+// warps); the sum is in thread 0.
+__device__ __forceinline__ FF block_sum_ff(FF v, FF* sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    v = warp_sum_ff(v);
+    if (lane == 0) sh[w] = v;
+    __syncthreads();
+    if (w == 0) {
+        v = lane < kNhBlock / 32 ? sh[lane] : FF{0.f, 0.f};
+#pragma unroll
+        for (int o = kNhBlock / 64; o > 0; o >>= 1)
+            v = ff_plus(v, FF{__shfl_down_sync(0xffffffffu, v.h, o),
+                              __shfl_down_sync(0xffffffffu, v.l, o)});
+    }
+    return v;
+}
+
 template <int kForce, int kBonded>
-__global__ void __launch_bounds__(kNhBlock) k_nh_step(const __grid_constant__ NhParams p) {
+__device__ __forceinline__ void nh_step(const NhParams& p) {
     // dependent launch: the previous launch's state, force and velocity
     // scales are read only after it has completed
     griddep_wait();
     griddep_launch_dependents();
     __shared__ FF s_ke[kNhBlock / 32];
     __shared__ bool s_last;
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x;
     Drift d;
     d.on = p.kick_drift != 0;
     d.s1 = d.on ? p.nh->s1 : 1.0f;
@@ -193,7 +220,7 @@ __global__ void __launch_bounds__(kNhBlock) k_nh_step(const __grid_constant__ Nh
             deposit_drift(p, d, i0 + tid);
         return;
     }
-#pragma unroll 2
+#pragma unroll (kBonded == 2 ? 2 : 1)
     for (int i = blockIdx.x * kNhBlock + tid; i < p.n; i += gridDim.x * kNhBlock) {
         const uint32_t m = p.meta[i];
         float x, y, z, vx, vy, vz;
@@ -217,36 +244,31 @@ __global__ void __launch_bounds__(kNhBlock) k_nh_step(const __grid_constant__ Nh
     // the kinetic-energy sum in float-float on the FP32 pipe (this GPU's FP64
     // rate is 1/64 of its FP32 rate): warp, block, then the blocks' partials
     // in a fixed order
-    ke = warp_sum_ff(ke);
-    if (lane == 0) s_ke[tid >> 5] = ke;
-    __syncthreads();
+    ke = block_sum_ff(ke, s_ke);
     if (tid == 0) {
-        FF b = s_ke[0];
-        for (int k = 1; k < kNhBlock / 32; ++k) b = ff_plus(b, s_ke[k]);
-        p.part[blockIdx.x] = make_float2(b.h, b.l);
+        p.part[blockIdx.x] = make_float2(ke.h, ke.l);
         __threadfence();
         s_last = atomicAdd(&p.nh->ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!s_last) return;
     // the last block sums the partials in a fixed order (strided per thread,
-    // then the same shuffle tree and warp order as above)
+    // then the same tree as above)
     __threadfence();
+    double xi = 0.0, eta = 0.0;
+    if (tid == 0) {
+        xi = p.nh->xi;
+        eta = p.nh->eta;
+    }
     FF v{0.f, 0.f};
     for (int k = tid; k < (int)gridDim.x; k += kNhBlock) {
         const float2 q = __ldcg(&p.part[k]);
         v = ff_plus(v, FF{q.x, q.y});
     }
-    v = warp_sum_ff(v);
-    __syncthreads();
-    if (lane == 0) s_ke[tid >> 5] = v;
-    __syncthreads();
+    v = block_sum_ff(v, s_ke);
     if (tid != 0) return;
-    FF tot = s_ke[0];
-    for (int k = 1; k < kNhBlock / 32; ++k) tot = ff_plus(tot, s_ke[k]);
-    const double sum = ff_to_double(tot);
+    const double sum = ff_to_double(v);
     double K = 0.5 * p.t.mass * sum;
-    double xi = p.nh->xi, eta = p.nh->eta;
     p.nh->ke = K;
     const double a = nh_half(p.t, xi, eta, K);  // the end of step n - 1
     const double b = nh_half(p.t, xi, eta, K);  // the start of step n
@@ -257,22 +279,34 @@ __global__ void __launch_bounds__(kNhBlock) k_nh_step(const __grid_constant__ Nh
     p.nh->ticket = 0u;
 }
 
+template <int kForce, int kBonded>
+__global__ void __launch_bounds__(kNhBlock, kNhPerSM) k_nh_step(const __grid_constant__ NhParams p) {
+    nh_step<kForce, kBonded>(p);
+}
+
+// With dihedrals 48 registers are too few.
+template <int kForce>
+__global__ void __launch_bounds__(kNhBlock) k_nh_step_dihedrals(const __grid_constant__ NhParams p) {
+    nh_step<kForce, 2>(p);
+}
+
+// A fixed grid (it depends only on n and the bonded terms): the summation order
+// of the kinetic energy is the same on every GPU.
+int nh_blocks(int n, int bonded) {
+    return std::min((n + kNhBlock - 1) / kNhBlock, kNhGrid[bonded]);
+}
+
 template <int kForce>
 void launch_nh_e(const NhParams& p, int bonded, cudaStream_t s) {
-    const int blocks = nh_blocks(p.n);
-    if (bonded == 2) launch_pdl(k_nh_step<kForce, 2>, blocks, kNhBlock, 0, s, p);
+    const int blocks = nh_blocks(p.n, bonded);
+    if (bonded == 2) launch_pdl(k_nh_step_dihedrals<kForce>, blocks, kNhBlock, 0, s, p);
     else if (bonded == 1) launch_pdl(k_nh_step<kForce, 1>, blocks, kNhBlock, 0, s, p);
     else launch_pdl(k_nh_step<kForce, 0>, blocks, kNhBlock, 0, s, p);
 }
 
 }  // namespace
 
-int nh_blocks(int n) {
-    // a fixed grid (it depends only on n): the summation order of the kinetic
-    // energy is the same on every GPU
-    const int b = (n + kNhBlock - 1) / kNhBlock;
-    return b < kNhGrid ? b : kNhGrid;
-}
+int nh_max_blocks(int n) { return std::max({nh_blocks(n, 0), nh_blocks(n, 1), nh_blocks(n, 2)}); }
 
 void launch_nh_step(const NhParams& p, cudaStream_t s) {
     if (p.n <= 0) return;

@@ -37,7 +37,7 @@ struct NhParams {
     int force_kick;  // F at the (new) positions; v += dt/(2m) F; K; thermostat half steps
 };
 
-int nh_blocks(int n);
+int nh_max_blocks(int n);  // of a launch, whatever the bonded terms
 void launch_nh_step(const NhParams& p, cudaStream_t s);
 
 }  // namespace hpf

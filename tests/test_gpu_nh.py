@@ -191,3 +191,23 @@ def test_empty_system_steps(hpf_gpu):
     s.set_state(z, z, np.zeros(0, np.int32), np.zeros((0, 2), np.int32))
     s.step(5)
     assert s.get_state()[2] == 5
+
+
+@pytest.mark.parametrize("n", [255, 257, 760 * 256 - 31, 760 * 256, 760 * 256 + 1, 2 * 760 * 256 + 300])
+def test_every_bead_counts_once_in_the_kinetic_energy(hpf_gpu, orc, n):
+    """Free beads at the edges of the blocks' shares and of the grid, the last
+    bead of each share 30 times as fast.  With tau = 0.01 a step changes xi by
+    dt / tau^2 = 100 times the relative excess of K: a fast bead left out or
+    counted twice shows as 0.2 or more, K's FP32 roundings (at most four of
+    2^-24 per bead and step) as 2.4e-5 a step."""
+    w = W.Workload("free", [(n, [0])], 12.0, 8, 1, [[0.0]], 0.0, field_every=2, steps=2)
+    d = W.generate(w)
+    fast = sorted({0, n - 1} | {i for i in (255, 256, 760 * 256 - 1, 760 * 256) if i < n})
+    d["vel"][fast] *= 30.0
+    s, pp = make(hpf_gpu, w, d, nh_tau=0.01)
+    s.step(2)
+    xi, eta = s.get_thermostat()
+    _, _, (xo, eo), _ = orc.run_nh(orc.make_params(**pp), d["pos"], d["vel"], d["type"], d["bonds"],
+                                   0, 2, xe=(0.0, 0.0))
+    assert abs(xi - xo) <= 1e-4 * max(1.0, abs(xo))
+    assert abs(eta - eo) <= 1e-6 * max(1.0, abs(xo))
