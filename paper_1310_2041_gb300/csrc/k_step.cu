@@ -3,8 +3,19 @@
 
 namespace hpf {
 
-constexpr int kStepBlock = 512;
 constexpr int kHaloMax = 16;  // most steps fused into one launch
+
+// Threads of a halo-form CTA (k_step): kStepBlock where the halo is at most
+// kNarrowHalo beads a side, kWideBlock where the redundant rim would cost more
+// than the finer CTAs give.  Four CTAs of 256 leave less of the chip idle in the last
+// wave than two of 512 (160k beads, 4 steps: 318 CTAs for 304 places against 646
+// for 608; 120 -> 110.5 us for 20 steps with their fields).  256 against 512
+// threads, same steps: halo 2 to 10 -4 to -12 % (160k and 600k beads, bonds
+// or angles), halo 15 and 16 0 to -12 %, halo 20 +2 % at 600k beads, halo 30
+// +14 %.
+constexpr int kStepBlock = 256;
+constexpr int kWideBlock = 512;
+constexpr int kNarrowHalo = kHaloMax;  // always met by bonds alone
 
 int step_halo_max() { return kHaloMax; }
 
@@ -51,13 +62,13 @@ void launch_forces(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const f
 
 // ------------------------------------------------------------------ A6 fused steps
 //
-// One CTA advances a window of kStepBlock consecutive beads (whole chains or
+// One CTA advances a window of kB consecutive beads (whole chains or
 // not) by n_sub steps without leaving the chip: positions live in registers,
 // bonded neighbours are exchanged through shared memory, and the frozen field
 // is sampled through a per-bead cache.  A bead's update after k steps depends
 // on beads up to k places away along its chain, so the outer `halo` beads on
 // each side are recomputed redundantly (bit-identically, the noise is keyed by
-// tag and step) and only the inner kStepBlock - 2 halo beads are written back.
+// tag and step) and only the inner kB - 2 halo beads are written back.
 //
 // Field cache: inside one cell the interpolated gradient is the trilinear
 // polynomial c0 + c1 fx + c2 fy + c3 fz + c4 fx fy + c5 fx fz + c6 fy fz
@@ -68,8 +79,9 @@ void launch_forces(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const f
 // h = 1, dt = 0.01 -- so most sub-steps read six shared float4s instead of
 // gathering eight corners from L1/L2.
 constexpr int kCachePlanes = 6;
-constexpr size_t kStepSmem = sizeof(float4) * kCachePlanes * kStepBlock +
-                             sizeof(float) * 3 * 2 * kStepBlock;
+constexpr size_t step_smem(int block) {
+    return sizeof(float4) * kCachePlanes * block + sizeof(float) * 3 * 2 * block;
+}
 
 // The cell polynomial's coefficients from its corners into cache slot t
 // (component-major: planes 2j, 2j + 1 hold c0..c7 of component j; kForce 1:
@@ -93,7 +105,7 @@ template <int kForce>
 __device__ __forceinline__ void fill_cell_cache(const float4* __restrict__ Gt, const MeshGeom& g,
                                                 float flx, float fly, float flz,
                                                 float4* __restrict__ cache, int t,
-                                                int stride = kStepBlock) {
+                                                int stride) {
     if (kForce == 2) {
         float c[6];
         stag_vertex_coefs(Gt, g, flx, fly, flz, c);
@@ -115,7 +127,7 @@ template <int kForce>
 __device__ __forceinline__ void eval_cell_cache(const float4* __restrict__ cache, int t, float fx,
                                                 float fy, float fz, float& Fx, float& Fy,
                                                 float& Fz, const MeshGeom& g,
-                                                int stride = kStepBlock) {
+                                                int stride) {
     if (kForce == 2) {
         const float4 lo = cache[t], hi = cache[stride + t];
         const float c[6] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y};
@@ -144,28 +156,31 @@ __device__ __forceinline__ void eval_cell_cache(const float4* __restrict__ cache
 // form no cycle.  With two position buffers a warp can run at most one
 // sub-step ahead of a neighbour, which has by then finished reading the buffer
 // it is about to overwrite.
-static_assert(kStepBlock / 32 <= 16, "named barriers 1..15 cover at most 16 warps");
+static_assert(kWideBlock / 32 <= 16, "named barriers 1..15 cover at most 16 warps");
+template <int kB>
 __device__ __forceinline__ void neighbour_sync(int w) {
-    constexpr int kWarps = kStepBlock / 32;
+    constexpr int kWarps = kB / 32;
     if (w > 0) asm volatile("bar.sync %0, 64;" ::"r"(w) : "memory");
     if (w + 1 < kWarps) asm volatile("bar.sync %0, 64;" ::"r"(w + 1) : "memory");
 }
 
-template <int kTherm, int kForce, int kBonded>
-__global__ void __launch_bounds__(kStepBlock, 2) k_step(StateBuf in, StateBuf out,
+template <int kB, int kTherm, int kForce, int kBonded>
+__global__ void __launch_bounds__(kB, 1024 / kB) k_step(StateBuf in, StateBuf out,
                                                         const uint32_t* __restrict__ meta, int n,
                                                         int halo, int n_sub, long long step0,
                                                         MeshGeom g, const float4* __restrict__ G,
                                                         StepConsts c,
                                                         unsigned long long* __restrict__ D_next,
                                                         int* __restrict__ flag) {
+    griddep_wait();
+    griddep_launch_dependents();
     extern __shared__ float4 smem4[];
-    float4* cache = smem4;                                   // [kCachePlanes][kStepBlock]
-    float* sx = reinterpret_cast<float*>(smem4 + kCachePlanes * kStepBlock);  // [2][block]
-    float* sy = sx + 2 * kStepBlock;
-    float* sz = sy + 2 * kStepBlock;
+    float4* cache = smem4;                                   // [kCachePlanes][kB]
+    float* sx = reinterpret_cast<float*>(smem4 + kCachePlanes * kB);  // [2][block]
+    float* sy = sx + 2 * kB;
+    float* sz = sy + 2 * kB;
     const int t = threadIdx.x;
-    const int payload = kStepBlock - 2 * halo;
+    const int payload = kB - 2 * halo;
     const long long i = (long long)blockIdx.x * payload - halo + t;
     const bool live = (i >= 0 && i < n);
     float x = 0.f, y = 0.f, z = 0.f, vx = 0.f, vy = 0.f, vz = 0.f;
@@ -181,10 +196,10 @@ __global__ void __launch_bounds__(kStepBlock, 2) k_step(StateBuf in, StateBuf ou
     }
     // out-of-range threads only fill their shared-memory slot
     const bool has_prev = live && (m & kBondPrev) && t > 0;
-    const bool has_next = live && (m & kBondNext) && t + 1 < kStepBlock;
+    const bool has_next = live && (m & kBondNext) && t + 1 < kB;
     // bond flags of the whole window, for the angles centred at the neighbours
     // and the dihedrals through them
-    __shared__ unsigned char s_bonds[kStepBlock];
+    __shared__ unsigned char s_bonds[kB];
     int back = 0, fwd = 0;  // consecutive bonds backwards / forwards inside the window (<= 3)
     if (kBonded >= 1) {
         s_bonds[t] = (unsigned char)((has_prev ? 1 : 0) | (has_next ? 2 : 0));
@@ -211,23 +226,23 @@ __global__ void __launch_bounds__(kStepBlock, 2) k_step(StateBuf in, StateBuf ou
     float cfx = __int_as_float(0x7fc00000), cfy = cfx, cfz = cfx;  // cached cell: none
     for (int k = 0; k < n_sub; ++k) {
         const int b = k & 1;
-        sx[b * kStepBlock + t] = x;
-        sy[b * kStepBlock + t] = y;
-        sz[b * kStepBlock + t] = z;
-        neighbour_sync(t >> 5);
+        sx[b * kB + t] = x;
+        sy[b * kB + t] = y;
+        sz[b * kB + t] = z;
+        neighbour_sync<kB>(t >> 5);
         const float s0 = __fmul_rn(x, g.inv_h[0]), s1 = __fmul_rn(y, g.inv_h[1]),
                     s2 = __fmul_rn(z, g.inv_h[2]);
         const float flx = cache_key<kForce>(s0), fly = cache_key<kForce>(s1),
                     flz = cache_key<kForce>(s2);
         if (flx != cfx || fly != cfy || flz != cfz) {
-            fill_cell_cache<kForce>(Gt, g, flx, fly, flz, cache, t);
+            fill_cell_cache<kForce>(Gt, g, flx, fly, flz, cache, t, kB);
             cfx = flx;
             cfy = fly;
             cfz = flz;
         }
         float fx = -c.fric * vx, fy = -c.fric * vy, fz = -c.fric * vz;
         eval_cell_cache<kForce>(cache, t, __fsub_rn(s0, flx), __fsub_rn(s1, fly),
-                                __fsub_rn(s2, flz), fx, fy, fz, g);
+                                __fsub_rn(s2, flz), fx, fy, fz, g, kB);
         if (kTherm == 1) {
             float nx, ny, nz;
             gauss3(c, tag, step0 + k, nx, ny, nz);
@@ -236,20 +251,20 @@ __global__ void __launch_bounds__(kStepBlock, 2) k_step(StateBuf in, StateBuf ou
             fz = fmaf(c.sigma, nz, fz);
         }
         const int tp = has_prev ? t - 1 : t, tn = has_next ? t + 1 : t;
-        bond_force(x - sx[b * kStepBlock + tp], y - sy[b * kStepBlock + tp],
-                   z - sz[b * kStepBlock + tp], has_prev ? c.two_k : 0.0f, c.r0, fx, fy, fz);
-        bond_force(x - sx[b * kStepBlock + tn], y - sy[b * kStepBlock + tn],
-                   z - sz[b * kStepBlock + tn], has_next ? c.two_k : 0.0f, c.r0, fx, fy, fz);
+        bond_force(x - sx[b * kB + tp], y - sy[b * kB + tp],
+                   z - sz[b * kB + tp], has_prev ? c.two_k : 0.0f, c.r0, fx, fy, fz);
+        bond_force(x - sx[b * kB + tn], y - sy[b * kB + tn],
+                   z - sz[b * kB + tn], has_next ? c.two_k : 0.0f, c.r0, fx, fy, fz);
         if (kBonded >= 1) {
             // the three angles this bead belongs to: centred at t - 1, t and t + 1
             const int tp2 = (has_prev && t >= 2) ? t - 2 : t;
-            const int tn2 = (has_next && t + 2 < kStepBlock) ? t + 2 : t;
+            const int tn2 = (has_next && t + 2 < kB) ? t + 2 : t;
             const bool left = has_prev && t >= 2 && (s_bonds[t - 1] & 1);
-            const bool right = has_next && t + 2 < kStepBlock && (s_bonds[t + 1] & 2);
-            const float xp = sx[b * kStepBlock + tp], yp = sy[b * kStepBlock + tp],
-                        zp = sz[b * kStepBlock + tp];
-            const float xn = sx[b * kStepBlock + tn], yn = sy[b * kStepBlock + tn],
-                        zn = sz[b * kStepBlock + tn];
+            const bool right = has_next && t + 2 < kB && (s_bonds[t + 1] & 2);
+            const float xp = sx[b * kB + tp], yp = sy[b * kB + tp],
+                        zp = sz[b * kB + tp];
+            const float xn = sx[b * kB + tn], yn = sy[b * kB + tn],
+                        zn = sz[b * kB + tn];
             float ax, ay, az, bx, by, bz;
             // centred at t: this bead takes minus both end shares
             angle_force(xp - x, yp - y, zp - z, xn - x, yn - y, zn - z,
@@ -259,22 +274,22 @@ __global__ void __launch_bounds__(kStepBlock, 2) k_step(StateBuf in, StateBuf ou
             fy -= ay + by;
             fz -= az + bz;
             // centred at t - 1 (ends t - 2 and t): this bead is end b
-            angle_force(sx[b * kStepBlock + tp2] - xp, sy[b * kStepBlock + tp2] - yp,
-                        sz[b * kStepBlock + tp2] - zp, x - xp, y - yp, z - zp,
+            angle_force(sx[b * kB + tp2] - xp, sy[b * kB + tp2] - yp,
+                        sz[b * kB + tp2] - zp, x - xp, y - yp, z - zp,
                         left ? c.two_ka : 0.0f, c, ax, ay, az, bx, by, bz);
             fx += bx;
             fy += by;
             fz += bz;
             // centred at t + 1 (ends t and t + 2): this bead is end a
-            angle_force(x - xn, y - yn, z - zn, sx[b * kStepBlock + tn2] - xn,
-                        sy[b * kStepBlock + tn2] - yn, sz[b * kStepBlock + tn2] - zn,
+            angle_force(x - xn, y - yn, z - zn, sx[b * kB + tn2] - xn,
+                        sy[b * kB + tn2] - yn, sz[b * kB + tn2] - zn,
                         right ? c.two_ka : 0.0f, c, ax, ay, az, bx, by, bz);
             fx += ax;
             fy += ay;
             fz += az;
         }
         if (kBonded == 2) {
-            const int o = b * kStepBlock + t;
+            const int o = b * kB + t;
             dihedral_forces_of(
                 [&](int d) { return make_float3(sx[o + d], sy[o + d], sz[o + d]); }, back, fwd, c,
                 fx, fy, fz);
@@ -296,7 +311,7 @@ __global__ void __launch_bounds__(kStepBlock, 2) k_step(StateBuf in, StateBuf ou
         y = fmaf(c.dt, vy, y);
         z = fmaf(c.dt, vz, z);
     }
-    const bool mine = live && t >= halo && t < kStepBlock - halo;
+    const bool mine = live && t >= halo && t < kB - halo;
     if (mine) {
         out.x[i] = x;
         out.y[i] = y;
@@ -315,22 +330,34 @@ __global__ void __launch_bounds__(kStepBlock, 2) k_step(StateBuf in, StateBuf ou
     if (D_next) scatter_paired(D_next, g, x, y, z, m, mine);
 }
 
-template <int kTherm, int kForce, int kBonded>
-static void launch_step_t(StateBuf in, StateBuf out, const uint32_t* meta, int n, int n_sub,
+template <int kB, int kTherm, int kForce, int kBonded>
+static void launch_step_b(StateBuf in, StateBuf out, const uint32_t* meta, int n, int halo, int n_sub,
                           long long step0, MeshGeom g, const float4* G, StepConsts c,
                           unsigned long long* D_next, int* flag, cudaStream_t s) {
     static std::once_flag attr[64];
     once_per_device(attr, [] {
-        cudaFuncSetAttribute(k_step<kTherm, kForce, kBonded>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepSmem);
+        cudaFuncSetAttribute(k_step<kB, kTherm, kForce, kBonded>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step_smem(kB));
     });
+    const int payload = kB - 2 * halo;
+    const int blocks = (n + payload - 1) / payload;
+    launch_pdl(k_step<kB, kTherm, kForce, kBonded>, dim3(blocks), dim3(kB), step_smem(kB), s, in, out,
+               meta, n, halo, n_sub, step0, g, G, c, D_next, flag);
+}
+
+template <int kTherm, int kForce, int kBonded>
+static void launch_step_t(StateBuf in, StateBuf out, const uint32_t* meta, int n, int n_sub,
+                          long long step0, MeshGeom g, const float4* G, StepConsts c,
+                          unsigned long long* D_next, int* flag, cudaStream_t s) {
     // a bead's update after k sub-steps depends on beads up to k (bonds), 2k
     // (angles) or 3k (dihedrals) places away along its chain
     const int halo = (kBonded + 1) * n_sub;
-    const int payload = kStepBlock - 2 * halo;
-    const int blocks = (n + payload - 1) / payload;
-    k_step<kTherm, kForce, kBonded><<<blocks, kStepBlock, kStepSmem, s>>>(
-        in, out, meta, n, halo, n_sub, step0, g, G, c, D_next, flag);
+    if (kBonded == 0 || halo <= kNarrowHalo)
+        launch_step_b<kStepBlock, kTherm, kForce, kBonded>(in, out, meta, n, halo, n_sub, step0, g, G,
+                                                           c, D_next, flag, s);
+    else if constexpr (kBonded > 0)
+        launch_step_b<kWideBlock, kTherm, kForce, kBonded>(in, out, meta, n, halo, n_sub, step0, g, G,
+                                                           c, D_next, flag, s);
 }
 
 template <int kTherm, int kForce>
