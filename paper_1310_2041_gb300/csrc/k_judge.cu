@@ -3,7 +3,7 @@
 //
 // One pass over the beads gathers both fields at once (sixteen corner loads in
 // flight per bead) and sums |Fa - Fb|^2 and |Fb|^2: two force passes through
-// memory, an FP64 error pass and a one-warp sum over its 1216 partials took
+// memory, an FP64 error pass and a one-warp sum over 1216 partials took
 // 18.6 + 18.6 + 37 + 74 us at 1M beads.  A bead's terms are formed in
 // float-float (the difference exactly, squares with their errors, about
 // 2^-45 relative) and added to the thread's FP64 sums, one addition per sum
@@ -17,7 +17,12 @@ namespace hpf {
 namespace {
 
 constexpr int kJudgeBlock = 256;
-constexpr int kJudgeGrid = 1216;  // eight blocks on each of 152 SMs, whatever the device
+// One wave of three blocks (80 registers: all sixteen corner loads of a bead in
+// flight) on each of 152 SMs, whatever the device.  A learned window of 1M
+// beads with its judge: 1012 us at 304 or 456 blocks, 1019 at 608 (4 per SM),
+// 1030 at 760 (5), 1034 at 1216 (48 registers, two waves).
+constexpr int kJudgePerSM = 3;
+constexpr int kJudgeGrid = kJudgePerSM * 152;
 
 struct JudgeScratch {
     unsigned ticket;
@@ -51,7 +56,7 @@ __device__ __forceinline__ void block_sum2(double& e, double& r, double (*sh)[kJ
     }
 }
 
-__global__ void __launch_bounds__(kJudgeBlock) k_judge(StateBuf st, const uint32_t* __restrict__ meta,
+__global__ void __launch_bounds__(kJudgeBlock, kJudgePerSM) k_judge(StateBuf st, const uint32_t* __restrict__ meta,
                                                        int n, MeshGeom g,
                                                        const float4* __restrict__ Ga,
                                                        const float4* __restrict__ Gb, int mode,
