@@ -213,8 +213,8 @@ hpf_status hpf_selftest_timeout(hpf_ctx* ctx, double* seconds);
 /* The field stencil runs on shared-memory tiles of the mesh, staged by TMA
  * tensor copies when the mesh allows it (Mx even, n_species <= 4), or untiled
  * (one ghosted node, or two real nodes, per thread).  The kernel is chosen
- * the first time the field is computed, by timing the eight candidates on
- * this mesh (that first refresh synchronises once).  shape[0..2] = tile
+ * from the mesh and the species count the first time the field is computed.
+ * shape[0..2] = tile
  * (x, y, z); (0, 0, 0) for the one-node untiled kernel (and before the first
  * refresh), (2, 1, 1) for the node-pair kernel; *uses_tma = 1 if the tiles
  * are staged by TMA, 0 otherwise.  Either pointer may be NULL.
@@ -223,7 +223,7 @@ hpf_status hpf_field_tile(const hpf_ctx* ctx, int32_t shape[3], int32_t* uses_tm
 
 /* Pin the stencil to candidate `tile` (0 .. 7: tiles (32,8,4), (32,8,8),
  * (16,16,4), (64,4,4), (16,16,8), (32,4,8), untiled one node per thread,
- * untiled node pairs) instead of autotuning; -1 autotunes again at the next
+ * untiled node pairs) instead of the chosen one; -1 chooses again at the next
  * field.  Every candidate computes the same bits.  Errors: HPF_ERR_INVALID. */
 hpf_status hpf_set_field_tile(hpf_ctx* ctx, int32_t tile);
 

@@ -53,7 +53,7 @@ struct hpf_ctx {
     float4* G = nullptr;              // field mesh (ghosted)
     float4* field_stage = nullptr;    // dense copy of the field for hpf_field's output
     FieldCoef* d_coef = nullptr;      // the stencil coefficients in device memory
-    int field_tile = -1;              // tiled stencil shape chosen by the autotuner (-1: not yet)
+    int field_tile = -1;              // stencil shape (-1: not chosen yet)
     int tmap_tile = -1;               // tile the tensor maps below were encoded for
     bool tmap_ok = false;             // TMA usable for this mesh
     CUtensorMap tmap[2];              // over mesh buffers 0 and 1
@@ -394,56 +394,6 @@ void fill_field_rep(hpf_ctx* c, int tile, int dm, TiledFieldRep& fr, int& blocks
                         blocks);
 }
 
-// Time every candidate tile on this launch shape and keep the fastest.  The
-// candidates compute the same field (the last launch leaves it in place).
-template <class Params, class Fill>
-int autotune_tile(cudaStream_t s, int S, Fill fill) {
-    if (S > 4) return -1;
-    // Each candidate timed launch by launch (an event between launches, so
-    // what counts is a launch's own duration, as in a step loop where the
-    // next kernel waits on the field), the median of kReps launches per
-    // round, the best of kRounds interleaved rounds (a single timing of a few
-    // launches picked a 1.5x slower tile often enough to matter).
-    constexpr int kRounds = 3, kReps = 5;
-    cudaEvent_t ev[kReps + 1];
-    int made = 0;
-    for (; made <= kReps; ++made)
-        if (cudaEventCreate(&ev[made]) != cudaSuccess) break;
-    if (made <= kReps) {
-        for (int k = 0; k < made; ++k) cudaEventDestroy(ev[k]);
-        cudaGetLastError();
-        return 0;
-    }
-    const int cands = field_tile_candidates();
-    std::vector<float> score(cands, 1e30f);
-    for (int round = 0; round < kRounds; ++round) {
-        for (int t = 0; t < cands; ++t) {
-            Params p;
-            fill(t, p);
-            launch_field_tiled(p, S, t, s);  // warm
-            cudaEventRecord(ev[0], s);
-            for (int rep = 0; rep < kReps; ++rep) {
-                launch_field_tiled(p, S, t, s);
-                cudaEventRecord(ev[rep + 1], s);
-            }
-            if (cudaEventSynchronize(ev[kReps]) != cudaSuccess) continue;
-            float d[kReps];
-            bool ok = true;
-            for (int rep = 0; rep < kReps; ++rep)
-                ok = ok && cudaEventElapsedTime(&d[rep], ev[rep], ev[rep + 1]) == cudaSuccess;
-            if (!ok) continue;
-            std::sort(d, d + kReps);
-            score[t] = std::min(score[t], d[kReps / 2]);
-        }
-    }
-    int best = 0;
-    for (int t = 1; t < cands; ++t)
-        if (score[t] < score[best]) best = t;
-    cudaGetLastError();
-    for (int k = 0; k <= kReps; ++k) cudaEventDestroy(ev[k]);
-    return best;
-}
-
 // The context's mesh holds the density of the current positions afterwards:
 // scatter into the other buffer (cleared first unless known zero) and flip.
 hpf_status scatter_current(hpf_ctx* c) {
@@ -472,13 +422,7 @@ hpf_status run_field(hpf_ctx* c) {
     if (c->S <= 4) {
         // the tiled (TMA-staged) stencil with one replica; a batch runs the same
         // kernel, so contexts and batch members agree bit for bit
-        if (c->field_tile < 0)
-            c->field_tile = autotune_tile<SingleFieldParams>(c->stream, c->S, [&](int t, SingleFieldParams& p) {
-                memset(&p, 0, sizeof p);
-                p.R = 1;
-                p.flag = c->dflag;
-                fill_field_rep(c, t, c->dmesh, p.rep[0], p.blocks);
-            });
+        if (c->field_tile < 0) c->field_tile = field_tile_for(c->geom, c->S);
         StageScope sc(c, HPF_STAGE_FIELD, 1);
         SingleFieldParams p;
         memset(&p, 0, sizeof p);
@@ -1540,7 +1484,7 @@ hpf_status bfail(hpf_batch* b, hpf_status s, const char* msg) {
 
 // The batched stencil over all replicas, each reading its mesh buffer
 // dmesh ^ flip: one tiled launch per distinct tile shape among the replicas
-// (each replica keeps the shape the autotuner picked for its mesh).
+// (field_tile_for each replica's mesh).
 void launch_batch_fields(hpf_batch* b, int flip) {
     const int S = b->rep[0]->S;
     std::vector<int> shapes;
@@ -1557,50 +1501,6 @@ void launch_batch_fields(hpf_batch* b, int flip) {
         }
         launch_field_tiled(p, S, t, b->stream);
     }
-}
-
-// Tile shapes: every candidate timed on each replica's own mesh gives a shape
-// per replica; the grouped launches this needs (one per distinct shape) are
-// then timed against the best single shape for all replicas in one launch,
-// and the faster of the two is kept.
-void batch_autotune(hpf_batch* b) {
-    const int S = b->rep[0]->S;
-    std::vector<int> per(b->R, 0);
-    for (int r = 0; r < b->R; ++r) {
-        hpf_ctx* c = b->rep[r];
-        per[r] = autotune_tile<TiledFieldParams>(b->stream, S, [&](int t, TiledFieldParams& p) {
-            memset(&p, 0, sizeof p);
-            p.flag = c->dflag;
-            p.R = 1;
-            fill_field_rep(c, t, c->dmesh, p.rep[0], p.blocks);
-        });
-    }
-    const int uni = autotune_tile<TiledFieldParams>(b->stream, S, [&](int t, TiledFieldParams& p) {
-        memset(&p, 0, sizeof p);
-        p.flag = b->rep[0]->dflag;
-        for (int r = 0; r < b->R; ++r) {
-            hpf_ctx* c = b->rep[r];
-            fill_field_rep(c, t, c->dmesh, p.rep[p.R++], p.blocks);
-        }
-    });
-    cudaEvent_t e0, e1;
-    float ms[2] = {0.f, 0.f};
-    if (cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess) {
-        for (int k = 0; k < 2; ++k) {
-            b->rep_tile = k == 0 ? per : std::vector<int>(b->R, uni);
-            launch_batch_fields(b, 0);  // warm
-            cudaEventRecord(e0, b->stream);
-            for (int rep = 0; rep < 3; ++rep) launch_batch_fields(b, 0);
-            cudaEventRecord(e1, b->stream);
-            if (cudaEventSynchronize(e1) != cudaSuccess ||
-                cudaEventElapsedTime(&ms[k], e0, e1) != cudaSuccess)
-                ms[k] = 0.f;
-        }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-    }
-    cudaGetLastError();
-    b->rep_tile = (ms[0] > 0.f && ms[0] < ms[1]) ? per : std::vector<int>(b->R, uni);
 }
 
 // Batched refresh of the replicas whose field is due (all of them in steady state).
@@ -1628,7 +1528,8 @@ hpf_status batch_refresh(hpf_batch* b) {
         }
         return HPF_OK;
     }
-    if (b->rep_tile.empty()) batch_autotune(b);
+    if (b->rep_tile.empty())
+        for (auto* c : b->rep) b->rep_tile.push_back(field_tile_for(c->geom, c->S));
     {
         StageScope sc(c0, HPF_STAGE_FIELD, 1);
         launch_batch_fields(b, 0);

@@ -1123,6 +1123,7 @@ void launch_step_warp_lerp(const SingleStepParams& p, const float4* G2, int j0, 
                            int max_seg, int therm, cudaStream_t s);
 void launch_field_batch(const BatchFieldParams& p, int S, cudaStream_t s);
 int field_tile_candidates();
+int field_tile_for(const MeshGeom& g, int S);  // the shape for a mesh and species count
 bool field_tile_is_plain(int id);
 void field_tile_shape(int id, int out[3]);
 void launch_field_tiled(const TiledFieldParams& p, int S, int tile, cudaStream_t s);

@@ -9,7 +9,9 @@
 // 16 bytes), else by plain loads.  TMA has no periodic mode: box elements
 // outside the mesh arrive as zeros and are then replaced by their periodic
 // images with plain loads (only tiles on the mesh boundary have any).  The
-// tile shape is chosen per mesh by timing the candidates (hpf_api.cu).
+// untiled shapes, which load neighbours through L1 and L2, turned out faster at
+// every mesh size (field_tile_for); the staged ones run when asked for by
+// hpf_set_field_tile.
 #include <cuda.h>
 
 #include "chunk_pipe.cuh"
@@ -25,7 +27,24 @@ constexpr int kTileCandidates = 8;
 constexpr int kTileShapes[kTileCandidates][3] = {
     {32, 8, 4}, {32, 8, 8}, {16, 16, 4}, {64, 4, 4}, {16, 16, 8}, {32, 4, 8}, {0, 0, 0},
     {2, 1, 1}};
+constexpr int kPlainTile = 6;
 constexpr int kPairTile = 7;
+
+// The shape for a mesh: one node per thread, except that a large mesh of one
+// species takes pairs (its loads are the longer part; 16 bytes each).  Kernel
+// times in us, best staged shape / one node / pair:
+//   S = 1: 15^3 7.1 / 2.8 / 3.6, 70^3 9.2 / 5.2 / 5.8, 140^3 27.3 / 21.7 / 21.3,
+//          256^3 130 / 116 / 112
+//   S = 2: 15^3 12.4 / 3.5 / 5.0, 41^3 13.0 / 4.0 / 5.4, 70^3 15.8 / 7.9 / 9.3,
+//          140^3 52 / 40 / 47, 256^3 261 / 223 / 254
+//   S = 3: 70^3 22.5 / 10.3 / 12.5, 140^3 85 / 58 / 67
+//   S = 4: 15^3 22.6 / 5.3 / 8.2, 70^3 30 / 13.3 / 17.7, 140^3 128 / 81 / 112
+// 64 meshes of 27^3 to 46^3 in one launch: 23.5 / 29.9 (one node / pair).
+// Timing the candidates on the device instead took 2.8 ms of a context's
+// first step and 190 ms of a batch's, and now and then kept the pairs.
+int field_tile_for(const MeshGeom& g, int S) {
+    return S == 1 && g.mx % 2 == 0 && g.nodes >= (1 << 21) ? kPairTile : kPlainTile;
+}
 
 int field_tile_candidates() { return kTileCandidates; }
 
@@ -187,10 +206,15 @@ __global__ void __launch_bounds__(TX * TY) k_field_tiled(const __grid_constant__
     }
 }
 
-// The untiled candidate: one thread per node of the ghosted array, neighbours
-// loaded directly (through L1/L2), same arithmetic as the tiled kernel.
+// The untiled stencil: one thread per node of the ghosted array, neighbours
+// loaded directly (through L1/L2), same arithmetic as the tiled kernel.  Small
+// meshes are one chain of dependent latencies: with 42 registers (six blocks
+// per SM) all loads of a node are in flight at once (3.56 -> 3.27 us at 15^3,
+// 8.2 -> 7.9 at 70^3, S = 2); a batch of many meshes fills the chip and takes eight
+// (24.6 -> 23.5).  Two or four nodes in z per thread, sharing their loads, were
+// slower (8.8 and 9.1 us at 70^3).
 template <int S, int kCap>
-__global__ void __launch_bounds__(256) k_field_plain(const __grid_constant__ TiledFieldParamsT<kCap> p) {
+__global__ void __launch_bounds__(256, kCap == 1 ? 6 : 8) k_field_plain(const __grid_constant__ TiledFieldParamsT<kCap> p) {
     griddep_wait();
     griddep_launch_dependents();
     const int lo = field_replica(p);
@@ -241,7 +265,7 @@ __global__ void __launch_bounds__(256) k_field_plain(const __grid_constant__ Til
 // rows are read as int64 pairs (7 loads per species for two nodes); an odd
 // extent uses scalar loads and a last pair of one node.  Each node writes its
 // ghost copies itself (x = 0 also at x = Mx, and so on), so no ghosted-index
-// arithmetic is needed.  Same arithmetic as the other candidates.
+// arithmetic is needed.  Same arithmetic as the other shapes.
 template <int S, int kCap>
 __global__ void __launch_bounds__(256) k_field_pair(const __grid_constant__ TiledFieldParamsT<kCap> p) {
     griddep_wait();

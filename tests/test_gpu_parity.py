@@ -622,3 +622,17 @@ def test_bounded_wait_gives_up_and_the_context_survives(hpf_gpu, orc):
     po, vo, _ = orc.run(oparams(orc, pp), d["pos"], d["vel"], d["type"], d["bonds"], 0, 10)
     assert step == 10
     assert np.max(np.abs(pos - po)) <= 1e-4 and np.max(np.abs(vel - vo)) <= 1e-4
+
+
+@pytest.mark.parametrize("S,mesh,shape", [(1, 128, (2, 1, 1)), (1, 129, (0, 0, 0)), (1, 126, (0, 0, 0)),
+                                          (2, 128, (0, 0, 0)), (4, 5, (0, 0, 0))])
+def test_the_stencil_is_chosen_by_mesh_and_species(hpf_gpu, S, mesh, shape):
+    """Node pairs for large even meshes of one species, one node per thread
+    otherwise; the same field, bit for bit, as the other of the two."""
+    w = W.Workload("mix", [(40 * S, [k % S for k in range(5)])], float(mesh), mesh, S,
+                   np.full((S, S), 0.7).tolist(), 0.1, field_every=1, steps=1)
+    s, d, _ = make(hpf_gpu, w)
+    F = s.field(D_in=s.scatter_density())
+    assert s.field_tile() == (shape, False)
+    s.force_field_tile(7 if shape == (0, 0, 0) else 6)
+    assert np.array_equal(F, s.field(D_in=s.scatter_density()))
