@@ -688,7 +688,7 @@ hpf_status energy_launch(hpf_ctx* c) {
                            c->nh ? reinterpret_cast<const double*>(c->nh) : nullptr, c->h_nh};
         if (c->obs_step == c->step) {
             // the bead terms came with the step launch: node sums and combination
-            StageScope sc(c, HPF_STAGE_ENERGY, 2);
+            StageScope sc(c, HPF_STAGE_ENERGY, energy_nodes_launches(c->S));
             launch_energy_nodes_only(c->n, c->geom, Dm, c->ec, c->obs_part, c->obs_nb,
                                      c->partials, eo, c->stream);
         } else {
@@ -771,6 +771,7 @@ hpf_status hpf_init(const hpf_params* params, void* stream, hpf_ctx** out) {
     e = e ? e : cudaMalloc(&c->partials,
                            sizeof(double) * energy_partials_needed(c->n, c->geom.nodes,
                                                                    c->p.n_species));
+    e = e ? e : cudaMemsetAsync(c->partials, 0, 2 * sizeof(double), c->stream);  // the ticket
     e = e ? e : cudaMallocHost(&c->h_out6, sizeof(double) * 8);
     e = e ? e : cudaEventCreateWithFlags(&c->energy_ev, cudaEventDisableTiming);
     e = e ? e : cudaMalloc(&c->obs_part, sizeof(float2) * kBeadVals * step_warp_grid_cap());

@@ -1139,6 +1139,7 @@ bool make_mesh_tensor_map(CUtensorMap* map, const long long* D, const MeshGeom& 
 void tile_grid(const MeshGeom& g, int tile, int* tiles_x, int* tiles_y, int* blocks);
 int energy_partials_needed(int n, int nodes, int S);
 int energy_launches(int n, int S);  // kernels launch_energy issues
+int energy_nodes_launches(int S);   // and launch_energy_nodes_only
 void launch_energy_nodes_only(int n, MeshGeom g, const long long* D, const EnergyConsts& e,
                               const float2* bead_part, int nb_bead, double* partials,
                               const EnergyOut& out, cudaStream_t s);

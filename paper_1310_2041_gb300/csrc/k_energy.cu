@@ -7,13 +7,14 @@ namespace hpf {
 // ------------------------------------------------------------------ A7 FP64 observables
 
 constexpr int kRedBlock = 256;    // the bead and node kernels
-constexpr int kFinalBlock = 1024;  // the one block that combines their partials
+constexpr int kFinalBlock = 1024;  // the one block that combines their partials (more than three species)
 // Grid-stride shares (on average) of a bead or node thread: small, so that a
 // million beads make about 2000 blocks, which the SMs take in several waves
 // with little left over for the last one (at 8 beads a thread the 489 blocks
-// of a million beads came to just over one wave of three blocks per SM).
-constexpr int kBeadsPerThread = 2;
-constexpr int kNodesPerThread = 2;
+// of a million beads came to just over one wave of three blocks per SM); more
+// beads give longer shares, so that the last block's sum over the blocks stays short.
+constexpr int kPerThread = 2;
+constexpr int kMaxBlocks = 2048;
 
 // Exact unsigned 128-bit sums (the field energy's node sums).
 struct U128 {
@@ -96,7 +97,7 @@ __device__ __forceinline__ FF dihedral_energy_ff(const StateBuf& st, int i, cons
 // (the FP32 force already limits them to ~1e-7) and are summed in float-float
 // over the thread's beads, its warp and its block, into one float-float
 // partial per observable and block (kinetic energy without the factor m/2 and
-// momentum without m, both applied in FP64 in k_energy_final).
+// momentum without m, both applied in FP64 in energy_combine).
 // Block blk of nb bead blocks (grid-stride over the beads within them).
 // kBonded: bonded_level(c).
 template <int kBonded>
@@ -264,101 +265,74 @@ __global__ void __launch_bounds__(kRedBlock) k_energy_nodes(const long long* __r
     griddep_launch_dependents();
 }
 
-// One launch for the bead and node sums: blocks 0 .. nn - 1 take the nodes
-// (kN species; 0: none), the rest the beads, so the two run side by side.
-template <int kN, int kBonded>
-__global__ void __launch_bounds__(kRedBlock, kBonded == 0 ? 4 : 3) k_energy_main(StateBuf st,
-                                                              const uint32_t* __restrict__ meta,
-                                                              int n, MeshGeom g,
-                                                              const float4* __restrict__ G,
-                                                              StepConsts c, long long step,
-                                                              EnergyConsts e,
-                                                              float2* __restrict__ bead_part,
-                                                              int nb, const long long* __restrict__ D,
-                                                              unsigned long long* __restrict__ node_part,
-                                                              int nn) {
-    constexpr int kQ = kN * (kN + 1) / 2 + 2;
-    constexpr int kBytes = (int)sizeof(U128) * kQ > (int)sizeof(FF) * kBeadVals
-                               ? (int)sizeof(U128) * kQ
-                               : (int)sizeof(FF) * kBeadVals;
-    __shared__ __align__(16) unsigned char sm[kBytes * (kRedBlock / 32)];
-    int blk = (int)blockIdx.x;
-    if constexpr (kN > 0) {
-        if (blk < nn) {
-            energy_nodes_block<kN>(D, g.nodes, node_part, blk, nn,
-                                   reinterpret_cast<U128(*)[kRedBlock / 32]>(sm));
-            griddep_launch_dependents();
-            return;
-        }
-        blk -= nn;
-    }
-    energy_beads_block<kBonded>(st, meta, n, g, G, c, step, e, bead_part, blk, nb,
-                       reinterpret_cast<FF(*)[kRedBlock / 32]>(sm));
-    // the combining kernel may be scheduled once every block is here
-    griddep_launch_dependents();
-}
+// One block of kB threads: the bead partials (float-float) and the node
+// partials (exact 128-bit) summed over the blocks in a fixed order -- each
+// thread a strided share of the blocks, its loads all in flight together, then
+// its warp, then each value by one warp over the warps' sums -- and combined in
+// FP64, the three independent parts by three warps, then written to the host.
+template <int kS, int kB>
+struct CombineSmem {
+    static constexpr int kQ = kS * (kS + 1) / 2 + 2;
+    FF f[kBeadVals][kB / 32];
+    U128 u[kQ][kB / 32];
+    double res[kBeadVals + kQ];
+};
 
-// One block: the bead partials (float-float) and the node partials (exact
-// 128-bit) summed over the blocks in a fixed order -- each thread a strided
-// share of the blocks, its loads all in flight together, then its warp, then
-// one lane per value over the warps -- and combined in FP64, then written to the host.
-template <int kS>
-__global__ void __launch_bounds__(kFinalBlock) k_energy_final(const float2* __restrict__ bead_part,
-                                                              int nb,
-                                                              const unsigned long long* __restrict__ node_part,
-                                                              int nn, int nodes, EnergyConsts e,
-                                                              EnergyOut out) {
+template <int kS, int kB>
+__device__ __forceinline__ void energy_combine(const float2* bead_part, int nb,
+                                               const unsigned long long* node_part, int nn,
+                                               int nodes, const EnergyConsts& e,
+                                               const EnergyOut& out, CombineSmem<kS, kB>& sh) {
     constexpr int kP = kS * (kS + 1) / 2;
     constexpr int kQ = kP + 2;
-    constexpr int kW = kFinalBlock / 32;
-    __shared__ FF shf[kBeadVals][kW];
-    __shared__ U128 shu[kQ][kW];
-    __shared__ double res[kBeadVals + kQ];
-    griddep_wait();  // launched programmatically after the partial sums
+    constexpr int kW = kB / 32;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     FF acc[kBeadVals];
 #pragma unroll
     for (int k = 0; k < kBeadVals; ++k) acc[k] = FF{0.f, 0.f};
-    for (int b = threadIdx.x; b < nb; b += kFinalBlock) {
+    for (int b = t; b < nb; b += kB) {
         float2 p[kBeadVals];
 #pragma unroll
-        for (int k = 0; k < kBeadVals; ++k) p[k] = bead_part[(size_t)b * kBeadVals + k];
+        for (int k = 0; k < kBeadVals; ++k) p[k] = __ldcg(&bead_part[(size_t)b * kBeadVals + k]);
 #pragma unroll
         for (int k = 0; k < kBeadVals; ++k) acc[k] = ff_plus(acc[k], FF{p[k].x, p[k].y});
     }
     U128 qa[kQ];
 #pragma unroll
     for (int q = 0; q < kQ; ++q) qa[q] = U128{0ull, 0ull};
-    for (int b = threadIdx.x; b < nn; b += kFinalBlock) {
+    for (int b = t; b < nn; b += kB) {
         U128 p[kQ];
 #pragma unroll
-        for (int q = 0; q < kQ; ++q)
-            p[q] = U128{node_part[((size_t)b * kQ + q) * 2], node_part[((size_t)b * kQ + q) * 2 + 1]};
+        for (int q = 0; q < kQ; ++q) {
+            const ulonglong2 v =
+                __ldcg(reinterpret_cast<const ulonglong2*>(node_part) + (size_t)b * kQ + q);
+            p[q] = U128{v.x, v.y};
+        }
 #pragma unroll
         for (int q = 0; q < kQ; ++q) u128_add(qa[q], p[q]);
     }
-    const int w = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < kBeadVals; ++k) {
         acc[k] = warp_sum_ff(acc[k]);
-        if ((threadIdx.x & 31) == 0) shf[k][w] = acc[k];
+        if (lane == 0) sh.f[k][w] = acc[k];
     }
 #pragma unroll
     for (int q = 0; q < kQ; ++q) {
         qa[q] = warp_sum_u128(qa[q]);
-        if ((threadIdx.x & 31) == 0) shu[q][w] = qa[q];
+        if (lane == 0) sh.u[q][w] = qa[q];
     }
     __syncthreads();
-    const int t = threadIdx.x;
-    if (t < kBeadVals) {
-        FF r = shf[t][0];
-        for (int j = 1; j < kW; ++j) r = ff_plus(r, shf[t][j]);
-        res[t] = ff_to_double(r);
-    } else if (t >= 32 && t < 32 + kQ) {  // another warp, so that both run at once
-        U128 r = shu[t - 32][0];
-        for (int j = 1; j < kW; ++j) u128_add(r, shu[t - 32][j]);
-        res[kBeadVals + t - 32] = u128_to_double(r);
+    for (int v = w; v < kBeadVals + kQ; v += kW) {
+        double r;
+        if (v < kBeadVals)
+            r = ff_to_double(warp_sum_ff(lane < kW ? sh.f[v][lane] : FF{0.f, 0.f}));
+        else
+            r = u128_to_double(warp_sum_u128(lane < kW ? sh.u[v - kBeadVals][lane] : U128{0ull, 0ull}));
+        if (lane == 0) sh.res[v] = r;
     }
     __syncthreads();
+    const double* res = sh.res;
+    const double ke = 0.5 * e.mass * res[0], ub = res[1];
     if (t == 0) {
         double q_chi = 0.0;
         int q = 0;
@@ -370,13 +344,14 @@ __global__ void __launch_bounds__(kFinalBlock) k_energy_final(const float2* __re
         const double w_f = e.w_scale * (0.5 * e.kT * pc * pc * q_chi +
                                         0.5 * e.inv_kappa * (pc * pc * t2 - 2.0 * pc * t1 +
                                                              (double)nodes));
-        const double ke = 0.5 * e.mass * res[0], ub = res[1];
-        const double px = e.mass * res[2], py = e.mass * res[3], pz = e.mass * res[4];
         out.out6[0] = ke;
         out.out6[1] = ub;
         out.out6[2] = w_f;
         out.out6[3] = ke + ub + w_f;
+    } else if (t == 32) {
+        const double px = e.mass * res[2], py = e.mass * res[3], pz = e.mass * res[4];
         out.out6[4] = sqrt(px * px + py * py + pz * pz);
+    } else if (t == 64) {
         out.out6[5] = e.n > 0 ? 2.0 * ke / (3.0 * (double)e.n) : 0.0;
         *out.h_flag = *out.flag;
         if (out.nh) {
@@ -386,99 +361,151 @@ __global__ void __launch_bounds__(kFinalBlock) k_energy_final(const float2* __re
     }
 }
 
-static int energy_blocks(int count, int per_thread);
-
-int energy_launches(int n, int S) { return S <= 3 ? 2 : (n > 0 ? 3 : 2); }
-
-int energy_partials_needed(int n, int nodes, int S) {
-    // bead partials (doubles), then per node block (S (S + 1) / 2 + 2) sums of two words
-    return energy_blocks(n, kBeadsPerThread) * kBeadVals +
-           energy_blocks(nodes, kNodesPerThread) * 2 * (S * (S + 1) / 2 + 2) + 1;
+// One launch for the bead and node sums and, with kN species (kN > 0), the
+// observables: blocks 0 .. nn - 1 take the nodes, the rest the beads, so the
+// two run side by side, and the last of them to finish (ticket, left at zero)
+// combines the partials of all.  A second launch of one block for that took
+// 9 us more, half of it before its first load: 6.2 + 9.0 -> 12.1 us for 10k beads,
+// 7.1 + 9.0 -> 13.0 for 70^3 nodes and given bead partials, 22.2 + 8.3 -> 29.2 for 200k
+// beads with dihedrals, and the gap between the two.  nb bead blocks; nb_part partials of them (formed elsewhere when nb is
+// 0).  kN 0: the beads alone.
+template <int kN, int kBonded>
+__global__ void __launch_bounds__(kRedBlock, kBonded == 0 ? 4 : 3) k_energy_main(
+    StateBuf st, const uint32_t* __restrict__ meta, int n, MeshGeom g, const float4* __restrict__ G,
+    StepConsts c, long long step, const __grid_constant__ EnergyConsts e, float2* bead_part, int nb,
+    int nb_part, const long long* __restrict__ D, unsigned long long* node_part, int nn,
+    unsigned* ticket, const __grid_constant__ EnergyOut out) {
+    constexpr int kQ = kN * (kN + 1) / 2 + 2;
+    constexpr int kS = kN > 0 ? kN : 1;  // without nodes the combination is not instantiated
+    union Smem {
+        U128 u[kQ][kRedBlock / 32];
+        FF f[kBeadVals][kRedBlock / 32];
+        CombineSmem<kS, kRedBlock> combine;
+    };
+    __shared__ __align__(16) unsigned char sm[sizeof(Smem)];
+    __shared__ bool s_last;
+    Smem& sh = *reinterpret_cast<Smem*>(sm);
+    griddep_wait();
+    griddep_launch_dependents();
+    const int blk = (int)blockIdx.x;
+    if (kN > 0 && blk < nn)
+        energy_nodes_block<kS>(D, g.nodes, node_part, blk, nn, sh.u);
+    else
+        energy_beads_block<kBonded>(st, meta, n, g, G, c, step, e, bead_part, kN > 0 ? blk - nn : blk,
+                                    nb, sh.f);
+    if constexpr (kN > 0) {
+        if (threadIdx.x < 32) {  // the warp that wrote the block's partials
+            __threadfence();
+            __syncwarp();
+            if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        }
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        if (threadIdx.x == 0) *ticket = 0u;
+        energy_combine<kS, kRedBlock>(bead_part, nb_part, node_part, nn, g.nodes, e, out, sh.combine);
+    }
 }
 
-// Blocks of the energy reductions: each thread takes a grid-stride share (at
-// most 8 beads or nodes per thread on average), independent of the device so
-// the summation order, and with it every FP64 bit, is the same on any GPU.
-static int energy_blocks(int count, int per_thread) {
-    const int per_block = kRedBlock * per_thread;
-    return (count + per_block - 1) / per_block;
+// The combination as a launch of its own (more than three species).
+template <int kS>
+__global__ void __launch_bounds__(kFinalBlock) k_energy_final(const float2* bead_part, int nb,
+                                                              const unsigned long long* node_part,
+                                                              int nn, int nodes,
+                                                              const __grid_constant__ EnergyConsts e,
+                                                              const __grid_constant__ EnergyOut out) {
+    __shared__ CombineSmem<kS, kFinalBlock> sh;
+    griddep_wait();  // launched programmatically after the partial sums
+    energy_combine<kS, kFinalBlock>(bead_part, nb, node_part, nn, nodes, e, out, sh);
+}
+
+// Blocks of the energy reductions: each thread takes a grid-stride share,
+// independent of the device so the summation order, and with it every FP64
+// bit, is the same on any GPU.
+static int energy_blocks(int count) {
+    const int b = (count + kRedBlock * kPerThread - 1) / (kRedBlock * kPerThread);
+    return b < kMaxBlocks ? b : kMaxBlocks;
+}
+
+int energy_launches(int n, int S) { return S <= 3 ? 1 : (n > 0 ? 3 : 2); }
+
+// Doubles: the ticket (and padding), per node block S (S + 1) / 2 + 2 sums of
+// two words, then the bead partials.
+constexpr int kTicketWords = 2;
+
+int energy_partials_needed(int n, int nodes, int S) {
+    return kTicketWords + energy_blocks(nodes) * 2 * (S * (S + 1) / 2 + 2) +
+           energy_blocks(n) * kBeadVals;
+}
+
+// The launches; nb_given >= 0: bead partials formed elsewhere.
+static void launch_sums(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const float4* G,
+                        const StepConsts& c, long long step, const long long* D,
+                        const EnergyConsts& e, const float2* given, int nb_given, double* partials,
+                        const EnergyOut& out, cudaStream_t s) {
+    const int nb = nb_given >= 0 ? 0 : energy_blocks(n);
+    const int nn = energy_blocks(g.nodes);
+    const int nb_part = nb_given >= 0 ? nb_given : nb;
+    unsigned* ticket = reinterpret_cast<unsigned*>(partials);
+    unsigned long long* node_part = reinterpret_cast<unsigned long long*>(partials + kTicketWords);
+    // kBeadVals float-float pairs (one double's room each) per block
+    float2* bead_part = nb_given >= 0
+                            ? const_cast<float2*>(given)
+                            : reinterpret_cast<float2*>(node_part + (size_t)nn * 2 *
+                                                                        (e.S * (e.S + 1) / 2 + 2));
+    // up to three species: one launch; more species: the beads, the node sums
+    // and the combination in launches of their own
+    const int bonded = bonded_level(c);
+#define HPF_MAIN_B(k, B, blocks)                                                                 \
+    launch_pdl(k_energy_main<k, B>, dim3(blocks), dim3(kRedBlock), 0, s, st, meta, n, g, G, c, step, \
+               e, bead_part, nb, nb_part, D, node_part, nn, ticket, out)
+#define HPF_MAIN(k, blocks)                         \
+    if (bonded == 2) HPF_MAIN_B(k, 2, blocks);      \
+    else if (bonded == 1) HPF_MAIN_B(k, 1, blocks); \
+    else HPF_MAIN_B(k, 0, blocks);
+    if (e.S <= 3) {
+        if (e.S == 1) {
+            HPF_MAIN(1, nn + nb)
+        } else if (e.S == 2) {
+            HPF_MAIN(2, nn + nb)
+        } else {
+            HPF_MAIN(3, nn + nb)
+        }
+        return;
+    }
+    if (nb > 0) {
+        HPF_MAIN(0, nb)
+    }
+#undef HPF_MAIN
+#undef HPF_MAIN_B
+    switch (e.S) {
+#define HPF_NODES(k)                                                                         \
+    case k:                                                                                  \
+        k_energy_nodes<k><<<nn, kRedBlock, 0, s>>>(D, g.nodes, node_part);                   \
+        launch_pdl(k_energy_final<k>, dim3(1), dim3(kFinalBlock), 0, s,                      \
+                   (const float2*)bead_part, nb_part, (const unsigned long long*)node_part, nn, \
+                   g.nodes, e, out);                                                         \
+        break;
+        HPF_NODES(4) HPF_NODES(5) HPF_NODES(6) HPF_NODES(7) HPF_NODES(8)
+#undef HPF_NODES
+    }
 }
 
 void launch_energy(StateBuf st, const uint32_t* meta, int n, MeshGeom g, const float4* G,
                    StepConsts c, long long step, const long long* D, const EnergyConsts& e,
                    double* partials, const EnergyOut& out, cudaStream_t s) {
-    const int nb = energy_blocks(n, kBeadsPerThread);
-    const int nn = energy_blocks(g.nodes, kNodesPerThread);
-    // bead partials: kBeadVals float-float pairs (one double's room each) per block
-    float2* bead_part = reinterpret_cast<float2*>(partials);
-    unsigned long long* node_part =
-        reinterpret_cast<unsigned long long*>(partials + (size_t)nb * kBeadVals);
-    // up to three species: node and bead sums in one launch; more species:
-    // the node sums in a launch of their own, after the beads
-    const int bonded = bonded_level(c);
-#define HPF_MAIN_B(k, B, blocks, nn_)                                                             \
-    k_energy_main<k, B><<<blocks, kRedBlock, 0, s>>>(st, meta, n, g, G, c, step, e, bead_part, nb, \
-                                                     D, node_part, nn_)
-#define HPF_MAIN(k, blocks, nn_)                           \
-    if (bonded == 2) HPF_MAIN_B(k, 2, blocks, nn_);        \
-    else if (bonded == 1) HPF_MAIN_B(k, 1, blocks, nn_);   \
-    else HPF_MAIN_B(k, 0, blocks, nn_);
-    if (e.S == 1) {
-        HPF_MAIN(1, nn + nb, nn)
-    } else if (e.S == 2) {
-        HPF_MAIN(2, nn + nb, nn)
-    } else if (e.S == 3) {
-        HPF_MAIN(3, nn + nb, nn)
-    } else {
-        if (nb > 0) {
-            HPF_MAIN(0, nb, 0)
-        }
-        switch (e.S) {
-#define HPF_NODES(k)                                                                     \
-    case k: k_energy_nodes<k><<<nn, kRedBlock, 0, s>>>(D, g.nodes, node_part); break;
-            HPF_NODES(4) HPF_NODES(5) HPF_NODES(6) HPF_NODES(7) HPF_NODES(8)
-#undef HPF_NODES
-        }
-    }
-#undef HPF_MAIN
-#undef HPF_MAIN_B
-    switch (e.S) {
-#define HPF_FINAL(k)                                                                        \
-    case k:                                                                                 \
-        launch_pdl(k_energy_final<k>, dim3(1), dim3(kFinalBlock), 0, s, (const float2*)bead_part, \
-                   nb, (const unsigned long long*)node_part, nn, g.nodes, e, out);         \
-        break;
-        HPF_FINAL(1) HPF_FINAL(2) HPF_FINAL(3) HPF_FINAL(4)
-        HPF_FINAL(5) HPF_FINAL(6) HPF_FINAL(7) HPF_FINAL(8)
-#undef HPF_FINAL
-    }
+    launch_sums(st, meta, n, g, G, c, step, D, e, nullptr, -1, partials, out, s);
 }
 
 // The node sums and the combination, with bead partials formed elsewhere
 // (nb_bead CTAs' worth, by the step launch that ended at this state).
+int energy_nodes_launches(int S) { return S <= 3 ? 1 : 2; }
+
 void launch_energy_nodes_only(int n, MeshGeom g, const long long* D, const EnergyConsts& e,
                               const float2* bead_part, int nb_bead, double* partials,
                               const EnergyOut& out, cudaStream_t s) {
-    const int nb = energy_blocks(n, kBeadsPerThread);
-    const int nn = energy_blocks(g.nodes, kNodesPerThread);
-    unsigned long long* node_part =
-        reinterpret_cast<unsigned long long*>(partials + (size_t)nb * kBeadVals);
-    switch (e.S) {
-#define HPF_ONLY(k)                                                                         \
-    case k:                                                                                 \
-        if (k <= 3)                                                                         \
-            k_energy_main<(k <= 3 ? k : 0), 0><<<nn, kRedBlock, 0, s>>>(                       \
-                StateBuf{}, nullptr, 0, g, nullptr, StepConsts{}, 0, e, nullptr, 0, D,      \
-                node_part, nn);                                                             \
-        else                                                                                \
-            k_energy_nodes<k><<<nn, kRedBlock, 0, s>>>(D, g.nodes, node_part);              \
-        launch_pdl(k_energy_final<k>, dim3(1), dim3(kFinalBlock), 0, s, bead_part, nb_bead, \
-                   (const unsigned long long*)node_part, nn, g.nodes, e, out);             \
-        break;
-        HPF_ONLY(1) HPF_ONLY(2) HPF_ONLY(3) HPF_ONLY(4)
-        HPF_ONLY(5) HPF_ONLY(6) HPF_ONLY(7) HPF_ONLY(8)
-#undef HPF_ONLY
-    }
+    launch_sums(StateBuf{}, nullptr, n, g, nullptr, StepConsts{}, 0, D, e, bead_part, nb_bead,
+                partials, out, s);
 }
 
 }  // namespace hpf
