@@ -73,26 +73,25 @@ __device__ __forceinline__ void tile_origin(const PropGeom& g, int t, int& x0, i
 // propagated gradient with flipped, transposed weights, no bias), multiplied by
 // the SiLU derivative of the layer below in the epilogue, on the
 // fifth-generation tensor cores.  A CTA (one warpgroup) works on tiles of
-// 8 x 16 x 4 voxels of the plain channels-last layout [V][16]; a
+// 8 x 16 x 2 voxels of the plain channels-last layout [V][16]; a
 // z-plane of a tile is 128 voxels = the 128 rows of one MMA (eight
 // x-consecutive voxels per 8-row core-matrix group, one group per y row).
-// The periodic 10 x 18 x 6 input box sits in shared memory as two planes of
+// The periodic 10 x 18 x 4 input box sits in shared memory as two planes of
 // 8-channel halves (16 bytes per voxel): the canonical K-major layout without
 // swizzle, so the box shifted by any in-plane offset (dy, dx) is a matrix
 // descriptor that starts at the shifted voxel (K halves one plane apart,
 // 8-row groups one box row apart).
 //
-// Each input plane z (box planes -1 .. 4 of the tile) feeds the output planes
+// Each input plane z (box planes -1 .. 2 of the tile) feeds the output planes
 // z + 1, z and z - 1 through the kernel offsets dz = -1, 0, +1 (an output
 // voxel n sums W[d] in(n + d)).  So the weights of one in-plane offset are
 // stacked for the three dz values as N = 3 x 16 columns, and the accumulators
-// of the four output planes sit in tensor memory in reverse order, 16 columns
-// each: the three planes an input plane feeds are then 48 consecutive columns,
-// and one tcgen05.mma (M 128, N 48, K 16, BF16 in, FP32 accumulate) per input
-// plane and in-plane offset updates all three; at the tile's first and last
-// input planes fewer planes exist (N = 16 or 32).  That is 6 x 9 MMAs per
-// tile instead of 27 x 4 of width 16, and every MMA reads its A operand once
-// for three output planes.  The accumulators are cleared by tcgen05.st
+// of the output planes sit in tensor memory in reverse order, 16 columns
+// each: the planes an input plane feeds are then consecutive columns,
+// and one tcgen05.mma (M 128, K 16, BF16 in, FP32 accumulate) per input
+// plane and in-plane offset updates them all (N = 32 inside the tile, 16 at its
+// first and last input planes).  That is 4 x 9 MMAs per tile instead of 27 x 2
+// of width 16, and an MMA reads its A operand once for two output planes.  The accumulators are cleared by tcgen05.st
 // before the tile's MMAs, which then all accumulate.
 //
 // One thread issues the MMAs and commits them to an mbarrier; all eight warps
@@ -100,13 +99,18 @@ __device__ __forceinline__ void tile_origin(const PropGeom& g, int t, int& x0, i
 // bounded (kTcWaitLimit polls);
 // a wait that gives up sets kFlagTimeout and the CTA stops after releasing
 // its tensor memory.
-constexpr int kTcX = 8, kTcY = 16, kTcZ = 4;
+// Two z-planes a tile: six CTAs fit an SM (37 KB each), and 70^3 voxels, 1575
+// tiles, take 1.7 rounds of them; with four planes (48 KB, four CTAs, 810 tiles)
+// the second of two rounds was one third full.  A training step at 70^3: 168.1 us at
+// four planes, 162.5 at two, 175.6 at six (three CTAs).
+constexpr int kTcX = 8, kTcY = 16, kTcZ = 2;
+constexpr int kTcPerSM = 6;
 constexpr int kTcBX = kTcX + 2, kTcBY = kTcY + 2, kTcBZ = kTcZ + 2;
 constexpr int kTcPlane = kTcBX * kTcBY;   // box voxels per z-plane
-constexpr int kTcBox = kTcPlane * kTcBZ;  // 1080 voxels per channel half
+constexpr int kTcBox = kTcPlane * kTcBZ;  // voxels per channel half
 constexpr int kTcInPlane = 9;             // in-plane offsets (dy, dx)
 constexpr int kTcRows16 = 48;             // B rows per in-plane offset: (dz, co)
-constexpr int kTcCols = 64;               // accumulator columns per set: 4 planes x 16
+constexpr int kTcCols = 16 * kTcZ;        // accumulator columns per set (a power of two from 32)
 constexpr unsigned kTcWaitLimit = 1u << 22;
 constexpr int kTcThreads = 256;          // two warps per tensor-memory lane quarter
 constexpr int kTcWCopies = 8;            // replicas of each packed weight image (spread L2 reads)
@@ -213,9 +217,11 @@ __device__ __forceinline__ void tc_zero_cols16(uint32_t taddr) {
         : "memory");
 }
 
-// g SiLU'(z).
+// g SiLU'(z), to be rounded to BF16, by the hardware's exponential and
+// reciprocal: with the full expf and division they were a quarter of the
+// kernel's time (a training step at 70^3 171.9 -> 167.5 us).
 __device__ __forceinline__ float silu_backward(float g, float z) {
-    const float s = 1.0f / (1.0f + expf(-z));
+    const float s = __fdividef(1.0f, 1.0f + __expf(-z));
     return g * s * (1.0f + z * (1.0f - s));
 }
 
@@ -271,7 +277,7 @@ __device__ __forceinline__ void tc_epilogue(uint32_t tcol, const PropGeom& g, in
 // [27][16 out][16 in], offset index 9 dz_index + in-plane offset (dy, dx);
 // K = 16 input channels of the planar layout [2][V][8].
 template <int kBuf>
-__global__ void __launch_bounds__(kTcThreads, kBuf == 1 ? 4 : 1)
+__global__ void __launch_bounds__(kTcThreads, kBuf == 1 ? kTcPerSM : 1)
     k_conv_tc(const __nv_bfloat16* __restrict__ in, const uint4* __restrict__ Wp,
               const float* __restrict__ z_in, __nv_bfloat16* __restrict__ gz_out, PropGeom g,
               int n_tiles, int* __restrict__ flag) {
@@ -416,7 +422,7 @@ __global__ void __launch_bounds__(kTcThreads, kBuf == 1 ? 4 : 1)
             // epilogue of the previous tile while this one is on the tensor cores
             const uint32_t accp = tmem + (uint32_t)(kTcCols * (b ^ 1));
 #pragma unroll 1
-            for (int p = 2 * (w >> 2); p < 2 * (w >> 2) + 2; ++p)
+            for (int p = (kTcZ / 2) * (w >> 2); p < (kTcZ / 2) * (w >> 2) + kTcZ / 2; ++p)
                 tc_epilogue(accp + (uint32_t)(16 * (kTcZ - 1 - p)), g, px0, py0, pz0 + p, z_in,
                             gz_out);
         }
@@ -434,7 +440,7 @@ __global__ void __launch_bounds__(kTcThreads, kBuf == 1 ? 4 : 1)
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t accp = tmem + (uint32_t)(kTcCols * pb);
 #pragma unroll 1
-            for (int p = 2 * (w >> 2); p < 2 * (w >> 2) + 2; ++p)
+            for (int p = (kTcZ / 2) * (w >> 2); p < (kTcZ / 2) * (w >> 2) + kTcZ / 2; ++p)
                 tc_epilogue(accp + (uint32_t)(16 * (kTcZ - 1 - p)), g, px0, py0, pz0 + p, z_in,
                             gz_out);
         }
@@ -459,8 +465,8 @@ int conv_tc_tiles(const PropGeom& g) {
     return ((g.mx + kTcX - 1) / kTcX) * ((g.my + kTcY - 1) / kTcY) * ((g.mz + kTcZ - 1) / kTcZ);
 }
 
-// One tile per CTA, single-buffered (48 KB of shared memory and 64
-// tensor-memory columns per CTA, four CTAs per SM overlap one another's box
+// One tile per CTA, single-buffered (37 KB of shared memory and 32
+// tensor-memory columns per CTA, six CTAs per SM overlap one another's box
 // loads, MMAs and epilogues); the attribute is set once per device.
 void conv_tc_setup() {
     static std::once_flag once[64];
