@@ -38,8 +38,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     return false;
 }
 
-// A CTA walks a run of chunks of kChunk consecutive beads, one bead per
-// thread, with kChunkHalo more staged on both sides for the chain neighbours.
+// A CTA walks a run of chunks of kC consecutive beads, one bead per thread, with kChunkHalo more staged on both sides for the chain neighbours.
 // The bead arrays are streamed by one bulk copy per array and chunk
 // (cp.async.bulk, completion on the stage's mbarrier), kChunkStages chunks
 // deep, so that a thread's only exposed latency is the field gather: with
@@ -48,14 +47,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 // in front of their first and behind their last element (kBeadPad and
 // bead_stride), so every copy starts on a 16-byte boundary and none needs a
 // bounds check.
-constexpr int kChunk = 256;
 constexpr int kChunkHalo = 4;
-constexpr int kSpan = kChunk + 2 * kChunkHalo;
 constexpr int kChunkStages = 3;
 static_assert(kChunkHalo <= kBeadPad && kChunkHalo * 4 % 16 == 0, "copies start at the halo");
 
-template <int kArrays>
+template <int kArrays, int kC>
 struct ChunkPipe {
+    static constexpr int kSpan = kC + 2 * kChunkHalo;
     float (*stage)[kArrays][kSpan];  // [kChunkStages]
     uint32_t bar;                    // shared address of the stages' mbarriers
     int first, count;                // this CTA's chunks
@@ -65,7 +63,7 @@ struct ChunkPipe {
     __device__ __forceinline__ void begin(float* smem, unsigned long long* bars, int n) {
         stage = reinterpret_cast<float(*)[kArrays][kSpan]>(smem);
         bar = smem_u32(bars);
-        const long long chunks = (n + kChunk - 1) / kChunk;
+        const long long chunks = (n + kC - 1) / kC;
         first = (int)(chunks * blockIdx.x / gridDim.x);
         count = (int)(chunks * (blockIdx.x + 1) / gridDim.x) - first;
         if (threadIdx.x == 0) {
@@ -90,13 +88,13 @@ struct ChunkPipe {
             asm volatile(
                 "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
                 "[%3];" ::"r"(smem_u32(&stage[s][lane][0])),
-                "l"(reinterpret_cast<const float*>(src) + (long long)(first + i) * kChunk - kChunkHalo),
+                "l"(reinterpret_cast<const float*>(src) + (long long)(first + i) * kC - kChunkHalo),
                 "r"(kBytes), "r"(b)
                 : "memory");
     }
 
     // First bead of chunk i.
-    __device__ __forceinline__ int bead0(int i) const { return (first + i) * kChunk; }
+    __device__ __forceinline__ int bead0(int i) const { return (first + i) * kC; }
     __device__ __forceinline__ bool wait(int i) const {
         return mbar_wait(bar + 8 * (i % kChunkStages), (i / kChunkStages) & 1);
     }

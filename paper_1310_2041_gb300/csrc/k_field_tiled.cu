@@ -28,6 +28,7 @@ constexpr int kTileShapes[kTileCandidates][3] = {
     {32, 8, 4}, {32, 8, 8}, {16, 16, 4}, {64, 4, 4}, {16, 16, 8}, {32, 4, 8}, {0, 0, 0},
     {2, 1, 1}};
 constexpr int kPlainTile = 6;
+constexpr int kPlainBlock = 128;
 constexpr int kPairTile = 7;
 
 // The shape for a mesh: one node per thread, except that a large mesh of one
@@ -208,19 +209,20 @@ __global__ void __launch_bounds__(TX * TY) k_field_tiled(const __grid_constant__
 
 // The untiled stencil: one thread per node of the ghosted array, neighbours
 // loaded directly (through L1/L2), same arithmetic as the tiled kernel.  Small
-// meshes are one chain of dependent latencies: with 42 registers (six blocks
+// meshes are one chain of dependent latencies: with 42 registers (1536 threads
 // per SM) all loads of a node are in flight at once (3.56 -> 3.27 us at 15^3,
-// 8.2 -> 7.9 at 70^3, S = 2); a batch of many meshes fills the chip and takes eight
-// (24.6 -> 23.5).  Two or four nodes in z per thread, sharing their loads, were
+// 8.2 -> 7.9 at 70^3, S = 2); a batch of many meshes fills the chip and takes 2048
+// (24.6 -> 23.5).  Blocks of 128 instead of 256 spread a small mesh over more SMs
+// (10k beads, 20 refreshes and steps: -3 us).  Two or four nodes in z per thread, sharing their loads, were
 // slower (8.8 and 9.1 us at 70^3).
 template <int S, int kCap>
-__global__ void __launch_bounds__(256, kCap == 1 ? 6 : 8) k_field_plain(const __grid_constant__ TiledFieldParamsT<kCap> p) {
+__global__ void __launch_bounds__(kPlainBlock, kCap == 1 ? 12 : 16) k_field_plain(const __grid_constant__ TiledFieldParamsT<kCap> p) {
     griddep_wait();
     griddep_launch_dependents();
     const int lo = field_replica(p);
     const TiledFieldRep& r = p.rep[lo];
     const MeshGeom& g = r.g;
-    const int pnode = ((int)blockIdx.x - r.blk_begin) * 256 + threadIdx.x;
+    const int pnode = ((int)blockIdx.x - r.blk_begin) * kPlainBlock + threadIdx.x;
     if (pnode >= g.gnodes) return;
     const int px = pnode % g.gx, py = (pnode / g.gx) % (g.my + 1), pz = pnode / g.gxy;
     const int x = px == g.mx ? 0 : px, y = py == g.my ? 0 : py, z = pz == g.mz ? 0 : pz;
@@ -376,8 +378,8 @@ static void launch_for_species(const TiledFieldParamsT<kCap>& p, int tile, cudaS
             else k_field_pair<S, kCap><<<p.blocks, 256, 0, s>>>(p);
             break;
         default:
-            if (kCap == 1) launch_pdl(k_field_plain<S, kCap>, p.blocks, 256, 0, s, p);
-            else k_field_plain<S, kCap><<<p.blocks, 256, 0, s>>>(p);
+            if (kCap == 1) launch_pdl(k_field_plain<S, kCap>, p.blocks, kPlainBlock, 0, s, p);
+            else k_field_plain<S, kCap><<<p.blocks, kPlainBlock, 0, s>>>(p);
             break;
     }
 }
@@ -463,10 +465,10 @@ void tile_grid(const MeshGeom& g, int tile, int* tiles_x, int* tiles_y, int* blo
         *blocks = (((g.mx + 1) >> 1) * g.my * g.mz + 255) / 256;
         return;
     }
-    if (t[0] == 0) {  // untiled: 256 nodes of the ghosted array per block
+    if (t[0] == 0) {  // untiled: kPlainBlock nodes of the ghosted array per block
         *tiles_x = 0;
         *tiles_y = 0;
-        *blocks = (g.gnodes + 255) / 256;
+        *blocks = (g.gnodes + kPlainBlock - 1) / kPlainBlock;
         return;
     }
     const int nx = (g.mx + 1 + t[0] - 1) / t[0];

@@ -20,7 +20,16 @@ namespace hpf {
 namespace {
 
 constexpr int kOneArrays = 7;  // x y z vx vy vz meta
-constexpr int kOnePerSM = 3;    // resident CTAs (80 registers; four, at 64, spill)
+// Beads (threads) of a CTA's chunk, and in a system of at most four small ones
+// an SM.  Small systems are one chain of latencies, to which a chunk's gather
+// and deposit on one SM add; 256 against 128, 20 steps of one launch and one
+// field: 5k beads 134.9 / 123.8 us, 10k 135.8 / 124.9, 30k 158 / 150, 80k 204 / 201;
+// past one chunk for every resident CTA the small ones lose: 120k 247 / 276, 1M
+// 472 / 513.
+constexpr int kChunk = 256;
+constexpr int kSmallChunk = 128;
+constexpr int kSmallPerSM = 4;
+constexpr int kOnePerSM = 3;      // resident CTAs of 256 threads (80 registers; four, at 64, spill)
 
 struct OneParams {
     const void* src[kOneArrays];
@@ -34,12 +43,15 @@ struct OneParams {
     int* flag;
 };
 
-template <int kTherm, bool kWarp>
-__global__ void __launch_bounds__(kChunk, kOnePerSM) k_step_one(const __grid_constant__ OneParams p) {
+template <int kC, int kTherm, bool kWarp>
+__global__ void __launch_bounds__(kC, kOnePerSM * 256 / kC)
+    k_step_one(const __grid_constant__ OneParams p) {
+    using Pipe = ChunkPipe<kOneArrays, kC>;
+    constexpr int kSpan = Pipe::kSpan;
     __shared__ __align__(128) float smem[kChunkStages * kOneArrays * kSpan];
     __shared__ __align__(8) unsigned long long bars[kChunkStages];
     const int tid = threadIdx.x;
-    ChunkPipe<kOneArrays> pipe;
+    Pipe pipe;
     pipe.begin(smem, bars, p.n);
     griddep_wait();
     griddep_launch_dependents();
@@ -173,16 +185,21 @@ void launch_step_one(StateBuf in, StateBuf out, const uint32_t* meta, int n, lon
     once_per_device(once, [dev] {
         cudaDeviceGetAttribute(&sms[dev & 63], cudaDevAttrMultiProcessorCount, dev);
     });
-    const int chunks = (n + kChunk - 1) / kChunk, cap = kOnePerSM * (sms[dev & 63] > 0 ? sms[dev & 63] : 1);
+    const int n_sm = sms[dev & 63] > 0 ? sms[dev & 63] : 1;
+    const bool small = n <= kSmallPerSM * kSmallChunk * n_sm;
+    const int chunk = small ? kSmallChunk : kChunk;
+    const int chunks = (n + chunk - 1) / chunk, cap = kOnePerSM * 256 / chunk * n_sm;
     const int blocks = chunks < cap ? chunks : cap;
     const OneParams p{{in.x, in.y, in.z, in.vx, in.vy, in.vz, meta}, out, n, step, g, G, c, D_next,
                       flag};
     const int th = step_thermostat(c);
-#define HPF_ONE(T, W) launch_pdl(k_step_one<T, W>, dim3(blocks), dim3(kChunk), 0, s, p)
+#define HPF_ONE_C(C, T, W) launch_pdl(k_step_one<C, T, W>, dim3(blocks), dim3(C), 0, s, p)
+#define HPF_ONE(T, W) small ? HPF_ONE_C(kSmallChunk, T, W) : HPF_ONE_C(kChunk, T, W)
     if (th == 1) warp_order ? HPF_ONE(1, true) : HPF_ONE(1, false);
     else if (th == 2) warp_order ? HPF_ONE(2, true) : HPF_ONE(2, false);
     else warp_order ? HPF_ONE(0, true) : HPF_ONE(0, false);
 #undef HPF_ONE
+#undef HPF_ONE_C
 }
 
 }  // namespace hpf

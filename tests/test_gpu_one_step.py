@@ -50,3 +50,20 @@ def test_single_steps_give_the_bits_of_a_period(hpf_gpu, name):
             out.append(s.get_state() + (s.scatter_density(),))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("free", [127, 128, 129, 77824, 77825, 116737])
+def test_chunk_sizes_give_the_bits_of_a_period(hpf_gpu, free):
+    """Both sides of the small chunks' edges, of the system size up to which
+    they are used and of the size one chunk per resident CTA covers."""
+    w = solvent_blend(1, 7, free - 7, max(4.0, (free / 3.0) ** (1.0 / 3.0)), 4 if free < 200 else 32)
+    d = W.generate(w)
+    out = []
+    for calls in ((4, 4), (1,) * 8):
+        with hpf_gpu.System(hpf_gpu.make_params(**w.params())) as s:
+            s.set_state(d["pos"], d["vel"], d["type"], d["bonds"])
+            for n in calls:
+                s.step(n)
+            out.append(s.get_state() + (s.scatter_density(),))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
