@@ -915,6 +915,23 @@ __device__ __forceinline__ int uniform_warp() {
     return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
 }
 
+// The segment a warp takes in the round that starts at segment r.  A block's
+// warps take neighbouring segments (which share cells in L1), but those of a
+// partial round are dealt out over all blocks, the later half's (the second
+// CTA of an SM) on other schedulers, so that every SM gets its share.  A
+// second or later round of less than two segments a block stays with neighbouring warps: it
+// is over sooner that way (160k beads 75.2 / 77.5 us dealt out, 320k 105.6 /
+// 110; two launches of 10 steps with their fields).  Together / dealt out:
+// 5k beads 42.6 / 39.2, 40k 49.8 / 46.2, 120k 61.2 / 58.7, 240k 90.8 / 86.5,
+// 1M 254.8 / 252.9; 200k with dihedrals, four launches, 214 / 189.
+__device__ __forceinline__ int segment_of(int r, int total, int warp) {
+    constexpr int kWarps = kWarpBlock / 32;
+    const int rem = total - r, grid = (int)gridDim.x, block = (int)blockIdx.x;
+    if (rem >= grid * kWarps || (r > 0 && rem < 2 * grid)) return r + block * kWarps + warp;
+    const int slot = (warp + (2 * block >= grid ? kWarps - 2 : 0)) % kWarps;
+    return r + slot * grid + block;
+}
+
 // All replicas of a batch in one persistent launch (a single context is a
 // batch of one): the warps walk the concatenated segment lists; each
 // segment's replica (warp-uniform) selects its record in the kernel parameter
@@ -939,7 +956,7 @@ __global__ void __launch_bounds__(kWarpBlock, 2) k_step_warp_batch(
     const int total = s_off[p.R];
     const int warps_total = gridDim.x * (kWarpBlock / 32);
     const long long step0 = p.step_dev ? *p.step_dev : p.step0;
-    for (int w = blockIdx.x * (kWarpBlock / 32) + uniform_warp(); w < total; w += warps_total) {
+    for (int r = 0, w; (w = segment_of(r, total, uniform_warp())) < total; r += warps_total) {
         int lo = 0;  // replica r with s_off[r] <= w < s_off[r + 1]
         if (kCap > 1) {
             int hi = p.R - 1;
@@ -983,7 +1000,7 @@ __global__ void __launch_bounds__(kWarpBlock, 2) k_step_warp_obs(
     FF acc[kBeadVals];
 #pragma unroll
     for (int k = 0; k < kBeadVals; ++k) acc[k] = FF{0.f, 0.f};
-    for (int w = blockIdx.x * (kWarpBlock / 32) + uniform_warp(); w < total; w += warps_total)
+    for (int r = 0, w; (w = segment_of(r, total, uniform_warp())) < total; r += warps_total)
         advance_pairs<kTherm, 1>(rp.st[p.cur], rp.st[p.cur ^ 1], rp.meta, rp.seg_start[w],
                                     rp.seg_count[w], p.n_sub, step0, rp.g, rp.G, rp.c,
                                     p.fuse ? rp.D[p.dnext] : nullptr, p.flag, &o, acc);
@@ -1021,7 +1038,7 @@ __global__ void __launch_bounds__(kWarpBlock, 2) k_step_warp_lerp(
     const BatchStepRep& rp = p.rep[0];
     const int total = *rp.n_seg;
     const int warps_total = gridDim.x * (kWarpBlock / 32);
-    for (int w = blockIdx.x * (kWarpBlock / 32) + (tid >> 5); w < total; w += warps_total)
+    for (int r = 0, w; (w = segment_of(r, total, tid >> 5)) < total; r += warps_total)
         advance_segment<kTherm, 0, kBonded, 1>(rp.st[p.cur], rp.st[p.cur ^ 1], rp.meta,
                                                rp.seg_start[w], rp.seg_count[w], p.n_sub,
                                                p.step0, rp.g, rp.G, rp.c,
@@ -1126,8 +1143,7 @@ void launch_step_warp_batch(const BatchStepParams& p, int max_seg_total, int the
                             cudaStream_t s) {
     if (max_seg_total <= 0 || p.n_sub <= 0) return;
     const int cap = warp_grid_cap();
-    const int need = (max_seg_total + kWarpBlock / 32 - 1) / (kWarpBlock / 32);
-    const int blocks = need < cap ? need : cap;
+    const int blocks = max_seg_total < cap ? max_seg_total : cap;
     launch_warp(p, blocks, therm, p.rep[0].c.force_mode, s);  // replicas share the force mode
 }
 
@@ -1135,8 +1151,7 @@ void launch_step_warp_lerp(const SingleStepParams& p, const float4* G2, int j0, 
                            int max_seg, int therm, cudaStream_t s) {
     if (max_seg <= 0 || p.n_sub <= 0) return;
     const int cap = warp_grid_cap();
-    const int need = (max_seg + kWarpBlock / 32 - 1) / (kWarpBlock / 32);
-    const int blocks = need < cap ? need : cap;
+    const int blocks = max_seg < cap ? max_seg : cap;
     const int bonded = bonded_level(p.rep[0].c);
     if (therm == 1) {
         if (bonded == 2) launch_lerp_k<1, 2>(p, G2, j0, inv_k, blocks, s);
@@ -1159,8 +1174,7 @@ int launch_step_warp_obs(const SingleStepParams& p, int max_seg, int therm, floa
                          float half_dt_m, const BondFF& bond, cudaStream_t s) {
     if (max_seg <= 0 || p.n_sub <= 0) return 0;
     const int cap = warp_grid_cap();
-    const int need = (max_seg + kWarpBlock / 32 - 1) / (kWarpBlock / 32);
-    const int blocks = need < cap ? need : cap;
+    const int blocks = max_seg < cap ? max_seg : cap;
     const ObsArgs o{part, half_dt_m, bond};
     if (therm == 1) launch_pdl(k_step_warp_obs<1>, blocks, kWarpBlock, 0, s, p, o);
     else launch_pdl(k_step_warp_obs<0>, blocks, kWarpBlock, 0, s, p, o);
@@ -1171,8 +1185,7 @@ void launch_step_warp_single(const SingleStepParams& p, int max_seg, int therm,
                              cudaStream_t s) {
     if (max_seg <= 0 || p.n_sub <= 0) return;
     const int cap = warp_grid_cap();
-    const int need = (max_seg + kWarpBlock / 32 - 1) / (kWarpBlock / 32);
-    const int blocks = need < cap ? need : cap;
+    const int blocks = max_seg < cap ? max_seg : cap;
     launch_warp(p, blocks, therm, p.rep[0].c.force_mode, s);
 }
 

@@ -67,3 +67,20 @@ def test_chunk_sizes_give_the_bits_of_a_period(hpf_gpu, free):
             out.append(s.get_state() + (s.scatter_density(),))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("chains", [3 * 304 - 1, 3 * 2432, 3 * 2432 + 1, 3 * 2700, 3 * 3300])
+def test_rounds_of_segments_give_the_bits_of_single_steps(hpf_gpu, chains):
+    """Three chains of 20 fill a segment: counts of segments below, at and
+    beyond one round of the warps, with short and long last rounds."""
+    w = W.diblock(chains, 9, 11, (chains * 20 / 3.0) ** (1.0 / 3.0), 30, 1.0, field_every=4)
+    d = W.generate(w)
+    out = []
+    for calls in ((4, 4), (1,) * 8):
+        with hpf_gpu.System(hpf_gpu.make_params(**w.params())) as s:
+            s.set_state(d["pos"], d["vel"], d["type"], d["bonds"])
+            for n in calls:
+                s.step(n)
+            out.append(s.get_state() + (s.scatter_density(),))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
