@@ -412,7 +412,9 @@ __device__ __forceinline__ void scatter_bead(unsigned long long* __restrict__ Dt
 // the other, the even lane the four corners at the lower x, the odd lane the
 // four at the upper one, so that an instruction's two words of a bead mostly lie in one
 // 32-byte sector.  The L2 takes these reductions sector by sector: 8M
-// of them cost 41 us one to a sector and 25 us two to a sector.
+// of them cost 41 us one to a sector and 25 us two to a sector.  A 10-step
+// launch of 1M beads with its deposit took 118 us before and 109 after, a 5-step
+// launch of 8.1M 620 and 548, the one-step kernel's 47 and 39.
 __device__ __forceinline__ void scatter_paired(unsigned long long* __restrict__ D, const MeshGeom& g,
                                                float x, float y, float z, uint32_t m, bool on) {
     const AxisCoord ax = axis_coord(x, g.inv_h[0], g.mx, g.inv_m[0]);

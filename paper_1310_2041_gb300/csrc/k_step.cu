@@ -523,7 +523,8 @@ __device__ __forceinline__ void kick_bead(Bead& b, float f0, float f1, float f2,
 // multiply-add on float pairs), and the two cell polynomials live in 48
 // registers, paired coefficient by coefficient, instead of shared memory: no
 // loads per evaluation, and the L1 keeps the space.  91.4M -> 75.0M
-// instructions and 124 -> 118 us per 10-step launch of 1M beads (L1 data pipe
+// instructions and 124 -> 118 us per 10-step launch of 1M beads, 107 with today's
+// deposit and uniform segment bounds (L1 data pipe
 // 56 -> 34 %).  What bounds it now is latency at 16 warps per SM: the refills
 // (a warp meets about one per sub-step; 1.7 of 6.8 stall cycles per
 // instruction) and dependent arithmetic.  Starting a refill's loads a
