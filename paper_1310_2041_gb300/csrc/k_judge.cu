@@ -4,7 +4,7 @@
 // One pass over the beads gathers both fields at once (sixteen corner loads in
 // flight per bead) and sums |Fa - Fb|^2 and |Fb|^2: two force passes through
 // memory, an FP64 error pass and a one-warp sum over 1216 partials took
-// 18.6 + 18.6 + 37 + 74 us at 1M beads, this pass 35.  A bead's terms are formed in
+// 18.6 + 18.6 + 37 + 74 us at 1M beads, this pass 37.  A bead's terms are formed in
 // float-float (the difference exactly, squares with their errors, about
 // 2^-45 relative) and added to the thread's FP64 sums, one addition per sum
 // and bead instead of eight FP64 operations per component (this GPU's FP64
