@@ -70,4 +70,13 @@ __device__ __forceinline__ float cell_poly(const float4 lo, const float4 hi, flo
     return fmaf(fz, lo.w, v);
 }
 
+// Friction and field force of one component, -fric v - poly in one rounding.
+// Written out, here and in the packed form (pair_force): left to the compiler
+// the product is fused in one kernel and not in another, and a run's bits then
+// depend on which kernel its steps go through (seen at gamma m = 0.7, whose
+// products round; at 1 they are exact).
+__device__ __forceinline__ float drag_field(float fric, float v, float poly) {
+    return fmaf(-fric, v, -poly);
+}
+
 }  // namespace hpf

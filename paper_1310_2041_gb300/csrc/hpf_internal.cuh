@@ -751,20 +751,26 @@ __host__ __device__ __forceinline__ BondFF bond_ff(const EnergyConsts& e) {
 // typical bond force).  kOrder fixes the rounding of |d|^2 where two kernels
 // have to form the same bits: kLaneBond the bond between the two beads of a
 // lane of the warp form, kCrossBond the one to the next lane's first bead (the
-// two orders are the ones every release of the warp kernel has had); 0 leaves
-// it to the compiler.
-constexpr int kLaneBond = 1, kCrossBond = 2;
+// two orders are the ones every release of the warp kernel has had), kChainBond
+// a bond of the halo form, whose share goes into the sum so far by one fma; 0
+// leaves it to the compiler.
+constexpr int kLaneBond = 1, kCrossBond = 2, kChainBond = 3;
 template <int kOrder = 0>
 __device__ __forceinline__ void bond_force(float dx, float dy, float dz, float two_k, float r0,
                                            float& fx, float& fy, float& fz) {
     float rr = dx * dx + dy * dy + dz * dz;
     if (kOrder == kLaneBond) rr = fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
-    if (kOrder == kCrossBond) rr = fmaf(dz, dz, fmaf(dx, dx, __fmul_rn(dy, dy)));
+    if (kOrder == kCrossBond || kOrder == kChainBond)
+        rr = fmaf(dz, dz, fmaf(dx, dx, __fmul_rn(dy, dy)));
     // r^2 is clamped so that a masked bond (two_k = 0, zero vector) adds exactly zero
     const float r2 = fmaxf(rr, 1e-30f);
     const float ir = rsqrtf(r2);
     const float s = -two_k * fmaf(-r0, ir, 1.0f);
-    if (kOrder != 0) {  // a share on its own: rounded before it is summed
+    if (kOrder == kChainBond) {
+        fx = fmaf(s, dx, fx);
+        fy = fmaf(s, dy, fy);
+        fz = fmaf(s, dz, fz);
+    } else if (kOrder != 0) {  // a share on its own: rounded before it is summed
         fx = __fmul_rn(s, dx);
         fy = __fmul_rn(s, dy);
         fz = __fmul_rn(s, dz);

@@ -112,14 +112,13 @@ __global__ void __launch_bounds__(kC, kOnePerSM * 256 / kC)
                 if (coll) gauss3(c, tag, p.step, gx, gy, gz);
             }
             const float f0 = __fsub_rn(s0, flx), f1 = __fsub_rn(s1, fly), f2 = __fsub_rn(s2, flz);
-            float fx = -c.fric * vx, fy = -c.fric * vy, fz = -c.fric * vz;
             float4 lo, hi;
             cell_coefs(HPF_CORNERS(k, x), lo, hi);
-            fx -= cell_poly(lo, hi, f0, f1, f2);
+            float fx = drag_field(c.fric, vx, cell_poly(lo, hi, f0, f1, f2));
             cell_coefs(HPF_CORNERS(k, y), lo, hi);
-            fy -= cell_poly(lo, hi, f0, f1, f2);
+            float fy = drag_field(c.fric, vy, cell_poly(lo, hi, f0, f1, f2));
             cell_coefs(HPF_CORNERS(k, z), lo, hi);
-            fz -= cell_poly(lo, hi, f0, f1, f2);
+            float fz = drag_field(c.fric, vz, cell_poly(lo, hi, f0, f1, f2));
             if (kTherm == 1) {
                 fx = fmaf(c.sigma, gx, fx);
                 fy = fmaf(c.sigma, gy, fy);
@@ -131,17 +130,17 @@ __global__ void __launch_bounds__(kC, kOnePerSM * 256 / kC)
                 fz += nz;
             } else {
                 if (m & kBondPrev)
-                    bond_force(x - s[0][e - 1], y - s[1][e - 1], z - s[2][e - 1], c.two_k, c.r0, fx,
-                               fy, fz);
+                    bond_force<kChainBond>(x - s[0][e - 1], y - s[1][e - 1], z - s[2][e - 1], c.two_k,
+                                           c.r0, fx, fy, fz);
                 if (m & kBondNext)
-                    bond_force(x - s[0][e + 1], y - s[1][e + 1], z - s[2][e + 1], c.two_k, c.r0, fx,
-                               fy, fz);
+                    bond_force<kChainBond>(x - s[0][e + 1], y - s[1][e + 1], z - s[2][e + 1], c.two_k,
+                                           c.r0, fx, fy, fz);
             }
             if (kTherm == 2 && coll) {
                 const float h = 0.5f * c.dt_m;
-                vx = fmaf(h, fx, c.sig_v * gx);
-                vy = fmaf(h, fy, c.sig_v * gy);
-                vz = fmaf(h, fz, c.sig_v * gz);
+                vx = fmaf(h, fx, __fmul_rn(c.sig_v, gx));
+                vy = fmaf(h, fy, __fmul_rn(c.sig_v, gy));
+                vz = fmaf(h, fz, __fmul_rn(c.sig_v, gz));
             } else {
                 vx = fmaf(c.dt_m, fx, vx);
                 vy = fmaf(c.dt_m, fy, vy);

@@ -123,11 +123,18 @@ __device__ __forceinline__ float cache_key(float s) {
     return kForce == 2 ? stag_vertex(s) : floorf(s);
 }
 
+// Friction and field force of a bead with velocity (vx, vy, vz) from its cached
+// cell, at the offset (fx, fy, fz).
 template <int kForce>
 __device__ __forceinline__ void eval_cell_cache(const float4* __restrict__ cache, int t, float fx,
-                                                float fy, float fz, float& Fx, float& Fy,
-                                                float& Fz, const MeshGeom& g,
-                                                int stride) {
+                                                float fy, float fz, float fric, float vx, float vy,
+                                                float vz, float& Fx, float& Fy, float& Fz,
+                                                const MeshGeom& g, int stride) {
+    if (kForce != 0) {
+        Fx = __fmul_rn(-fric, vx);
+        Fy = __fmul_rn(-fric, vy);
+        Fz = __fmul_rn(-fric, vz);
+    }
     if (kForce == 2) {
         const float4 lo = cache[t], hi = cache[stride + t];
         const float c[6] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y};
@@ -143,9 +150,9 @@ __device__ __forceinline__ void eval_cell_cache(const float4* __restrict__ cache
         Fy = fmaf(-g.inv_h[1], dy, Fy);
         Fz = fmaf(-g.inv_h[2], dz, Fz);
     } else {
-        Fx -= cell_poly(cache[0 * stride + t], cache[1 * stride + t], fx, fy, fz);
-        Fy -= cell_poly(cache[2 * stride + t], cache[3 * stride + t], fx, fy, fz);
-        Fz -= cell_poly(cache[4 * stride + t], cache[5 * stride + t], fx, fy, fz);
+        Fx = drag_field(fric, vx, cell_poly(cache[0 * stride + t], cache[1 * stride + t], fx, fy, fz));
+        Fy = drag_field(fric, vy, cell_poly(cache[2 * stride + t], cache[3 * stride + t], fx, fy, fz));
+        Fz = drag_field(fric, vz, cell_poly(cache[4 * stride + t], cache[5 * stride + t], fx, fy, fz));
     }
 }
 
@@ -240,9 +247,9 @@ __global__ void __launch_bounds__(kB, 1024 / kB) k_step(StateBuf in, StateBuf ou
             cfy = fly;
             cfz = flz;
         }
-        float fx = -c.fric * vx, fy = -c.fric * vy, fz = -c.fric * vz;
+        float fx, fy, fz;
         eval_cell_cache<kForce>(cache, t, __fsub_rn(s0, flx), __fsub_rn(s1, fly),
-                                __fsub_rn(s2, flz), fx, fy, fz, g, kB);
+                                __fsub_rn(s2, flz), c.fric, vx, vy, vz, fx, fy, fz, g, kB);
         if (kTherm == 1) {
             float nx, ny, nz;
             gauss3(c, tag, step0 + k, nx, ny, nz);
@@ -251,10 +258,10 @@ __global__ void __launch_bounds__(kB, 1024 / kB) k_step(StateBuf in, StateBuf ou
             fz = fmaf(c.sigma, nz, fz);
         }
         const int tp = has_prev ? t - 1 : t, tn = has_next ? t + 1 : t;
-        bond_force(x - sx[b * kB + tp], y - sy[b * kB + tp],
-                   z - sz[b * kB + tp], has_prev ? c.two_k : 0.0f, c.r0, fx, fy, fz);
-        bond_force(x - sx[b * kB + tn], y - sy[b * kB + tn],
-                   z - sz[b * kB + tn], has_next ? c.two_k : 0.0f, c.r0, fx, fy, fz);
+        bond_force<kChainBond>(x - sx[b * kB + tp], y - sy[b * kB + tp], z - sz[b * kB + tp],
+                               has_prev ? c.two_k : 0.0f, c.r0, fx, fy, fz);
+        bond_force<kChainBond>(x - sx[b * kB + tn], y - sy[b * kB + tn], z - sz[b * kB + tn],
+                               has_next ? c.two_k : 0.0f, c.r0, fx, fy, fz);
         if (kBonded >= 1) {
             // the three angles this bead belongs to: centred at t - 1, t and t + 1
             const int tp2 = (has_prev && t >= 2) ? t - 2 : t;
@@ -299,9 +306,9 @@ __global__ void __launch_bounds__(kB, 1024 / kB) k_step(StateBuf in, StateBuf ou
             float nx, ny, nz;
             gauss3(c, tag, step0 + k, nx, ny, nz);
             const float h = 0.5f * c.dt_m;
-            vx = fmaf(h, fx, c.sig_v * nx);
-            vy = fmaf(h, fy, c.sig_v * ny);
-            vz = fmaf(h, fz, c.sig_v * nz);
+            vx = fmaf(h, fx, __fmul_rn(c.sig_v, nx));
+            vy = fmaf(h, fy, __fmul_rn(c.sig_v, ny));
+            vz = fmaf(h, fz, __fmul_rn(c.sig_v, nz));
         } else {
             vx = fmaf(c.dt_m, fx, vx);
             vy = fmaf(c.dt_m, fy, vy);
@@ -461,9 +468,6 @@ __device__ __forceinline__ void bead_force(const Bead& b, float f0, float f1, fl
                                            const StepConsts& c, const MeshGeom& g,
                                            const float4* __restrict__ cache, int slot, float a,
                                            float& fx, float& fy, float& fz) {
-    fx = -c.fric * b.vx;
-    fy = -c.fric * b.vy;
-    fz = -c.fric * b.vz;
     if (kLerp) {
         // the field (1 - a) G0 + a G2: P0 + a (P2 - P0) of the two cached polynomials
         constexpr int st = 2 * kWarpBlock;
@@ -474,11 +478,12 @@ __device__ __forceinline__ void bead_force(const Bead& b, float f0, float f1, fl
         const float p2x = cell_poly(c2[0 * st + slot], c2[1 * st + slot], f0, f1, f2);
         const float p2y = cell_poly(c2[2 * st + slot], c2[3 * st + slot], f0, f1, f2);
         const float p2z = cell_poly(c2[4 * st + slot], c2[5 * st + slot], f0, f1, f2);
-        fx -= fmaf(a, p2x - p0x, p0x);
-        fy -= fmaf(a, p2y - p0y, p0y);
-        fz -= fmaf(a, p2z - p0z, p0z);
+        fx = drag_field(c.fric, b.vx, fmaf(a, p2x - p0x, p0x));
+        fy = drag_field(c.fric, b.vy, fmaf(a, p2y - p0y, p0y));
+        fz = drag_field(c.fric, b.vz, fmaf(a, p2z - p0z, p0z));
     } else {
-        eval_cell_cache<kForce>(cache, slot, f0, f1, f2, fx, fy, fz, g, 2 * kWarpBlock);
+        eval_cell_cache<kForce>(cache, slot, f0, f1, f2, c.fric, b.vx, b.vy, b.vz, fx, fy, fz, g,
+                                2 * kWarpBlock);
     }
     if (kTherm == 1) {
         fx = fmaf(c.sigma, nx, fx);
@@ -503,9 +508,9 @@ __device__ __forceinline__ void kick_bead(Bead& b, float f0, float f1, float f2,
                                       fx, fy, fz);
     if (kTherm == 2 && coll) {
         const float h = 0.5f * c.dt_m;
-        b.vx = fmaf(h, fx, c.sig_v * nx);
-        b.vy = fmaf(h, fy, c.sig_v * ny);
-        b.vz = fmaf(h, fz, c.sig_v * nz);
+        b.vx = fmaf(h, fx, __fmul_rn(c.sig_v, nx));
+        b.vy = fmaf(h, fy, __fmul_rn(c.sig_v, ny));
+        b.vz = fmaf(h, fz, __fmul_rn(c.sig_v, nz));
     } else {
         b.vx = fmaf(c.dt_m, fx, b.vx);
         b.vy = fmaf(c.dt_m, fy, b.vy);
@@ -543,17 +548,15 @@ __device__ __forceinline__ float2 pair_sub(float2 a, float2 b) {  // a - b
     return __ffma2_rn(b, both(-1.0f), a);
 }
 
-// -(cell polynomials) added to f: cell_poly of both beads.
-__device__ __forceinline__ float2 pair_poly(float2 f, const float2 (&c)[8], float2 fx, float2 fy,
-                                            float2 fz) {
+// cell_poly of both beads.
+__device__ __forceinline__ float2 pair_poly(const float2 (&c)[8], float2 fx, float2 fy, float2 fz) {
     float2 a = __ffma2_rn(fz, c[7], c[4]);
     a = __ffma2_rn(fy, a, c[1]);
     a = __ffma2_rn(fz, c[5], a);
     const float2 b = __ffma2_rn(fz, c[6], c[2]);
     float2 v = __ffma2_rn(fx, a, c[0]);
     v = __ffma2_rn(fy, b, v);
-    v = __ffma2_rn(fz, c[3], v);
-    return pair_sub(f, v);
+    return __ffma2_rn(fz, c[3], v);
 }
 
 template <int kBead>
@@ -591,27 +594,27 @@ __device__ __forceinline__ float2 pair_uniform(uint32_t r0, uint32_t r1) {
                       both(-0.999999940395355224609375f));
 }
 
-// The Box-Muller radius sqrt(-2 ln u) of both, negated (log_unit's two forms).
-__device__ __forceinline__ float2 pair_radius_neg(float2 u) {
+// The Box-Muller radius sqrt(-2 ln u) of both (log_unit's two forms).
+__device__ __forceinline__ float2 pair_radius(float2 u) {
     const float2 d = __ffma2_rn(u, both(-1.0f), both(1.0f));
     const float2 t = __ffma2_rn(__ffma2_rn(d, both(1.0f / 3.0f), both(0.5f)), d, both(1.0f));
     const float2 series = __fmul2_rn(d, t);
     const float2 l = __fmul2_rn(make_float2(d.x <= 0.015625f ? series.x : -__logf(u.x),
                                             d.y <= 0.015625f ? series.y : -__logf(u.y)),
                                 both(2.0f));
-    return __fmul2_rn(l, make_float2(-rsqrtf(l.x), -rsqrtf(l.y)));
+    return __fmul2_rn(l, make_float2(rsqrtf(l.x), rsqrtf(l.y)));
 }
 
-// gauss3 of both beads.
-__device__ __forceinline__ void pair_gauss3(const StepConsts& c, uint32_t tag0, uint32_t tag1,
+// Minus gauss3 of both beads.
+__device__ __forceinline__ void pair_gauss3_neg(const StepConsts& c, uint32_t tag0, uint32_t tag1,
                                             long long step, float2& gx, float2& gy, float2& gz) {
     uint32_t a0 = tag0 + c.tag_base, a1 = (uint32_t)step,
              a2 = (uint32_t)((unsigned long long)step >> 32), a3 = 0u;
     uint32_t b0 = tag1 + c.tag_base, b1 = a1, b2 = a2, b3 = 0u;
     philox4x32_10(a0, a1, a2, a3, c.rk0, c.rk1);
     philox4x32_10(b0, b1, b2, b3, c.rk0, c.rk1);
-    const float2 a = pair_radius_neg(pair_uniform(a0, b0));
-    const float2 b = pair_radius_neg(pair_uniform(a2, b2));
+    const float2 a = pair_radius(pair_uniform(a0, b0));
+    const float2 b = pair_radius(pair_uniform(a2, b2));
     const float2 t1 = __fmul2_rn(__fadd2_rn(pair_uniform(a1, b1), both(-0.5f)),
                                  both(6.28318530717958648f));
     const float2 t3 = __fmul2_rn(__fadd2_rn(pair_uniform(a3, b3), both(-0.5f)),
@@ -624,11 +627,11 @@ __device__ __forceinline__ void pair_gauss3(const StepConsts& c, uint32_t tag0, 
     gz = __fmul2_rn(b, make_float2(__cosf(t3.x), __cosf(t3.y)));
 }
 
-// The bond forces of a segment (warp_bonded_forces<0>), the lane's two bonds as
+// Minus the bond forces of a segment (warp_bonded_forces<0>), the lane's two bonds as
 // a pair: the in-lane one (2l, 2l + 1) and the one to the next lane.  The pairs
 // (dx, dy'), (dy, dx'), (dz, dz') give each its own order of |d|^2 (kLaneBond,
 // kCrossBond).
-__device__ __forceinline__ void pair_bonds(const Pair& b, bool p0, float2 minus_k,
+__device__ __forceinline__ void pair_bonds(const Pair& b, bool p0, float2 two_k,
                                            const StepConsts& c, float2& wx, float2& wy,
                                            float2& wz) {
     const float dx = __shfl_down_sync(0xffffffffu, b.x.x, 1);
@@ -639,7 +642,7 @@ __device__ __forceinline__ void pair_bonds(const Pair& b, bool p0, float2 minus_
     const float2 C = make_float2(__fsub_rn(b.z.x, b.z.y), __fsub_rn(b.z.y, dz));
     const float2 rr = __ffma2_rn(C, C, __ffma2_rn(B, B, __fmul2_rn(A, A)));
     const float2 ir = make_float2(rsqrtf(fmaxf(rr.x, 1e-30f)), rsqrtf(fmaxf(rr.y, 1e-30f)));
-    const float2 s = __fmul2_rn(minus_k, __ffma2_rn(both(-c.r0), ir, both(1.0f)));
+    const float2 s = __fmul2_rn(two_k, __ffma2_rn(both(-c.r0), ir, both(1.0f)));
     const float2 fa = __fmul2_rn(s, A), fb = __fmul2_rn(s, B), fc = __fmul2_rn(s, C);
     const float ux = __shfl_up_sync(0xffffffffu, fb.y, 1);  // the previous lane's share
     const float uy = __shfl_up_sync(0xffffffffu, fa.y, 1);
@@ -649,21 +652,22 @@ __device__ __forceinline__ void pair_bonds(const Pair& b, bool p0, float2 minus_
     wz = make_float2(p0 ? __fsub_rn(fc.x, uz) : fc.x, __fsub_rn(fc.y, fc.x));
 }
 
-// The forces on a lane's two beads at their positions: field, friction, bonds
-// and step `step`'s noise.  coll0, coll1 (Andersen): the bead collides
-// and (gx, gy, gz) holds its normals.
+// Minus the forces on a lane's two beads at their positions: field, friction,
+// bonds and step `step`'s noise.  Opposite sums round alike, and with this sign
+// friction and field are one fma, as in drag_field, without a negation.  The
+// bonds come last: their shuffles then wait behind the refills (1M beads, 20 steps
+// 255.0 -> 254.1 us).  (gx, gy, gz): minus the normals (Langevin), or with
+// coll0, coll1 (Andersen: the bead collides) its normals.
 struct PairForce {
-    float2 fx, fy, fz, gx, gy, gz;
+    float2 nx, ny, nz, gx, gy, gz;
     bool coll0, coll1;
 };
 
 template <int kTherm>
-__device__ __forceinline__ PairForce pair_force(Pair& b, bool p0, float2 minus_k, long long step,
+__device__ __forceinline__ PairForce pair_force(Pair& b, bool p0, float2 two_k, long long step,
                                                 const MeshGeom& g, const float4* __restrict__ G,
                                                 const StepConsts& c) {
     PairForce r;
-    float2 wx, wy, wz;
-    pair_bonds(b, p0, minus_k, c, wx, wy, wz);
     const float2 s0 = __fmul2_rn(b.x, both(g.inv_h[0])), s1 = __fmul2_rn(b.y, both(g.inv_h[1])),
                  s2 = __fmul2_rn(b.z, both(g.inv_h[2]));
     const float2 l0 = pair_floor(s0), l1 = pair_floor(s1), l2 = pair_floor(s2);
@@ -678,45 +682,48 @@ __device__ __forceinline__ PairForce pair_force(Pair& b, bool p0, float2 minus_k
     r.gx = r.gy = r.gz = both(0.f);
     r.coll0 = r.coll1 = false;
     const uint32_t t0 = b.m0 & kTagMask, t1 = b.m1 & kTagMask;
-    if (kTherm == 1) pair_gauss3(c, t0, t1, step, r.gx, r.gy, r.gz);
+    if (kTherm == 1) pair_gauss3_neg(c, t0, t1, step, r.gx, r.gy, r.gz);
     if (kTherm == 2) {
         r.coll0 = andersen_collides(c, t0, step);
         r.coll1 = andersen_collides(c, t1, step);
         if (r.coll0) gauss3(c, t0, step, r.gx.x, r.gy.x, r.gz.x);
         if (r.coll1) gauss3(c, t1, step, r.gx.y, r.gy.y, r.gz.y);
     }
-    const float2 fric = both(-c.fric);
-    r.fx = pair_poly(__fmul2_rn(fric, b.vx), b.kx, f0, f1, f2);
-    r.fy = pair_poly(__fmul2_rn(fric, b.vy), b.ky, f0, f1, f2);
-    r.fz = pair_poly(__fmul2_rn(fric, b.vz), b.kz, f0, f1, f2);
+    const float2 fric = both(c.fric);
+    r.nx = __ffma2_rn(fric, b.vx, pair_poly(b.kx, f0, f1, f2));
+    r.ny = __ffma2_rn(fric, b.vy, pair_poly(b.ky, f0, f1, f2));
+    r.nz = __ffma2_rn(fric, b.vz, pair_poly(b.kz, f0, f1, f2));
     if (kTherm == 1) {
-        r.fx = __ffma2_rn(both(c.sigma), r.gx, r.fx);
-        r.fy = __ffma2_rn(both(c.sigma), r.gy, r.fy);
-        r.fz = __ffma2_rn(both(c.sigma), r.gz, r.fz);
+        const float2 sigma = both(c.sigma);
+        r.nx = __ffma2_rn(sigma, r.gx, r.nx);
+        r.ny = __ffma2_rn(sigma, r.gy, r.ny);
+        r.nz = __ffma2_rn(sigma, r.gz, r.nz);
     }
-    r.fx = __fadd2_rn(r.fx, wx);
-    r.fy = __fadd2_rn(r.fy, wy);
-    r.fz = __fadd2_rn(r.fz, wz);
+    float2 wx, wy, wz;
+    pair_bonds(b, p0, two_k, c, wx, wy, wz);
+    r.nx = __fadd2_rn(r.nx, wx);
+    r.ny = __fadd2_rn(r.ny, wy);
+    r.nz = __fadd2_rn(r.nz, wz);
     return r;
 }
 
 // Kick by those forces (a colliding bead: redrawn velocity, second half kick) and drift.
 template <int kTherm>
 __device__ __forceinline__ void pair_move(Pair& b, const PairForce& r, const StepConsts& c) {
-    b.vx = __ffma2_rn(both(c.dt_m), r.fx, b.vx);
-    b.vy = __ffma2_rn(both(c.dt_m), r.fy, b.vy);
-    b.vz = __ffma2_rn(both(c.dt_m), r.fz, b.vz);
+    b.vx = __ffma2_rn(both(-c.dt_m), r.nx, b.vx);
+    b.vy = __ffma2_rn(both(-c.dt_m), r.ny, b.vy);
+    b.vz = __ffma2_rn(both(-c.dt_m), r.nz, b.vz);
     if (kTherm == 2) {
-        const float h = 0.5f * c.dt_m;
+        const float h = -0.5f * c.dt_m;
         if (r.coll0) {
-            b.vx.x = fmaf(h, r.fx.x, __fmul_rn(c.sig_v, r.gx.x));
-            b.vy.x = fmaf(h, r.fy.x, __fmul_rn(c.sig_v, r.gy.x));
-            b.vz.x = fmaf(h, r.fz.x, __fmul_rn(c.sig_v, r.gz.x));
+            b.vx.x = fmaf(h, r.nx.x, __fmul_rn(c.sig_v, r.gx.x));
+            b.vy.x = fmaf(h, r.ny.x, __fmul_rn(c.sig_v, r.gy.x));
+            b.vz.x = fmaf(h, r.nz.x, __fmul_rn(c.sig_v, r.gz.x));
         }
         if (r.coll1) {
-            b.vx.y = fmaf(h, r.fx.y, __fmul_rn(c.sig_v, r.gx.y));
-            b.vy.y = fmaf(h, r.fy.y, __fmul_rn(c.sig_v, r.gy.y));
-            b.vz.y = fmaf(h, r.fz.y, __fmul_rn(c.sig_v, r.gz.y));
+            b.vx.y = fmaf(h, r.nx.y, __fmul_rn(c.sig_v, r.gx.y));
+            b.vy.y = fmaf(h, r.ny.y, __fmul_rn(c.sig_v, r.gy.y));
+            b.vz.y = fmaf(h, r.nz.y, __fmul_rn(c.sig_v, r.gz.y));
         }
     }
     b.x = __ffma2_rn(both(c.dt), b.vx, b.x);
@@ -755,10 +762,10 @@ struct ObsArgs {
 
 template <int kTherm>
 __device__ __forceinline__ void observe_segment(Pair& b, bool a0, bool a1, bool p0, bool n0, bool n1,
-                                                float2 minus_k, long long step, const MeshGeom& g,
+                                                float2 two_k, long long step, const MeshGeom& g,
                                                 const float4* __restrict__ G, const StepConsts& c,
                                                 const ObsArgs& o, FF* acc) {
-    const PairForce r = pair_force<kTherm>(b, p0, minus_k, step, g, G, c);
+    const PairForce r = pair_force<kTherm>(b, p0, two_k, step, g, G, c);
     // the next lane's first bead (every lane takes part in the shuffles)
     const float qx = __shfl_down_sync(0xffffffffu, b.x.x, 1);
     const float qy = __shfl_down_sync(0xffffffffu, b.y.x, 1);
@@ -767,9 +774,9 @@ __device__ __forceinline__ void observe_segment(Pair& b, bool a0, bool a1, bool 
     if (n0) bond_energy_ff(b.x.x, b.y.x, b.z.x, b.x.y, b.y.y, b.z.y, o.bond, uh, ul);
     if (n1) bond_energy_ff(b.x.y, b.y.y, b.z.y, qx, qy, qz, o.bond, uh, ul);
     acc[1] = FF{uh, ul};
-    const float2 hf = both(o.half_dt_m);
-    const float2 ux = __ffma2_rn(hf, r.fx, b.vx), uy = __ffma2_rn(hf, r.fy, b.vy),
-                 uz = __ffma2_rn(hf, r.fz, b.vz);
+    const float2 hf = both(-o.half_dt_m);
+    const float2 ux = __ffma2_rn(hf, r.nx, b.vx), uy = __ffma2_rn(hf, r.ny, b.vy),
+                 uz = __ffma2_rn(hf, r.nz, b.vz);
     if (a0) {
         acc[0] = ff_plus(acc[0], fmaf(ux.x, ux.x, fmaf(uy.x, uy.x, __fmul_rn(uz.x, uz.x))));
         acc[2] = ff_plus(acc[2], ux.x);
@@ -814,11 +821,11 @@ __device__ __forceinline__ void advance_pairs(const StateBuf& in, const StateBuf
     // whole chains: every flagged neighbour is inside the segment
     const bool p0 = (b.m0 & kBondPrev) != 0, n0 = (b.m0 & kBondNext) != 0;
     const bool n1 = (b.m1 & kBondNext) != 0;  // b1's previous bond is b0's next
-    const float2 minus_k = make_float2(n0 ? -c.two_k : 0.f, n1 ? -c.two_k : 0.f);
+    const float2 two_k = make_float2(n0 ? c.two_k : 0.f, n1 ? c.two_k : 0.f);
     for (int k = 0; k < n_sub; ++k)
-        pair_move<kTherm>(b, pair_force<kTherm>(b, p0, minus_k, step0 + k, g, G, c), c);
+        pair_move<kTherm>(b, pair_force<kTherm>(b, p0, two_k, step0 + k, g, G, c), c);
     if constexpr (kObs != 0)
-        observe_segment<kTherm>(b, a0, a1, p0, n0, n1, minus_k, step0 + n_sub, g, G, c, *obs,
+        observe_segment<kTherm>(b, a0, a1, p0, n0, n1, two_k, step0 + n_sub, g, G, c, *obs,
                                 obs_acc);
     if (a0)
         finish_bead(Bead{b.x.x, b.y.x, b.z.x, b.vx.x, b.vy.x, b.vz.x, b.m0, 0.f, 0.f, 0.f}, i, out, g,

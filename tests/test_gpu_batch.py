@@ -126,3 +126,21 @@ def test_batch_energy_is_every_replicas_energy(hpf_gpu, orc):
         assert E[r][2] == pytest.approx(eo[2], rel=1e-12)
         assert E[r][0] == pytest.approx(eo[0], rel=1e-6)
     b.close()
+
+
+@pytest.mark.parametrize("fe", [1, 4])
+def test_batch_is_bitwise_the_independent_runs_with_rounding_friction(hpf_gpu, fe):
+    """gamma m and dt / m whose products round; with a refresh every step a
+    context's steps go through the one-step kernel, a replica's through the
+    field-period kernel."""
+    ws = [W.diblock(90, 8, 12, 8.7, 9, 0.3, field_every=fe, seed=11, gamma=0.7, mass=1.3),
+          W.diblock(150, 8, 12, 10.3, 10, 1.7, field_every=fe, seed=13, gamma=0.7, mass=1.3)]
+    b, data, _, stream = make_batch(hpf_gpu, ws)
+    b.step(24)
+    stream.synchronize()
+    for r, (w, d) in enumerate(zip(ws, data)):
+        pos, vel, _ = b.replica(r).get_state()
+        pi, vi, _ = independent(hpf_gpu, w, d, 24)
+        np.testing.assert_array_equal(pos, pi)
+        np.testing.assert_array_equal(vel, vi)
+    b.close()

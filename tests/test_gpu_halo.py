@@ -37,3 +37,24 @@ def test_launch_lengths_give_the_same_bits(hpf_gpu, chains, length, bonded):
             out.append(s.get_state() + (s.scatter_density(),))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("bonded", list(BONDED))
+@pytest.mark.parametrize("force_mode", [0, 1, 2])
+def test_launch_lengths_give_the_same_bits_with_rounding_friction(hpf_gpu, force_mode, bonded):
+    """gamma m and dt / m whose products round, every field force."""
+    chains, length = 11, 133
+    box = float((chains * length / 3.0) ** (1.0 / 3.0))
+    w = W.diblock(chains, length // 2, length - length // 2, box, round(box), 1.0, field_every=16,
+                  dt=0.004, gamma=0.7, mass=1.3)
+    d = W.with_bond_angles(w, W.generate(w))
+    out = []
+    for calls in ((16, 16), (2, 5, 6, 3) * 2, (1,) * 32):
+        with hpf_gpu.System(hpf_gpu.make_params(**{**w.params(), **BONDED[bonded],
+                                                   "force_mode": force_mode})) as s:
+            s.set_state(d["pos"], d["vel"], d["type"], d["bonds"])
+            for n in calls:
+                s.step(n)
+            out.append(s.get_state() + (s.scatter_density(),))
+    for a, b, c in zip(*out):
+        assert np.array_equal(a, b) and np.array_equal(a, c)

@@ -84,3 +84,21 @@ def test_rounds_of_segments_give_the_bits_of_single_steps(hpf_gpu, chains):
             out.append(s.get_state() + (s.scatter_density(),))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("name", ["256_solvent", "odd_chains", "andersen", "long", "long_andersen", "200k"])
+def test_friction_that_rounds_gives_the_bits_of_a_period(hpf_gpu, name):
+    """gamma m and dt / m whose products round (above all factors are 1): every
+    kernel fuses the friction with the field, so the bits still agree."""
+    w, extra = SYSTEMS[name]
+    d = W.generate(w)
+    pos = (d["pos"] + 0.05 * np.random.default_rng(1).normal(size=d["pos"].shape)).astype(np.float32)
+    out = []
+    for calls in ((4, 4), (1,) * 8):
+        with hpf_gpu.System(hpf_gpu.make_params(**{**w.params(), **extra, "gamma": 0.7, "mass": 1.3})) as s:
+            s.set_state(pos, d["vel"], d["type"], d["bonds"])
+            for n in calls:
+                s.step(n)
+            out.append(s.get_state() + (s.scatter_density(),))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
