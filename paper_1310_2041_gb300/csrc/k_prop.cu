@@ -1990,11 +1990,13 @@ hpf_status prop_read_loss(hpf_prop* p, double* loss) {
     return HPF_OK;
 }
 
-// A device (or managed) array of the current device.
+// A device (or managed) array of the current device that kernels can read and
+// write in place: an unaligned one goes through the staging buffers instead.
 bool prop_on_device(const void* ptr) {
     cudaPointerAttributes a;
     int dev = -1;
-    const bool ok = cudaPointerGetAttributes(&a, ptr) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
+    const bool ok = (reinterpret_cast<uintptr_t>(ptr) & 3u) == 0 &&
+                    cudaPointerGetAttributes(&a, ptr) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
                     (a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev));
     cudaGetLastError();
     return ok;

@@ -1,0 +1,64 @@
+"""Callers' arrays in device memory: used in place where kernels can use them,
+through staging buffers where they cannot, with the same bits either way."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_1310_2041_gb300 import learned
+
+pytestmark = pytest.mark.gpu
+
+MESH = (9, 18, 7)  # x, y, z
+GRID = MESH[::-1]
+
+
+def densities(seed, channels):
+    return np.random.default_rng(seed).uniform(0.2, 0.8, (channels,) + GRID).astype(np.float32)
+
+
+def at_byte(a, shift):
+    """A device copy of a that starts `shift` bytes into an allocation: (the allocation, its address)."""
+    import torch
+    raw = torch.zeros(a.nbytes + 64, dtype=torch.uint8, device="cuda")
+    raw[shift:shift + a.nbytes] = torch.from_numpy(np.ascontiguousarray(a).view(np.uint8).reshape(-1)).cuda()
+    torch.cuda.synchronize()
+    return raw, raw.data_ptr() + shift
+
+
+def network(hpf):
+    net = hpf.Propagator(MESH)
+    net.set_weights(learned.init_params(3))
+    net.scale = 4.0
+    return net
+
+
+@pytest.mark.parametrize("shift", [0, 4, 2, 1])
+def test_training_reads_device_arrays_at_any_address(hpf_gpu, shift):
+    x, nxt = densities(1, 4), densities(2, 2)
+    with network(hpf_gpu) as net:
+        loss, grads = net.backward(x, nxt)
+        net.train_step(x, nxt, 1e-3)
+        weights = net.get_weights()
+    (kx, px), (kn, pn) = at_byte(x, shift), at_byte(nxt, shift)
+    with network(hpf_gpu) as net:
+        g, got = np.empty_like(grads), ctypes.c_double()
+        assert net.lib.hpf_prop_backward(net.h, px, pn, g.ctypes.data, ctypes.byref(got)) == 0
+        assert net.lib.hpf_prop_train_step(net.h, px, pn, 1e-3, None) == 0
+        assert got.value == loss and np.array_equal(g, grads)
+        assert np.array_equal(net.get_weights(), weights)
+    del kx, kn
+
+
+@pytest.mark.parametrize("shift_in,shift_out", [(0, 0), (4, 8), (2, 0), (0, 2), (1, 3)])
+def test_predictions_at_any_address(hpf_gpu, shift_in, shift_out):
+    import torch
+    x = densities(1, 4)
+    with network(hpf_gpu) as net:
+        want = net.forward(x)
+        (keep, px), (out, po) = at_byte(x, shift_in), at_byte(np.zeros_like(want), shift_out)
+        assert net.lib.hpf_prop_forward(net.h, px, po) == 0
+        torch.cuda.synchronize()
+        got = out[shift_out:shift_out + want.nbytes].cpu().numpy().view(np.float32).reshape(want.shape)
+        assert np.array_equal(got, want)
+        del keep
