@@ -6,6 +6,7 @@
 #include <chrono>
 #include <cstdarg>
 #include <cstdio>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -200,6 +201,53 @@ hpf_status copy_out(hpf_ctx* c, void* dst, const void* src, size_t bytes) {
 }
 
 }  // namespace
+
+// The allocation that holds a device address: the driver's cuMemGetAddressRange.
+static bool address_range(uintptr_t p, uintptr_t* base, size_t* size) {
+    typedef CUresult (*Fn)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static Fn fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault,
+                                             &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<Fn>(f);
+        else
+            cudaGetLastError();
+    });
+    CUdeviceptr b = 0;
+    if (!fn || fn(&b, size, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    *base = (uintptr_t)b;
+    return true;
+}
+
+Placed hpf::placed(const void* ptr, size_t bytes, bool managed) {
+    if (bytes == 0) return Placed::kInPlace;
+    cudaPointerAttributes a;
+    int dev = -1;
+    if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return Placed::kCopied;
+    }
+    if (!(a.type == cudaMemoryTypeDevice || (managed && a.type == cudaMemoryTypeManaged)))
+        return Placed::kCopied;
+    // An array that runs on into a neighbouring allocation is the copy's to
+    // judge, as a tensor over several mapped pieces is one too.
+    const uintptr_t p0 = reinterpret_cast<uintptr_t>(ptr), end = p0 + bytes;
+    uintptr_t p = p0, base = 0;
+    size_t size = 0;
+    while (address_range(p, &base, &size) && base + size > p) {
+        if (base + size >= end)
+            return p == p0 && (p0 & 3u) == 0 &&
+                           (a.type == cudaMemoryTypeManaged || a.device == dev)
+                       ? Placed::kInPlace
+                       : Placed::kCopied;
+        p = base + size;
+    }
+    return p == p0 ? Placed::kCopied : Placed::kShort;
+}
 
 // The mesh and field parameters (shared with the allocation-free entry point).
 hpf_status hpf::validate_field_params(const hpf_params* p) {
@@ -1089,18 +1137,6 @@ hpf_status hpf_apply_state(hpf_ctx* c, int64_t step) {
     return HPF_OK;
 }
 
-// Whether kernels may write n floats at p in place of a copy: memory of the
-// current device, aligned.
-static bool device_floats(const void* p) {
-    cudaPointerAttributes a;
-    int dev = -1;
-    const bool ok = cudaPointerGetAttributes(&a, p) == cudaSuccess &&
-                    cudaGetDevice(&dev) == cudaSuccess && a.type == cudaMemoryTypeDevice &&
-                    a.device == dev && (reinterpret_cast<uintptr_t>(p) & 3u) == 0;
-    if (!ok) cudaGetLastError();
-    return ok;
-}
-
 hpf_status hpf_get_state(hpf_ctx* c, float* pos, float* vel, int64_t* step) {
     if (!c) return HPF_ERR_INVALID;
     if (!c->has_state) return fail(c, HPF_ERR_STATE, "no state loaded");
@@ -1108,7 +1144,12 @@ hpf_status hpf_get_state(hpf_ctx* c, float* pos, float* vel, int64_t* step) {
     // memory above all) take the staged arrays and a copy
     const size_t bytes = sizeof(float) * 3 * (size_t)c->n;
     const uintptr_t pa = reinterpret_cast<uintptr_t>(pos), va = reinterpret_cast<uintptr_t>(vel);
-    const bool direct = (!pos || device_floats(pos)) && (!vel || device_floats(vel)) &&
+    const Placed pp = pos ? placed(pos, bytes, false) : Placed::kInPlace;
+    const Placed vp = vel ? placed(vel, bytes, false) : Placed::kInPlace;
+    if (pp == Placed::kShort || vp == Placed::kShort)
+        return fail(c, HPF_ERR_CUDA, "%s ends before its %zu bytes",
+                    pp == Placed::kShort ? "pos" : "vel", bytes);
+    const bool direct = pp == Placed::kInPlace && vp == Placed::kInPlace &&
                         (!pos || !vel || pa + bytes <= va || va + bytes <= pa);
     float* pt = direct ? pos : (pos ? c->out_f : nullptr);
     float* vt = direct ? vel : (vel ? c->out_f + 3 * (size_t)c->n : nullptr);

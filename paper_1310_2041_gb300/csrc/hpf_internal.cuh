@@ -1068,6 +1068,13 @@ struct EnergyOut {
     double* h_nh;
 };
 
+// What a caller's array of `bytes` at p allows: kernels may use it in place
+// (aligned memory of the current device, inside one allocation; managed memory
+// too if asked for), it goes through a copy (all other memory), or it is
+// device memory that ends before `bytes`, which no kernel may touch.
+enum class Placed { kInPlace, kCopied, kShort };
+Placed placed(const void* p, size_t bytes, bool managed);
+
 // Mesh, box, species, rho0, kT, 1/kappa and chi of a parameter block:
 // HPF_OK or HPF_ERR_INVALID.
 hpf_status validate_field_params(const hpf_params* p);

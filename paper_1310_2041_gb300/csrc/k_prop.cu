@@ -1990,16 +1990,15 @@ hpf_status prop_read_loss(hpf_prop* p, double* loss) {
     return HPF_OK;
 }
 
-// A device (or managed) array of the current device that kernels can read and
-// write in place: an unaligned one goes through the staging buffers instead.
-bool prop_on_device(const void* ptr) {
-    cudaPointerAttributes a;
-    int dev = -1;
-    const bool ok = (reinterpret_cast<uintptr_t>(ptr) & 3u) == 0 &&
-                    cudaPointerGetAttributes(&a, ptr) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
-                    (a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev));
-    cudaGetLastError();
-    return ok;
+// Whether the kernels read n floats at src in place (*src stays) or from the
+// staging buffer dst, filled here.
+hpf_status prop_input(hpf_prop* p, float* dst, const float** src, size_t n) {
+    const Placed at = placed(*src, sizeof(float) * n, true);
+    if (at == Placed::kInPlace) return HPF_OK;
+    if (at == Placed::kShort) return HPF_ERR_CUDA;
+    const float* from = *src;
+    *src = dst;
+    return prop_stage(p, dst, from, n);
 }
 
 hpf_status prop_launched(hpf_prop* p) {
@@ -2231,13 +2230,16 @@ hpf_status hpf_prop_forward(hpf_prop* p, const float* x, float* dphi) {
     // device arrays of the current device are read and written in place (the
     // input is consumed by the first kernel, so x may even alias dphi); host
     // arrays go through the handle's staging buffers
-    const bool dev_in = prop_on_device(x), dev_out = prop_on_device(dphi);
-    hpf_status s = HPF_OK;
-    if (!dev_in && (s = prop_stage(p, p->xin, x, (size_t)p->g.V * 4)) != HPF_OK) return s;
-    prop_predict(p, dev_in ? x : p->xin, dev_out ? dphi : p->yout, p->stream, p->flag);
+    const size_t out_bytes = sizeof(float) * 2 * p->g.V;
+    const Placed out = placed(dphi, out_bytes, true);
+    if (out == Placed::kShort) return HPF_ERR_CUDA;
+    hpf_status s = prop_input(p, p->xin, &x, (size_t)p->g.V * 4);
+    if (s != HPF_OK) return s;
+    prop_predict(p, x, out == Placed::kInPlace ? dphi : p->yout, p->stream, p->flag);
     if ((s = prop_launched(p)) != HPF_OK) return s;
-    if (dev_out) return HPF_OK;  // the wait status comes with the next synchronising call
-    if ((s = prop_copy_out(p, dphi, p->yout, sizeof(float) * 2 * p->g.V)) != HPF_OK) return s;
+    // in place: the wait status comes with the next synchronising call
+    if (out == Placed::kInPlace) return HPF_OK;
+    if ((s = prop_copy_out(p, dphi, p->yout, out_bytes)) != HPF_OK) return s;
     return prop_flag_status(p);  // the host copy has synchronised: the status is known
 }
 
@@ -2265,15 +2267,8 @@ hpf_status hpf_prop_rollout(hpf_prop* p, const float* x, int32_t steps, float* p
 // the handle's staging buffers.
 static hpf_status prop_gradients(hpf_prop* p, const float* x, const float* phi_next,
                                  const AdamArgs& adam) {
-    hpf_status s = HPF_OK;
-    if (!prop_on_device(x)) {
-        s = prop_stage(p, p->xin, x, (size_t)p->g.V * 4);
-        x = p->xin;
-    }
-    if (s == HPF_OK && !prop_on_device(phi_next)) {
-        s = prop_stage(p, p->tin, phi_next, (size_t)p->g.V * 2);
-        phi_next = p->tin;
-    }
+    hpf_status s = prop_input(p, p->xin, &x, (size_t)p->g.V * 4);
+    if (s == HPF_OK) s = prop_input(p, p->tin, &phi_next, (size_t)p->g.V * 2);
     if (s != HPF_OK) return s;
     prop_forward(p, x, phi_next, p->stream, p->flag);
     prop_backward(p, adam);

@@ -5,12 +5,13 @@ import ctypes
 import numpy as np
 import pytest
 
-from paper_1310_2041_gb300 import learned
+from paper_1310_2041_gb300 import learned, workloads as W
 
 pytestmark = pytest.mark.gpu
 
 MESH = (9, 18, 7)  # x, y, z
 GRID = MESH[::-1]
+CUDA_ERROR = 2  # HPF_ERR_CUDA
 
 
 def densities(seed, channels):
@@ -62,3 +63,46 @@ def test_predictions_at_any_address(hpf_gpu, shift_in, shift_out):
         got = out[shift_out:shift_out + want.nbytes].cpu().numpy().view(np.float32).reshape(want.shape)
         assert np.array_equal(got, want)
         del keep
+
+
+SEGMENT = 12 << 20  # a tensor of this size has an allocation of its own
+
+
+def address_near_an_end(nbytes):
+    """(an allocation, the address `nbytes` before its end)."""
+    import torch
+    raw = torch.zeros(SEGMENT, dtype=torch.uint8, device="cuda")
+    return raw, raw.data_ptr() + SEGMENT - nbytes
+
+
+def test_device_arrays_that_are_too_short_are_refused(hpf_gpu):
+    """A state, a prediction or a training input whose allocation ends inside it
+    is an error (the staging copies refused it); nothing is launched on it."""
+    import torch
+    w = W.diblock(33, 4, 3, 4.4, 4, 1.0)
+    d = W.generate(w)
+    n = w.n_beads
+    raw, short = address_near_an_end(12 * n - 4)
+    whole = torch.zeros((n, 3), device="cuda")
+    with hpf_gpu.System(hpf_gpu.make_params(**w.params())) as s:
+        s.set_state(d["pos"], d["vel"], d["type"], d["bonds"])
+        assert s.lib.hpf_get_state(s.h, short, whole.data_ptr(), None) == CUDA_ERROR
+        assert s.lib.hpf_get_state(s.h, whole.data_ptr(), short, None) == CUDA_ERROR
+        assert np.array_equal(s.get_state()[0], d["pos"])
+        assert s.lib.hpf_get_state(s.h, raw.data_ptr() + SEGMENT - 12 * n, None, None) == 0
+    last = raw[SEGMENT - 12 * n:].cpu().numpy().view(np.float32).reshape(n, 3)
+    assert np.array_equal(last, d["pos"])
+    assert not raw[:SEGMENT - 12 * n].any()
+    x, nxt = densities(1, 4), densities(2, 2)
+    xd, nd = torch.from_numpy(x).cuda(), torch.from_numpy(nxt).cuda()
+    with network(hpf_gpu) as net:
+        before = net.get_weights()
+        for px, pn in ((short, nd.data_ptr()), (xd.data_ptr(), short)):
+            assert net.lib.hpf_prop_train_step(net.h, px, pn, 1e-3, None) == CUDA_ERROR
+            assert net.lib.hpf_prop_forward(net.h, px, pn) == CUDA_ERROR
+        assert np.array_equal(net.get_weights(), before)
+        net.train_step(xd, nd, 1e-3)
+        stepped = net.get_weights()
+    with network(hpf_gpu) as net:  # the refused steps do not count in Adam's bias correction
+        net.train_step(x, nxt, 1e-3)
+        assert np.array_equal(net.get_weights(), stepped)
