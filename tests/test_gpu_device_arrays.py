@@ -106,3 +106,55 @@ def test_device_arrays_that_are_too_short_are_refused(hpf_gpu):
     with network(hpf_gpu) as net:  # the refused steps do not count in Adam's bias correction
         net.train_step(x, nxt, 1e-3)
         assert np.array_equal(net.get_weights(), stepped)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 255, 257, 1003])
+def test_states_are_read_back_to_any_memory(hpf_gpu, n):
+    """Device outputs that kernels can write in place, alone and side by side in
+    one allocation, and those that take the copies: beside a host output,
+    overlapping, unaligned."""
+    import torch
+    w = W.Workload("free", [(n, [0])], 8.0, 8, 1, [[0.0]], 0.1, field_every=2, steps=2)
+    d = W.generate(w)
+    with hpf_gpu.System(hpf_gpu.make_params(**w.params())) as s:
+        s.set_state(d["pos"], d["vel"], d["type"], d["bonds"])
+        s.step(3)
+        pos, vel, _ = s.get_state()
+
+        def read(p, v):
+            assert s.lib.hpf_get_state(s.h, p, v, None) == 0
+
+        def buffers(words):
+            raw = torch.full((words,), -7.0, device="cuda")
+            torch.cuda.synchronize()
+            return raw, raw.data_ptr()
+
+        def floats(raw, first, count=3 * n):
+            return raw[first:first + count].cpu().numpy()
+
+        p, v, _ = s.get_state(torch.empty((n, 3), device="cuda"), torch.empty((n, 3), device="cuda"))
+        assert np.array_equal(p.cpu(), pos) and np.array_equal(v.cpu(), vel)
+        for gap in (0, 1):  # side by side in one allocation, velocities first
+            raw, a = buffers(6 * n + gap + 2)
+            read(a + 4 * (1 + 3 * n + gap), a + 4)
+            assert np.array_equal(floats(raw, 1), vel.reshape(-1))
+            assert np.array_equal(floats(raw, 1 + 3 * n + gap), pos.reshape(-1))
+            assert floats(raw, 0, 1) == -7 and floats(raw, 6 * n + gap + 1, 1) == -7
+            assert gap == 0 or floats(raw, 3 * n + 1, 1) == -7
+        raw, a = buffers(6 * n)  # one alone
+        read(a, None)
+        assert np.array_equal(floats(raw, 0), pos.reshape(-1)) and np.all(floats(raw, 3 * n) == -7)
+        read(None, a + 12 * n)
+        assert np.array_equal(floats(raw, 0), pos.reshape(-1))
+        assert np.array_equal(floats(raw, 3 * n), vel.reshape(-1))
+        host = np.zeros((n, 3), np.float32)  # one on the host
+        raw, a = buffers(3 * n)
+        read(a, host.ctypes.data)
+        assert np.array_equal(floats(raw, 0), pos.reshape(-1)) and np.array_equal(host, vel)
+        raw, a = buffers(3 * n + 1)  # overlapping: velocities are copied last
+        read(a, a + 4)
+        assert floats(raw, 0, 1) == pos[0, 0] and np.array_equal(floats(raw, 1), vel.reshape(-1))
+        raw, a = at_byte(np.zeros((2, n, 3), np.float32), 2)  # unaligned
+        read(a, a + 12 * n)
+        got = raw[2:2 + 24 * n].cpu().numpy().view(np.float32).reshape(2, n, 3)
+        assert np.array_equal(got[0], pos) and np.array_equal(got[1], vel)
