@@ -1900,9 +1900,9 @@ hpf_status ensure_learned(hpf_ctx* c) {
     return HPF_OK;
 }
 
-// The judge's eps of the fields Ga (candidate) and Gb at the current
-// positions; waits for the stream.
-hpf_status judge_fields(hpf_ctx* c, const float4* Ga, const float4* Gb, double* eps) {
+// The judge's sums of the fields Ga (candidate) and Gb at the current
+// positions, and the error word so far to hflag[0].
+hpf_status judge_fields(hpf_ctx* c, const float4* Ga, const float4* Gb) {
     LearnedBufs* L = c->learned;
     {
         StageScope sc(c, HPF_STAGE_OTHER, 1);
@@ -1910,12 +1910,13 @@ hpf_status judge_fields(hpf_ctx* c, const float4* Ga, const float4* Gb, double* 
                      L->h_acc, c->dflag, c->hflag, c->stream);
     }
     LAUNCH_CHECK(c);
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    const hpf_status s = flag_status(c, c->hflag[0]);
-    if (s != HPF_OK) return s;
-    const double e2 = L->h_acc[0], r2 = L->h_acc[1];
-    *eps = r2 > 0.0 ? sqrt(e2 / r2) : (e2 > 0.0 ? INFINITY : 0.0);
     return HPF_OK;
+}
+
+// eps from the judge's sums, which the stream has reached.
+double judge_eps(const hpf_ctx* c) {
+    const double e2 = c->learned->h_acc[0], r2 = c->learned->h_acc[1];
+    return r2 > 0.0 ? sqrt(e2 / r2) : (e2 > 0.0 ? INFINITY : 0.0);
 }
 
 // eps of a candidate density against the true density of the current
@@ -1935,7 +1936,11 @@ hpf_status judge_mesh(hpf_ctx* c, bool have_G2, double* eps) {
         }
         if ((s = field_from(c, L->Dp, L->tmap, L->tmap_ok, nullptr, L->G2)) != HPF_OK) return s;
     }
-    return judge_fields(c, L->G2, c->G, eps);
+    if ((s = judge_fields(c, L->G2, c->G)) != HPF_OK) return s;
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    if ((s = flag_status(c, c->hflag[0])) != HPF_OK) return s;
+    *eps = judge_eps(c);
+    return HPF_OK;
 }
 
 // K steps with a true scatter and field refresh at every step (the plain
@@ -2042,10 +2047,15 @@ hpf_status hpf_judge_density_pair(hpf_ctx* c, const float* phi_cand, const float
     CUtensorMap none;
     memset(&none, 0, sizeof none);
     if ((s = field_from(c, L->Dp, none, false, nullptr, L->G2)) != HPF_OK) return s;
+    c->field_valid = false;  // until the last refresh below
     if ((s = field_from(c, L->Dbase, none, false, nullptr)) != HPF_OK) return s;
-    if ((s = judge_fields(c, L->G2, c->G, eps)) != HPF_OK) return s;
-    // the field of the true density back in force
-    return run_field(c);
+    if ((s = judge_fields(c, L->G2, c->G)) != HPF_OK) return s;
+    // the field of the true density back in force, before the stream is waited
+    // for: its error word counts too, and an error leaves it in place
+    if ((s = run_field(c)) != HPF_OK) return s;
+    if ((s = check_flags(c)) != HPF_OK) return s;
+    *eps = judge_eps(c);
+    return HPF_OK;
 }
 
 hpf_status hpf_step_learned(hpf_ctx* c, hpf_prop* prop, int32_t n_windows, int32_t K, double tol,

@@ -692,3 +692,26 @@ def test_judge_density_pair(hpf_gpu):
         e_true = s.judge_density(cand)
         assert e_true > 1e-3
         assert abs(e_pair - e_true) <= 1e-5 * e_true + 1e-7
+
+
+def test_judge_density_pair_waits_for_the_field_it_restores(hpf_gpu):
+    """The call synchronises: nothing of it, the refresh that puts the true
+    density's field back among it (50 us and more on this mesh), is left on the
+    stream when it returns, and that refresh's field is the true one."""
+    import torch
+    w = W.diblock(50, 5, 5, 192.0, 192, 1.0)
+    d = W.generate(w)
+    with hpf_gpu.System(hpf_gpu.make_params(**w.params()), stream=torch.cuda.Stream()) as s:
+        s.set_state(d["pos"], d["vel"], d["type"], d["bonds"])
+        true = torch.empty(s.mesh_shape, device="cuda")
+        s.density_phi(true)
+        cand = true + 0.5
+        torch.cuda.synchronize()
+        want = s.forces(hpf_gpu.FORCE_FIELD)
+        stream = torch.cuda.ExternalStream(s.stream)
+        left = []
+        for _ in range(3):
+            assert s.judge_density_pair(cand, cand) == 0.0
+            left.append(not stream.query())
+        assert not any(left)
+        assert np.array_equal(s.forces(hpf_gpu.FORCE_FIELD), want)
