@@ -2,14 +2,13 @@
 // density is from that of the reference, over all beads.
 //
 // One pass over the beads gathers both fields at once (sixteen corner loads in
-// flight per bead) and sums |Fa - Fb|^2 and |Fb|^2: two force passes through
-// memory, an FP64 error pass and a one-warp sum over 1216 partials took
-// 18.6 + 18.6 + 37 + 74 us at 1M beads, this pass 37.  A bead's terms are formed in
-// float-float (the difference exactly, squares with their errors, about
-// 2^-45 relative) and added to the thread's FP64 sums, one addition per sum
-// and bead instead of eight FP64 operations per component (this GPU's FP64
-// rate is 1/64 of its FP32 rate).  The last block to finish adds the block
-// sums in order and writes them to the host.
+// flight per bead) and sums |Fa - Fb|^2 and |Fb|^2 in FP64, one rounding per
+// square: two force passes through memory, an error pass and a one-warp sum over
+// 1216 partials took 18.6 + 18.6 + 37 + 74 us at 1M beads.  A call with its
+// stencils and synchronisation takes 75.6 us; with a bead's squares in float-float
+// instead (about 2^-45 relative), 69.6, which is not worth bits that the error
+// pass had.  The last block to finish adds the block sums in order and writes
+// them to the host.
 #include "hpf_internal.cuh"
 
 namespace hpf {
@@ -18,7 +17,8 @@ namespace {
 
 constexpr int kJudgeBlock = 256;
 // One wave of three blocks (80 registers: all sixteen corner loads of a bead in
-// flight) on each of 152 SMs, whatever the device.  A learned window of 1M
+// flight) on each of 152 SMs, and the same number on any other device, so that the
+// sums are taken in the same order, to the same bits, everywhere.  A learned window of 1M
 // beads with its judge: 1012 us at 304 or 456 blocks, 1019 at 608 (4 per SM),
 // 1030 at 760 (5), 1034 at 1216 (48 registers, two waves).
 constexpr int kJudgePerSM = 3;
@@ -28,13 +28,6 @@ struct JudgeScratch {
     unsigned ticket;
     double part[kJudgeGrid][2];
 };
-
-// v^2 of v = h + l in float-float, added to a.
-__device__ __forceinline__ FF ff_square_plus(FF a, float h, float l) {
-    const float p = __fmul_rn(h, h);
-    const float e = fmaf(2.0f * h, l, fmaf(h, h, -p));
-    return ff_plus(a, FF{p, e});
-}
 
 __device__ __forceinline__ void block_sum2(double& e, double& r, double (*sh)[kJudgeBlock / 32]) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -82,16 +75,10 @@ __global__ void __launch_bounds__(kJudgeBlock, kJudgePerSM) k_judge(StateBuf st,
             gather_field_mode(Ga + off, g, mode, x, y, z, a[0], a[1], a[2]);
             gather_field_mode(Gb + off, g, mode, x, y, z, b[0], b[1], b[2]);
         }
-        FF fe{0.f, 0.f}, fr{0.f, 0.f};
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            float h, l;
-            two_sum(a[k], -b[k], h, l);
-            fe = ff_square_plus(fe, h, l);
-            fr = ff_square_plus(fr, b[k], 0.f);
-        }
-        e += ff_to_double(fe);
-        r += ff_to_double(fr);
+        const double b0 = b[0], b1 = b[1], b2 = b[2];
+        const double d0 = (double)a[0] - b0, d1 = (double)a[1] - b1, d2 = (double)a[2] - b2;
+        e = fma(d0, d0, fma(d1, d1, fma(d2, d2, e)));
+        r = fma(b0, b0, fma(b1, b1, fma(b2, b2, r)));
     }
     block_sum2(e, r, sh);
     if (threadIdx.x == 0) {

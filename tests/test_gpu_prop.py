@@ -715,3 +715,63 @@ def test_judge_density_pair_waits_for_the_field_it_restores(hpf_gpu):
             left.append(not stream.query())
         assert not any(left)
         assert np.array_equal(s.forces(hpf_gpu.FORCE_FIELD), want)
+
+
+def force_pair(hpf, s, pp, cand):
+    """The FP32 field forces of a candidate density and of the true one, as FP64."""
+    h = [np.float64(np.float32(pp["box"][a])) / pp["mesh"][a] for a in range(3)]
+    inv_phi_c = 1.0 / (2.0 ** -39 / (pp["rho0"] * (h[0] * h[1] * h[2])))
+    Dc = np.maximum(np.rint(cand.astype(np.float64) * inv_phi_c), 0).astype(np.int64)
+    D = s.scatter_density()
+    s.field(D_in=Dc)
+    Fc = s.forces(hpf.FORCE_FIELD).astype(np.float64)
+    s.field(D_in=D)
+    return Fc, s.forces(hpf.FORCE_FIELD).astype(np.float64)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3])
+def test_judge_sums_in_fp64(hpf_gpu, n):
+    """eps of a few beads from their FP32 forces to FP64 rounding: a bead's three
+    squares enter each sum by one rounding each (2^-53 of it at most), so the
+    root of the quotient is off by at most (3 n + 3 n) / 2 + 1/2 + 1 of them."""
+    w = W.Workload("few", [(n, [0])], 5.0, 5, 1, [[0.0]], 0.5, field_every=1, steps=1)
+    pp = w.params()
+    worst = 0.0
+    for seed in range(40):
+        rng = np.random.default_rng(seed)
+        d = W.generate(w)
+        pos = rng.uniform(0.0, 5.0, (n, 3)).astype(np.float32)
+        with hpf_gpu.System(hpf_gpu.make_params(**pp)) as s:
+            s.set_state(pos, d["vel"], d["type"], d["bonds"])
+            cand = (s.density_phi() + rng.uniform(0.0, 0.3, s.mesh_shape)).astype(np.float32)
+            eps = s.judge_density(cand)
+            Fc, Ft = force_pair(hpf_gpu, s, pp, cand)
+            diff = (Fc - Ft).astype(np.longdouble)
+            want = np.sqrt((diff ** 2).sum() / (Ft.astype(np.longdouble) ** 2).sum())
+            worst = max(worst, float(abs(eps - want) / want))
+    assert worst <= (3 * n + 1.5) * 2.0 ** -53 * 1.001
+
+
+@pytest.mark.parametrize("n", [456 * 256 - 1, 456 * 256 + 1, 2 * 456 * 256 + 77])
+def test_judge_counts_every_bead_once(hpf_gpu, n):
+    """Beads at both ends of the grid's rounds, each judged by a candidate that
+    differs from the true density around that bead alone: left out or counted
+    twice it changes eps by its share of the few beads there, the FP32 forces'
+    summation by 1e-12 at most."""
+    w = W.Workload("free", [(n, [0])], 40.0, 40, 1, [[0.0]], 0.5, field_every=1, steps=1)
+    pp, d = w.params(), W.generate(w)
+    with hpf_gpu.System(hpf_gpu.make_params(**pp)) as s:
+        s.set_state(d["pos"], d["vel"], d["type"], d["bonds"])
+        true = s.density_phi()
+        order = s.order()
+        for slot in sorted({0, 456 * 256 - 1, 456 * 256, 2 * 456 * 256, n - 1}):
+            if slot >= n:
+                continue
+            cand = true.copy()
+            x, y, z = np.floor(d["pos"][order[slot]]).astype(int) % 40
+            cand[0, z, y, x] += 0.5
+            eps = s.judge_density(cand)
+            Fc, Ft = force_pair(hpf_gpu, s, pp, cand)
+            want = np.linalg.norm(Fc - Ft) / np.linalg.norm(Ft)
+            assert eps == pytest.approx(want, rel=1e-12)
+            assert np.any(Fc[order[slot]] != Ft[order[slot]])
