@@ -375,9 +375,12 @@ void derive_constants(hpf_ctx* c) {
     };
     split(e.ff_angle_k, p.angle_k);
     split(e.ff_cos0, p.angle_cos0);
-    split(e.ff_dih_k, p.dihedral_k);
-    split(e.ff_dih_cd, cos(p.dihedral_delta));
-    split(e.ff_dih_sd, sin(p.dihedral_delta));
+    e.dih_k = p.dihedral_k;
+    e.dih_cd = cos(p.dihedral_delta);
+    e.dih_sd = sin(p.dihedral_delta);
+    split(e.ff_dih_k, e.dih_k);
+    split(e.ff_dih_cd, e.dih_cd);
+    split(e.ff_dih_sd, e.dih_sd);
     e.inv_kappa = p.inv_kappa;
     e.phi_c = phi_c;
     e.w_scale = p.rho0 * vol;

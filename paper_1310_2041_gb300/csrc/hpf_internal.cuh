@@ -118,7 +118,9 @@ struct EnergyConsts {
     double angle_k, cos0;  // angle potential
     int angle_form;        // 0 cosine, 1 harmonic (theta0)
     double theta0;
-    int dih_n;             // dihedral potential k [1 + cos(n phi - delta)]
+    double dih_k;          // dihedral potential k [1 + cos(n phi - delta)]
+    int dih_n;
+    double dih_cd, dih_sd;  // cos delta, sin delta
     // float-float pairs (high, low) of angle_k, cos0, the dihedral's k, cos delta, sin delta
     float ff_angle_k[2], ff_cos0[2], ff_dih_k[2], ff_dih_cd[2], ff_dih_sd[2];
 };

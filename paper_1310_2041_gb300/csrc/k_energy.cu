@@ -66,12 +66,83 @@ __device__ __forceinline__ FF angle_energy_ff(const StateBuf& st, int i, const E
 // Dihedral energy k [1 + cos(n phi - delta)] of the quadruplet i .. i + 3: cos
 // phi = A.B / (|A||B|), sin phi = |b2| b1.B / (|A||B|) with A = b1 x b2, B =
 // b2 x b3, and cos(n phi), sin(n phi) by the n-th power of cos phi + i sin phi.
-__device__ __forceinline__ FF dihedral_energy_ff(const StateBuf& st, int i, const EnergyConsts& e) {
-    const FF3 b1 = bond_ff3(st, i, i + 1), b2 = bond_ff3(st, i + 1, i + 2),
-              b3 = bond_ff3(st, i + 2, i + 3);
-    const FF3 A = ff_cross(b1, b2), B = ff_cross(b2, b3);
+// In FP64: the quadruplets that the float-float form leaves.
+__device__ __noinline__ double dihedral_energy_fp64(const StateBuf& st, int i,
+                                                    const EnergyConsts& e) {
+    double b[3][3];  // bond vectors
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        b[k][0] = (double)st.x[i + k + 1] - st.x[i + k];
+        b[k][1] = (double)st.y[i + k + 1] - st.y[i + k];
+        b[k][2] = (double)st.z[i + k + 1] - st.z[i + k];
+    }
+    double A[3], B[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int u = (a + 1) % 3, v = (a + 2) % 3;
+        A[a] = b[0][u] * b[1][v] - b[0][v] * b[1][u];
+        B[a] = b[1][u] * b[2][v] - b[1][v] * b[2][u];
+    }
+    const double AA = A[0] * A[0] + A[1] * A[1] + A[2] * A[2];
+    const double BB = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
+    const double L = norm_fp64(b[1][0] * b[1][0] + b[1][1] * b[1][1] + b[1][2] * b[1][2]);
+    const double den = norm_fp64(AA) * norm_fp64(BB);
+    const double cp = (A[0] * B[0] + A[1] * B[1] + A[2] * B[2]) / den;
+    const double sp = L * (b[0][0] * B[0] + b[0][1] * B[1] + b[0][2] * B[2]) / den;
+    double cn = cp, sn = sp;
+    for (int k = 1; k < e.dih_n; ++k) {
+        const double t = cn * cp - sn * sp;
+        sn = sn * cp + cn * sp;
+        cn = t;
+    }
+    return e.dih_k * (1.0 + cn * e.dih_cd + sn * e.dih_sd);
+}
+
+// a + s b with s near the value that leaves only a's part across b, rounded to 13
+// bits so that s b is exact wherever b's components are FP32 numbers; ibb = 1 / b.b.
+// cc: the length squared of the result.
+__device__ __forceinline__ FF3 across(const FF3& a, const FF3& b, float ibb, float& cc) {
+    const float d = fmaf(a.z.h, b.z.h, fmaf(a.y.h, b.y.h, __fmul_rn(a.x.h, b.x.h)));
+    const float s = __uint_as_float((__float_as_uint(__fmul_rn(-d, ibb)) + 0x400u) & 0xfffff800u);
+    auto add = [s](FF u, FF v) {
+        const float p = __fmul_rn(s, v.h);
+        return ff_plus(u, FF{p, fmaf(s, v.l, fmaf(s, v.h, -p))});
+    };
+    const FF3 c{add(a.x, b.x), add(a.y, b.y), add(a.z, b.z)};
+    cc = fmaf(c.z.h, c.z.h, fmaf(c.y.h, c.y.h, __fmul_rn(c.x.h, c.x.h)));
+    return c;
+}
+
+// The same in float-float; false where it would be less accurate than the FP64
+// form.  In a nearly straight triplet the two halves of a cross product cancel,
+// and with them goes what 48 bits have less than 53.  Adding a multiple of b2 to b1
+// (and to b3) changes neither A, B nor b1.B, and without its part along b2
+// nothing cancels.  FP64 takes over where even so |A| is below a fifth of the
+// factors' product (within about 0.02 degrees of straight, exactly straight ones,
+// whose angle is undefined, among them) or |A|^2 leaves the range in which FP32
+// holds a product's low half (bonds below 3e-5 or beyond 3e7).  A lane there costs
+// a launch 10 us, so the line must lie where thermal chains hardly come: with
+// b1 +- b2 in place of the projection 1 in 4000 quadruplets crossed it.  Largest
+// error per k against 80-bit arithmetic over 200,000 quadruplets each, n = 3, FP64
+// form / this one: angles of 100 to 140 degrees 2.8e-13 / 1.0e-13, all angles alike
+// 2.8e-13 / 1.0e-13, 177 to 179 degrees 2.5e-13 / 1.0e-13, 179 to 180 degrees
+// 1.2e-11 / 8.6e-12 (b1 and b3 as they are: 1.0e-13, 1.3e-12, 2.4e-12, 1.7e-7).
+__device__ __forceinline__ bool dihedral_energy_ff(const StateBuf& st, int i, const EnergyConsts& e,
+                                                   FF& energy) {
+    constexpr float kTau2 = 1.0f / 25.0f;
+    constexpr float kLow = 8.673617379884035e-19f, kHigh = 1.2676506002282294e30f;  // 2^-60, 2^100
+    const FF3 b2 = bond_ff3(st, i + 1, i + 2);
     const FF b22 = ff_dot(b2, b2);
-    const FF inv = ff_mul(ff_rsqrt(ff_dot(A, A)), ff_rsqrt(ff_dot(B, B)));
+    const float ibb = __fdividef(1.0f, b22.h);
+    float c1, c3;
+    const FF3 b1 = across(bond_ff3(st, i, i + 1), b2, ibb, c1);
+    const FF3 b3 = across(bond_ff3(st, i + 2, i + 3), b2, ibb, c3);
+    const FF3 A = ff_cross(b1, b2), B = ff_cross(b2, b3);
+    const FF AA = ff_dot(A, A), BB = ff_dot(B, B);
+    if (!(AA.h >= kTau2 * c1 * b22.h && BB.h >= kTau2 * c3 * b22.h && fminf(AA.h, BB.h) >= kLow &&
+          fmaxf(AA.h, BB.h) <= kHigh))
+        return false;
+    const FF inv = ff_mul(ff_rsqrt(AA), ff_rsqrt(BB));
     const FF cp = ff_mul(ff_dot(A, B), inv);
     const FF sp = ff_mul(ff_mul(ff_mul(b22, ff_rsqrt(b22)), ff_dot(b1, B)), inv);
     FF cn = cp, sn = sp;
@@ -82,7 +153,8 @@ __device__ __forceinline__ FF dihedral_energy_ff(const StateBuf& st, int i, cons
     }
     const FF v = ff_plus(ff_plus(FF{1.0f, 0.f}, ff_mul(cn, ff_of(e.ff_dih_cd))),
                          ff_mul(sn, ff_of(e.ff_dih_sd)));
-    return ff_mul(ff_of(e.ff_dih_k), v);
+    energy = ff_mul(ff_of(e.ff_dih_k), v);
+    return true;
 }
 
 // Per bead: F_n with the terms the step kernel's kick uses (bonds, the field
@@ -109,7 +181,7 @@ __device__ __forceinline__ void energy_beads_block(const StateBuf& st,
                                                    const EnergyConsts& e,
                                                    float2* __restrict__ partials, int blk, int nb,
                                                    FF (*sh)[kRedBlock / 32]) {
-    double ub = 0.0;           // harmonic angle energies (FP64)
+    double ub = 0.0;           // harmonic angles and the dihedrals left to FP64
     float uh = 0.f, ul = 0.f;  // the other bonded energies, float-float
     FF kf{0.f, 0.f}, pfx{0.f, 0.f}, pfy{0.f, 0.f}, pfz{0.f, 0.f};
     for (int i = blk * kRedBlock + threadIdx.x; i < n; i += nb * kRedBlock) {
@@ -153,9 +225,14 @@ __device__ __forceinline__ void energy_beads_block(const StateBuf& st,
                 [&](int d) { return make_float3(st.x[i + d], st.y[i + d], st.z[i + d]); }, back,
                 fwd, c, fx, fy, fz);
             if (fwd == 3) {  // the one starting here, once
-                const FF u = ff_plus(FF{uh, ul}, dihedral_energy_ff(st, i, e));
-                uh = u.h;
-                ul = u.l;
+                FF u;
+                if (dihedral_energy_ff(st, i, e, u)) {
+                    u = ff_plus(FF{uh, ul}, u);
+                    uh = u.h;
+                    ul = u.l;
+                } else {
+                    ub += dihedral_energy_fp64(st, i, e);
+                }
             }
         }
         const float4* Gt = G + (size_t)((m >> kTypeShift) & kTypeMask) * g.gnodes;

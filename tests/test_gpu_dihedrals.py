@@ -189,3 +189,57 @@ def test_invalid_dihedral_parameters_are_rejected(hpf_gpu):
             hpf_gpu.System(hpf_gpu.make_params(**dict(w.params(), **bad)))
     # the multiplicity is not checked without dihedrals
     hpf_gpu.System(hpf_gpu.make_params(**dict(w.params(), dihedral_k=0.0, dihedral_n=0))).close()
+
+
+def quadruplets(rng, count, angles, bond, box):
+    """Chains of four beads with bond angles in the given range, any torsion, the
+    bond lengths a tenth apart; FP32."""
+    out = np.empty((count, 4, 3), np.float32)
+    unit = lambda v: v / np.linalg.norm(v)  # noqa: E731
+    for p in out:
+        x, t = rng.uniform(0.0, box, 3), unit(rng.normal(size=3))
+        p[0] = x
+        for k in range(1, 4):
+            if k > 1:
+                th = np.radians(rng.uniform(*angles))
+                q = rng.normal(size=3)
+                t = -np.cos(th) * t + np.sin(th) * unit(q - (q @ t) * t)
+            x = x + bond * (1.0 + 0.1 * rng.normal()) * t
+            p[k] = x
+    return out
+
+
+def dihedral_terms(p, n):
+    """1 + cos(n phi) of each chain in long doubles."""
+    b = np.diff(p.astype(np.longdouble), axis=1)
+    A, B = np.cross(b[:, 0], b[:, 1]), np.cross(b[:, 1], b[:, 2])
+    norm = lambda v: np.sqrt((v * v).sum(1))  # noqa: E731
+    z = ((A * B).sum(1) + 1j * norm(b[:, 1]) * (b[:, 0] * B).sum(1)) / (norm(A) * norm(B))
+    return 1 + np.prod([z] * n, axis=0).real
+
+
+@pytest.mark.parametrize("angles,bond,box,rms", [
+    ((100.0, 140.0), 0.7, 3.0, 1e-13),
+    ((179.6, 179.8), 0.7, 3.0, 1e-12),
+    ((100.0, 140.0), 7e-10, 1e-9, 1e-13),
+    ((100.0, 140.0), 7e8, 1e9, 1e-13),
+], ids=["bent", "straight", "short", "long"])
+def test_energies_of_single_dihedrals(hpf_gpu, angles, bond, box, rms):
+    """Each of 512 quadruplets by itself (n = 3), an error per k as FP64 has it
+    from the FP32 positions: lengths to 3e-14 (one Newton step), three of them in a
+    phase that is taken three times, 5e-14 rms; nearly straight ones cancel 1 /
+    sin theta (250) of b1.B's 2^-53 once more, 8e-14 rms with a tail to 5e-12."""
+    rng = np.random.default_rng(9)
+    size = max(8.0, 4.0 * box)
+    w = W.Workload("one", [(1, [0] * 4)], size, 4, 1, [[0.0]], 0.0, field_every=1, steps=1)
+    pars = hpf_gpu.make_params(**{**w.params(), "bond_k": 0.0, "dihedral_k": 1.0, "dihedral_n": 3,
+                                  "dt": 1e-6, "rho0": 4.0 / size ** 3})
+    d = W.generate(w)
+    err = []
+    with hpf_gpu.Batch([pars] * 64) as b:
+        for _ in range(8):
+            p = quadruplets(rng, 64, angles, bond, box)
+            for r in range(64):
+                b.replica(r).set_state(p[r], d["vel"], d["type"], d["bonds"])
+            err.append(b.energy()[:, 1] - dihedral_terms(p, 3))
+    assert np.sqrt(np.mean(np.concatenate(err).astype(np.float64) ** 2)) <= rms
