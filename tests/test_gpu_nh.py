@@ -211,3 +211,21 @@ def test_every_bead_counts_once_in_the_kinetic_energy(hpf_gpu, orc, n):
                                    0, 2, xe=(0.0, 0.0))
     assert abs(xi - xo) <= 1e-4 * max(1.0, abs(xo))
     assert abs(eta - eo) <= 1e-6 * max(1.0, abs(xo))
+
+
+@pytest.mark.parametrize("n", [912 * 256 - 31, 912 * 256, 912 * 256 + 1, 2 * 912 * 256 + 300])
+def test_every_bead_counts_once_beside_dihedrals(hpf_gpu, orc, n):
+    """The same in the kernel with dihedrals, whose grid and loop are its own: five
+    chains of eight beads among free ones, bent as a thermal chain."""
+    w = W.Workload("mixed", [(5, [0] * 8), (n - 40, [0])], 12.0, 8, 1, [[0.0]], 0.0, field_every=2,
+                   steps=2, dt=0.002)
+    d = W.with_bond_angles(w, W.generate(w))
+    fast = sorted({0, n - 1} | {i for i in (255, 256, 912 * 256 - 1, 912 * 256) if i < n})
+    d["vel"][fast] *= 30.0
+    s, pp = make(hpf_gpu, w, d, nh_tau=0.002, angle_k=4.0, angle_cos0=-0.5, dihedral_k=0.5, dihedral_n=3)
+    s.step(2)
+    xi, eta = s.get_thermostat()
+    _, _, (xo, eo), _ = orc.run_nh(orc.make_params(**pp), d["pos"], d["vel"], d["type"], d["bonds"],
+                                   0, 2, xe=(0.0, 0.0))
+    assert abs(xi - xo) <= 1e-4 * max(1.0, abs(xo))
+    assert abs(eta - eo) <= 1e-6 * max(1.0, abs(xo))
