@@ -146,9 +146,6 @@ hpf_status hpf_set_state(hpf_ctx* ctx, const float* pos, const float* vel, const
  * Errors: HPF_ERR_INVALID, HPF_ERR_STATE (no hpf_set_state yet), HPF_ERR_CUDA. */
 hpf_status hpf_update_state(hpf_ctx* ctx, const float* pos, const float* vel, int64_t step);
 
-/* Copy the state out in tag order (either pointer may be NULL) and the step
- * number.  Synchronises the stream.
- * Errors: HPF_ERR_STATE, HPF_ERR_NONFINITE (state became non-finite), HPF_ERR_CUDA. */
 /* Pipelined replacement of positions and velocities, for callers that feed
  * a new state every few steps and want its upload to overlap the GPU work of
  * the previous one (double buffering).  hpf_upload_state starts the copy of
@@ -170,6 +167,11 @@ hpf_status hpf_update_state(hpf_ctx* ctx, const float* pos, const float* vel, in
 hpf_status hpf_upload_state(hpf_ctx* ctx, const float* pos, const float* vel);
 hpf_status hpf_apply_state(hpf_ctx* ctx, int64_t step);
 
+/* Copy the state out in tag order (either pointer may be NULL) and the step
+ * number.  Aligned device arrays that do not overlap are written in place,
+ * others through a copy.  Synchronises the stream.
+ * Errors: HPF_ERR_STATE, HPF_ERR_NONFINITE (state became non-finite), HPF_ERR_CUDA
+ * (also for a device array whose allocation ends inside it). */
 hpf_status hpf_get_state(hpf_ctx* ctx, float* pos, float* vel, int64_t* step);
 
 /* The library's storage order: order[i] is the tag of storage slot i.
@@ -210,11 +212,11 @@ hpf_status hpf_field(hpf_ctx* ctx, const int64_t* D_in, float* field_out);
  * Errors: HPF_ERR_INVALID, HPF_ERR_CUDA. */
 hpf_status hpf_selftest_timeout(hpf_ctx* ctx, double* seconds);
 
-/* The field stencil runs on shared-memory tiles of the mesh, staged by TMA
- * tensor copies when the mesh allows it (Mx even, n_species <= 4), or untiled
- * (one ghosted node, or two real nodes, per thread).  The kernel is chosen
- * from the mesh and the species count the first time the field is computed.
- * shape[0..2] = tile
+/* The field stencil computes one ghosted node per thread, or two real nodes
+ * for large even meshes of one species; the kernel is chosen from the mesh and
+ * the species count the first time the field is computed.  Slower ones on
+ * shared-memory tiles, staged by TMA tensor copies when the mesh allows it (Mx
+ * even, n_species <= 4), run only by hpf_set_field_tile.  shape[0..2] = tile
  * (x, y, z); (0, 0, 0) for the one-node untiled kernel (and before the first
  * refresh), (2, 1, 1) for the node-pair kernel; *uses_tma = 1 if the tiles
  * are staged by TMA, 0 otherwise.  Either pointer may be NULL.
@@ -323,10 +325,10 @@ hpf_status hpf_step_partial(hpf_ctx* ctx, int32_t n_steps, int32_t* steps_done, 
  * out[4] |total momentum| of v_n, out[5] kinetic temperature 2 KE / (3 N).
  * Errors: HPF_ERR_INVALID (out NULL), HPF_ERR_STATE, HPF_ERR_NONFINITE, HPF_ERR_CUDA. */
 hpf_status hpf_energy(hpf_ctx* ctx, double out[6]);
-/* hpf_energy in two halves: hpf_energy_start enqueues the kernels and the
- * copy of the six values (and of the kernels' error word) to pinned mirrors
+/* hpf_energy in two halves: hpf_energy_start enqueues the kernels, the last of
+ * which writes the six values (and the kernels' error word) to pinned mirrors,
  * on the context's stream and returns; hpf_energy_finish waits for those
- * copies only and returns the values of the step at which hpf_energy_start
+ * kernels only and returns the values of the step at which hpf_energy_start
  * was called, with the errors raised up to that point.  Work enqueued
  * between the two (hpf_upload_state, hpf_apply_state and hpf_step of the
  * next step) may still be running when it returns, so the next step's work
@@ -533,8 +535,9 @@ hpf_status hpf_prop_rollout(hpf_prop* prop, const float* x, int32_t steps, float
  * and its gradient with respect to the parameter vector (back-propagation
  * through the same BF16 kernels: data gradients with flipped, transposed
  * weights, weight gradients as tensor-core voxel reductions).  phi_next is
- * [2][Mz][My][Mx]; grads [param_count] and loss may be NULL.  Synchronises
- * when loss is given or grads is host memory. */
+ * [2][Mz][My][Mx]; grads [param_count] and loss may be NULL.  x and phi_next on
+ * the current device are read in place, as hpf_prop_forward reads x.
+ * Synchronises when loss is given or grads is host memory. */
 hpf_status hpf_prop_backward(hpf_prop* prop, const float* x, const float* phi_next, float* grads,
                              double* loss);
 

@@ -471,8 +471,8 @@ hpf_status scatter_current(hpf_ctx* c) {
 // target of the next scatter.
 hpf_status run_field(hpf_ctx* c) {
     if (c->S <= 4) {
-        // the tiled (TMA-staged) stencil with one replica; a batch runs the same
-        // kernel, so contexts and batch members agree bit for bit
+        // the stencil chosen for the mesh, with one replica; a batch runs the same
+        // kernels, so contexts and batch members agree bit for bit
         if (c->field_tile < 0) c->field_tile = field_tile_for(c->geom, c->S);
         StageScope sc(c, HPF_STAGE_FIELD, 1);
         SingleFieldParams p;
@@ -1528,7 +1528,7 @@ hpf_status bfail(hpf_batch* b, hpf_status s, const char* msg) {
 }
 
 // The batched stencil over all replicas, each reading its mesh buffer
-// dmesh ^ flip: one tiled launch per distinct tile shape among the replicas
+// dmesh ^ flip: one launch per distinct stencil among the replicas
 // (field_tile_for each replica's mesh).
 void launch_batch_fields(hpf_batch* b, int flip) {
     const int S = b->rep[0]->S;

@@ -20,7 +20,7 @@ namespace hpf {
 
 // Candidate tiles (x, y, z): a CTA has x * y threads, each computing z nodes
 // along a z column.  Shape {0, 0, 0} is the untiled one-node-per-thread stencil
-// with direct L1/L2 loads, so the autotuner can never pick a slower kernel.
+// with direct L1/L2 loads, the one that field_tile_for takes nearly always.
 // Shape {2, 1, 1} is the untiled two-nodes-per-thread stencil (16-byte pair
 // loads, ghost copies written directly).
 constexpr int kTileCandidates = 8;
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(TX * TY) k_field_tiled(const __grid_constant__
 
 // The untiled stencil: one thread per node of the ghosted array, neighbours
 // loaded directly (through L1/L2), same arithmetic as the tiled kernel.  Small
-// meshes are one chain of dependent latencies: with 42 registers (1536 threads
+// meshes are one chain of dependent latencies: with 40 registers (1536 threads
 // per SM) all loads of a node are in flight at once (3.56 -> 3.27 us at 15^3,
 // 8.2 -> 7.9 at 70^3, S = 2); a batch of many meshes fills the chip and takes 2048
 // (24.6 -> 23.5).  Blocks of 128 instead of 256 spread a small mesh over more SMs

@@ -4,10 +4,10 @@
 // One pass over the beads gathers both fields at once (sixteen corner loads in
 // flight per bead) and sums |Fa - Fb|^2 and |Fb|^2 in FP64, one rounding per
 // square: two force passes through memory, an error pass and a one-warp sum over
-// 1216 partials took 18.6 + 18.6 + 37 + 74 us at 1M beads.  A call with its
-// stencils and synchronisation takes 75.6 us; with a bead's squares in float-float
-// instead (about 2^-45 relative), 69.6, which is not worth bits that the error
-// pass had.  The last block to finish adds the block sums in order and writes
+// 1216 partials took 18.6 + 18.6 + 37 + 74 us at 1M beads, this pass 43, the FP64
+// pipe 74 % busy.  A call with its stencils and synchronisation takes 75.6 us; with
+// a bead's squares in float-float instead (about 2^-45 relative, 37 us a pass),
+// 69.6, which is not worth bits that the error pass had.  The last block to finish adds the block sums in order and writes
 // them to the host.
 #include "hpf_internal.cuh"
 

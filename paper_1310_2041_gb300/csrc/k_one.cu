@@ -13,8 +13,10 @@
 // the warp form's bond sums, else that of the halo form, so that a run gives
 // the same bits whichever kernel its steps go through.  1M beads, step and
 // deposit: 60 us with the warp kernel, 39 here, of which the deposit's
-// reductions are 11 and the rest is bound by the L1's data pipe (the eight
-// corner loads touch 22 sectors each).
+// reductions are 11.  No unit is full: the eight corner loads touch 22 sectors each
+// (L1 data pipe 58 % of the launch), the L2 is 52 % busy with them and the deposit,
+// and at 24 warps an SM a warp waits for its loads in 3.5 of the 11.8 cycles between
+// its instructions.
 #include "cell_poly.cuh"
 #include "chunk_pipe.cuh"
 

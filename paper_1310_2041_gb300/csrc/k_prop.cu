@@ -102,7 +102,9 @@ __device__ __forceinline__ void tile_origin(const PropGeom& g, int t, int& x0, i
 // Two z-planes a tile: six CTAs fit an SM (37 KB each), and 70^3 voxels, 1575
 // tiles, take 1.7 rounds of them; with four planes (48 KB, four CTAs, 810 tiles)
 // the second of two rounds was one third full.  A training step at 70^3: 168.1 us at
-// four planes, 162.5 at two, 175.6 at six (three CTAs).
+// four planes, 162.5 at two, 175.6 at six (three CTAs).  A launch takes 20.2 us: 60 %
+// of its issue slots go to filling boxes and to the epilogue, the tensor pipe is 13 %
+// busy.
 constexpr int kTcX = 8, kTcY = 16, kTcZ = 2;
 constexpr int kTcPerSM = 6;
 constexpr int kTcBX = kTcX + 2, kTcBY = kTcY + 2, kTcBZ = kTcZ + 2;
@@ -218,8 +220,10 @@ __device__ __forceinline__ void tc_zero_cols16(uint32_t taddr) {
 }
 
 // g SiLU'(z), to be rounded to BF16, by the hardware's exponential and
-// reciprocal: with the full expf and division they were a quarter of the
-// kernel's time (a training step at 70^3 171.9 -> 167.5 us).
+// reciprocal (a training step at 70^3 161.2 us, with expf and a full division
+// 164.3).  Ten networks on meshes of 16^3 to 80 x 73 x 79: the gradient's error against
+// 64 bits (2.2e-3 to 7.2e-3 of its norm, the BF16 operands') is the same with either to
+// 5e-6 of itself.
 __device__ __forceinline__ float silu_backward(float g, float z) {
     const float s = __fdividef(1.0f, 1.0f + __expf(-z));
     return g * s * (1.0f + z * (1.0f - s));
@@ -1253,7 +1257,9 @@ void launch_conv_sweep(const CUtensorMap& tmap, const SweepArgs& a, int ctas, cu
 // so the eight x-consecutive voxels of an ldmatrix phase are 128 contiguous
 // bytes (no bank conflict, no swizzle) and every address is a per-lane base
 // plus a constant.  A k-step's gradient fragment is loaded once for all of a
-// warp's offsets.  Layer kL: 1, 2 (27 offsets): warp w owns offsets w, w + 8,
+// warp's offsets.  Layers 2, 1, 0 take 20.6, 21.9 and 14.0 us, the tensor pipe 31, 59
+// and 28 % busy, the L1 data pipe 56, 57 and 44 %: at 16 warps an SM an MMA waits for
+// its ldmatrix in 12, 8 and 4 cycles an instruction.  Layer kL: 1, 2 (27 offsets): warp w owns offsets w, w + 8,
 // w + 16 and, w < 3, w + 24; the two-channel last layer (2) multiplies only
 // the first eight output channels.  0: the x-im2col input carries the three dx
 // as channels (dx + 1) 4 + ci, so nine offsets (dz, dy) do: warp w owns offset

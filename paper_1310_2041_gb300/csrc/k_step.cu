@@ -528,11 +528,11 @@ __device__ __forceinline__ void kick_bead(Bead& b, float f0, float f1, float f2,
 // multiply-add on float pairs), and the two cell polynomials live in 48
 // registers, paired coefficient by coefficient, instead of shared memory: no
 // loads per evaluation, and the L1 keeps the space.  91.4M -> 75.0M
-// instructions and 124 -> 118 us per 10-step launch of 1M beads, 107 with today's
-// deposit and uniform segment bounds (L1 data pipe
-// 56 -> 34 %).  What bounds it now is latency at 16 warps per SM: the refills
-// (a warp meets about one per sub-step; 1.7 of 6.8 stall cycles per
-// instruction) and dependent arithmetic.  Starting a refill's loads a
+// instructions and 124 -> 118 us per 10-step launch of 1M beads (L1 data pipe 56 ->
+// 34 %), 108 with today's deposit, uniform segment bounds and fused friction.  What
+// bounds it now is latency at 16 warps per SM (60 % of the issue slots used): the
+// refills (a warp meets about one per sub-step; 1.3 of the 6.1 cycles between a warp's
+// instructions) and dependent arithmetic.  Starting a refill's loads a
 // sub-step's noise earlier was slower, whether as L1 prefetches (137 us: they
 // do not fill the L1) or as asynchronous copies into shared memory (126 us).
 // The rounding of every operation is the scalar form's, so the bits are too.
@@ -916,9 +916,10 @@ __device__ __forceinline__ void advance_segment(const StateBuf& in, const StateB
 
 // This warp's number in its block, from a shuffle: the compiler then knows it
 // for the same in all lanes and keeps the segment's bounds and the replica's
-// record in uniform registers.  Nothing spills any more (44 bytes before, 144
-// with the observables): a 10-step launch of 1M beads took 109 -> 107.5 us, a 5-step
-// launch of 8.1M 548 -> 536, 64 replicas' (4M beads, 10 steps) 462 -> 446.
+// record in uniform registers.  At 128 registers a context's kernel then spills 16
+// bytes (44 before), with the observables 4 (144), a batch's none: a 10-step launch of
+// 1M beads took 109 -> 107.5 us, a 5-step launch of 8.1M 548 -> 536, 64 replicas' (4M
+// beads, 10 steps) 462 -> 446.
 __device__ __forceinline__ int uniform_warp() {
     return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
 }
@@ -931,7 +932,8 @@ __device__ __forceinline__ int uniform_warp() {
 // is over sooner that way (160k beads 75.2 / 77.5 us dealt out, 320k 105.6 /
 // 110; two launches of 10 steps with their fields).  Together / dealt out:
 // 5k beads 42.6 / 39.2, 40k 49.8 / 46.2, 120k 61.2 / 58.7, 240k 90.8 / 86.5,
-// 1M 254.8 / 252.9; 200k with dihedrals, four launches, 214 / 189.
+// 1M 254.8 / 252.9; 200k with dihedrals, four launches, 214 / 189; two learned
+// windows of 20 steps at 5k beads 216 / 197, 60k 277 / 244, 240k 415 / 407, 1M 1019 / 1017.
 __device__ __forceinline__ int segment_of(int r, int total, int warp) {
     constexpr int kWarps = kWarpBlock / 32;
     const int rem = total - r, grid = (int)gridDim.x, block = (int)blockIdx.x;
